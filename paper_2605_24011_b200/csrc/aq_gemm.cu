@@ -179,8 +179,6 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* slab, bool have, int
             for (int i = 0; i < 4; ++i) { dmw[0][i] = 0; dmw[1][i] = 0; }
         }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar_pempty_slot);   // packed bytes are in registers now
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t as = ai % GM_ASTAGES;
@@ -213,7 +211,13 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* slab, bool have, int
         }
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_afull + 8 * as);
+        if (lane == 0) {
+            mbar_arrive(bar_afull + 8 * as);
+            // The packed slot is given back only here: its refill is written through the asynchronous proxy, which may
+            // overtake shared-memory loads that have been issued but not returned.  By now every lane has used what it
+            // loaded, and the fence above stands between those reads and the refill.
+            if (h == 1) mbar_arrive(bar_pempty_slot);
+        }
     }
     return true;
 }
