@@ -7,31 +7,39 @@
 // launch, so the pass runs as one cooperative grid of one CTA per SM:
 //
 //   * Work.  Consecutive ops that read the same input vector form a phase.
-//     Every op's units (16 rows x 256 k) are dealt as contiguous runs to the
-//     CTAs; inside a CTA the runs of a phase are concatenated into one list
-//     and consumer warp w takes positions w, w + 15, w + 30 ... of it, so all
-//     warps of a CTA reach the end of a phase within one unit of each other
-//     and a warp never "switches ops": every unit comes with a descriptor.
-//   * Weight stream.  Which bytes a warp will need does not depend on any
-//     activation, so a 16th warp (lane w serves consumer warp w) keeps every
-//     consumer's private ring of bulk copies (cp.async.bulk + mbarrier, L2
-//     evict-first) full, running ahead across op and phase boundaries, and
-//     writes each unit's descriptor (op, unit index) beside it.
-//   * Sums and dependencies.  A unit's 16 row sums leave the warp as ONE
-//     64-bit red.add each: the sum in 2^-24 fixed point in the upper 52 bits
-//     plus 1 in the lower 12 bits.  A row is complete when its count equals the
-//     number of k-slabs of the matrix, so whoever needs a value polls the value
+//     Every op's units (128 rows x 256 k) are dealt as contiguous runs to the
+//     CTAs.  Inside a CTA five roles pass the units on (aq_decode_tc.cuh has the
+//     arithmetic), so that none waits for another's latency:
+//       - the feeder (one thread) keeps a ring of bulk copies (cp.async.bulk +
+//         mbarrier, L2 evict-first) full;
+//       - eight unpack warps turn codes into tensor-core operands in TMEM, in two
+//         to five stages.  Neither depends on any activation: they run ahead
+//         across op and phase boundaries, so a phase starts with its first units
+//         waiting in TMEM;
+//       - the issuer (one thread) starts a unit's tensor-core instructions;
+//       - eight collect warps form a phase's input, read the units' sums back,
+//         apply scales and minima and add the rows up in memory;
+//       - two record warps write the caller's copies of a phase's input.
+//     Four warps that each did all of this in turn, step after step, needed 1404
+//     us for a 7B-shaped pass of one token (software-pipelined: 1398); the roles
+//     834, the mma.sync kernel before them 1044 (3.4 against 2.7 TB/s).
+//   * Sums and dependencies.  A row's sum over a unit leaves its lane as ONE
+//     64-bit red.add: the sum in 2^-24 fixed point in the upper 52 bits plus 1 in
+//     the lower 12.  A row is complete when its count equals the number of
+//     k-slabs of the matrix, so whoever needs a value polls the value
 //     itself: no arrival counters, no fences, no release, and the result does
 //     not depend on the order of the additions.  A CTA starts a phase as soon
 //     as the elements IT reads are complete, not when the whole op is.
 //   * Glue.  At the start of a phase each CTA forms, in shared memory, the
-//     rounded input vector for the k-slabs its warps will touch (RMS scaling /
-//     SiLU(g)*u / plain) with one round trip to L2, and writes its share of the
-//     float32 buffer and of the rounded vector to the caller's workspace,
-//     where every op's input and output stay readable.  For one token the
-//     vector is stored already spread out as the B operand of the tensor-core
-//     instruction (non-zero only in the column of its block), so a warp picks
-//     its operand up with eight 16-byte loads.
+//     rounded input vector for the k-slabs its units touch (RMS scaling /
+//     SiLU(g)*u / plain) with one round trip to L2.  Its share of the float32
+//     buffer and of the rounded vector goes to the caller's workspace, where
+//     every op's input and output stay readable.
+//
+// What bounds it now (7B shapes, one token): between two boundaries a unit takes
+// 304 ns per SM, HBM's rate is 323; a boundary costs 3.3 us, of which the ring
+// (160 KB per SM, 3.6 us of HBM) hides the weights' part.  With 8 tokens a unit
+// takes 0.8 us (applying block scales to 8 columns and 1024 red.adds per unit).
 //
 // Every wait is bounded: when one runs out the kernel raises a status word,
 // gives copies in flight time to land and returns.
@@ -43,23 +51,45 @@
 #include <mutex>
 #include <vector>
 
-#include "aq_gemv_core.cuh"
+#include "aq_decode_tc.cuh"
 #include "aq_internal.h"
 
 namespace aq {
 
 typedef unsigned long long u64;
 
-constexpr int DS_WARPS = 15;                // consumer warps
-constexpr int DS_CTHREADS = DS_WARPS * 32;  // consumer threads
-constexpr int DS_THREADS = DS_CTHREADS + 32;   // + the copy warp
-constexpr int DS_SLOTS = 5;                 // ring depth per warp (units)
-constexpr int DS_SLOT_BYTES = 2560;         // the largest unit (4-bit: 2 fragments of 1280 B)
-constexpr int DS_MAX_SLOTS = 6;             // staged slabs per phase per CTA (one token; fewer with more tokens)
-constexpr int DS_XS_BYTES = DS_MAX_SLOTS * 4224;   // staged input (see ds_slab_bytes)
+// Warps by role (a warp reaches the TMEM lanes of its quarter only: unpack and collect teams start at multiples of four).
+// At most five warps per scheduler leave 96 registers per thread.
+constexpr int DS_UNPACK_WARPS = 8;          // two teams of four: one per half (128 k) of a unit
+constexpr int DS_COLLECT_WARPS = 8;         // two teams of four, taking units in turn
+constexpr int DS_RECORD_WARPS = 2;
+constexpr int DS_COLLECT0 = DS_UNPACK_WARPS, DS_ISSUER = DS_COLLECT0 + DS_COLLECT_WARPS, DS_FEEDER = DS_ISSUER + 1, DS_RECORD0 = DS_FEEDER + 1;
+constexpr int DS_WARPS = DS_RECORD0 + DS_RECORD_WARPS;
+constexpr int DS_THREADS = DS_WARPS * 32;
+constexpr int DS_CTHREADS = DS_COLLECT_WARPS * 32;
+constexpr int DS_FRAGS = 8;                 // 16-row tiles of a unit
+constexpr int DS_QUEUE = 16;                // units in flight at most
+constexpr int DS_RING_BYTES = 160 * 1024;   // packed units in flight
+constexpr int DS_MAX_SLOTS = 6;             // staged slabs per phase per CTA
+constexpr int DS_XS_BYTES = DS_MAX_SLOTS * dt_slab_bytes(AQ_DECODE_MAX_M);
+// A unit's operands and sums in TMEM: A of both halves, D of both halves.
+template <int MT> struct DsStage {
+    static constexpr int COLS = 2 * (DtShape<MT>::A_COLS + DtShape<MT>::D_COLS);   // 96 / 256
+    static constexpr int N = 512 / COLS;                                           // 5 / 2 stages
+};
+constexpr int DS_MAX_STAGES = 5;
 constexpr int DS_MAX_PHASE_OPS = 8;
 constexpr int DS_RMS_HOLD = 4;              // groups of four elements per thread kept in registers by the one-token RMS path
-constexpr int DS_DESC_BITS_SHIFT = 8;       // descriptor word 0: op inside the phase | code width << 8
+// Several tokens: up to this many elements (M K) every CTA reads the rows whole for the row norms, above it the norms come from
+// shares.  Whole rows cost 8 M K bytes from the same lines of L2, shares one more trip through L2 and a wait for the slowest
+// CTA.  Measured on passes of 18 and 8 blocks: K = 1024, M = 8 500 us whole, 595 us shares; K = 4096, M = 4 (16384) 425
+// against 441; K = 4096, M = 8 (32768) 634 against 588.
+constexpr int64_t DS_WHOLE_ROWS = 16384;
+constexpr int DS_RECS = 4;                  // phase records held in shared memory
+constexpr int DS_DESC_FIRST = 8;            // descriptor word 0: op inside the phase | the op's first k-slab << 3 ...
+constexpr int DS_DESC_BITS_SHIFT = 8;       // ... | code width << 8 ...
+constexpr int DS_DESC_PHASE_SHIFT = 12;     // ... and the phase from bit 12 on
+constexpr uint32_t DS_DESC_END = 0xFFFFFFFFu;   // ... or: the stream is over
 constexpr u64 DS_WAIT_NS_DEFAULT = 2000000000ull;   // every wait gives up after two seconds
 
 // A packed sum: bits [12, 64) hold the value in units of 2^-24 (two's complement), bits [0, 12) the number of
@@ -69,26 +99,16 @@ constexpr u64 DS_CNT_MASK = (1ull << DS_CNT_BITS) - 1;
 constexpr int DS_MAX_CONTRIB = (1 << DS_CNT_BITS) - 1;
 constexpr float DS_FIX_ONE = 16777216.f;            // 2^24
 constexpr float DS_FIX_MAX = 134217600.f;           // just below 2^27: what the 52-bit field holds with room to add
-constexpr int DS_RES_PLAIN = 0x100;
-
-// Shared-memory bytes of one staged slab (256 k): one token is stored spread out
-// as B operands (32 lanes x 8 blocks x 16 B) plus 8 block sums, padded to a multiple of 128 bytes (the readers form
-// addresses with an XOR); several tokens are stored plainly, [token][256] halves.
-__host__ __device__ constexpr int ds_slab_bytes(int M) { return M == 1 ? 4096 + 128 : M * 512; }
 
 __device__ int g_decode_status = 0;   // nonzero: a bounded wait ran out (1 = an input never completed, 2 = a copy)
 
 struct DsOp {
-    const uint8_t* frags;
     u64* dst;              // packed sums [M][N]
     const void* res;       // [M][N] added once (by the k-slab-0 units), or null: packed sums that are complete before the
-                           // phase starts, or plain float32 when bit 8 of `bits` is set (the program input)
+                           // phase starts, or plain float32 when res_plain is set (the program input)
     int32_t N;             // true rows
-    int32_t NT;            // 16-row tiles
-    uint32_t nt_magic;     // floor(2^32 / NT) + 1: u / NT = umulhi(u, magic) or one more (u < 2^26); 0 when NT = 1
-    int32_t bits;          // code width | DS_RES_PLAIN
-    int32_t units_q;       // KP * NT = units_q * (number of CTAs) + units_r
-    int32_t units_r_rot;   // units_r | rot << 16: CTA c takes the run of slot (c + rot) mod (number of CTAs)
+    int32_t res_plain;
+    u64 pad_;
 };
 
 struct DsPhase {
@@ -110,36 +130,27 @@ struct DsPhase {
     u64 pad2_;
     DsOp ops[DS_MAX_PHASE_OPS];
 };
-static_assert(sizeof(DsOp) == 48, "DsOp layout");
+static_assert(sizeof(DsOp) == 32, "DsOp layout");
 static_assert(sizeof(DsPhase) % 16 == 0, "a phase record is fetched with one bulk copy");
 
-// What the copy stream needs to know of an op / a phase, small enough to keep the
-// whole program's worth in shared memory (a cursor then advances in tens of cycles).
-struct DsMiniOp {
+// What the feeder needs to know of an op, in the order of the program.
+struct DsFeedOp {
     const uint8_t* frags;
-    uint32_t q_bits;       // units_q | bits << 28
-    uint32_t r_rot;        // units_r | rot << 16
-    int32_t NT;
-    uint32_t nt_magic;
+    int32_t units_q;       // KP NT8 = units_q * (number of CTAs) + units_r (NT8: 128-row tiles)
+    int32_t units_r_rot;   // units_r | rot << 16: CTA c takes the run of slot (c + rot) mod (number of CTAs)
+    int32_t NT;            // 16-row tiles
+    uint32_t word0;        // descriptor word 0 without the first-slab bit
     int32_t pad_[2];
 };
-struct DsMiniPhase {
-    int32_t op_first;      // index into the mini-op table
-    int32_t op_count;
-    int32_t pad_[2];
-};
-static_assert(sizeof(DsMiniOp) == 32 && sizeof(DsMiniPhase) == 16, "mini tables are copied as 16-byte items");
-constexpr int DS_MINI_BYTES = 10240;
-
+static_assert(sizeof(DsFeedOp) == 32, "DsFeedOp layout");
 // What one CTA needs to know of one phase besides the phase record: worked out on the host, since it depends on
 // nothing but the shapes (a single thread doing this in the kernel sat on every phase's critical path).
 struct DsCtaPhase {
     int32_t total;                          // units of the phase dealt to this CTA
     int32_t n_slots;                        // staged slabs
     int32_t slab_of_slot[DS_MAX_SLOTS];     // the pair-slabs staged for the phase, ascending
-    int32_t xoff[DS_MAX_PHASE_OPS];         // per op: (slot of its first slab) - (that slab): slab P sits in slot xoff + P
 };
-static_assert(sizeof(DsCtaPhase) == 64, "DsCtaPhase layout");
+static_assert(sizeof(DsCtaPhase) == 32, "DsCtaPhase layout");
 
 // A stretch of a buffer no phase reads: converted to float32 for the caller once the last phase is done.
 struct DsTail {
@@ -154,13 +165,14 @@ constexpr int DS_TAIL_CHUNK = 2048;
 
 struct DsArgs {
     const DsPhase* phases;
-    const DsMiniPhase* mini_phases;   // n_phases entries, followed by
-    const DsMiniOp* mini_ops;         // n_mini_ops entries (contiguous: one copy brings both)
+    const DsFeedOp* feed_ops;         // n_ops entries and a spare one
+    const int16_t* xoff;              // [op][CTA]: (slot of the CTA's first slab) - (that slab): slab P is staged in slot xoff + P
+    const int32_t* unit_total;        // [CTA]: its units over all phases
     const DsTail* tails;
     const DsCtaPhase* ctab;           // [phase][CTA]
     u64 wait_ns;
     int n_phases;
-    int n_mini_ops;
+    int n_ops;
     int n_tails;
     int M;
     // the caller's rounded output: the tail chunks that convert [out_src, out_src + out_n) also write it (null: nobody does)
@@ -189,15 +201,6 @@ __device__ __forceinline__ bool ds_mbar_try(uint32_t bar, uint32_t parity) {
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool ds_mbar_test(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ void ds_bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t pol) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
@@ -208,23 +211,32 @@ __device__ __forceinline__ uint64_t ds_now_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait on a shared-memory barrier; false when wait_ns passed.
-__device__ __forceinline__ bool ds_mbar_wait(uint32_t bar, uint32_t parity, u64 wait_ns) {
+// Bounded wait on a shared-memory barrier; false when wait_ns passed (the status is raised) or another role gave up.
+__device__ __forceinline__ bool ds_mbar_wait(uint32_t bar, uint32_t parity, u64 wait_ns, int* abort_flag) {
     if (ds_mbar_try(bar, parity)) return true;
     const uint64_t t0 = ds_now_ns();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
             if (ds_mbar_try(bar, parity)) return true;
-        if (ds_now_ns() - t0 > wait_ns) return false;
+        if (*reinterpret_cast<volatile int*>(abort_flag) != 0) return false;
+        if (ds_now_ns() - t0 > wait_ns) {
+            atomicCAS(&g_decode_status, 0, 2);
+            *reinterpret_cast<volatile int*>(abort_flag) = 1;
+            return false;
+        }
     }
 }
-// Barrier among the consumer warps only (the copy warp never joins).
-__device__ __forceinline__ void ds_consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(DS_CTHREADS) : "memory"); }
-// The same barrier, returning the OR of `flag` over all consumer threads: every thread gets the same answer, so a
+// The same by a whole warp, with one answer for all of it.
+__device__ __forceinline__ bool ds_warp_wait(uint32_t bar, uint32_t parity, u64 wait_ns, int* abort_flag) {
+    return __all_sync(0xffffffffu, ds_mbar_wait(bar, parity, wait_ns, abort_flag));
+}
+// Barrier among the collect warps only.
+__device__ __forceinline__ void ds_collect_sync() { asm volatile("bar.sync 1, %0;" ::"n"(DS_CTHREADS) : "memory"); }
+// The same barrier, returning the OR of `flag` over all collect threads: every thread gets the same answer, so a
 // decision to leave the phase loop is taken by all warps or by none (a flag read after a plain barrier could change
 // between two threads' reads).
-__device__ __forceinline__ bool ds_consumer_sync_or(int flag) {
+__device__ __forceinline__ bool ds_collect_sync_or(int flag) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
@@ -285,52 +297,6 @@ __device__ __forceinline__ bool ds_quad_complete(const u64* p, DsQuad& q, uint32
     return ok;
 }
 
-// ---- the CTA's share of an op --------------------------------------------------------
-// Every op's units are dealt on their own: with n = q G + r units and G CTAs, slot
-// s takes q + 1 units if s < r, else q; CTA c takes slot (c + rot) mod G, where rot
-// moves on from op to op so that the odd units do not always land on the same CTAs.
-__device__ __forceinline__ void ds_cta_run(int q, int r_rot, int& a, int& b) {
-    const int r = r_rot & 0xFFFF, rot = r_rot >> 16;
-    int s = (int)blockIdx.x + rot;
-    if (s >= (int)gridDim.x) s -= (int)gridDim.x;
-    a = q * s + min(s, r);
-    b = a + q + (s < r ? 1 : 0);
-}
-
-// The copy stream's position: consumer w reads positions w, w + DS_WARPS, ... of the list made of the CTA's runs
-// of the phase's ops, one after the other.
-struct DsCursor {
-    int ph, oi;            // phase (n_phases: past the end) and op inside it
-    int pos, base;         // position in the phase's list; position at which op oi's run starts
-    int a, len;            // op oi's run: first unit, number of units
-    const uint8_t* frags;
-    int ub;                // bytes per unit
-    int NT;                // the op's row tiles and the magic number that divides by them
-    uint32_t magic;
-    uint32_t word0;        // op inside the phase | bits << 8, for the unit's descriptor
-};
-__device__ __forceinline__ void ds_cursor_load(DsCursor& c, const DsMiniPhase* mp, const DsMiniOp* mo) {
-    const DsMiniOp op = mo[mp[c.ph].op_first + c.oi];
-    int a, b;
-    ds_cta_run((int)(op.q_bits & 0x0FFFFFFFu), (int)op.r_rot, a, b);
-    c.a = a; c.len = b - a;
-    c.frags = op.frags;
-    c.ub = 2 * frag_bytes((int)(op.q_bits >> 28));
-    c.NT = op.NT; c.magic = op.nt_magic;
-    c.word0 = (uint32_t)c.oi | ((op.q_bits >> 28) << DS_DESC_BITS_SHIFT);
-}
-// Moves (ph, oi, base) on until op oi's run contains pos; a new phase starts again at position `lane`.
-__device__ __forceinline__ void ds_cursor_settle(DsCursor& c, const DsMiniPhase* mp, const DsMiniOp* mo, int n_phases, int lane) {
-    while (c.ph < n_phases && c.pos - c.base >= c.len) {
-        c.base += c.len;
-        if (++c.oi >= mp[c.ph].op_count) {
-            ++c.ph; c.oi = 0; c.base = 0; c.pos = lane;
-            if (c.ph >= n_phases) return;
-        }
-        ds_cursor_load(c, mp, mo);
-    }
-}
-
 // ---- glue arithmetic --------------------------------------------------------------
 __device__ __forceinline__ float ds_silu_mul(float g, float u) { return g / (1.f + expf(-g)) * u; }
 
@@ -352,296 +318,398 @@ __device__ __forceinline__ uint2 ds_round4(const float4& v, float* sum) {
     return r;
 }
 
+// The four values of ds_round4's result.
+template <bool BF16>
+__device__ __forceinline__ float4 ds_values4(const uint2& r) {
+    float2 a, b;
+    if constexpr (BF16) { a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.x)); b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.y)); }
+    else { a = __half22float2(*reinterpret_cast<const __half2*>(&r.x)); b = __half22float2(*reinterpret_cast<const __half2*>(&r.y)); }
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
 // ---- shared memory ------------------------------------------------------------------
 struct DsShared {
-    alignas(128) uint8_t ring[DS_WARPS][DS_SLOTS][DS_SLOT_BYTES];
-    alignas(128) uint8_t xs[DS_XS_BYTES];   // staged input slabs
-    alignas(16) uint8_t mini[DS_MINI_BYTES];   // [DsMiniPhase x n_phases][DsMiniOp x n_mini_ops] when they fit
-    alignas(16) DsPhase rec[2];             // descriptors of the current and the next phase
-    alignas(8) uint64_t full[DS_WARPS][DS_SLOTS];    // copy landed
-    alignas(8) uint64_t empty[DS_WARPS][DS_SLOTS];   // consumer has read the slot
-    alignas(8) uint64_t rec_bar[2];
-    alignas(16) uint4 desc[DS_WARPS][DS_SLOTS];      // the unit in the slot: (op | bits << 8, pair-slab, row tile, -)
-    alignas(16) DsCtaPhase ctab[2];         // this CTA's tables of the current and the next phase
-    float red[AQ_DECODE_MAX_M][DS_WARPS];
-    float scale[AQ_DECODE_MAX_M];
+    alignas(128) uint8_t ring[DS_RING_BYTES];
+    alignas(128) uint8_t zlow[DT_ZERO_BYTES];   // (zeros below and above the slabs: see dt_issue)
+    alignas(128) uint8_t xs[DS_XS_BYTES];       // staged input slabs
+    alignas(128) uint8_t zhigh[DT_ZERO_BYTES];
+    alignas(128) uint8_t dm[DS_MAX_STAGES][2 * DS_FRAGS][SCALE_BYTES];   // the staged units' scales and minima
+    alignas(16) DsPhase rec[DS_RECS];       // phase records, fetched two phases ahead
+    alignas(16) DsCtaPhase ctab[DS_RECS];   // this CTA's tables of the same phases
+    alignas(16) uint4 desc[DS_QUEUE];       // units in the ring: (word 0, byte offset of the staged slab, 128-row tile, offset in the
+                                            // ring | size of half a unit / 256 << 20)
+    alignas(16) uint4 sdesc[DS_MAX_STAGES]; // the same of the units in TMEM
+    alignas(8) uint64_t full[DS_QUEUE];     // the unit's copies have landed
+    alignas(8) uint64_t empty[DS_QUEUE];    // the unpack warps have read it
+    alignas(8) uint64_t stored[DS_MAX_STAGES];   // ... and stored its A operand
+    alignas(8) uint64_t done[DS_MAX_STAGES];     // its tensor-core instructions have completed
+    alignas(8) uint64_t taken[DS_MAX_STAGES];    // its sums have been read
+    alignas(8) uint64_t rec_bar[DS_RECS];
+    uint32_t qsize[DS_QUEUE];               // (the feeder's) ring bytes of the units in flight
+    float red[AQ_DECODE_MAX_M][DS_COLLECT_WARPS];
+    float scale[DS_RECS][AQ_DECODE_MAX_M];  // row scales of the phases (1 / rms)
+    uint32_t tmem;
+    int xphase;                             // phases whose input is staged
+    int recorded[DS_RECORD_WARPS];          // phases whose caller's copies are written
     int abort_flag;
 };
+static_assert(sizeof(DsShared) <= 227 * 1024, "fits an SM");
 
-// Writes 4 rounded elements (k .. k+3 of slab-local index) of the staged vector.
+// One packed red.add per token of the lane's row.  When `res` is given its value (complete, same shape as out) rides along.
 template <int MT>
-__device__ __forceinline__ void ds_store4(uint8_t* slab, int M, int m, int kl, uint2 r) {
-    if constexpr (MT == 1) {
-        const int bk = kl >> 5, t = (kl >> 3) & 3;
-        *reinterpret_cast<uint2*>(slab + ds_spread_offset(bk * 4 + t, bk) + (kl & 7) * 2) = r;
-    } else {
-        *reinterpret_cast<uint2*>(slab + ((size_t)m * 256 + kl) * 2) = r;
-    }
-}
-
-// The x operand of one pair-slab from its staged copy in shared memory.
-template <int MT, bool BF16>
-__device__ __forceinline__ void ds_load_x_operand(XOperand<MT>& xo, const uint8_t* slab, int M, int lane) {
-    if constexpr (MT == 1) {   // (the B registers are read from the slab where they are used)
-        const float2 xs = *reinterpret_cast<const float2*>(slab + 4096 + (lane & 3) * 8);
-        xo.X0[0] = xs.x; xo.X1[0] = xs.y;
-    } else {
-        const uint16_t* x = reinterpret_cast<const uint16_t*>(slab);
-        fill_x_operand<MT, BF16>(xo, lane, [&](int tok, int kk) {
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (tok < M) v = *reinterpret_cast<const uint4*>(x + tok * 256 + kk);
-            return v;
-        });
-    }
-}
-
-// Cross-lane reduction of a unit's partial sums and one packed red.add per (token, row).  When `res` is given its
-// value (complete, same shape as out) rides along.  Free of branches when res is null (bounds are predicates), so
-// that the compiler can weave it into the next unit's arithmetic.
-__device__ __forceinline__ void ds_red_add_if(u64* p, u64 v, bool on) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %2, 0;\n\t"
-        "@p red.relaxed.gpu.global.add.u64 [%0], %1;\n\t}"
-        ::"l"(p), "l"(v), "r"((uint32_t)on) : "memory");
-}
-template <int MT>
-__device__ __forceinline__ void ds_unit_commit(const float (&acc)[4], u64* out, const void* res, bool res_plain, int64_t ld, int row0,
-                                               int N, int M, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    auto put = [&](int tok, int row, float v, bool lane_on) {
-        const bool on = lane_on && tok < M && row < N;
-        const int64_t o = (int64_t)tok * ld + row;
-        u64 w = ds_pack(v);
-        if (res != nullptr && on) {
+__device__ __forceinline__ void ds_commit(const float (&acc)[MT], u64* out, const void* res, bool res_plain, int row, int N, int M) {
+    if (row >= N) return;
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+        if (m >= M) break;
+        const int64_t o = (int64_t)m * N + row;
+        u64 w = ds_pack(acc[m]);
+        if (res != nullptr) {
             if (res_plain) w += ds_pack(__ldcg(reinterpret_cast<const float*>(res) + o)) - 1ull;
             else w += ds_ld1(reinterpret_cast<const u64*>(res) + o) & ~DS_CNT_MASK;
         }
-        ds_red_add_if(out + o, w, on);
-    };
-    if constexpr (MT == 1) {
-        const float v0 = acc[0] + acc[1], v1 = acc[2] + acc[3];
-        float keep = (t & 1) ? v1 : v0;
-        const float send = (t & 1) ? v0 : v1;
-        keep += __shfl_xor_sync(0xffffffffu, send, 1);
-        keep += __shfl_xor_sync(0xffffffffu, keep, 2);
-        put(0, row0 + g + 8 * (t & 1), keep, t < 2);
-    } else if constexpr (MT == 2) {
-        float kA = (t & 1) ? acc[1] : acc[0], kB = (t & 1) ? acc[3] : acc[2];
-        const float sA = (t & 1) ? acc[0] : acc[1], sB = (t & 1) ? acc[2] : acc[3];
-        kA += __shfl_xor_sync(0xffffffffu, sA, 1);
-        kB += __shfl_xor_sync(0xffffffffu, sB, 1);
-        float v = (t & 2) ? kB : kA;
-        const float s = (t & 2) ? kA : kB;
-        v += __shfl_xor_sync(0xffffffffu, s, 2);
-        put(t & 1, row0 + g + 8 * (t >> 1), v, true);
-    } else if constexpr (MT == 4) {
-        float c[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) c[i] = acc[i] + __shfl_xor_sync(0xffffffffu, acc[i], 2);
-        const int tk = 2 * (t & 1);
-        const int hi = t >> 1;
-        put(tk, row0 + g + 8 * hi, hi ? c[2] : c[0], true);
-        put(tk + 1, row0 + g + 8 * hi, hi ? c[3] : c[1], true);
-    } else {
-        const int tk = 2 * t;
-        put(tk, row0 + g, acc[0], true); put(tk, row0 + g + 8, acc[2], true);
-        put(tk + 1, row0 + g, acc[1], true); put(tk + 1, row0 + g + 8, acc[3], true);
+        ds_red_add(out + o, w);
     }
 }
 
-// A unit whose sums have not left the warp yet: they do at the start of the next unit's arithmetic, where the
-// shuffles, the conversion and the red.add hide behind tensor-core work instead of standing between two units.
-struct DsPending {
-    float acc[4];
-    u64* out;
-    int row0, N;
-    bool on;
-};
-template <int MT>
-__device__ __forceinline__ void ds_flush(DsPending& pd, int M, int lane) {
-    if (pd.on) ds_unit_commit<MT>(pd.acc, pd.out, nullptr, false, pd.N, pd.row0, pd.N, M, lane);   // (pd.on is the same in every lane)
-    pd.on = false;
+// ---- the roles ------------------------------------------------------------------------
+// The CTA's units [a, b) of an op: slot s takes q + 1 units if s < r, else q.
+__device__ __forceinline__ void ds_cta_run(int q, int r_rot, int& a, int& b) {
+    const int r = r_rot & 0xFFFF, rot = r_rot >> 16;
+    int s = (int)blockIdx.x + rot;
+    if (s >= (int)gridDim.x) s -= (int)gridDim.x;
+    a = q * s + min(s, r);
+    b = a + q + (s < r ? 1 : 0);
 }
 
-// One unit: the previous unit's commit, then this unit's multiply-accumulate.
-template <int BITS, int MT, bool BF16>
-__device__ __forceinline__ void ds_unit_body(const uint8_t* unit, const uint8_t* xseg, XOperand<MT>& xo, DsPending& pd, int M, int lane,
-                                             float (&acc)[4]) {
-    ds_load_x_operand<MT, BF16>(xo, xseg, M, lane);
-    const uint32_t xlane = ds_spread_lane_base(xseg, lane);
-    ds_flush<MT>(pd, M, lane);
-    unit_mac<BITS, MT, BF16, MT == 1>(unit, xo, lane, acc, xlane);
+// The feeder (one thread): every unit of the CTA, op by op, into the ring as soon as there is room.
+__device__ __forceinline__ void ds_feed(DsShared& sh, const DsArgs& a) {
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    uint32_t head = 0, room = DS_RING_BYTES;   // next byte of the ring, free bytes
+    uint32_t nq = 0, tail = 0;                 // units copied, units known to have been read
+    auto wait_tail = [&]() -> bool {
+        const uint32_t e = tail % DS_QUEUE;
+        if (!ds_mbar_wait(ds_smem(&sh.empty[e]), (tail / DS_QUEUE) & 1u, 2 * a.wait_ns, &sh.abort_flag)) return false;
+        room += sh.qsize[e];
+        ++tail;
+        return true;
+    };
+    DsFeedOp next = a.feed_ops[0];             // (one op ahead: the latency hides behind an op's copies)
+    int next_off = a.xoff[blockIdx.x];
+    for (int o = 0; o < a.n_ops; ++o) {
+        const DsFeedOp run = next;
+        const int slab = next_off * dt_slab_bytes(a.M);
+        next = a.feed_ops[o + 1];
+        next_off = a.xoff[(size_t)(o + 1) * gridDim.x + blockIdx.x];
+        int u0, u1;
+        ds_cta_run(run.units_q, run.units_r_rot, u0, u1);
+        const int fb = frag_bytes((int)(run.word0 >> DS_DESC_BITS_SHIFT) & 7), NT8 = (run.NT + DS_FRAGS - 1) / DS_FRAGS;
+        int P = u0 / NT8, R = u0 - P * NT8;
+        for (int u = u0; u < u1; ++u) {
+            const uint32_t half = (uint32_t)(min(DS_FRAGS, run.NT - R * DS_FRAGS) * fb), need = 2 * half;
+            const bool wrap = head + need > DS_RING_BYTES;             // (a unit lies in one piece)
+            const uint32_t pad = wrap ? DS_RING_BYTES - head : 0u;
+            while (room < need + pad || nq - tail == DS_QUEUE)
+                if (!wait_tail()) return;
+            if (wrap) head = 0;
+            const uint32_t e = nq % DS_QUEUE, bar = ds_smem(&sh.full[e]);
+            sh.qsize[e] = need + pad;
+            // (ordered before the copies' arrival by the release of expect_tx)
+            sh.desc[e] = make_uint4(run.word0 | (P == 0 ? (uint32_t)DS_DESC_FIRST : 0u), (uint32_t)(slab + P * dt_slab_bytes(a.M)), (uint32_t)R,
+                                    head | ((half >> 8) << 20));
+            ds_expect_tx(bar, need);
+            const uint8_t* src = run.frags + frag_index(2 * P, R * DS_FRAGS, run.NT) * fb;
+            ds_bulk_load(ds_smem(sh.ring) + head, src, half, bar, pol);
+            ds_bulk_load(ds_smem(sh.ring) + head + half, src + (int64_t)run.NT * fb, half, bar, pol);
+            room -= need + pad;
+            head += need;
+            ++nq;
+            if (++R == NT8) { R = 0; ++P; }
+        }
+    }
+    while (nq - tail >= DS_QUEUE)
+        if (!wait_tail()) return;
+    sh.desc[nq % DS_QUEUE] = make_uint4(DS_DESC_END, 0u, 0u, 0u);
+    ds_mbar_arrive(ds_smem(&sh.full[nq % DS_QUEUE]));
+}
+
+// An unpack warp: its two fragments (rows 32 quarter .. + 31) of half `half` of every unit.
+template <int MT, bool BF16>
+__device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint32_t tmem, int half, int quarter, int lane) {
+    using ST = DsStage<MT>;
+    using SH = DtShape<MT>;
+    uint32_t stage = 0, use = 0;   // TMEM stage and how often the stages have gone round
+    for (uint32_t n = 0;; ++n) {
+        const uint32_t e = n % DS_QUEUE;
+        if (!ds_warp_wait(ds_smem(&sh.full[e]), (n / DS_QUEUE) & 1u, wait_ns, &sh.abort_flag)) return;
+        const uint4 d = sh.desc[e];
+        if (d.x == DS_DESC_END) return;
+        const int bits = (int)(d.x >> DS_DESC_BITS_SHIFT) & 7, fb = frag_bytes(bits);
+        // (row tiles past the matrix's last one: whatever lies there; their rows are not written)
+        const uint8_t* fr = sh.ring + (d.w & 0xFFFFFu) + (half ? (d.w >> 20) << 8 : 0u) + (uint32_t)(quarter * 2 * fb);
+        const uint4 dm = *reinterpret_cast<const uint4*>(fr + (lane >> 4) * fb + (lane & 15) * 16);
+        const uint32_t ta = tmem + stage * ST::COLS + (uint32_t)(half * SH::A_COLS) + ((uint32_t)(quarter * 32) << 16);
+        // the stage is free once its last unit's sums have been read
+        auto stage_free = [&]() { return use == 0 || ds_warp_wait(ds_smem(&sh.taken[stage]), (use - 1) & 1u, wait_ns, &sh.abort_flag); };
+        if constexpr (MT == 1) {
+            uint32_t va[16], vb[16];
+            if (bits == 2) dt_unpack2<2>(fr, lane, va, vb);
+            else if (bits == 3) dt_unpack2<3>(fr, lane, va, vb);
+            else dt_unpack2<4>(fr, lane, va, vb);
+            if (!stage_free()) return;
+            tc_fence_after();
+            tmem_st_16x128(ta, va);
+            tmem_st_16x128(ta + (16u << 16), vb);
+        } else {
+            uint32_t v[32];
+            auto unpack = [&](const uint8_t* f) {
+                if (bits == 2) dt_unpack1<2, BF16>(f, lane, v);
+                else if (bits == 3) dt_unpack1<3, BF16>(f, lane, v);
+                else dt_unpack1<4, BF16>(f, lane, v);
+            };
+            unpack(fr);
+            if (!stage_free()) return;
+            tc_fence_after();
+            tmem_st_16x128(ta, v);
+            unpack(fr + fb);
+            tmem_st_16x128(ta + (16u << 16), v);
+        }
+        *reinterpret_cast<uint4*>(&sh.dm[stage][half * DS_FRAGS + quarter * 2 + (lane >> 4)][(lane & 15) * 16]) = dm;
+        if (half == 0 && quarter == 0 && lane == 0) sh.sdesc[stage] = d;
+        tmem_st_wait();          // (everything read from the ring has been used: the slot may be refilled)
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+            ds_mbar_arrive(ds_smem(&sh.empty[e]));
+            ds_mbar_arrive(ds_smem(&sh.stored[stage]));
+        }
+        if (++stage == ST::N) { stage = 0; ++use; }
+    }
+}
+
+// Waits until *count exceeds `value`; returns the count (not above `value`: gave up).  One answer for the whole warp.
+__device__ __forceinline__ int ds_wait_count(const int* count, int value, u64 wait_ns, int* abort_flag) {
+    const uint32_t addr = ds_smem(count);
+    const uint64_t t0 = ds_now_ns();
+    for (;;) {
+        int v = 0;
+#pragma unroll 1
+        for (int i = 0; i < 256; ++i) {
+            asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+            v = __shfl_sync(0xffffffffu, v, 0);
+            if (v > value) return v;
+        }
+        const bool stop = *reinterpret_cast<volatile int*>(abort_flag) != 0 || ds_now_ns() - t0 > wait_ns;
+        if (__any_sync(0xffffffffu, stop)) {
+            if (*reinterpret_cast<volatile int*>(abort_flag) == 0) { atomicCAS(&g_decode_status, 0, 2); *reinterpret_cast<volatile int*>(abort_flag) = 1; }
+            return v;
+        }
+    }
+}
+
+// The issuer (one warp, one elected thread): a unit's instructions once its A operand and the phase's input are there.
+template <int MT, bool BF16>
+__device__ __forceinline__ void ds_issue_units(DsShared& sh, const DsArgs& a, uint32_t tmem) {
+    using ST = DsStage<MT>;
+    uint32_t stage = 0, use = 0;
+    int ready = 0;   // phases whose input is staged
+    const uint32_t zlow = ds_smem(sh.zlow), zhigh = ds_smem(sh.zhigh), xs = ds_smem(sh.xs);
+    for (int left = a.unit_total[blockIdx.x]; left > 0; --left) {
+        if (!ds_warp_wait(ds_smem(&sh.stored[stage]), use & 1u, 2 * a.wait_ns, &sh.abort_flag)) return;
+        const uint2 d = *reinterpret_cast<const uint2*>(&sh.sdesc[stage]);
+        const int ph = (int)(d.x >> DS_DESC_PHASE_SHIFT);
+        if (ready <= ph) {
+            ready = ds_wait_count(&sh.xphase, ph, 2 * a.wait_ns, &sh.abort_flag);
+            if (ready <= ph) return;
+        }
+        const uint32_t x = __shfl_sync(0xffffffffu, xs + d.y, 0);
+        const uint32_t t0 = __shfl_sync(0xffffffffu, tmem + stage * ST::COLS, 0);
+        tc_fence_after();
+        if (elect_one()) {
+            dt_issue<MT, BF16>(t0, t0 + 2 * DtShape<MT>::A_COLS, x, zlow, zhigh);
+            umma_commit(ds_smem(&sh.done[stage]));
+        }
+        __syncwarp();
+        if (++stage == ST::N) { stage = 0; ++use; }
+    }
+}
+
+// How the waits for other CTAs' sums end: a counter of rounds, the time of the first late one.
+struct DsPatience {
+    uint32_t spins = 0;
+    uint64_t t0 = 0;
+    // after a round of readings that found something incomplete: true when the wait has to end
+    __device__ __forceinline__ bool over(DsShared& sh, u64 wait_ns) {
+        if ((++spins & 7u) != 0) return false;
+        if (*reinterpret_cast<volatile int*>(&g_decode_status) != 0) { sh.abort_flag = 1; return true; }
+        const uint64_t t = ds_now_ns();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > wait_ns) { atomicCAS(&g_decode_status, 0, 1); sh.abort_flag = 1; return true; }
+        return false;
+    }
+};
+// Four consecutive source elements at offset o, complete; zeros after a failed wait.
+__device__ __forceinline__ float4 ds_source4(DsShared& sh, const u64* p, const float* pf, uint32_t expect, int64_t o, u64 wait_ns, DsPatience& pat) {
+    if (p == nullptr) return __ldcg(reinterpret_cast<const float4*>(pf + o));
+    DsQuad q;
+    for (;;) {
+        ds_ld_quad(p + o, q);
+        if (ds_quad_ready(q, expect)) return ds_quad_value(q);
+        if (pat.over(sh, wait_ns)) return make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// A record warp: this CTA's share of the caller's copies (the float32 source buffers and the rounded input of every
+// phase), written while the phase's units are at work.
+template <bool BF16>
+__device__ __forceinline__ void ds_record(DsShared& sh, const DsArgs& a, int rw, int lane) {
+    for (int ph = 0; ph < a.n_phases; ++ph) {
+        const int pb = ph % DS_RECS;
+        if (!ds_warp_wait(ds_smem(&sh.rec_bar[pb]), (uint32_t)(ph / DS_RECS) & 1u, 2 * a.wait_ns, &sh.abort_flag)) return;
+        if (ds_wait_count(&sh.xphase, ph, 2 * a.wait_ns, &sh.abort_flag) <= ph) return;   // (the row scales are there then)
+        const DsPhase& P = sh.rec[pb];
+        const int q4 = P.K >> 2;                                  // groups of 4 elements per token
+        const int g0 = (int)(((int64_t)q4 * blockIdx.x) / gridDim.x), share = (int)(((int64_t)q4 * (blockIdx.x + 1)) / gridDim.x) - g0;
+        const bool two = (P.in_op == AQ_IN_SILU_MUL);
+        DsPatience pat;
+        for (int it = rw * 32 + lane; it < share * a.M; it += DS_RECORD_WARPS * 32) {
+            const int m = it / share;
+            const int64_t o = (int64_t)m * P.K + 4 * (int64_t)(g0 + it - m * share);
+            float4 v = ds_source4(sh, P.src, P.src_f, P.expect, o, a.wait_ns, pat);
+            if (P.rec) *reinterpret_cast<float4*>(P.rec + o) = v;
+            if (two) {
+                const float4 t = ds_source4(sh, P.src2, P.src2_f, P.expect2, o, a.wait_ns, pat);
+                if (P.rec2) *reinterpret_cast<float4*>(P.rec2 + o) = t;
+                v = make_float4(ds_silu_mul(v.x, t.x), ds_silu_mul(v.y, t.y), ds_silu_mul(v.z, t.z), ds_silu_mul(v.w, t.w));
+            } else {
+                const float sc = (P.in_op == AQ_IN_RMSNORM) ? sh.scale[pb][m] : 1.f;
+                v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+            }
+            float sum;
+            *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(P.stage) + o) = ds_round4<BF16>(v, &sum);
+        }
+        __syncwarp();
+        if (lane == 0) asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(ds_smem(&sh.recorded[rw])), "r"(ph + 1) : "memory");
+    }
 }
 
 // ---- the kernel ---------------------------------------------------------------------
 template <int MT, bool BF16>
 __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArgs a) {
+    using ST = DsStage<MT>;
     extern __shared__ __align__(128) uint8_t ds_smem_raw[];
     DsShared& sh = *reinterpret_cast<DsShared*>(ds_smem_raw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int quarter = warp & 3;   // (a warp reaches the TMEM lanes of its quarter only)
     const int M = a.M;
-    const int slab_bytes = ds_slab_bytes(M);
     const u64 wait_ns = a.wait_ns;
 
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
-        ds_mbar_init(ds_smem(&sh.rec_bar[0]), 1);
-        ds_mbar_init(ds_smem(&sh.rec_bar[1]), 1);
-    }
-    if (warp < DS_WARPS && lane == 0) {
+        sh.xphase = 0;
 #pragma unroll
-        for (int s = 0; s < DS_SLOTS; ++s) {
-            ds_mbar_init(ds_smem(&sh.full[warp][s]), 1);
-            ds_mbar_init(ds_smem(&sh.empty[warp][s]), 1);
+        for (int i = 0; i < DS_RECORD_WARPS; ++i) sh.recorded[i] = 0;
+#pragma unroll 1
+        for (int i = 0; i < DS_RECS; ++i) ds_mbar_init(ds_smem(&sh.rec_bar[i]), 1);
+#pragma unroll 1
+        for (int i = 0; i < DS_QUEUE; ++i) {
+            ds_mbar_init(ds_smem(&sh.full[i]), 1);
+            ds_mbar_init(ds_smem(&sh.empty[i]), DS_UNPACK_WARPS);
+        }
+#pragma unroll 1
+        for (int i = 0; i < DS_MAX_STAGES; ++i) {
+            ds_mbar_init(ds_smem(&sh.stored[i]), DS_UNPACK_WARPS);
+            ds_mbar_init(ds_smem(&sh.done[i]), 1);
+            ds_mbar_init(ds_smem(&sh.taken[i]), 4);
         }
     }
-    // one-token slabs keep zeros everywhere but in the chunks the stagers rewrite every phase
-    for (int i = threadIdx.x; i < DS_XS_BYTES / 16; i += (int)blockDim.x)
-        reinterpret_cast<uint4*>(sh.xs)[i] = make_uint4(0, 0, 0, 0);
-    // the copy stream's tables: into shared memory when they fit
-    const int mini_items = a.n_phases + 2 * a.n_mini_ops;   // in 16-byte pieces
-    const bool mini_in_smem = mini_items * 16 <= DS_MINI_BYTES;
-    if (mini_in_smem)
-        for (int i = threadIdx.x; i < mini_items; i += (int)blockDim.x)
-            reinterpret_cast<uint4*>(sh.mini)[i] = __ldg(reinterpret_cast<const uint4*>(a.mini_phases) + i);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ds_smem(&sh.tmem)), "n"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // the slabs keep zeros everywhere but in the elements the stagers rewrite every phase (rows of absent tokens; one
+    // token: every row but the first)
+    for (int i = threadIdx.x; i < (DS_XS_BYTES + 2 * DT_ZERO_BYTES) / 16; i += DS_THREADS)
+        reinterpret_cast<uint4*>(sh.zlow)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+    tc_fence_before();
     __syncthreads();
-    const DsMiniPhase* mp = mini_in_smem ? reinterpret_cast<const DsMiniPhase*>(sh.mini) : a.mini_phases;
-    const DsMiniOp* mo = mini_in_smem ? reinterpret_cast<const DsMiniOp*>(sh.mini + (size_t)a.n_phases * 16) : a.mini_ops;
+    tc_fence_after();
+    const uint32_t tmem = sh.tmem;
 
-    uint64_t pol, pol_keep;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
-
-    if (warp == DS_WARPS) {
-        // ================= the copy warp: lane w keeps consumer warp w's ring full =================
-        DsCursor c;
-        c.ph = a.n_phases; c.oi = 0; c.pos = 0; c.base = 0; c.a = 0; c.len = 0; c.frags = nullptr; c.ub = 0;
-        c.NT = 1; c.magic = 0; c.word0 = 0;
-        if (lane < DS_WARPS && a.n_phases > 0) {
-            c.ph = 0; c.pos = lane;
-            ds_cursor_load(c, mp, mo);
-            ds_cursor_settle(c, mp, mo, a.n_phases, lane);
-        }
-        uint32_t iseq = 0;   // copies issued for this consumer
-        uint64_t t_progress = ds_now_ns();
-        uint32_t idle = 0;
-        for (;;) {
-            const bool active = c.ph < a.n_phases;
-            bool moved = false;
-            if (active) {
-                // the n-th copy into a slot (n >= 1) waits for the consumer's arrival after its (n-1)-th read
-                const uint32_t slot = iseq % DS_SLOTS, n = iseq / DS_SLOTS;
-                const bool is_free = (n == 0) || ds_mbar_test(ds_smem(&sh.empty[lane][slot]), (n - 1) & 1u);
-                if (is_free) {
-                    const uint32_t u = (uint32_t)(c.a + (c.pos - c.base));
-                    int Pk = c.magic ? (int)__umulhi(u, c.magic) : (int)u;   // u / NT (no magic: NT = 1)
-                    int R = (int)u - Pk * c.NT;
-                    if (R < 0) { --Pk; R += c.NT; }
-                    // (ordered before the copy's arrival by the release of expect_tx)
-                    sh.desc[lane][slot] = make_uint4(c.word0, (uint32_t)Pk, (uint32_t)R, 0u);
-                    const uint32_t bar = ds_smem(&sh.full[lane][slot]);
-                    ds_expect_tx(bar, (uint32_t)c.ub);
-                    ds_bulk_load(ds_smem(&sh.ring[lane][slot][0]), c.frags + (int64_t)u * c.ub, (uint32_t)c.ub, bar, pol);
-                    ++iseq;
-                    c.pos += DS_WARPS;
-                    ds_cursor_settle(c, mp, mo, a.n_phases, lane);
-                    moved = true;
-                }
-            }
-            if (!__any_sync(0xffffffffu, active)) break;
-            if (__any_sync(0xffffffffu, moved)) { idle = 0; continue; }
-            __nanosleep(200);   // a consumer needs about half a microsecond per unit: no need to spin on its barriers
-            if ((++idle & 255u) == 0) {   // nothing to do for a while: stop if the CTA gave up, or after the time limit
-                if (*reinterpret_cast<volatile int*>(&sh.abort_flag)) break;
-                const uint64_t t = ds_now_ns();
-                if (idle == 256u) t_progress = t;
-                else if (t - t_progress > 2 * wait_ns) { atomicCAS(&g_decode_status, 0, 2); sh.abort_flag = 1; break; }
-            }
-        }
-        return;
-    }
-
-    // ================= consumer warps =================
+    if (warp < DS_UNPACK_WARPS) {
+        ds_unpack_units<MT, BF16>(sh, wait_ns, tmem, warp >> 2, quarter, lane);
+    } else if (warp == DS_ISSUER) {
+        ds_issue_units<MT, BF16>(sh, a, tmem);
+    } else if (warp == DS_FEEDER) {
+        if (lane == 0) ds_feed(sh, a);
+        __syncwarp();
+    } else if (warp >= DS_RECORD0) {
+        ds_record<BF16>(sh, a, warp - DS_RECORD0, lane);
+    } else {
+    // ================= collect warps =================
+    const int ctid = (int)threadIdx.x - DS_COLLECT0 * 32, cwarp = warp - DS_COLLECT0;
     auto fetch_record = [&](int q) {   // the phase's record and this CTA's tables for it, on one barrier
-        const uint32_t bar = ds_smem(&sh.rec_bar[q & 1]);
+        const uint32_t bar = ds_smem(&sh.rec_bar[q % DS_RECS]);
+        uint64_t pol_keep;
+        asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
         ds_expect_tx(bar, (uint32_t)(sizeof(DsPhase) + sizeof(DsCtaPhase)));
-        ds_bulk_load(ds_smem(&sh.rec[q & 1]), a.phases + q, (uint32_t)sizeof(DsPhase), bar, pol_keep);
-        ds_bulk_load(ds_smem(&sh.ctab[q & 1]), a.ctab + (size_t)q * gridDim.x + blockIdx.x, (uint32_t)sizeof(DsCtaPhase), bar, pol_keep);
+        ds_bulk_load(ds_smem(&sh.rec[q % DS_RECS]), a.phases + q, (uint32_t)sizeof(DsPhase), bar, pol_keep);
+        ds_bulk_load(ds_smem(&sh.ctab[q % DS_RECS]), a.ctab + (size_t)q * gridDim.x + blockIdx.x, (uint32_t)sizeof(DsCtaPhase), bar, pol_keep);
     };
-    if (threadIdx.x == 0) {
+    if (ctid == 0) {
         if (a.n_phases > 0) fetch_record(0);
         if (a.n_phases > 1) fetch_record(1);
     }
-
-    uint32_t cslot = 0, cparity = 0;   // next ring slot to consume and the parity of its `full` barrier
-    bool dead = false;                 // this warp gave up on a wait
-    XOperand<MT> xo;
-    DsPending pd;
-    pd.on = false; pd.out = nullptr; pd.row0 = 0; pd.N = 0;
-    pd.acc[0] = pd.acc[1] = pd.acc[2] = pd.acc[3] = 0.f;
+    uint32_t stage = 0, use = 0;       // TMEM stage of the next unit, and how often the stages have gone round
+    uint32_t turn = 0;                 // the team whose unit that is
 
 #pragma unroll 1
     for (int ph = 0; ph < a.n_phases; ++ph) {
-        const int pb = ph & 1;
+        const int pb = ph % DS_RECS;
         const DsPhase& P = sh.rec[pb];
         const DsCtaPhase& C = sh.ctab[pb];
-        // -- the phase's descriptors (fetched one phase ahead) --
-        if (!ds_mbar_wait(ds_smem(&sh.rec_bar[pb]), (uint32_t)(ph >> 1) & 1u, wait_ns)) {
-            atomicCAS(&g_decode_status, 0, 2);
-            sh.abort_flag = 1;
+        // -- the phase's descriptors (fetched two phases ahead) --
+        ds_mbar_wait(ds_smem(&sh.rec_bar[pb]), (uint32_t)(ph / DS_RECS) & 1u, wait_ns, &sh.abort_flag);
+        if (cwarp == 0 && ph + 2 < a.n_phases) {   // slot of phase ph - 2: the collect warps are through with it, and the record warps?
+#pragma unroll
+            for (int i = 0; i < DS_RECORD_WARPS; ++i)
+                if (ph >= 2) ds_wait_count(&sh.recorded[i], ph - 2, wait_ns, &sh.abort_flag);
+            if (lane == 0) fetch_record(ph + 2);
         }
-        // every warp is through with phase ph - 1: the staged slabs and its record slot are free
-        if (ds_consumer_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
-        if (threadIdx.x == 0 && ph >= 1 && ph + 1 < a.n_phases) fetch_record(ph + 1);
+        // every warp is through with phase ph - 1: the staged slabs are free
+        if (ds_collect_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
 
-        // -- form the rounded input vector: slabs this CTA reads -> shared memory, its share -> workspace --
+        // -- form the rounded input vector for the slabs this CTA reads --
         {
             const int n_slots = C.n_slots;
             const int q4 = P.K >> 2;                                  // groups of 4 elements per token
-            const int g0 = (int)(((int64_t)q4 * blockIdx.x) / gridDim.x), g1 = (int)(((int64_t)q4 * (blockIdx.x + 1)) / gridDim.x);
-            uint16_t* stage_out = reinterpret_cast<uint16_t*>(P.stage);
             const uint32_t expect = P.expect, expect2 = P.expect2;
-            uint32_t spins = 0;
-            uint64_t t_wait0 = 0;
-            // after a round of readings that found something incomplete: true when the wait has to end
-            auto give_up = [&]() -> bool {
-                if ((++spins & 7u) != 0) return false;
-                if (*reinterpret_cast<volatile int*>(&g_decode_status) != 0) { sh.abort_flag = 1; return true; }
-                const uint64_t t = ds_now_ns();
-                if (t_wait0 == 0) t_wait0 = t;
-                if (t - t_wait0 > wait_ns) { atomicCAS(&g_decode_status, 0, 1); sh.abort_flag = 1; return true; }
-                return false;
-            };
-            // four consecutive source elements (group i4 of token m), complete; zeros after a failed wait
-            auto source4 = [&](const u64* p, const float* pf, uint32_t ex, int m, int i4) -> float4 {
-                const int64_t o = (int64_t)m * P.K + 4 * (int64_t)i4;
-                if (p == nullptr) return __ldcg(reinterpret_cast<const float4*>(pf + o));
-                DsQuad q;
-                for (;;) {
-                    ds_ld_quad(p + o, q);
-                    if (ds_quad_ready(q, ex)) return ds_quad_value(q);
-                    if (give_up()) return make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            };
+            DsPatience pat;
             // stores group i4 (elements 4 i4 ..) of token m into slab copy `sl`; whole warps call this together
-            auto place = [&](uint8_t* sl, int m, int i4, float4 v, bool rec) {
+            auto place = [&](uint8_t* sl, int m, int i4, float4 v) {
                 float sum;
                 const uint2 r = ds_round4<BF16>(v, &sum);   // v is zero past the end of the row: padding stages zeros
-                if constexpr (MT == 1) {   // block sums: 8 consecutive groups = 8 consecutive lanes
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-                }
                 const int kl = (i4 * 4) & 255;
-                if (sl) {
-                    ds_store4<MT>(sl, M, m, kl, r);
-                    if constexpr (MT == 1) {
-                        if ((lane & 7) == 0) *reinterpret_cast<float*>(sl + 4096 + (kl >> 5) * 4) = sum;
-                    }
+                // block sums (and, for one token, the largest magnitude): 8 consecutive groups = 8 consecutive lanes
+                sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+                if constexpr (MT == 1) {
+                    const float4 f = ds_values4<BF16>(r);
+                    float mx = fmaxf(fmaxf(fabsf(f.x), fabsf(f.y)), fmaxf(fabsf(f.z), fabsf(f.w)));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                    const uint32_t sc = dt_fix_scale(mx);
+                    dt_stage4_fix(sl, kl, f, sc);
+                    if ((lane & 7) == 0) reinterpret_cast<float2*>(sl + DT_SUMS<1>)[kl >> 5] = make_float2(sum, dt_fix_step(sc));
+                } else {
+                    dt_stage4(sl, m, kl, r);
+                    if ((lane & 7) == 0) reinterpret_cast<float*>(sl + DT_SUMS<MT>)[(kl >> 5) * 8 + m] = sum;
                 }
-                if (rec) *reinterpret_cast<uint2*>(stage_out + (int64_t)m * P.K + i4 * 4) = r;
             };
             if (P.in_op == AQ_IN_RMSNORM && MT == 1 && q4 <= DS_RMS_HOLD * DS_CTHREADS) {
                 // one token, row held in registers: one trip to L2 once the row is complete (all of a thread's readings
@@ -656,26 +724,26 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                         bool ready = true;
 #pragma unroll
                         for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                            const int i4 = threadIdx.x + n * DS_CTHREADS;
+                            const int i4 = ctid + n * DS_CTHREADS;
                             if (i4 < q4) ds_ld_quad(P.src + 4 * (int64_t)i4, q[n]);
                         }
 #pragma unroll
                         for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                            const int i4 = threadIdx.x + n * DS_CTHREADS;
+                            const int i4 = ctid + n * DS_CTHREADS;
                             if (i4 < q4) ready = ready && ds_quad_ready(q[n], expect);
                         }
-                        if (ready || give_up()) break;
+                        if (ready || pat.over(sh, wait_ns)) break;
                     }
                     const bool failed = *reinterpret_cast<volatile int*>(&sh.abort_flag) != 0;
 #pragma unroll
                     for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                        const int i4 = threadIdx.x + n * DS_CTHREADS;
+                        const int i4 = ctid + n * DS_CTHREADS;
                         v[n] = (i4 < q4 && !failed) ? ds_quad_value(q[n]) : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 } else {
 #pragma unroll
                     for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                        const int i4 = threadIdx.x + n * DS_CTHREADS;
+                        const int i4 = ctid + n * DS_CTHREADS;
                         v[n] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (i4 < q4) v[n] = __ldcg(reinterpret_cast<const float4*>(P.src_f) + i4);
                     }
@@ -689,196 +757,231 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                 }
 #pragma unroll
                 for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
-                if (lane == 0) sh.red[0][warp] = ss;
-                ds_consumer_sync();
+                if (lane == 0) sh.red[0][cwarp] = ss;
+                ds_collect_sync();
                 float tot = 0.f;
 #pragma unroll
-                for (int w = 0; w < DS_WARPS; ++w) tot += sh.red[0][w];
+                for (int w = 0; w < DS_COLLECT_WARPS; ++w) tot += sh.red[0][w];
                 const float scale = rsqrtf(tot / (float)P.K + 1e-6f);
+                if (ctid == 0) sh.scale[pb][0] = scale;
 #pragma unroll
                 for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                    const int i4 = threadIdx.x + n * DS_CTHREADS;
+                    const int i4 = ctid + n * DS_CTHREADS;
                     if (n * DS_CTHREADS < q4) {   // the same for every thread: warps stay whole
-                        const bool mine = i4 >= g0 && i4 < g1;
-                        if (mine && P.rec) reinterpret_cast<float4*>(P.rec)[i4] = v[n];
-                        const int slab = i4 >> 6;
+                        const int slab = i4 >> 6;   // (a warp's 32 groups are half a slab)
                         int sl = -1;
 #pragma unroll
                         for (int x = 0; x < DS_MAX_SLOTS; ++x) sl = (x < n_slots && slabs[x] == slab) ? x : sl;
-                        // most of the row is read for its sum of squares only: a warp (its 32 groups are half a slab)
-                        // whose groups are neither staged nor part of this CTA's share of the caller's copy rounds nothing
-                        const int wg = i4 - lane;
-                        if (sl >= 0 || (wg < g1 && wg + 32 > g0))
-                            place(sl >= 0 ? sh.xs + (size_t)sl * slab_bytes : nullptr, 0, i4,
-                                  make_float4(v[n].x * scale, v[n].y * scale, v[n].z * scale, v[n].w * scale), mine);
+                        if (sl >= 0)
+                            place(sh.xs + (size_t)sl * dt_slab_bytes(MT), 0, i4, make_float4(v[n].x * scale, v[n].y * scale, v[n].z * scale, v[n].w * scale));
                     }
                 }
             } else {
                 bool normed = false;
                 if constexpr (MT > 1) {
                 if (P.in_op == AQ_IN_RMSNORM && P.norm != nullptr) {
-                    // Row norms from shares: this CTA sums the squares of its share of every token row (one group of
-                    // four per thread, one trip to L2), publishes the M partial sums as (float | 1 << 32) words, and
-                    // gathers every CTA's words; all sums run in a fixed order, so every CTA gets the same norms.
-                    float* part = &sh.red[0][0];
-                    float* gathered = reinterpret_cast<float*>(sh.xs);   // [CTA][M]: the slab area is not in use yet
-                    const int share = g1 - g0, n_items = share * M;      // (the host made sure n_items fits sh.red)
-                    if ((int)threadIdx.x < n_items) {
-                        const int m = (int)threadIdx.x / share, i4 = g0 + (int)threadIdx.x - m * share;
-                        const float4 v = source4(P.src, P.src_f, expect, m, i4);
-                        part[threadIdx.x] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
-                    }
-                    ds_consumer_sync();
-                    if ((int)threadIdx.x < M) {
+                    // Row norms from shares, a warp per token row: it sums the squares of this CTA's share of the row,
+                    // publishes the sum as a (float | 1 << 32) word and gathers every CTA's word; all sums run in a fixed
+                    // order, so every CTA gets the same norms.
+                    if (cwarp < M) {
+                        const int g0 = (int)(((int64_t)q4 * blockIdx.x) / gridDim.x), g1 = (int)(((int64_t)q4 * (blockIdx.x + 1)) / gridDim.x);
                         float ss = 0.f;
-                        for (int j = 0; j < share; ++j) ss += part[threadIdx.x * share + j];
-                        const u64 w = (u64)__float_as_uint(ss) | (1ull << 32);
-                        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(P.norm + (size_t)blockIdx.x * M + threadIdx.x), "l"(w) : "memory");
-                    }
-                    const int n_words = (int)gridDim.x * M;
-                    for (int it = threadIdx.x; it < n_words; it += DS_CTHREADS) {
-                        u64 w;
-                        for (;;) {
-                            w = ds_ld1(P.norm + it);
-                            if ((w >> 32) != 0 || give_up()) break;
-                        }
-                        gathered[it] = __uint_as_float((uint32_t)w);
-                    }
-                    ds_consumer_sync();
-                    if ((int)threadIdx.x < M) {
-                        float tot = 0.f;
-                        for (int c = 0; c < (int)gridDim.x; ++c) tot += gathered[c * M + threadIdx.x];
-                        sh.scale[threadIdx.x] = rsqrtf(tot / (float)P.K + 1e-6f);
-                    }
-                    ds_consumer_sync();
-                    normed = true;
-                }
-                }
-                if (P.in_op == AQ_IN_RMSNORM && !normed) {
-                    for (int m = 0; m < M; ++m) {
-                        float ss = 0.f;
-                        for (int i = threadIdx.x; i < q4; i += DS_CTHREADS) {
-                            const float4 v = source4(P.src, P.src_f, expect, m, i);
+                        for (int g = g0 + lane; g < g1; g += 32) {
+                            const float4 v = ds_source4(sh, P.src, P.src_f, expect, (int64_t)cwarp * P.K + 4 * (int64_t)g, wait_ns, pat);
                             ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
                         }
                         __syncwarp();
 #pragma unroll
                         for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
-                        if (lane == 0) sh.red[m][warp] = ss;
-                    }
-                    ds_consumer_sync();
-                    if ((int)threadIdx.x < M) {
+                        u64* row = P.norm + (size_t)cwarp * AQ_NORM_MAX_CTAS;
+                        if (lane == 0) {
+                            const u64 w = (u64)__float_as_uint(ss) | (1ull << 32);
+                            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(row + blockIdx.x), "l"(w) : "memory");
+                        }
+                        constexpr int NW = AQ_NORM_MAX_CTAS / 32;
+                        u64 w[NW];
+                        for (;;) {
+                            bool ready = true;
+#pragma unroll
+                            for (int i = 0; i < NW; ++i) { w[i] = 1ull << 32; if (lane + 32 * i < (int)gridDim.x) w[i] = ds_ld1(row + lane + 32 * i); }
+#pragma unroll
+                            for (int i = 0; i < NW; ++i) ready = ready && (w[i] >> 32) != 0;
+                            if (ready || pat.over(sh, wait_ns)) break;
+                        }
+                        __syncwarp();
                         float tot = 0.f;
 #pragma unroll
-                        for (int w = 0; w < DS_WARPS; ++w) tot += sh.red[threadIdx.x][w];
-                        sh.scale[threadIdx.x] = rsqrtf(tot / (float)P.K + 1e-6f);
+                        for (int i = 0; i < NW; ++i) tot += __uint_as_float((uint32_t)w[i]);
+#pragma unroll
+                        for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
+                        if (lane == 0) sh.scale[pb][cwarp] = rsqrtf(tot / (float)P.K + 1e-6f);
                     }
-                    ds_consumer_sync();
+                    ds_collect_sync();
+                    normed = true;
                 }
-                // one list of work: first the slabs this CTA reads, then its share of the caller's copies
-                const int per_slab = 64 * M;
-                const int n_a = n_slots * per_slab;
-                const int n_b = (g1 - g0) * M;
-                const int n_all = n_a + n_b;
-                const bool two = (P.in_op == AQ_IN_SILU_MUL);
-                for (int it0 = 0; it0 < n_all; it0 += DS_CTHREADS) {
-                    const int it = it0 + threadIdx.x;
-                    int m = 0, i4 = 0;
-                    bool valid = false;
-                    uint8_t* sl = nullptr;
-                    if (it < n_a) {
-                        const int s_ = it / per_slab, w = it - s_ * per_slab;
-                        m = w >> 6;
-                        i4 = C.slab_of_slot[s_] * 64 + (w & 63);
-                        sl = sh.xs + (size_t)s_ * slab_bytes;
-                        valid = i4 < q4;
-                    } else if (it < n_all) {
-                        const int w = it - n_a;
-                        m = w / (g1 - g0);
-                        i4 = g0 + w - m * (g1 - g0);
-                        valid = true;
+                }
+                if (P.in_op == AQ_IN_RMSNORM && !normed) {
+                    if constexpr (MT < 4) {
+                        for (int m = 0; m < M; ++m) {
+                            float ss = 0.f;
+                            for (int i = ctid; i < q4; i += DS_CTHREADS) {
+                                const float4 v = ds_source4(sh, P.src, P.src_f, expect, (int64_t)m * P.K + 4 * (int64_t)i, wait_ns, pat);
+                                ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
+                            }
+                            __syncwarp();
+#pragma unroll
+                            for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
+                            if (lane == 0) sh.red[m][cwarp] = ss;
+                        }
+                    } else {
+                        // two tokens at a time: both readings go out together and are repeated together until complete
+                        for (int m = 0; m < M; m += 2) {
+                            float ss[2] = {0.f, 0.f};
+                            const bool second = m + 1 < M;
+                            for (int i = ctid; i < q4; i += DS_CTHREADS) {
+                                const int64_t o = (int64_t)m * P.K + 4 * (int64_t)i;
+                                float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
+                                if (P.src == nullptr) {
+                                    v = __ldcg(reinterpret_cast<const float4*>(P.src_f + o));
+                                    if (second) u = __ldcg(reinterpret_cast<const float4*>(P.src_f + o + P.K));
+                                } else {
+                                    DsQuad qa, qb;
+                                    for (;;) {
+                                        ds_ld_quad(P.src + o, qa);
+                                        if (second) ds_ld_quad(P.src + o + P.K, qb);
+                                        const bool ready = ds_quad_ready(qa, expect) && (!second || ds_quad_ready(qb, expect));
+                                        if (ready || pat.over(sh, wait_ns)) break;
+                                    }
+                                    v = ds_quad_value(qa);
+                                    if (second) u = ds_quad_value(qb);
+                                }
+                                ss[0] = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, ss[0]))));
+                                ss[1] = fmaf(u.w, u.w, fmaf(u.z, u.z, fmaf(u.y, u.y, fmaf(u.x, u.x, ss[1]))));
+                            }
+                            __syncwarp();
+#pragma unroll
+                            for (int x = 0; x < 2; ++x) {
+#pragma unroll
+                                for (int d = 16; d > 0; d >>= 1) ss[x] += __shfl_xor_sync(0xffffffffu, ss[x], d);
+                                if (lane == 0 && m + x < M) sh.red[m + x][cwarp] = ss[x];
+                            }
+                        }
                     }
-                    const bool share = it >= n_a;
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (valid) {
-                        // both sources' readings go out together and are repeated together until complete
-                        const int64_t o = (int64_t)m * P.K + 4 * (int64_t)i4;
-                        float4 s = make_float4(0.f, 0.f, 0.f, 0.f), t = s;
-                        DsQuad qa, qb;
-                        for (;;) {
-                            if (P.src) ds_ld_quad(P.src + o, qa);
-                            else s = __ldcg(reinterpret_cast<const float4*>(P.src_f + o));
-                            if (two) {
-                                if (P.src2) ds_ld_quad(P.src2 + o, qb);
-                                else t = __ldcg(reinterpret_cast<const float4*>(P.src2_f + o));
-                            }
-                            bool ready = true;
-                            if (P.src) ready = ds_quad_ready(qa, expect);
-                            if (two && P.src2) ready = ready && ds_quad_ready(qb, expect2);
-                            if (ready) {
-                                if (P.src) s = ds_quad_value(qa);
-                                if (two && P.src2) t = ds_quad_value(qb);
-                                break;
-                            }
-                            if (give_up()) { s = t = make_float4(0.f, 0.f, 0.f, 0.f); break; }
+                    ds_collect_sync();
+                    if (ctid < M) {
+                        float tot = 0.f;
+#pragma unroll
+                        for (int w = 0; w < DS_COLLECT_WARPS; ++w) tot += sh.red[ctid][w];
+                        sh.scale[pb][ctid] = rsqrtf(tot / (float)P.K + 1e-6f);
+                    }
+                    ds_collect_sync();
+                }
+                // half a slab of one token (32 groups) per warp and item, NB items in flight
+                constexpr int NB = MT == 1 ? 1 : 2;
+                const int n_items = 2 * n_slots * M;
+                const uint32_t by_m = (65536u + (uint32_t)M - 1) / (uint32_t)M;   // (v * by_m) >> 16 = v / M for v < 64
+                const bool two = (P.in_op == AQ_IN_SILU_MUL), rms = (P.in_op == AQ_IN_RMSNORM);
+                for (int it0 = cwarp; it0 < n_items; it0 += NB * DS_COLLECT_WARPS) {
+                    int slot[NB], m[NB], i4[NB];
+                    bool on[NB];
+#pragma unroll
+                    for (int n = 0; n < NB; ++n) {
+                        const int it = it0 + n * DS_COLLECT_WARPS, v = it >> 1;
+                        slot[n] = (int)(((uint32_t)v * by_m) >> 16);
+                        m[n] = v - slot[n] * M;
+                        i4[n] = 0; on[n] = false;
+                        if (it < n_items) {
+                            i4[n] = C.slab_of_slot[slot[n]] * 64 + (it & 1) * 32 + lane;
+                            on[n] = i4[n] < q4;
                         }
-                        if (share && P.rec) *reinterpret_cast<float4*>(P.rec + o) = s;
-                        if (two) {
-                            if (share && P.rec2) *reinterpret_cast<float4*>(P.rec2 + o) = t;
-                            v = make_float4(ds_silu_mul(s.x, t.x), ds_silu_mul(s.y, t.y), ds_silu_mul(s.z, t.z), ds_silu_mul(s.w, t.w));
-                        } else {
-                            const float sc = (P.in_op == AQ_IN_RMSNORM) ? sh.scale[m] : 1.f;
-                            v = make_float4(s.x * sc, s.y * sc, s.z * sc, s.w * sc);
+                    }
+                    // all readings go out together and are repeated together until complete
+                    float4 s[NB], t[NB];
+                    DsQuad qa[NB], qb[NB];
+                    bool ready;
+                    for (;;) {
+                        ready = true;
+#pragma unroll
+                        for (int n = 0; n < NB; ++n) {
+                            const int64_t o = (int64_t)m[n] * P.K + 4 * (int64_t)i4[n];
+                            if (on[n]) {
+                                if (P.src) ds_ld_quad(P.src + o, qa[n]);
+                                else s[n] = __ldcg(reinterpret_cast<const float4*>(P.src_f + o));
+                                if (two) {
+                                    if (P.src2) ds_ld_quad(P.src2 + o, qb[n]);
+                                    else t[n] = __ldcg(reinterpret_cast<const float4*>(P.src2_f + o));
+                                }
+                            }
                         }
+#pragma unroll
+                        for (int n = 0; n < NB; ++n) {
+                            if (on[n] && P.src) ready = ready && ds_quad_ready(qa[n], expect);
+                            if (on[n] && two && P.src2) ready = ready && ds_quad_ready(qb[n], expect2);
+                        }
+                        if (ready || pat.over(sh, wait_ns)) break;
                     }
                     __syncwarp();
-                    if (it0 + (int)(threadIdx.x - lane) < n_a) {
-                        place(sl, m, i4, v, false);              // n_a is a multiple of 32: the whole warp is inside the slab items
-                    } else if (valid) {
-                        float sum;
-                        const uint2 r = ds_round4<BF16>(v, &sum);
-                        *reinterpret_cast<uint2*>(stage_out + (int64_t)m * P.K + i4 * 4) = r;
+#pragma unroll
+                    for (int n = 0; n < NB; ++n) {
+                        if (it0 + n * DS_COLLECT_WARPS >= n_items) break;
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (on[n] && ready) {
+                            v = P.src ? ds_quad_value(qa[n]) : s[n];
+                            if (two) {
+                                const float4 u = P.src2 ? ds_quad_value(qb[n]) : t[n];
+                                v = make_float4(ds_silu_mul(v.x, u.x), ds_silu_mul(v.y, u.y), ds_silu_mul(v.z, u.z), ds_silu_mul(v.w, u.w));
+                            } else if (rms) {
+                                const float sc = sh.scale[pb][m[n]];
+                                v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+                            }
+                        }
+                        __syncwarp();
+                        place(sh.xs + (size_t)slot[n] * dt_slab_bytes(MT), m[n], i4[n], v);
                     }
                 }
             }
         }
-        if (ds_consumer_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
+        fence_async_smem();   // (the tensor core reads the slabs through the asynchronous proxy)
+        if (ds_collect_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
+        if (ctid == 0) asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(ds_smem(&sh.xphase)), "r"(ph + 1) : "memory");
 
-        // -- consume this warp's units of the phase: positions warp, warp + 15, ... of the CTA's list --
+        // -- the sums of the phase's units, the two teams taking turns --
         const int total = C.total;
+        bool ok = true;
 #pragma unroll 1
-        for (int pos = warp; pos < total && !dead; pos += DS_WARPS) {
-            dead = __any_sync(0xffffffffu, !ds_mbar_wait(ds_smem(&sh.full[warp][cslot]), cparity, wait_ns));
-            if (dead) {
-                if (lane == 0) { atomicCAS(&g_decode_status, 0, 2); sh.abort_flag = 1; }
-                break;
+        for (int i = 0; i < total && ok; ++i) {
+            if (turn == (uint32_t)(cwarp >> 2)) {
+                ok = ds_warp_wait(ds_smem(&sh.stored[stage]), use & 1u, wait_ns, &sh.abort_flag) &&
+                     ds_warp_wait(ds_smem(&sh.done[stage]), use & 1u, wait_ns, &sh.abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const uint4 d = sh.sdesc[stage];
+                const int bits = (int)(d.x >> DS_DESC_BITS_SHIFT) & 7;
+                const float* sums = reinterpret_cast<const float*>(sh.xs + d.y + DT_SUMS<MT>);
+                const uint8_t* dmp = &sh.dm[stage][quarter * 2 + (lane >> 4)][(lane & 15) * 16];
+                const uint4 dm0 = *reinterpret_cast<const uint4*>(dmp), dm1 = *reinterpret_cast<const uint4*>(dmp + DS_FRAGS * SCALE_BYTES);
+                const uint32_t td = tmem + stage * ST::COLS + 2 * DtShape<MT>::A_COLS + ((uint32_t)(quarter * 32) << 16);
+                float acc[MT];
+#pragma unroll
+                for (int m = 0; m < MT; ++m) acc[m] = 0.f;
+                if (bits == 2) dt_collect<2, MT, BF16>(td, dm0, dm1, sums, acc);
+                else if (bits == 3) dt_collect<3, MT, BF16>(td, dm0, dm1, sums, acc);
+                else dt_collect<4, MT, BF16>(td, dm0, dm1, sums, acc);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ds_mbar_arrive(ds_smem(&sh.taken[stage]));
+                const DsOp& op = P.ops[d.x & (DS_MAX_PHASE_OPS - 1)];
+                ds_commit<MT>(acc, op.dst, (d.x & DS_DESC_FIRST) ? op.res : nullptr, op.res_plain != 0, (int)d.z * DT_ROWS + quarter * 32 + lane, op.N, M);
             }
-            const uint4 ds = sh.desc[warp][cslot];
-            const uint8_t* xseg = sh.xs + (size_t)(C.xoff[ds.x & 0xFFu] + (int)ds.y) * slab_bytes;
-            const uint8_t* unit = &sh.ring[warp][cslot][0];
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            const int bits = (int)(ds.x >> DS_DESC_BITS_SHIFT);
-            if (bits == 2) ds_unit_body<2, MT, BF16>(unit, xseg, xo, pd, M, lane, acc);
-            else if (bits == 3) ds_unit_body<3, MT, BF16>(unit, xseg, xo, pd, M, lane, acc);
-            else ds_unit_body<4, MT, BF16>(unit, xseg, xo, pd, M, lane, acc);
-            __syncwarp();        // every lane has read its part of the slot
-            if (lane == 0) ds_mbar_arrive(ds_smem(&sh.empty[warp][cslot]));
-            if (++cslot == DS_SLOTS) { cslot = 0; cparity ^= 1u; }
-            const DsOp& op = P.ops[ds.x & 0xFFu];
-            if (ds.y == 0 && op.res != nullptr) {   // (rare: the residual rides along with the first k-slab's sums)
-                ds_unit_commit<MT>(acc, op.dst, op.res, (op.bits & DS_RES_PLAIN) != 0, op.N, (int)ds.z * 16, op.N, M, lane);
-            } else {
-                pd.acc[0] = acc[0]; pd.acc[1] = acc[1]; pd.acc[2] = acc[2]; pd.acc[3] = acc[3];
-                pd.out = op.dst; pd.N = op.N; pd.row0 = (int)ds.z * 16; pd.on = true;
-            }
+            turn ^= 1u;
+            if (++stage == ST::N) { stage = 0; ++use; }
         }
-        ds_flush<MT>(pd, M, lane);   // nothing of this phase stays behind: other CTAs wait for these sums
     }
 
     // -- buffers no phase reads (and the last outputs): float32 copies for the caller, one chunk per warp --
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag) == 0) {
 #pragma unroll 1
-        for (int e = (int)blockIdx.x * DS_WARPS + warp; e < a.n_tails; e += (int)gridDim.x * DS_WARPS) {
+        for (int e = (int)blockIdx.x * DS_COLLECT_WARPS + cwarp; e < a.n_tails; e += (int)gridDim.x * DS_COLLECT_WARPS) {
             const DsTail T = a.tails[e];
             bool ok = true;
             for (int i = lane * 4; i < T.n && ok; i += 128) {      // n is a multiple of 4
@@ -898,8 +1001,16 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
         }
     }
 
-    // after a failed wait copies may still be on their way into this CTA's shared memory: give them time
+    }   // (collect warps)
+
+    // after a failed wait copies and tensor-core instructions may still be at work in this CTA: give them time
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag)) __nanosleep(500000);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512) : "memory");
+    }
 }
 
 // ---- host: plan, cache, launch -----------------------------------------------------
@@ -908,9 +1019,9 @@ namespace {
 struct DecodePlan {
     std::vector<uint8_t> key;
     std::vector<aq_handle_t> handles;
-    uint8_t* dev = nullptr;       // [phase records][mini phases, mini ops][tail chunks][per-CTA phase tables]
-    size_t phases_bytes = 0, mini_bytes = 0, tail_bytes = 0, ctab_bytes = 0;
-    int n_mini_ops = 0;
+    uint8_t* dev = nullptr;       // [phase records][ops][slab offsets][tail chunks][per-CTA phase tables][units per CTA]
+    size_t feed_at = 0, xoff_at = 0, tails_at = 0, ctab_at = 0, total_at = 0;   // (the phase records are at 0)
+    int n_ops = 0;
     int n_phases = 0;
     int n_tails = 0;
     int device = 0;
@@ -938,16 +1049,81 @@ template <typename T> void key_put(std::vector<uint8_t>& k, const T& v) {
 
 }  // namespace
 
+// How the units of the ops of one phase are dealt to the CTAs.  Every op's units are dealt on their own: with n = q G + r
+// units and G CTAs, row s of the table takes q + 1 units if s < r, else q; an op starts `rot` rows further on than the first
+// one, so that the odd units do not always land on the same CTAs.  It depends on the shapes alone, so the phases of equal
+// blocks share a table (made anew for each of them it was most of a program's first call).
+struct DealTable {
+    struct Op { int NT8, KP, q, r, rot; };
+    std::vector<Op> deal;
+    std::vector<DsCtaPhase> cta;    // [row]
+    std::vector<int16_t> xoff;      // [op][row]
+    int turn = 0;                   // rows the next phase starts further on
+    bool fits = false;              // no row needs more staged slabs than there is room for
+};
+// The table of ops[0 .. count), made if there is none yet; null when the kernel cannot take such a phase at all.
+const DealTable* deal_table(std::vector<DealTable>& tables, const aq_stack_op_t* ops, int count, int n_cta) {
+    DealTable t;
+    int64_t all = 0;
+    for (int i = 0; i < count; ++i) {
+        const aq_handle_s* h = ops[i].w;
+        const int NT8 = (h->NT + DS_FRAGS - 1) / DS_FRAGS;
+        const int64_t nu = (int64_t)h->KP * NT8;
+        all += nu;
+        if (all > (int64_t)1 << 26 || h->KP > DS_MAX_CONTRIB) return nullptr;
+        t.deal.push_back({NT8, h->KP, (int)(nu / n_cta), (int)(nu % n_cta), t.turn});
+        t.turn = (int)((t.turn + nu % n_cta) % n_cta);
+    }
+    for (const DealTable& o : tables) {
+        bool same = o.deal.size() == t.deal.size();
+        for (size_t i = 0; i < t.deal.size() && same; ++i) same = o.deal[i].NT8 == t.deal[i].NT8 && o.deal[i].KP == t.deal[i].KP;
+        if (same) return &o;
+    }
+    t.cta.resize(n_cta);
+    t.xoff.assign((size_t)count * n_cta, 0);
+    t.fits = true;
+    for (int c = 0; c < n_cta && t.fits; ++c) {
+        // the slabs the row reads, ascending, and where each op's first slab sits among them (an op's slabs are consecutive)
+        DsCtaPhase& T = t.cta[c];
+        memset(&T, 0, sizeof(T));
+        std::vector<int> need;
+        int lo[DS_MAX_PHASE_OPS];
+        for (int i = 0; i < count && t.fits; ++i) {
+            const DealTable::Op& d = t.deal[i];
+            const int sl = (c + d.rot) % n_cta, u0 = d.q * sl + std::min(sl, d.r), u1 = u0 + d.q + (sl < d.r ? 1 : 0);
+            T.total += u1 - u0;
+            lo[i] = u0 / d.NT8;
+            if (u0 == u1) continue;
+            const int hi = (u1 - 1) / d.NT8;
+            if (hi - lo[i] >= DS_MAX_SLOTS) t.fits = false;
+            else for (int x = lo[i]; x <= hi; ++x) need.push_back(x);
+        }
+        std::sort(need.begin(), need.end());
+        need.erase(std::unique(need.begin(), need.end()), need.end());
+        if ((int)need.size() > DS_MAX_SLOTS) t.fits = false;
+        if (!t.fits) break;
+        T.n_slots = (int32_t)need.size();
+        for (size_t x = 0; x < need.size(); ++x) T.slab_of_slot[x] = need[x];
+        for (int i = 0; i < count; ++i)
+            t.xoff[(size_t)i * n_cta + c] = (int16_t)(std::lower_bound(need.begin(), need.end(), lo[i]) - need.begin() - lo[i]);
+    }
+    tables.push_back(std::move(t));
+    return &tables.back();
+}
+
 // Device tables of a program: one record per phase (at most DS_MAX_PHASE_OPS ops that
 // read the same input vector) and the list of buffers nobody reads.  False when the program
 // does not fit this kernel.
 bool build_decode_tables(const aq_stack_t* p, const StackPlan& plan, int M, int n_cta, uint8_t* ws,
                          std::vector<DsPhase>& phases, std::vector<DsTail>& tails, std::vector<DsCtaPhase>& ctab,
-                         std::vector<char>& in_tails, int op_first, int op_end) {
+                         std::vector<DsFeedOp>& feed_ops, std::vector<int16_t>& xoff, std::vector<char>& in_tails, int op_first, int op_end) {
     if (M < 1 || M > AQ_DECODE_MAX_M || p->n_ops > 32000 || plan.pk_off.empty()) return false;
     phases.clear();
     tails.clear();
     ctab.clear();
+    feed_ops.clear();
+    xoff.clear();
+    std::vector<DealTable> tables;
     std::vector<int> writer(p->n_bufs, -1);         // op that writes the buffer
     std::vector<char> whole(p->n_bufs, 0);          // every CTA has seen the whole buffer complete (a normalised input)
     std::vector<char> recorded(p->n_bufs, 0);       // some phase writes the caller's float32 copy
@@ -976,61 +1152,33 @@ bool build_decode_tables(const aq_stack_t* p, const StackPlan& plan, int M, int 
             const int64_t K = p->buf_width[f.src];
             if (K > (int64_t)1 << 24 || n_cta > 32767) return false;
             DsPhase P;
-            std::vector<DsCtaPhase> ctab_phase;
-            int count = std::min(plast - first, DS_MAX_PHASE_OPS), rot_after = rot;
+            int count = std::min(plast - first, DS_MAX_PHASE_OPS);
+            const DealTable* tab = nullptr;
             for (; count >= 1; --count) {
-                memset(&P, 0, sizeof(P));
-                int r2 = rot;
-                int64_t off = 0;
-                bool ok = true;
-                for (int i = first; i < first + count && ok; ++i) {
-                    const aq_handle_s* h = p->ops[i].w;
-                    DsOp& d = P.ops[i - first];
-                    const int64_t nu = (int64_t)h->KP * h->NT;
-                    if (off + nu > (int64_t)1 << 26 || h->KP > DS_MAX_CONTRIB) { ok = false; break; }
-                    d.N = (int32_t)h->N; d.NT = h->NT; d.bits = h->bits;
-                    d.nt_magic = h->NT > 1 ? (uint32_t)(((uint64_t)1 << 32) / (uint64_t)h->NT + 1) : 0u;
-                    d.units_q = (int32_t)(nu / n_cta);
-                    d.units_r_rot = (int32_t)(nu % n_cta) | (r2 << 16);
-                    r2 = (int)((r2 + nu % n_cta) % n_cta);
-                    off += nu;
-                }
-                std::vector<DsCtaPhase> tab(ok ? n_cta : 0);
-                for (int c = 0; c < n_cta && ok; ++c) {
-                    // the slabs CTA c reads for the phase, ascending, and where each op's first slab sits among them
-                    DsCtaPhase& T = tab[c];
-                    memset(&T, 0, sizeof(T));
-                    std::vector<int64_t> need;
-                    int64_t lo[DS_MAX_PHASE_OPS];
-                    for (int i = 0; i < count; ++i) {
-                        const int64_t q = P.ops[i].units_q, r = P.ops[i].units_r_rot & 0xFFFF, ro = P.ops[i].units_r_rot >> 16;
-                        const int64_t sl = (c + ro) % n_cta;
-                        const int64_t u0 = q * sl + std::min(sl, r), u1 = u0 + q + (sl < r ? 1 : 0);
-                        T.total += (int32_t)(u1 - u0);
-                        lo[i] = -1;
-                        if (u0 < u1) {
-                            lo[i] = u0 / P.ops[i].NT;
-                            for (int64_t x = u0 / P.ops[i].NT; x <= (u1 - 1) / P.ops[i].NT; ++x) need.push_back(x);
-                        }
-                    }
-                    std::sort(need.begin(), need.end());
-                    need.erase(std::unique(need.begin(), need.end()), need.end());
-                    const int64_t slabs = (int64_t)need.size();
-                    if (slabs > DS_MAX_SLOTS || slabs * ds_slab_bytes(M) > DS_XS_BYTES) { ok = false; break; }
-                    T.n_slots = (int32_t)slabs;
-                    for (int64_t x = 0; x < slabs; ++x) T.slab_of_slot[x] = (int32_t)need[x];
-                    for (int i = 0; i < count; ++i) {
-                        if (lo[i] < 0) continue;
-                        const int64_t slot = std::lower_bound(need.begin(), need.end(), lo[i]) - need.begin();
-                        T.xoff[i] = (int32_t)(slot - lo[i]);   // (the op's slabs are consecutive, so are their slots)
-                    }
-                }
-                if (ok) ctab_phase = tab;
-                if (ok) { rot_after = r2; break; }
+                tab = deal_table(tables, p->ops + first, count, n_cta);
+                if (tab == nullptr) return false;
+                if (tab->fits) break;
             }
             if (count < 1) return false;
             const int last = first + count;
-            rot = rot_after;
+            // CTA c takes row (c + rot) mod (number of CTAs) of the table
+            memset(&P, 0, sizeof(P));
+            ctab.insert(ctab.end(), tab->cta.begin() + rot, tab->cta.end());
+            ctab.insert(ctab.end(), tab->cta.begin(), tab->cta.begin() + rot);
+            for (int i = 0; i < count; ++i) {
+                const aq_handle_s* h = p->ops[first + i].w;
+                DsFeedOp f2;
+                memset(&f2, 0, sizeof(f2));
+                f2.frags = h->frags; f2.NT = h->NT;
+                f2.units_q = tab->deal[i].q;
+                f2.units_r_rot = tab->deal[i].r | (((tab->deal[i].rot + rot) % n_cta) << 16);
+                f2.word0 = (uint32_t)i | ((uint32_t)h->bits << DS_DESC_BITS_SHIFT) | ((uint32_t)phases.size() << DS_DESC_PHASE_SHIFT);
+                feed_ops.push_back(f2);
+                const int16_t* x = tab->xoff.data() + (size_t)i * n_cta;
+                xoff.insert(xoff.end(), x + rot, x + n_cta);
+                xoff.insert(xoff.end(), x, x + rot);
+            }
+            rot = (rot + tab->turn) % n_cta;
             auto source = [&](int b, const u64*& sp, const float*& sf, float*& rec, uint32_t& ex) {
                 if (writer[b] < 0) { sp = nullptr; sf = plain(b); rec = nullptr; ex = 0; return; }   // the program input
                 sp = packed(b); sf = nullptr; ex = expect_of(b);
@@ -1044,30 +1192,27 @@ bool build_decode_tables(const aq_stack_t* p, const StackPlan& plan, int M, int 
             P.stage = ws + plan.in_off[first];
             P.K = (int32_t)K; P.in_op = f.in_op; P.op_count = count;
             // several tokens: the row norms come from per-CTA partial sums exchanged through the workspace (whole
-            // rows read by every CTA are 8 M K bytes per CTA from the same lines of L2); the partial sums of a CTA's
-            // share are added up through sh.red, hence the bound on the share
+            // rows read by every CTA are 8 M K bytes per CTA from the same lines of L2)
             P.norm = nullptr;
-            if (f.in_op == AQ_IN_RMSNORM && M >= 3 && !plan.nm_off.empty() && plan.nm_off[pfirst] != 0 && n_cta <= AQ_NORM_MAX_CTAS &&
-                (int64_t)M * ((K / 4 + n_cta - 1) / n_cta + 1) <= (int64_t)AQ_DECODE_MAX_M * DS_WARPS)
+            if (f.in_op == AQ_IN_RMSNORM && M >= 3 && (int64_t)M * K > DS_WHOLE_ROWS && !plan.nm_off.empty() && plan.nm_off[pfirst] != 0 && n_cta <= AQ_NORM_MAX_CTAS)
                 P.norm = reinterpret_cast<u64*>(ws + plan.nm_off[pfirst]);
             for (int i = first; i < last; ++i) {
                 const aq_stack_op_t& o = p->ops[i];
                 DsOp& d = P.ops[i - first];
-                d.frags = o.w->frags;
                 d.dst = packed(o.dst);
+                d.N = (int32_t)o.w->N;
                 d.res = nullptr;
                 if (o.out_op == AQ_OUT_ADD) {
                     // the residual is read without a wait: it must be complete for every CTA when the phase starts,
                     // i.e. the program input (plain float32) or an input that every CTA has already read as a whole
                     // (a normalised one)
-                    if (writer[o.res] < 0) { d.res = plain(o.res); d.bits |= DS_RES_PLAIN; }
+                    if (writer[o.res] < 0) { d.res = plain(o.res); d.res_plain = 1; }
                     else if (whole[o.res]) d.res = packed(o.res);
                     else return false;
                 }
             }
             for (int i = first; i < last; ++i) writer[p->ops[i].dst] = i;
             phases.push_back(P);
-            ctab.insert(ctab.end(), ctab_phase.begin(), ctab_phase.end());
             first = last;
         }
     }
@@ -1151,8 +1296,10 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
         std::vector<DsPhase> phases;
         std::vector<DsTail> tails;
         std::vector<DsCtaPhase> ctab;
+        std::vector<DsFeedOp> feed_ops;
+        std::vector<int16_t> xoff;
         std::vector<char> in_tails;
-        if (!build_decode_tables(p, plan, M, grid, ws, phases, tails, ctab, in_tails, op_first, op_end)) return 1;
+        if (!build_decode_tables(p, plan, M, grid, ws, phases, tails, ctab, feed_ops, xoff, in_tails, op_first, op_end)) return 1;
         if (g_plans.size() >= MAX_PLANS) {   // make room: the oldest plan no graph refers to
             size_t oldest = g_plans.size();
             for (size_t i = 0; i < g_plans.size(); ++i)
@@ -1166,39 +1313,30 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
         dp->device = dev;
         for (int i = 0; i < p->n_ops; ++i) dp->handles.push_back(p->ops[i].w);
         dp->in_tails = in_tails;
-        dp->phases_bytes = (phases.size() * sizeof(DsPhase) + 255) / 256 * 256;
-        std::vector<uint8_t> mini(phases.size() * sizeof(DsMiniPhase));
-        for (size_t i = 0; i < phases.size(); ++i) {
-            DsMiniPhase mph;
-            memset(&mph, 0, sizeof(mph));
-            mph.op_first = dp->n_mini_ops; mph.op_count = phases[i].op_count;
-            memcpy(mini.data() + i * sizeof(DsMiniPhase), &mph, sizeof(mph));
-            dp->n_mini_ops += phases[i].op_count;
-        }
-        for (size_t i = 0; i < phases.size(); ++i)
-            for (int j = 0; j < phases[i].op_count; ++j) {
-                DsMiniOp mop;
-                memset(&mop, 0, sizeof(mop));
-                mop.NT = phases[i].ops[j].NT; mop.nt_magic = phases[i].ops[j].nt_magic;
-                mop.frags = phases[i].ops[j].frags;
-                mop.q_bits = (uint32_t)phases[i].ops[j].units_q | ((uint32_t)(phases[i].ops[j].bits & 0xFF) << 28);
-                mop.r_rot = (uint32_t)phases[i].ops[j].units_r_rot;
-                const uint8_t* b = reinterpret_cast<const uint8_t*>(&mop);
-                mini.insert(mini.end(), b, b + sizeof(mop));
-            }
-        dp->mini_bytes = (mini.size() + 255) / 256 * 256;
-        dp->tail_bytes = (tails.size() * sizeof(DsTail) + 255) / 256 * 256;
         dp->n_phases = (int)phases.size();
         dp->n_tails = (int)tails.size();
-        dp->ctab_bytes = (ctab.size() * sizeof(DsCtaPhase) + 255) / 256 * 256;
-        cudaError_t e = cudaMalloc(&dp->dev, dp->phases_bytes + dp->mini_bytes + dp->tail_bytes + dp->ctab_bytes + 256);
-        if (e == cudaSuccess) e = cudaMemcpy(dp->dev, phases.data(), phases.size() * sizeof(DsPhase), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(dp->dev + dp->phases_bytes, mini.data(), mini.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && !tails.empty())
-            e = cudaMemcpy(dp->dev + dp->phases_bytes + dp->mini_bytes, tails.data(), tails.size() * sizeof(DsTail), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(dp->dev + dp->phases_bytes + dp->mini_bytes + dp->tail_bytes, ctab.data(), ctab.size() * sizeof(DsCtaPhase),
-                           cudaMemcpyHostToDevice);
+        // one table after the other, each at a multiple of 256 bytes
+        std::vector<uint8_t> image;
+        image.reserve(phases.size() * sizeof(DsPhase) + (feed_ops.size() + 1) * (sizeof(DsFeedOp) + 2 * grid) + tails.size() * sizeof(DsTail) + ctab.size() * sizeof(DsCtaPhase) + 4096);
+        auto add = [&](const void* data, size_t bytes) {
+            const size_t at = image.size();
+            image.resize((at + bytes + 255) / 256 * 256);
+            if (bytes) memcpy(image.data() + at, data, bytes);
+            return at;
+        };
+        std::vector<int32_t> unit_total(grid, 0);
+        for (size_t i = 0; i < ctab.size(); ++i) unit_total[i % grid] += ctab[i].total;
+        dp->n_ops = (int)feed_ops.size();
+        feed_ops.push_back(DsFeedOp{});   // (the feeder reads one op ahead)
+        xoff.resize(xoff.size() + grid, 0);
+        add(phases.data(), phases.size() * sizeof(DsPhase));
+        dp->feed_at = add(feed_ops.data(), feed_ops.size() * sizeof(DsFeedOp));
+        dp->xoff_at = add(xoff.data(), xoff.size() * sizeof(int16_t));
+        dp->tails_at = add(tails.data(), tails.size() * sizeof(DsTail));
+        dp->ctab_at = add(ctab.data(), ctab.size() * sizeof(DsCtaPhase));
+        dp->total_at = add(unit_total.data(), unit_total.size() * sizeof(int32_t));
+        cudaError_t e = cudaMalloc(&dp->dev, image.size());
+        if (e == cudaSuccess) e = cudaMemcpy(dp->dev, image.data(), image.size(), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) { cudaGetLastError(); drop_plan(dp); *err = e; return -1; }
         g_plans.push_back(dp);
     }
@@ -1207,11 +1345,12 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
 
     DsArgs a;
     a.phases = reinterpret_cast<const DsPhase*>(dp->dev);
-    a.mini_phases = reinterpret_cast<const DsMiniPhase*>(dp->dev + dp->phases_bytes);
-    a.mini_ops = reinterpret_cast<const DsMiniOp*>(dp->dev + dp->phases_bytes + (size_t)dp->n_phases * sizeof(DsMiniPhase));
-    a.tails = reinterpret_cast<const DsTail*>(dp->dev + dp->phases_bytes + dp->mini_bytes);
-    a.ctab = reinterpret_cast<const DsCtaPhase*>(dp->dev + dp->phases_bytes + dp->mini_bytes + dp->tail_bytes);
-    a.n_mini_ops = dp->n_mini_ops;
+    a.feed_ops = reinterpret_cast<const DsFeedOp*>(dp->dev + dp->feed_at);
+    a.xoff = reinterpret_cast<const int16_t*>(dp->dev + dp->xoff_at);
+    a.unit_total = reinterpret_cast<const int32_t*>(dp->dev + dp->total_at);
+    a.n_ops = dp->n_ops;
+    a.tails = reinterpret_cast<const DsTail*>(dp->dev + dp->tails_at);
+    a.ctab = reinterpret_cast<const DsCtaPhase*>(dp->dev + dp->ctab_at);
     a.n_phases = dp->n_phases;
     a.n_tails = dp->n_tails;
     a.M = M;

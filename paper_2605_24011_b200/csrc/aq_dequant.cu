@@ -33,7 +33,7 @@ template <> struct OutVec<__nv_bfloat16> {
 
 // lane (g,t): 8 decoded values of block j, row half hi
 template <int BITS>
-__device__ __forceinline__ void decode_unit(const LaneCodes<BITS>& lc, const uint8_t* fb, int g, int j, int hi,
+__device__ __forceinline__ void decode_unit(const SlotWords<BITS>& sw, const uint8_t* fb, int g, int j, int hi,
                                             float* w) {
     const __half2 dm = *reinterpret_cast<const __half2*>(fb + ((g + 8 * hi) * 4 + j) * 4);
     const float d = __low2float(dm), m = __high2float(dm);
@@ -41,7 +41,7 @@ __device__ __forceinline__ void decode_unit(const LaneCodes<BITS>& lc, const uin
     for (int i = 0; i < 4; ++i) {
         // the two codes as floats without a conversion: 2^23 + q has q in its low mantissa bits, and
         // (2^23 + q) - 2^23 is exact, so the value is the same as (float)q
-        const uint32_t p = code_pair<BITS>(lc, j, hi, i, 0u);
+        const uint32_t p = code_pair<BITS>(sw, j, hi, i, 0u);
         const float q0 = __uint_as_float((p & 0xffffu) | 0x4B000000u) - 8388608.f;
         const float q1 = __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7632)) - 8388608.f;
         w[2 * i] = fmaf(d, q0, m);
@@ -60,15 +60,17 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
     const int64_t u = f >> 1;
     const int64_t R = u % NT;
     const int64_t S = 2 * (u / NT) + par;
-    const uint8_t* fb = frags + f * FB;
+    const uint8_t* fb = frags + frag_index(S, R, NT) * FB;
     LaneCodes<BITS> lc;
     load_lane_codes<BITS>(lc, fb, lane);
+    SlotWords<BITS> sw;
+    sw.gather(lc);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
 #pragma unroll
         for (int hi = 0; hi < 2; ++hi) {
             float w[8];
-            decode_unit<BITS>(lc, fb, g, j, hi, w);
+            decode_unit<BITS>(sw, fb, g, j, hi, w);
             const int64_t row = R * 16 + g + 8 * hi;
             const int64_t k0 = S * 128 + 32 * j + 8 * t;
             if (row < N && k0 < K) {

@@ -179,6 +179,8 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* slab, bool have, int
             for (int i = 0; i < 4; ++i) { dmw[0][i] = 0; dmw[1][i] = 0; }
         }
     }
+    SlotWords<BITS> sw;
+    sw.gather(lc);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t as = ai % GM_ASTAGES;
@@ -195,7 +197,7 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* slab, bool have, int
                 const __half2 dm = *reinterpret_cast<const __half2*>(&dmw[hi][j]);
                 const __half2 d2 = __low2half2(dm), m2 = __high2half2(dm);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) o[jj][i] = dequant_pair(code_pair<BITS>(lc, j, hi, i, MAGIC), d2, m2);
+                for (int i = 0; i < 4; ++i) o[jj][i] = dequant_pair(code_pair<BITS>(sw, j, hi, i, MAGIC), d2, m2);
             }
             // Rows with odd g store block 2h + 1 first: the eight lanes that a 16-byte store serves together (g = 2q,
             // 2q + 1; t = 0..3) then hit eight different chunks of the swizzle atom instead of four twice.
@@ -299,10 +301,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
                     ok = mbar_wait(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
                     if (!ok) break;
                     mbar_expect_tx(bar_pfull + 8 * ps, (uint32_t)(n_rt * FB));
-                    for (int ft = 0; ft < n_rt; ++ft) {
-                        const int64_t f = (((int64_t)(s >> 1) * op.NT + rt0 + ft) * 2 + (s & 1));
-                        bulk_load(smem_u32(sP + ps * P_BYTES + ft * FB), op.frags + f * FB, FB, bar_pfull + 8 * ps);
-                    }
+                    bulk_load(smem_u32(sP + ps * P_BYTES), op.frags + frag_index(s, rt0, op.NT) * FB, (uint32_t)(n_rt * FB), bar_pfull + 8 * ps);
                     ++pi;
                 }
             }

@@ -43,7 +43,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 template <int BITS, int MT, bool BF16>
 __global__ void __launch_bounds__(GEMV_WARPS * 32, 2) gemv_kernel(const GemvArgs a) {
-    constexpr int UB = 2 * frag_bytes(BITS);
+    constexpr int FB = frag_bytes(BITS), UB = 2 * FB;
     constexpr int PIECES = UB / 16 / 32;   // 16-byte pieces per lane per unit
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -57,15 +57,23 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32, 2) gemv_kernel(const GemvArgs
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
 
-    auto issue = [&](int64_t u, int slot) {
-        const uint8_t* src = a.frags + u * UB;
+    // the next unit to copy: pair-slab and row tile
+    int64_t Pc = u0 / a.NT;
+    int Rc = (int)(u0 - Pc * a.NT);
+    auto issue = [&](int slot) {
+        const uint8_t* src = a.frags + frag_index(2 * Pc, Rc, a.NT) * FB;
+        const uint8_t* src2 = src + (int64_t)a.NT * FB - FB;   // (the second fragment's piece at offset o >= FB is src2 + o)
         const uint32_t dst = ring_s + slot * UB;
 #pragma unroll
-        for (int p = 0; p < PIECES; ++p) cp_async16(dst + (p * 32 + lane) * 16, src + (p * 32 + lane) * 16, pol);
+        for (int p = 0; p < PIECES; ++p) {
+            const int o = (p * 32 + lane) * 16;
+            cp_async16(dst + o, (o < FB ? src : src2) + o, pol);
+        }
+        if (++Rc == a.NT) { Rc = 0; ++Pc; }
     };
 #pragma unroll
     for (int s = 0; s < GEMV_STAGES - 1; ++s) {
-        if (u0 + s < u1) issue(u0 + s, s);
+        if (u0 + s < u1) issue(s);
         cp_async_commit();
     }
 
@@ -80,7 +88,7 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32, 2) gemv_kernel(const GemvArgs
         {   // refill the slot freed by the previous iteration
             const int64_t un = u + GEMV_STAGES - 1;
             int ns = slot + GEMV_STAGES - 1; if (ns >= GEMV_STAGES) ns -= GEMV_STAGES;
-            if (un < u1) issue(un, ns);
+            if (un < u1) issue(ns);
             cp_async_commit();
         }
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -155,7 +163,7 @@ constexpr int ROWS_STAGES = 2;
 
 template <int BITS, int MT, bool BF16>
 __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_rows_kernel(const GemvArgs a) {
-    constexpr int UB = 2 * frag_bytes(BITS);
+    constexpr int FB = frag_bytes(BITS), UB = 2 * FB;
     constexpr int PIECES = UB / 16 / 32;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ float sums[8 * 16];   // [token][row of the tile]
@@ -167,10 +175,14 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_rows_kernel(const GemvAr
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     auto issue = [&](int P, int slot) {
-        const uint8_t* src = a.frags + ((int64_t)P * a.NT + R) * UB;
+        const uint8_t* src = a.frags + frag_index(2 * P, R, a.NT) * FB;
+        const uint8_t* src2 = src + (int64_t)a.NT * FB - FB;
         const uint32_t dst = ring_s + slot * UB;
 #pragma unroll
-        for (int p = 0; p < PIECES; ++p) cp_async16(dst + (p * 32 + lane) * 16, src + (p * 32 + lane) * 16, pol);
+        for (int p = 0; p < PIECES; ++p) {
+            const int o = (p * 32 + lane) * 16;
+            cp_async16(dst + o, (o < FB ? src : src2) + o, pol);
+        }
     };
 #pragma unroll
     for (int i = 0; i < ROWS_STAGES; ++i) {

@@ -1,4 +1,4 @@
-// Device code shared by the decode kernels (single linear and whole stack):
+// Device code of the single-linear decode kernels:
 // the x operand of one 256-k pair-slab, one unit (16 rows x 256 k) of
 // multiply-accumulate on the tensor cores, and the commit of a unit's sums.
 //
@@ -51,16 +51,6 @@ __device__ __forceinline__ float sum8(const uint4& v) {
         s += f.x + f.y;
     }
     return s;
-}
-
-// Where the 16-byte chunk (block bk, quarter t) of a one-token slab staged in shared memory lives: in the
-// row of the lane (bk, t) that multiplies it, at a position rotated by the lane
-// so that the eight chunks a lane reads never collide on a bank.
-__device__ __forceinline__ int ds_spread_offset(int lane, int bk) { return lane * 128 + ((bk ^ (lane & 7)) * 16); }
-// The same place as a shared-memory address: with the slab 128-byte aligned, chunk bk of a lane is at
-// (slab + lane * 128 + (lane & 7) * 16) ^ (bk * 16), one XOR with a constant per block.
-__device__ __forceinline__ uint32_t ds_spread_lane_base(const uint8_t* slab, int lane) {
-    return (uint32_t)__cvta_generic_to_shared(slab) + (uint32_t)(lane * 128 + (lane & 7) * 16);
 }
 
 // Per-warp state for the x operand of one pair-slab (256 k = the 8 blocks of a unit).
@@ -144,14 +134,8 @@ __device__ __forceinline__ constexpr bool class_used_before(int c, int b0, int b
 //   MT >= 2: [row g, col 2t], [row g, col 2t+1], [row g+8, col 2t], [row g+8, col 2t+1]
 //            (columns are (block slot, token) pairs, both columns in one slot)
 //   MT == 1: the same four, where columns 2t, 2t+1 are two different blocks.
-//
-// With XS (one token only) the B registers are not taken from xo.b but read, block by block, from the spread-out
-// copy of the slab in shared memory (xlane = ds_spread_lane_base of that copy): 32 registers fewer per thread for one
-// 16-byte shared load per block.
-template <int BITS, int MT, bool BF16, bool XS = false>
-__device__ __forceinline__ void unit_mac(const uint8_t* unit, const XOperand<MT>& xo, int lane, float (&acc)[4],
-                                         uint32_t xlane = 0) {
-    static_assert(!XS || MT == 1, "the shared-memory x operand is the one-token layout");
+template <int BITS, int MT, bool BF16>
+__device__ __forceinline__ void unit_mac(const uint8_t* unit, const XOperand<MT>& xo, int lane, float (&acc)[4]) {
     using IP = InPlace<BITS>;
     constexpr int FB = frag_bytes(BITS);
     constexpr int BG = XOperand<MT>::BG;
@@ -161,19 +145,14 @@ __device__ __forceinline__ void unit_mac(const uint8_t* unit, const XOperand<MT>
     float cs[NCLS][4];
     LaneCodes<BITS> lc;
     IP ip;
+    SlotWords<BITS> sw;
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
         const int fi = b >> 2, j = b & 3;
         if (j == 0) {
             load_lane_codes<BITS>(lc, unit + fi * FB, lane);
-            if constexpr (!BF16) ip.prepare(lc);
-        }
-        uint32_t xb[4];
-        if constexpr (XS) {
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(xb[0]), "=r"(xb[1]), "=r"(xb[2]), "=r"(xb[3]) : "r"(xlane ^ (uint32_t)(b * 16)));
-        } else {
-            xb[0] = xo.b[b][0]; xb[1] = xo.b[b][1]; xb[2] = xo.b[b][2]; xb[3] = xo.b[b][3];
+            if constexpr (BF16) sw.gather(lc);
+            else ip.prepare(lc);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -181,13 +160,13 @@ __device__ __forceinline__ void unit_mac(const uint8_t* unit, const XOperand<MT>
             uint32_t a[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                if constexpr (BF16) a[r] = code_pair<BITS>(lc, j, r & 1, 2 * h + (r >> 1), MAGIC);
+                if constexpr (BF16) a[r] = code_pair<BITS>(sw, j, r & 1, 2 * h + (r >> 1), MAGIC);
                 else a[r] = ip.reg(f, r);
             }
             // the first instruction of a group that touches an accumulator set starts it from zero
             const int k = BF16 ? 0 : IP::cls(f);
             const bool first = BF16 ? (b % BG == 0 && h == 0) : !class_used_before<BITS>(k, b - b % BG, b, h);
-            mma16816<BF16>(cs[k], a, xb[2 * h], xb[2 * h + 1], first);
+            mma16816<BF16>(cs[k], a, xo.b[b][2 * h], xo.b[b][2 * h + 1], first);
         }
         if (b % BG == BG - 1) {
             // group of blocks [b - BG + 1, b] done: take the powers of two out, apply scale and min

@@ -10,25 +10,23 @@
 //     bytes [256,FB) : codes.  Slot s = g*4 + t (g = row mod 8, t = 0..3) owns,
 //                      for rows g and g+8 and each block j, the 8 codes
 //                      8t .. 8t+7 of that block.
-//   unit     = fragments of k-slabs 2P and 2P+1 for one row tile, contiguous.
-//   order    = [pair-slab P][row tile R][slab parity] ; N padded to 16, K to 256.
+//   order    = [k-slab S][row tile R] ; N padded to 16, K to 256.  The fragments of
+//              neighbouring row tiles are contiguous: 128 rows x 128 k, what a tensor
+//              core instruction of 128 rows wants, is one copy of 8 fragments.
+//   unit     = the fragments of k-slabs 2P and 2P+1 of one row tile.
 //
-// A slot's 64 codes are 32 pairs (two k-adjacent codes of one row: the even
-// one in the low half of a 32-bit word, the odd one in the high half, at the
-// same bit position).  Pair (j, hi, i) -- block j, row half hi, codes 2i, 2i+1
-// of the slot -- feeds tensor-core instruction f = 2j + (i >> 1) as A register
-// r = hi + 2 (i & 1).  The four registers of one instruction sit in four
-// different words at the SAME bit position, so the instruction sees
-// 2^pos * q in every element and the power of two is taken out afterwards:
-//   2-bit: word r (4 words at 256 + s*16), field f at bit 2f of each half.
-//   4-bit: word (f >> 2)*4 + r (piece p = f >> 2 at 256 + p*512 + s*16), field
-//          f & 3 at bit 4 (f & 3).
-//   3-bit: words 0..3 ("r-words", at 256 + s*16) hold f = 0..4 at bit 3f of
-//          word r; words 4,5 ("e-words", at 768 + s*8) hold f = 5,6,7: register
-//          r of f = 5 at bit 3 (r >> 1) of e-word r & 1, of f = 6 at bit
-//          6 + 3 (r >> 1), of f = 7 (r < 2) at bit 12; registers 2,3 of f = 7
-//          are spread over bit 15 of words {0,1,2} and {3,4,5} (code bit b in
-//          the b-th word of the triple).
+// A slot's 64 codes are 16 groups of 4: group (j, hi, h) = codes 4h .. 4h+3 of the
+// slot's block j, row half hi.  The four codes of a group sit in the four bytes of
+// ONE word at the SAME bit position pos(j, h), in the byte order 0, 2, 1, 3: a mask
+// gives four 8-bit operands, and the low (or, after a shift by 8, the high) bytes of
+// the two half words give a pair of k-adjacent codes as two 16-bit operands.  Either
+// way the operand is 2^pos * q, and the power of two is taken out elsewhere.
+//   4-bit: word 2j + hi, pos 4h.
+//   2-bit: word 2 (j & 1) + hi, pos 4h + 2 (j >> 1).
+//   3-bit: word 2j + hi, pos 4h for j < 3; the words of j = 3 are spread over the
+//          free bits 3 and 7 of every byte: bit b of word 6 + x, pos 4h, is bit
+//          3 + 4h of word 3x + b.
+//   words 0..3 lie at 256 + s*16; words 4.. at 768 + s*8 (3-bit) or 768 + s*16.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -41,22 +39,19 @@ constexpr int SLAB = 128;       // k per fragment
 constexpr int SCALE_BYTES = 256;
 
 __host__ __device__ constexpr int frag_bytes(int bits) { return 256 * (bits + 1); }
+__host__ __device__ constexpr int64_t frag_index(int64_t S, int64_t R, int64_t NT) { return S * NT + R; }
 
 // Home of bit tb of code c (0..7) of the slot's block j, row half hi: the index
 // of the slot's 32-bit word and the bit position in it.
 __host__ __device__ inline void slot_bit_home(int bits, int j, int hi, int c, int tb, int& widx, int& bitpos) {
-    const int half = c & 1, i = c >> 1;
-    const int f = 2 * j + (i >> 1), r = hi + 2 * (i & 1);
+    const int h = c >> 2;
+    const int byte = (c & 1) * 2 + ((c >> 1) & 1);   // codes 0, 1, 2, 3 of a group: bytes 0, 2, 1, 3
     if (bits == 2) {
-        widx = r; bitpos = 16 * half + 2 * f + tb;
-    } else if (bits == 4) {
-        widx = (f >> 2) * 4 + r; bitpos = 16 * half + 4 * (f & 3) + tb;
+        widx = 2 * (j & 1) + hi; bitpos = 8 * byte + 4 * h + 2 * (j >> 1) + tb;
+    } else if (bits == 4 || j < 3) {
+        widx = 2 * j + hi; bitpos = 8 * byte + 4 * h + tb;
     } else {
-        if (f <= 4) { widx = r; bitpos = 16 * half + 3 * f + tb; }
-        else if (f == 5) { widx = 4 + (r & 1); bitpos = 16 * half + 3 * (r >> 1) + tb; }
-        else if (f == 6) { widx = 4 + (r & 1); bitpos = 16 * half + 6 + 3 * (r >> 1) + tb; }
-        else if (r < 2) { widx = 4 + r; bitpos = 16 * half + 12 + tb; }
-        else { widx = (r == 2 ? 0 : 3) + tb; bitpos = 16 * half + 15; }
+        widx = 3 * hi + tb; bitpos = 8 * byte + 4 * h + 3;
     }
 }
 
@@ -101,99 +96,58 @@ __device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t mask, uint3
     return d;
 }
 
+// The words the groups are read from: the lane's own ones, for 3 bits with the two spread words gathered behind them.
+template <int BITS> struct SlotWords {
+    static constexpr int N = BITS == 2 ? 4 : 8;
+    uint32_t w[N];
+    __device__ __forceinline__ void gather(const LaneCodes<BITS>& lc) {
+#pragma unroll
+        for (int i = 0; i < 2 * BITS; ++i) w[i] = lc.w[i];
+        if constexpr (BITS == 3) {
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const uint32_t* T = lc.w + 3 * x;
+                uint32_t v = (T[0] >> 3) & 0x11111111u;
+                v = lop3_and_or(T[1] >> 2, 0x22222222u, v);
+                w[6 + x] = lop3_and_or(T[2] >> 1, 0x44444444u, v);
+            }
+        }
+    }
+    static __device__ __forceinline__ constexpr int word(int j, int hi) { return BITS == 2 ? 2 * (j & 1) + hi : 2 * j + hi; }
+    static __device__ __forceinline__ constexpr int pos(int j, int h) { return BITS == 2 ? 4 * h + 2 * (j >> 1) : 4 * h; }
+};
+
 // Pair i (codes 2i, 2i+1) of block j, row half hi (0: row g, 1: row g+8): the
 // two codes land in bits [0,BITS) and [16,16+BITS) of the result, OR-ed with
 // `orv` (0 for plain integers, a floating-point exponent pattern otherwise).
-// The general (shift + mask) reader; the fp16 decode path reads in place instead.
 template <int BITS>
-__device__ __forceinline__ uint32_t code_pair(const LaneCodes<BITS>& lc, int j, int hi, int i, uint32_t orv) {
-    const int f = 2 * j + (i >> 1), r = hi + 2 * (i & 1);
-    if constexpr (BITS == 2) {
-        return lop3_and_or(lc.w[r] >> (2 * f), 0x00030003u, orv);
-    } else if constexpr (BITS == 4) {
-        return lop3_and_or(lc.w[(f >> 2) * 4 + r] >> (4 * (f & 3)), 0x000F000Fu, orv);
-    } else {
-        if (f <= 4) return lop3_and_or(lc.w[r] >> (3 * f), 0x00070007u, orv);
-        if (f == 5) return lop3_and_or(lc.w[4 + (r & 1)] >> (3 * (r >> 1)), 0x00070007u, orv);
-        if (f == 6) return lop3_and_or(lc.w[4 + (r & 1)] >> (6 + 3 * (r >> 1)), 0x00070007u, orv);
-        if (r < 2) return lop3_and_or(lc.w[4 + r] >> 12, 0x00070007u, orv);
-        const uint32_t* T = lc.w + (r == 2 ? 0 : 3);
-        uint32_t v = lop3_and_or(T[0] >> 15, 0x00010001u, orv);
-        v = lop3_and_or(T[1] >> 14, 0x00020002u, v);
-        v = lop3_and_or(T[2] >> 13, 0x00040004u, v);
-        return v;
-    }
+__device__ __forceinline__ uint32_t code_pair(const SlotWords<BITS>& sw, int j, int hi, int i, uint32_t orv) {
+    constexpr uint32_t MASK = (1u << BITS) - 1u;
+    return lop3_and_or(sw.w[sw.word(j, hi)] >> (8 * (i & 1) + sw.pos(j, i >> 1)), MASK | (MASK << 16), orv);
 }
 
 // ---- in-place reader (fp16 operands) ----------------------------------------
 // A code left at bit position s of a half-word, everything else masked away,
 // IS the binary16 subnormal q * 2^(s - 24) as long as s + BITS <= 10.  One AND
-// per A register; a byte shift of the whole word brings the upper fields into
-// the mantissa.  InPlace<BITS> holds a lane's words and their shifted copies.
-template <int BITS> struct InPlace;
-
-template <> struct InPlace<2> {
-    static constexpr int NCLS = 5;                           // bit positions 0,2,4,6,8
-    uint32_t w[4], w8[4];
-    __device__ __forceinline__ void prepare(const LaneCodes<2>& lc) {
+// per A register; a byte shift of the whole word brings the other pair of its
+// group into place.  A register r = hi + 2 (i & 1) of instruction f = 2j + h is
+// pair i = 2h + (r >> 1) of block j, row half hi.
+template <int BITS> struct InPlace {
+    static constexpr int NCLS = BITS == 2 ? 4 : 2;           // bit positions 0,2,4,6 / 0,4
+    uint32_t w[SlotWords<BITS>::N], w8[SlotWords<BITS>::N];
+    __device__ __forceinline__ void prepare(const LaneCodes<BITS>& lc) {
+        SlotWords<BITS> sw;
+        sw.gather(lc);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) { w[r] = lc.w[r]; w8[r] = lc.w[r] >> 8; }
+        for (int i = 0; i < SlotWords<BITS>::N; ++i) { w[i] = sw.w[i]; w8[i] = sw.w[i] >> 8; }
     }
-    static __device__ __forceinline__ constexpr int pos(int f) { return f <= 4 ? 2 * f : 2 * f - 8; }
-    static __device__ __forceinline__ constexpr int cls(int f) { return pos(f) / 2; }
-    static __device__ __forceinline__ constexpr int cls_pos(int c) { return 2 * c; }
+    static __device__ __forceinline__ constexpr int pos(int f) { return SlotWords<BITS>::pos(f >> 1, f & 1); }
+    static __device__ __forceinline__ constexpr int cls(int f) { return BITS == 2 ? pos(f) / 2 : pos(f) / 4; }
+    static __device__ __forceinline__ constexpr int cls_pos(int c) { return BITS == 2 ? 2 * c : 4 * c; }
     __device__ __forceinline__ uint32_t reg(int f, int r) const {
-        return (f <= 4 ? w[r] : w8[r]) & (0x00030003u << pos(f));
-    }
-};
-
-template <> struct InPlace<4> {
-    static constexpr int NCLS = 2;                           // bit positions 0,4
-    uint32_t w[8], w8[8];
-    __device__ __forceinline__ void prepare(const LaneCodes<4>& lc) {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) { w[r] = lc.w[r]; w8[r] = lc.w[r] >> 8; }
-    }
-    static __device__ __forceinline__ constexpr int pos(int f) { return 4 * (f & 1); }
-    static __device__ __forceinline__ constexpr int cls(int f) { return f & 1; }
-    static __device__ __forceinline__ constexpr int cls_pos(int c) { return 4 * c; }
-    __device__ __forceinline__ uint32_t reg(int f, int r) const {
-        const int k = (f >> 2) * 4 + r;
-        return ((f & 2) ? w8[k] : w[k]) & (0x000F000Fu << pos(f));
-    }
-};
-
-template <> struct InPlace<3> {
-    static constexpr int NCLS = 5;                           // bit positions 0,1,3,4,6
-    uint32_t w[4], w8[4], e[2], e3[2], e8[2], sc[2];
-    __device__ __forceinline__ void prepare(const LaneCodes<3>& lc) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) { w[r] = lc.w[r]; w8[r] = lc.w[r] >> 8; }
-#pragma unroll
-        for (int x = 0; x < 2; ++x) { e[x] = lc.w[4 + x]; e3[x] = lc.w[4 + x] >> 3; e8[x] = lc.w[4 + x] >> 8; }
-        // the two pairs spread over bit 15 of three words each, gathered at bit position 4
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const uint32_t* T = lc.w + 3 * x;
-            uint32_t v = (T[0] >> 11) & 0x00100010u;
-            v = lop3_and_or(T[1] >> 10, 0x00200020u, v);
-            v = lop3_and_or(T[2] >> 9, 0x00400040u, v);
-            sc[x] = v;
-        }
-    }
-    static __device__ __forceinline__ constexpr int pos(int f) {
-        return f <= 2 ? 3 * f : f == 3 ? 1 : f == 4 ? 4 : f == 5 ? 0 : f == 6 ? 6 : 4;
-    }
-    static __device__ __forceinline__ constexpr int cls(int f) {
-        return pos(f) == 0 ? 0 : pos(f) == 1 ? 1 : pos(f) == 3 ? 2 : pos(f) == 4 ? 3 : 4;
-    }
-    static __device__ __forceinline__ constexpr int cls_pos(int c) { return c == 0 ? 0 : c == 1 ? 1 : c == 2 ? 3 : c == 3 ? 4 : 6; }
-    __device__ __forceinline__ uint32_t reg(int f, int r) const {
-        const uint32_t m = 0x00070007u << pos(f);
-        if (f <= 2) return w[r] & m;
-        if (f <= 4) return w8[r] & m;
-        if (f <= 6) return (r < 2 ? e[r] : e3[r - 2]) & m;
-        return r < 2 ? (e8[r] & m) : sc[r - 2];
+        constexpr uint32_t MASK = ((1u << BITS) - 1u) * 0x00010001u;
+        const int k = SlotWords<BITS>::word(f >> 1, r & 1);
+        return ((r >> 1) ? w8[k] : w[k]) & (MASK << pos(f));
     }
 };
 

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(128) pack_kernel(const float* __restrict__ W, 
     const int64_t u = f >> 1;
     const int R = (int)(u % NT);
     const int64_t S = 2 * (u / NT) + par;
-    uint8_t* fb = frags + f * FB;
+    uint8_t* fb = frags + frag_index(S, R, NT) * FB;
 
     uint32_t words[2 * BITS];
 #pragma unroll
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(128) pack_opt_kernel(const float* __restrict__
     const int64_t u = f >> 1;
     const int R = (int)(u % NT);
     const int64_t S = 2 * (u / NT) + par;
-    uint8_t* fb = frags + f * FB;
+    uint8_t* fb = frags + frag_index(S, R, NT) * FB;
 
     uint32_t words[2 * BITS];
 #pragma unroll
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(128) import_kernel(const uint8_t* __restrict__
     const int R = (int)(u % NT);
     const int64_t S = 2 * (u / NT) + par;
     const int64_t nb = K / 32;
-    uint8_t* fb = frags + f * FB;
+    uint8_t* fb = frags + frag_index(S, R, NT) * FB;
     uint32_t words[2 * BITS];
 #pragma unroll
     for (int i = 0; i < 2 * BITS; ++i) words[i] = 0;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(128) export_kernel(const uint8_t* __restrict__
     const int j = (int)(jb & 3), r = (int)(row & 15);
     const int64_t R = row >> 4;
     const int FB = frag_bytes(bits);
-    const uint8_t* fb = frags + (((S >> 1) * NT + R) * 2 + (S & 1)) * FB;
+    const uint8_t* fb = frags + frag_index(S, R, NT) * FB;
     const int rec_bytes = 4 + 4 * bits;
     uint8_t* rec = canon + idx * rec_bytes;
     const uint32_t dm = *reinterpret_cast<const uint32_t*>(fb + (r * 4 + j) * 4);

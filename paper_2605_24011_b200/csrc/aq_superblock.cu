@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(128) pack_sb_kernel(const float* __restrict__ 
                 if (jj == t) my_dm = (uint32_t)__half_as_ushort(dh) | ((uint32_t)__half_as_ushort(mh) << 16);
             }
             // this half of the lane's words: the other row half's bits are OR-ed in by the second pass over hi
-            uint8_t* fb = frags + (un * 2 + fi) * FB;
+            uint8_t* fb = frags + frag_index(2 * P + fi, R, NT) * FB;
             uint32_t* w0 = reinterpret_cast<uint32_t*>(fb + 256 + lane * 16);
             if (hi == 0) {
 #pragma unroll

@@ -1,0 +1,62 @@
+"""The one-launch decode kernel at the edges of its tiles and of its dispatch, op by op against the oracle.
+
+A unit is 128 rows x 256 k, a CTA's row tile of 128 rows may hold 1 to 8 fragments of 16, a row of a normalised input is
+kept in registers up to 4096 elements (one token), read whole by every CTA up to 16384 elements (M K) and summed from
+shares above that."""
+import numpy as np
+import pytest
+
+from oracle import aq_oracle as O
+from paper_2605_24011_b200 import synth
+from stack_check import check_program
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _run(M, K, N, dtype, bits, spread):
+    from paper_2605_24011_b200 import aq
+    # x0 [96] -> h [K]; two linears on rmsnorm(h) (one phase); silu(g) * u -> h + W (..): every glue, sources packed
+    shapes = [("in", K, 96), ("g", N, K), ("u", N, K), ("out", K, N), ("p", 40, K)]
+    handles, quant = {}, {}
+    for i, (nm, n, k) in enumerate(shapes):
+        W = synth.weights(n, k, 91, M, K, N, i, outliers=True)
+        b = bits[i % len(bits)]
+        handles[nm] = aq.aq_pack(b, 32, torch.from_numpy(W).cuda())
+        quant[(0, nm)] = O.quantize(W, b)
+    widths = [96, K, N, N, K, 40]
+    ops = [{"w": handles["in"], "src": 0, "dst": 1},
+           {"w": handles["g"], "src": 1, "dst": 2, "in_op": aq.AQ_IN_RMSNORM},
+           {"w": handles["u"], "src": 1, "dst": 3, "in_op": aq.AQ_IN_RMSNORM},
+           {"w": handles["out"], "src": 2, "src2": 3, "dst": 4, "in_op": aq.AQ_IN_SILU_MUL, "out_op": aq.AQ_OUT_ADD, "res": 1},
+           {"w": handles["p"], "src": 4, "dst": 5}]
+    prog = aq.Program(widths, ops)
+    tdt = torch.float16 if dtype == "f16" else torch.bfloat16
+    x = synth.activations(M, 96, 92, M, K) * 8.0
+    if spread:   # magnitudes of one block from 2^-12 to 2^4 of each other
+        x *= np.exp2(np.linspace(-12, 4, 96, dtype=np.float32))[None, ::-1]
+    x0 = torch.from_numpy(x).to(tdt).cuda()
+    ws = torch.empty(prog.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+    out = torch.empty((M, 40), dtype=tdt, device="cuda")
+    for _ in range(2):   # the second pass reuses the tables and the workspace
+        aq.aq_stack_forward(prog, x0, out, 5, M, ws)
+    aq.aq_check()
+    check_program(prog, [(0, nm) for nm, _, _ in shapes], ws, M, tdt, quant)
+    assert torch.equal(out, aq.stack_buffer(prog, ws, M, 5).to(tdt))
+
+
+@pytest.mark.parametrize("M,K", [(1, 4096), (1, 4128), (2, 4096), (2, 8224), (3, 5440), (3, 5472), (5, 3264), (5, 3296), (8, 2048), (8, 2080)])
+def test_row_norm_paths(M, K):
+    _run(M, K, 224, "f16", (2, 3, 4), False)
+
+
+@pytest.mark.parametrize("N", (32, 128, 160, 1152))
+@pytest.mark.parametrize("M,dtype", [(1, "f16"), (1, "bf16"), (4, "f16"), (8, "bf16")])
+def test_row_tiles(M, dtype, N):
+    _run(M, 288, N, dtype, (4, 2, 3), False)
+
+
+@pytest.mark.parametrize("bits", (2, 3, 4))
+@pytest.mark.parametrize("M,dtype", [(1, "f16"), (1, "bf16"), (2, "f16"), (6, "bf16")])
+def test_wide_magnitudes(M, dtype, bits):
+    _run(M, 512, 96, dtype, (bits,), True)
