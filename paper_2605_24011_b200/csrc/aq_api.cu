@@ -73,19 +73,27 @@ static aq_status_t new_handle(int bits, int block, int64_t N, int64_t K, aq_hand
     h->frags = nullptr; h->acc = nullptr; h->flags = nullptr; h->last_stream = nullptr;
     h->big = nullptr; h->big_bytes = 0; h->sb = nullptr;
     const size_t acc_bytes = (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float);
-    if (cudaMalloc(&h->frags, h->dev_bytes) != cudaSuccess || cudaMalloc(&h->acc, acc_bytes) != cudaSuccess ||
-        cudaMalloc(&h->flags, 256) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(h->frags); cudaFree(h->acc); cudaFree(h->flags);
-        delete h;
-        return AQ_ERR_ALLOC;
-    }
+    // one block: fragments, accumulators, flags (the last two start at zero: see clear_scratch)
+    const size_t frag_end = (h->dev_bytes + 255) / 256 * 256, acc_end = frag_end + (acc_bytes + 255) / 256 * 256;
+    h->block_bytes = acc_end + 256;
+    h->frags = static_cast<uint8_t*>(device_alloc(h->block_bytes, dev));
+    if (!h->frags) { delete h; return AQ_ERR_ALLOC; }
+    h->acc = reinterpret_cast<float*>(h->frags + frag_end);
+    h->flags = reinterpret_cast<int*>(h->frags + acc_end);
     *out = h;
     return AQ_OK;
 }
 
+static size_t sb_side_bytes(const aq_handle_s* h) { return (size_t)h->N * (size_t)(h->K / 256) * 32; }
+
+static cudaError_t clear_scratch(const aq_handle_s* h, cudaStream_t s) {
+    return cudaMemsetAsync(h->acc, 0, h->block_bytes - (size_t)(reinterpret_cast<uint8_t*>(h->acc) - h->frags), s);
+}
+
 static void destroy(aq_handle_s* h) {
-    cudaFree(h->frags); cudaFree(h->acc); cudaFree(h->flags); cudaFree(h->big); cudaFree(h->sb);
+    if (h->big) cudaFree(h->big);
+    device_release(h->sb, sb_side_bytes(h), h->device);
+    device_release(h->frags, h->block_bytes, h->device);
     h->magic = 0;
     delete h;
 }
@@ -105,8 +113,7 @@ aq_status_t aq_pack(int bits, int block, const float* W_dev, int64_t N, int64_t 
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(h->acc, 0, (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, 256, s);
+    cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack(h, W_dev, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
@@ -123,8 +130,7 @@ aq_status_t aq_pack_opt(int bits, int block, const float* W_dev, const float* F_
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(h->acc, 0, (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, 256, s);
+    cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack_opt(h, W_dev, F_dev, rounds, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
@@ -142,7 +148,8 @@ static aq_status_t new_sb_handle(int bits, int block, int sblock, int64_t N, int
     aq_handle_t h = nullptr;
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
-    if (cudaMalloc(&h->sb, (size_t)N * (size_t)(K / 256) * 32) != cudaSuccess) { cudaGetLastError(); destroy(h); return AQ_ERR_ALLOC; }
+    h->sb = static_cast<uint8_t*>(device_alloc(sb_side_bytes(h), h->device));
+    if (!h->sb) { destroy(h); return AQ_ERR_ALLOC; }
     *out = h;
     return AQ_OK;
 }
@@ -156,8 +163,7 @@ aq_status_t aq_pack_sb(int bits, int block, int sblock, const float* W_dev, int6
     aq_status_t st = new_sb_handle(bits, block, sblock, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(h->acc, 0, (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, 256, s);
+    cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack_sb(h, W_dev, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
@@ -177,15 +183,14 @@ aq_status_t aq_import_sb(int bits, int block, int sblock, int64_t N, int64_t K, 
     cudaStream_t s = (cudaStream_t)stream;
     const size_t plain_bytes = (size_t)N * (size_t)(K / 32) * (size_t)(4 + 4 * bits);
     const size_t plain_at = (nbytes + 255) / 256 * 256;
-    uint8_t* tmp = nullptr;
-    if (cudaMalloc(&tmp, plain_at + plain_bytes) != cudaSuccess) { cudaGetLastError(); destroy(h); return AQ_ERR_ALLOC; }
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device));
+    if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->acc, 0, (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, 256, s);
+    if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, true, s);
     if (e == cudaSuccess) e = launch_import(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    device_release(tmp, plain_at + plain_bytes, h->device);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
     *out = h;
@@ -202,14 +207,13 @@ aq_status_t aq_import(int bits, int block, int64_t N, int64_t K, const void* can
     if (st != AQ_OK) return st;
     if (nbytes != (size_t)N * (size_t)(K / 32) * (size_t)(4 + 4 * bits)) { destroy(h); return AQ_ERR_INVALID_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    uint8_t* tmp = nullptr;
-    if (cudaMalloc(&tmp, nbytes) != cudaSuccess) { cudaGetLastError(); destroy(h); return AQ_ERR_ALLOC; }
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(nbytes, h->device));
+    if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->acc, 0, (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, 256, s);
+    if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_import(h, tmp, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    device_release(tmp, nbytes, h->device);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
     *out = h;
@@ -230,13 +234,12 @@ aq_status_t aq_export(aq_handle_t h, void* canon_host, size_t cap, size_t* nbyte
     if (nbytes) *nbytes = need;
     if (!canon_host) return nbytes ? AQ_OK : AQ_ERR_INVALID_ARG;
     if (cap < need) return AQ_ERR_INVALID_ARG;
-    uint8_t* tmp = nullptr;
-    if (cudaMalloc(&tmp, need) != cudaSuccess) { cudaGetLastError(); return AQ_ERR_ALLOC; }
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(need, h->device));
+    if (!tmp) return AQ_ERR_ALLOC;
     cudaStream_t s = h->last_stream;
     cudaError_t e = launch_export(h, tmp, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(canon_host, tmp, need, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
+    device_release(tmp, need, h->device);
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }
@@ -249,14 +252,13 @@ aq_status_t aq_export_sb(aq_handle_t h, void* canon_host, size_t cap, size_t* nb
     if (cap < need) return AQ_ERR_INVALID_ARG;
     const size_t plain_bytes = (size_t)h->N * (size_t)(h->K / 32) * (size_t)(4 + 4 * h->bits);
     const size_t plain_at = (need + 255) / 256 * 256;
-    uint8_t* tmp = nullptr;
-    if (cudaMalloc(&tmp, plain_at + plain_bytes) != cudaSuccess) { cudaGetLastError(); return AQ_ERR_ALLOC; }
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device));
+    if (!tmp) return AQ_ERR_ALLOC;
     cudaStream_t s = h->last_stream;
     cudaError_t e = launch_export(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, false, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(canon_host, tmp, need, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(tmp);
+    if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
+    device_release(tmp, plain_at + plain_bytes, h->device);
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }

@@ -19,6 +19,7 @@ struct aq_handle_s {
     int KP;            // pair slabs of 256 k
     int64_t n_frags;   // NT * KP * 2
     size_t dev_bytes;  // n_frags * frag_bytes
+    size_t block_bytes;   // of the one device block that holds frags, acc and flags
     uint8_t* frags;    // DEVICE: fragment layout
     float* acc;        // DEVICE: [AQ_DECODE_MAX_M][NT*16] accumulation scratch, zero between calls
     uint8_t* sb;       // DEVICE: super-block parameters (32 bytes per row and super-block) of a handle made by aq_pack_sb /
@@ -142,6 +143,12 @@ cudaError_t launch_rope(void* x, int n_heads, int D, int64_t pos, float theta, a
 cudaError_t launch_attn_prepare(const float* q, const float* k, const float* v, void* q16, void* kc, void* vc, int M, int H, int Hkv,
                                 int64_t pos, int64_t Lmax, float theta, aq_dtype_t dt, cudaStream_t s);
 cudaError_t launch_kv_append(void* kc, void* vc, const void* k, const void* v, int n_kv, int D, int64_t pos, int64_t Lmax, cudaStream_t s);
+
+// memory (aq_memory.cu): device blocks out of a bounded cache (null: no memory left); a copy into pageable host memory, complete
+// when the call returns
+void* device_alloc(size_t bytes, int device);
+void device_release(void* p, size_t bytes, int device);
+cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t s);
 
 int current_device();               // cudaGetDevice, or -1
 int sm_count();                     // of the current device
