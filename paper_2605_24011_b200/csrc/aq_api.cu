@@ -1,8 +1,8 @@
 // C-ABI entry points of libaq: argument checks, handle ownership, dispatch.
 #include <cmath>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
+#include <cstdlib>
 #include <atomic>
 #include <new>
 
@@ -91,7 +91,7 @@ static cudaError_t clear_scratch(const aq_handle_s* h, cudaStream_t s) {
 }
 
 static void destroy(aq_handle_s* h) {
-    if (h->big) cudaFree(h->big);
+    device_release(h->big, h->big_bytes, h->device);
     device_release(h->sb, sb_side_bytes(h), h->device);
     device_release(h->frags, h->block_bytes, h->device);
     h->magic = 0;
@@ -302,32 +302,28 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
             if (e == cudaSuccess) e = launch_finalize(h->acc, h->acc, ld, y_dev, ydt, M, h->N, s);
         }
     } else {
-        // scratch owned by the handle: float32 sums when the output is half precision, the binary16 copy of bfloat16
-        // activations with its row scales and flag; allocated on the first such call and when a later one needs more
+        // scratch owned by the handle: float32 sums when the output is half precision, the activations in operand order,
+        // for bfloat16 with row scales; allocated on the first such call and when a later one needs more
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t out_bytes = (ydt == AQ_F32) ? 0 : up((size_t)M * h->N * sizeof(float));
-        const size_t x16_bytes = (xdt == AQ_BF16) ? up((size_t)M * h->K * 2) : 0;
-        const size_t rs_bytes = (xdt == AQ_BF16) ? up((size_t)M * sizeof(float) + 16) : 0;
+        const size_t x16_bytes = up((size_t)M * h->K * 2);
+        const size_t rs_bytes = (xdt == AQ_BF16) ? up((size_t)M * sizeof(float)) : 0;
         const size_t need = out_bytes + x16_bytes + rs_bytes;
         if (need > h->big_bytes) {
-            cudaFree(h->big);   // (waits for whatever still uses the old one)
-            h->big = nullptr; h->big_bytes = 0;
-            if (cudaMalloc(&h->big, need) != cudaSuccess) { cudaGetLastError(); return AQ_ERR_ALLOC; }
+            device_release(h->big, h->big_bytes, h->device);   // (waits for whatever still uses the old one)
+            h->big_bytes = 0;
+            h->big = static_cast<uint8_t*>(device_alloc(need, h->device));
+            if (!h->big) return AQ_ERR_ALLOC;
             h->big_bytes = need;
         }
         float* sums = (ydt == AQ_F32) ? (float*)y_dev : reinterpret_cast<float*>(h->big);
-        const void* xop = x_dev;
-        const float* rs = nullptr;
-        const int* flag = nullptr;
-        e = cudaSuccess;
-        if (xdt == AQ_BF16) {
-            void* x16 = h->big + out_bytes;
-            float* rsw = reinterpret_cast<float*>(h->big + out_bytes + x16_bytes);
-            int* fw = reinterpret_cast<int*>(h->big + out_bytes + x16_bytes + (size_t)M * sizeof(float));
-            e = launch_rows_to_f16(x_dev, x16, rsw, fw, M, h->K, s);
-            xop = x16; rs = rsw; flag = fw;
-        }
-        if (e == cudaSuccess) e = launch_gemm(h, xop, rs, flag, M, sums, h->N, nullptr, s);
+        void* x16 = h->big + out_bytes;
+        float* rs = (xdt == AQ_BF16) ? reinterpret_cast<float*>(h->big + out_bytes + x16_bytes) : nullptr;
+        const aq_handle_s* hc = h;
+        const int64_t ldo = h->N;
+        const bool preset = !gemm_stores_first(&hc, 1, M, s) && gemm_outputs_can_be_preset(&sums, &ldo, 1);
+        e = launch_operand_rows(x_dev, xdt, x16, rs, M, h->K, preset ? sums : nullptr, h->N, s);
+        if (e == cudaSuccess) e = launch_gemm(h, x16, rs, M, sums, h->N, preset, s);
         if (e == cudaSuccess && ydt != AQ_F32) e = launch_finalize(sums, nullptr, h->N, y_dev, ydt, M, h->N, s);
     }
     if (e != cudaSuccess) return cuda_fail(e);

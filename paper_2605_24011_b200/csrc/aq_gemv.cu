@@ -264,29 +264,42 @@ cudaError_t launch_gemv(const aq_handle_s* h, const void* x, aq_dtype_t xdt, int
     }
 }
 
-// y = cast(acc) for the first N columns of each row, then acc = 0.
+// y = cast(acc) for the first N columns of each row, then acc = 0.  Four elements per thread; blockIdx.y is the row.
 template <typename T>
-__global__ void finalize_kernel(const float* __restrict__ acc_in, float* __restrict__ acc_zero, int64_t ld,
-                                T* __restrict__ y, int M, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)M * N) return;
-    const int64_t m = i / N, n = i - m * N;
-    const float v = acc_in[m * ld + n];
-    if constexpr (sizeof(T) == 4) y[i] = v;
-    else if constexpr (std::is_same<T, __half>::value) y[i] = __float2half_rn(v);
-    else y[i] = __float2bfloat16_rn(v);
-    if (acc_zero) acc_zero[m * ld + n] = 0.f;
+__global__ void __launch_bounds__(256) finalize_kernel(const float* __restrict__ acc_in, float* __restrict__ acc_zero, int64_t ld, T* __restrict__ y, int64_t N) {
+    pdl_wait();   // the sums are the predecessor's output
+    const int64_t m = blockIdx.y, n = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
+    if (n >= N) return;
+    const float* a = acc_in + m * ld + n;
+    T* o = y + m * N + n;
+    auto cast = [](float v) -> T {
+        if constexpr (std::is_same<T, __half>::value) return __float2half_rn(v);
+        else if constexpr (std::is_same<T, __nv_bfloat16>::value) return __float2bfloat16_rn(v);
+        else return v;
+    };
+    if (((ld | N) & 3) == 0) {   // (rows of both stay aligned to four elements)
+        const float4 v = *reinterpret_cast<const float4*>(a);
+        struct __align__(4 * sizeof(T)) Four { T t[4]; } r;
+        r.t[0] = cast(v.x); r.t[1] = cast(v.y); r.t[2] = cast(v.z); r.t[3] = cast(v.w);
+        *reinterpret_cast<Four*>(o) = r;
+        if (acc_zero) *reinterpret_cast<float4*>(acc_zero + m * ld + n) = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
+    for (int i = 0; i < 4 && n + i < N; ++i) {
+        o[i] = cast(a[i]);
+        if (acc_zero) acc_zero[m * ld + n + i] = 0.f;
+    }
 }
 
 cudaError_t launch_finalize(const float* acc_in, float* acc_zero, int64_t ldacc, void* y, aq_dtype_t ydt, int M,
                             int64_t N, cudaStream_t s) {
-    const int64_t n = (int64_t)M * N;
-    const unsigned grid = (unsigned)((n + 255) / 256);
-    if (ydt == AQ_F16) finalize_kernel<__half><<<grid, 256, 0, s>>>(acc_in, acc_zero, ldacc, (__half*)y, M, N);
-    else if (ydt == AQ_BF16) finalize_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(acc_in, acc_zero, ldacc, (__nv_bfloat16*)y, M, N);
-    else finalize_kernel<float><<<grid, 256, 0, s>>>(acc_in, acc_zero, ldacc, (float*)y, M, N);
+    const dim3 grid((unsigned)((N + 1023) / 1024), (unsigned)M);
+    cudaError_t e;
+    if (ydt == AQ_F16) e = launch_pdl(finalize_kernel<__half>, grid, dim3(256), 0, s, acc_in, acc_zero, ldacc, (__half*)y, N);
+    else if (ydt == AQ_BF16) e = launch_pdl(finalize_kernel<__nv_bfloat16>, grid, dim3(256), 0, s, acc_in, acc_zero, ldacc, (__nv_bfloat16*)y, N);
+    else e = launch_pdl(finalize_kernel<float>, grid, dim3(256), 0, s, acc_in, acc_zero, ldacc, (float*)y, N);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace aq

@@ -56,19 +56,17 @@ cudaError_t launch_gemv(const aq_handle_s* h, const void* x, aq_dtype_t xdt, int
 cudaError_t launch_finalize(const float* acc_in, float* acc_zero, int64_t ldacc, void* y, aq_dtype_t ydt,
                             int M, int64_t N, cudaStream_t s);
 
-// prefill path: out[m][n] = (res ? res[m][n] : 0) + tok_scale[m] sum_k x16[m][k] w[n][k]; x16 binary16 [M][K];
-// tok_scale (with its flag, see launch_rows_to_f16) or null; out, res fp32 [M][ldo];
-// out need not be initialised (the launcher zeroes it when tiles are split over CTAs)
-cudaError_t launch_gemm(const aq_handle_s* h, const void* x16, const float* tok_scale, const int* scaled_flag, int M, float* out,
-                        int64_t ldo, const float* res, cudaStream_t s);
-// bfloat16 rows -> the binary16 operand of the GEMM, the per-row power of two they were divided by (1 unless a row
-// leaves binary16's range) and a flag that says whether any row has one
-cudaError_t launch_rows_to_f16(const void* x_bf16, void* x16, float* scale, int* flag, int M, int64_t K, cudaStream_t s);
+// prefill path: out[m][n] = (res ? res[m][n] : 0) + tok_scale[m] sum_k x[m][k] w[n][k]; x16 is x as binary16 [M][K] in operand
+// order (aq_tmem.cuh); tok_scale (see launch_operand_rows) or null; out, res fp32 [M][ldo];
+// with out_ready the caller has zeroed out where gemm_stores_first() is false, else the launcher does
+cudaError_t launch_gemm(const aq_handle_s* h, const void* x16, const float* tok_scale, int M, float* out, int64_t ldo, bool out_ready, cudaStream_t s);
+// rows of either type -> the operand of the GEMM; for bfloat16 also the per-row power of two they were divided by (1 unless a
+// row leaves binary16's range).  zero (or null): [M][zero_width] floats set to zero on the way (zero_width a multiple of 4)
+cudaError_t launch_operand_rows(const void* x, aq_dtype_t dt, void* x16, float* scale, int M, int64_t K, float* zero, int64_t zero_width, cudaStream_t s);
 // the same for up to AQ_GEMM_MAX_GROUP matrices of one K that read the same x, as one launch
 #define AQ_GEMM_MAX_GROUP 4
-cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x16, const float* tok_scale, const int* scaled_flag,
-                              int M, float* const* outs, const int64_t* ldos, const float* const* ress, bool outs_ready,
-                              cudaStream_t s);
+cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x16, const float* tok_scale, int M, float* const* outs,
+                              const int64_t* ldos, const float* const* ress, bool outs_ready, cudaStream_t s);
 bool gemm_outputs_can_be_preset(float* const* outs, const int64_t* ldos, int n);
 bool gemm_stores_first(const aq_handle_s* const* hs, int n, int M, cudaStream_t s);   // then only residuals need presetting
 
@@ -87,8 +85,6 @@ struct StackPlan {
                                     // partial sums of squares [AQ_NORM_MAX_CTAS][M] of 8 bytes, inside the region above; else 0
     std::vector<size_t> x16_off;    // per op (bfloat16, M > AQ_DECODE_MAX_M only): its phase's binary16 operand [M][K] ...
     std::vector<size_t> rs_off;     // ... the row scales [M] float32 ...
-    std::vector<size_t> flag_off;   // ... and the phase's "some row is scaled" flag (int), inside [flags_begin, flags_end)
-    size_t flags_begin = 0, flags_end = 0;
     size_t stage_off = 0;           // end of the float32 buffers
     size_t total = 0;
 };

@@ -149,6 +149,11 @@ template <int BITS> struct InPlace {
         const int k = SlotWords<BITS>::word(f >> 1, r & 1);
         return ((r >> 1) ? w8[k] : w[k]) & (MASK << pos(f));
     }
+    __device__ __forceinline__ uint32_t reg_or(int f, int r, uint32_t orv) const {
+        constexpr uint32_t MASK = ((1u << BITS) - 1u) * 0x00010001u;
+        const int k = SlotWords<BITS>::word(f >> 1, r & 1);
+        return lop3_and_or((r >> 1) ? w8[k] : w[k], MASK << pos(f), orv);
+    }
 };
 
 }  // namespace aq

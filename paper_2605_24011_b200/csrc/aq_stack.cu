@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "aq_internal.h"
+#include "aq_tmem.cuh"
 
 namespace aq {
 
@@ -66,16 +67,11 @@ static bool plan_stack(const aq_stack_t* p, int M, StackPlan& plan) {
     if (M > AQ_DECODE_MAX_M) {   // bfloat16 activations reach the tensor cores as binary16: a second staged vector per phase
         plan.x16_off.assign(p->n_ops, 0);
         plan.rs_off.assign(p->n_ops, 0);
-        plan.flag_off.assign(p->n_ops, 0);
-        plan.flags_begin = off;          // one int per phase, together: a single memset clears them
-        off += align_up((size_t)p->n_ops * sizeof(int), 256);
-        plan.flags_end = off;
         for (int i = 0; i < p->n_ops; ++i) {
             if (i > 0 && same_input(p->ops[i], p->ops[i - 1])) {
-                plan.x16_off[i] = plan.x16_off[i - 1]; plan.rs_off[i] = plan.rs_off[i - 1]; plan.flag_off[i] = plan.flag_off[i - 1];
+                plan.x16_off[i] = plan.x16_off[i - 1]; plan.rs_off[i] = plan.rs_off[i - 1];
                 continue;
             }
-            plan.flag_off[i] = plan.flags_begin + (size_t)i * sizeof(int);
             plan.x16_off[i] = off;
             off += align_up((size_t)M * p->buf_width[p->ops[i].src] * 2, 256);
             plan.rs_off[i] = off;
@@ -124,48 +120,63 @@ __global__ void narrow_kernel(const float* __restrict__ x, T* __restrict__ out, 
 
 // Rounds four values and stores them as one 8-byte word.
 template <typename T>
-__device__ __forceinline__ void store_round4(T* o, const float4& v) {
+__device__ __forceinline__ uint2 store_round4(T* o, const float4& v) {
     const T a = from_f32<T>(v.x), b = from_f32<T>(v.y), c = from_f32<T>(v.z), d = from_f32<T>(v.w);
     uint2 r;
     r.x = (uint32_t)*reinterpret_cast<const uint16_t*>(&a) | ((uint32_t)*reinterpret_cast<const uint16_t*>(&b) << 16);
     r.y = (uint32_t)*reinterpret_cast<const uint16_t*>(&c) | ((uint32_t)*reinterpret_cast<const uint16_t*>(&d) << 16);
     *reinterpret_cast<uint2*>(o) = r;
+    return r;
 }
 
-// x[m][k] = round(transform(src[m][k])); K is a multiple of 32, rows are 16-byte aligned.
+// x[m][k] = round(transform(src[m][k])); K is a multiple of 32, rows are 16-byte aligned.  x16 (or null): the same values in
+// the GEMM's operand order.
 // RMS scaling: one CTA per token row.  The other two forms have no row-wide term and
 // run as a flat grid over groups of four elements (blockIdx.y = 0).
 // Outputs the linears of a phase will add into: dst = src (the residual) or zero, n4 groups of four floats each.
+// CTAs from blockIdx.x = first on do this and nothing else.
 struct PresetList {
     float4* dst[8];
     const float4* src[8];
     int64_t n4[8];
     int n;
+    unsigned first;
+    unsigned ctas() const {   // enough to write a few megabytes at the rate of the device: four groups of four per thread
+        int64_t t = 0;
+        for (int q = 0; q < n; ++q) t += n4[q];
+        return (unsigned)std::min<int64_t>((t + 1023) / 1024, 2 * 148);
+    }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(256) stage_kernel(const float* __restrict__ src, const float* __restrict__ src2,
-                                                    int in_op, int64_t K, int64_t total4, T* __restrict__ x,
-                                                    const PresetList pre) {
-    pdl_wait();                 // the buffers read and preset here belong to the kernels before this one
-    pdl_launch_dependents();    // the linears of this phase may set themselves up meanwhile
+__device__ __forceinline__ void write_presets(const PresetList& pre) {
+    const int64_t step = (int64_t)(gridDim.x - pre.first) * 256;
     for (int q = 0; q < pre.n; ++q) {
         float4* d = pre.dst[q];
         const float4* r = pre.src[q];
-        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < pre.n4[q]; i += (int64_t)gridDim.x * 256)
+        for (int64_t i = (int64_t)(blockIdx.x - pre.first) * 256 + threadIdx.x; i < pre.n4[q]; i += step)
             d[i] = r ? r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) stage_kernel(const float* __restrict__ src, const float* __restrict__ src2,
+                                                    int in_op, int64_t K, int64_t total4, T* __restrict__ x, __half* __restrict__ x16,
+                                                    const PresetList pre) {
+    pdl_wait();                 // the buffers read and preset here belong to the kernels before this one
+    pdl_launch_dependents();    // the linears of this phase may set themselves up meanwhile
+    if (blockIdx.x >= pre.first) { write_presets(pre); return; }
     if (in_op != AQ_IN_RMSNORM) {
         const float4* s4 = reinterpret_cast<const float4*>(src);
         const float4* t4 = reinterpret_cast<const float4*>(src2);
-        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total4; i += (int64_t)gridDim.x * 256) {
+        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total4; i += (int64_t)pre.first * 256) {
             float4 v = s4[i];
             if (in_op == AQ_IN_SILU_MUL) {
                 const float4 u = t4[i];
                 v.x = v.x / (1.f + expf(-v.x)) * u.x; v.y = v.y / (1.f + expf(-v.y)) * u.y;
                 v.z = v.z / (1.f + expf(-v.z)) * u.z; v.w = v.w / (1.f + expf(-v.w)) * u.w;
             }
-            store_round4<T>(x + 4 * i, v);
+            const uint2 r = store_round4<T>(x + 4 * i, v);
+            if (x16) store_operand4(x16 + (4 * i / K) * K, 4 * i % K, r);
         }
         return;
     }
@@ -189,26 +200,21 @@ __global__ void __launch_bounds__(256) stage_kernel(const float* __restrict__ sr
     const float scale = rsqrtf(tot / (float)K + 1e-6f);
     for (int64_t k = threadIdx.x; k < q4; k += 256) {
         const float4 v = s4[k];
-        store_round4<T>(o + 4 * k, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
+        const uint2 r = store_round4<T>(o + 4 * k, make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
+        if (x16) store_operand4(x16 + m * K, 4 * k, r);
     }
 }
 
 // The same for bfloat16 activations on the tensor-core path, one CTA per token row: besides the rounded vector x
-// (kept for the caller) it writes the binary16 copy x16 the GEMM reads -- exact wherever a bfloat16 value lies
+// (kept for the caller) it writes the binary16 operand x16 the GEMM reads -- exact wherever a bfloat16 value lies
 // inside binary16's range; a row with a magnitude of 2^15 or more is divided by the power of two that brings its
-// largest one below 2^15, kept in scale[m] (1 otherwise) and undone by the GEMM's epilogue; *flag is raised then.
-// The flag must be zero when the kernel starts.
+// largest one below 2^15, kept in scale[m] (1 otherwise) and undone by the GEMM's epilogue.
 __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __restrict__ src, const float* __restrict__ src2, int in_op,
                                                               int64_t K, __nv_bfloat16* __restrict__ x, __half* __restrict__ x16,
-                                                              float* __restrict__ scale, int* __restrict__ flag, const PresetList pre) {
+                                                              float* __restrict__ scale, const PresetList pre) {
     pdl_wait();
     pdl_launch_dependents();
-    for (int q = 0; q < pre.n; ++q) {
-        float4* d = pre.dst[q];
-        const float4* r = pre.src[q];
-        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < pre.n4[q]; i += (int64_t)gridDim.x * 256)
-            d[i] = r ? r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (blockIdx.x >= pre.first) { write_presets(pre); return; }
     const int64_t m = blockIdx.x;
     const float4* s4 = reinterpret_cast<const float4*>(src + m * K);
     const float4* t4 = src2 ? reinterpret_cast<const float4*>(src2 + m * K) : nullptr;
@@ -252,7 +258,7 @@ __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __res
         const __half2 ha = __floats2half2_rn(fa.x, fa.y), hb = __floats2half2_rn(fb.x, fb.y);
         uint2 h;
         h.x = *reinterpret_cast<const uint32_t*>(&ha); h.y = *reinterpret_cast<const uint32_t*>(&hb);
-        *reinterpret_cast<uint2*>(hr + 4 * k) = h;
+        store_operand4(hr, 4 * k, h);
         mx = fmaxf(mx, fmaxf(fmaxf(fabsf(fa.x), fabsf(fa.y)), fmaxf(fabsf(fb.x), fabsf(fb.y))));
     }
 #pragma unroll
@@ -275,9 +281,8 @@ __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __res
             const __half2 ha = __floats2half2_rn(fa.x * inv, fa.y * inv), hb = __floats2half2_rn(fb.x * inv, fb.y * inv);
             uint2 h;
             h.x = *reinterpret_cast<const uint32_t*>(&ha); h.y = *reinterpret_cast<const uint32_t*>(&hb);
-            *reinterpret_cast<uint2*>(hr + 4 * k) = h;
+            store_operand4(hr, 4 * k, h);
         }
-        if (threadIdx.x == 0) *flag = 1;
     }
     if (threadIdx.x == 0) scale[m] = sc;
 }
@@ -292,10 +297,6 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
         const int64_t n = (int64_t)M * p->buf_width[0];
         widen_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x0, buf(0), n);
         count_launch();
-    }
-    if (!decode && dt == AQ_BF16) {   // the "a row was scaled" flags of all phases start at zero
-        e = cudaMemsetAsync(ws + plan.flags_begin, 0, plan.flags_end - plan.flags_begin, s);
-        if (e != cudaSuccess) return e;
     }
     if (decode) {   // one persistent kernel for the whole program, when it fits
         bool wrote_out = false;
@@ -363,13 +364,14 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
             const int64_t total4 = (int64_t)M * K / 4;
             const unsigned g = (f.in_op == AQ_IN_RMSNORM) ? (unsigned)M : (unsigned)std::min<int64_t>((total4 + 255) / 256, 4 * 148);
             const float* s2 = (f.in_op == AQ_IN_SILU_MUL) ? buf(f.src2) : nullptr;
-            if (decode) stage_kernel<T><<<g, 256, 0, s>>>(buf(f.src), s2, (int)f.in_op, K, total4, stage, pre);
+            pre.first = (!decode && dt == AQ_BF16) ? (unsigned)M : g;
+            if (decode) stage_kernel<T><<<g, 256, 0, s>>>(buf(f.src), s2, (int)f.in_op, K, total4, stage, nullptr, pre);
             else if (dt == AQ_BF16) {
-                int* flag = reinterpret_cast<int*>(ws + plan.flag_off[i]);
-                e = launch_pdl(stage_rows_bf16_kernel, dim3((unsigned)M), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K,
+                e = launch_pdl(stage_rows_bf16_kernel, dim3(pre.first + pre.ctas()), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K,
                                reinterpret_cast<__nv_bfloat16*>(stage), reinterpret_cast<__half*>(ws + plan.x16_off[i]),
-                               reinterpret_cast<float*>(ws + plan.rs_off[i]), flag, pre);
-            } else e = launch_pdl(stage_kernel<T>, dim3(g), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K, total4, stage, pre);
+                               reinterpret_cast<float*>(ws + plan.rs_off[i]), pre);
+            } else e = launch_pdl(stage_kernel<T>, dim3(pre.first + pre.ctas()), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K, total4, stage,
+                                reinterpret_cast<__half*>(ws + plan.x16_off[i]), pre);
             if (e != cudaSuccess) return e;
         }
         count_launch();
@@ -400,10 +402,8 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
                     ++n; ++j;
                 }
                 if (dt == AQ_BF16)
-                    e = launch_gemm_group(hs, n, ws + plan.x16_off[i], reinterpret_cast<const float*>(ws + plan.rs_off[i]),
-                                          reinterpret_cast<const int*>(ws + plan.flag_off[i]), M, outs, ldos, ress,
-                                          preset, s);
-                else e = launch_gemm_group(hs, n, stage, nullptr, nullptr, M, outs, ldos, ress, preset, s);
+                    e = launch_gemm_group(hs, n, ws + plan.x16_off[i], reinterpret_cast<const float*>(ws + plan.rs_off[i]), M, outs, ldos, ress, preset, s);
+                else e = launch_gemm_group(hs, n, ws + plan.x16_off[i], nullptr, M, outs, ldos, ress, preset, s);
                 if (e != cudaSuccess) return e;
             }
         }

@@ -1,0 +1,34 @@
+"""The prefill GEMM at the edges of its tiles: 256 rows (two row halves of 8 fragments), token tiles of up to 128 with two
+sets of accumulators up to 64, k-slabs of 128 in pairs."""
+import numpy as np
+import pytest
+
+from oracle import aq_oracle as O
+from paper_2605_24011_b200 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M", (9, 64, 65, 128, 129, 200, 257))
+@pytest.mark.parametrize("N,K,bits,dtype", [(16, 160, 2, "f16"), (136, 288, 3, "bf16"), (260, 512, 4, "f16"), (520, 96, 3, "f16"), (384, 1056, 2, "bf16")])
+def test_tile_edges(M, N, K, bits, dtype):
+    from paper_2605_24011_b200 import aq
+    tdt = torch.float16 if dtype == "f16" else torch.bfloat16
+    W = synth.weights(N, K, 97, N, K, outliers=True)
+    h = aq.aq_pack(bits, 32, torch.from_numpy(W).cuda())
+    x = torch.from_numpy(synth.activations(M, K, 98, M, K)).to(tdt).cuda()
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        aq.aq_linear(h, x, y)
+    aq.aq_check()
+    want, T = O.linear(*O.quantize(W, bits), x.double().cpu().numpy())
+    assert O.linear_excess(y.double().cpu().numpy(), want, T).max() <= 1.0
+    half = torch.full((M, N), float("nan"), dtype=tdt, device="cuda")   # up to 64 tokens the GEMM itself rounds: the tickets
+    for _ in range(2):                                                  # of shared tiles are zero again for the second call
+        aq.aq_linear(h, x, half)
+    aq.aq_check()
+    # two runs' float32 sums may differ by their order and then round to neighbouring values
+    ulp = 2.0 ** -10 if dtype == "f16" else 2.0 ** -7
+    a, b = half.double().cpu().numpy(), y.double().cpu().numpy()
+    assert np.all(np.abs(a - b) <= ulp * np.abs(b) + 1e-5 * T + 1e-7)
