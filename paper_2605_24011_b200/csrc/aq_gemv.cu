@@ -47,6 +47,8 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32, 2) gemv_kernel(const GemvArgs
     constexpr int PIECES = UB / 16 / 32;   // 16-byte pieces per lane per unit
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_wait();                 // (x, the sums and, right after packing, the weights are the predecessor's)
+    pdl_launch_dependents();
     uint8_t* ring = smem + (size_t)warp * GEMV_STAGES * UB;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
 
@@ -151,9 +153,9 @@ static cudaError_t launch_one(const GemvArgs& a, cudaStream_t s) {
     int grid = 2 * sm_count();
     const int64_t need = (warps_wanted + GEMV_WARPS - 1) / GEMV_WARPS;
     if (need < grid) grid = (int)need;
-    kern<<<grid, GEMV_WARPS * 32, SMEM, s>>>(a);
+    const cudaError_t e = launch_pdl(kern, dim3((unsigned)grid), dim3(GEMV_WARPS * 32), SMEM, s, a);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 // Small matrices (a few MB: the launch, not HBM, is what counts): one CTA per 16-row tile, its warps share the tile's
@@ -168,6 +170,8 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_rows_kernel(const GemvAr
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ float sums[8 * 16];   // [token][row of the tile]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_wait();
+    pdl_launch_dependents();
     const int R = blockIdx.x;
     const int KP = (int)(a.n_units / a.NT);
     uint8_t* ring = smem + (size_t)warp * ROWS_STAGES * UB;
@@ -224,21 +228,32 @@ template <int BITS, int MT, bool BF16>
 static cudaError_t launch_rows(const GemvArgs& a, cudaStream_t s) {
     constexpr int SMEM = GEMV_WARPS * ROWS_STAGES * 2 * frag_bytes(BITS);
     static_assert(SMEM <= 48 * 1024, "fits the default dynamic shared memory limit");
-    gemv_rows_kernel<BITS, MT, BF16><<<a.NT, GEMV_WARPS * 32, SMEM, s>>>(a);
+    const cudaError_t e = launch_pdl(gemv_rows_kernel<BITS, MT, BF16>, dim3((unsigned)a.NT), dim3(GEMV_WARPS * 32), SMEM, s, a);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
-// True when the row-tile kernel above is the better choice: outputs written by the kernel, one wave of CTAs, every
-// warp with a short run along k.
-static bool rows_kernel_fits(const GemvArgs& a) {
-    const int64_t KP = a.n_units / a.NT;
-    return a.y != nullptr && a.NT <= 4 * sm_count() && KP >= 2 && KP <= 8 * GEMV_WARPS;
+// True when the row-tile kernel above is the better choice: a warp has few units along k (x is fetched anew for each, and more
+// of it the more tokens there are) and the CTAs are few waves.  Measured, streaming kernel and cast / this, us:
+//   1 token:  2048 x 1024 5.6 / 2.3   4096 x 4096 5.7 / 4.1   16384 x 4096 11.2 / 9.2   2048 x 8192 7.3 / 4.9   512 x 8192 4.7 / 4.8
+//             4096 x 16384, 2 bits 11.3 / 9.7, 4 bits 11.7 / 14.0
+//   4 tokens: 4096 x 4096 6.4 / 6.3   11008 x 4096 10.3 / 9.7   16384 x 4096 12.7 / 13.0   4096 x 8192 8.9 / 10.2
+//   8 tokens: 4096 x 4096 7.0 / 6.6   9000 x 4096 9.9 / 11.5   2048 x 8192 7.0 / 7.6
+static bool rows_kernel_fits(int NT, int KP, int M, int bits) {
+    const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2);
+    if (NT > waves * sm_count() || KP < 2) return false;
+    if (KP <= 2 * GEMV_WARPS) return true;
+    if (M > 2 || 2 * NT < sm_count()) return false;
+    return KP <= (M == 1 && bits == 2 ? 8 : 4) * GEMV_WARPS;
 }
+
+// The kernel casts the outputs itself: any number of them from the row-tile kernel, few from the streaming kernel, whose last
+// CTA does it alone (about 0.1 us per 256 outputs; the cast as a launch of its own adds 1 us).
+bool gemv_writes_y(const aq_handle_s* h, int M) { return (int64_t)M * h->N <= 2048 || rows_kernel_fits(h->NT, h->KP, M, h->bits); }
 
 template <int BITS, bool BF16>
 static cudaError_t launch_mt(const GemvArgs& a, cudaStream_t s) {
-    if (rows_kernel_fits(a)) {
+    if (a.y != nullptr && rows_kernel_fits(a.NT, (int)(a.n_units / a.NT), a.M, BITS)) {
         if (a.M == 1) return launch_rows<BITS, 1, BF16>(a, s);
         if (a.M == 2) return launch_rows<BITS, 2, BF16>(a, s);
         if (a.M <= 4) return launch_rows<BITS, 4, BF16>(a, s);

@@ -53,6 +53,7 @@ cudaError_t launch_sb_records(const aq_handle_s* h, uint8_t* sbcanon_dev, uint8_
 cudaError_t launch_gemv(const aq_handle_s* h, const void* x, aq_dtype_t xdt, int M, float* acc,
                         int64_t ldacc, cudaStream_t s, void* y_fused = nullptr, aq_dtype_t ydt = AQ_F32);
 // y[m][n] = cast(acc[m][n]) for n < N, then acc = 0
+bool gemv_writes_y(const aq_handle_s* h, int M);   // launch_gemv can be given y
 cudaError_t launch_finalize(const float* acc_in, float* acc_zero, int64_t ldacc, void* y, aq_dtype_t ydt,
                             int M, int64_t N, cudaStream_t s);
 
