@@ -127,26 +127,40 @@ def _check(status: int, where: str):
 
 def _ptr(t) -> int:
     """Address of a torch tensor's storage (0 for None)."""
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        return _current_stream()
     return int(getattr(stream, "cuda_stream", stream))
 
 
-_DT = {"f16": AQ_F16, "bf16": AQ_BF16, "f32": AQ_F32}
+def _current_stream() -> int:
+    """Handle of torch's current stream (first call: finds the cheapest way to ask and takes this function's place).  A
+    linear of one token takes 5 us on the device, and building a Stream object on the way to its handle took 1.5 us."""
+    import torch
+    global _current_stream
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is None:
+        _current_stream = lambda: int(torch.cuda.current_stream().cuda_stream)
+    else:
+        _current_stream = lambda: raw(device())
+    return _current_stream()
+
+
+_DT = {"f16": AQ_F16, "bf16": AQ_BF16, "f32": AQ_F32}   # and torch's types from the first time one is asked for
 
 
 def dtype_code(t) -> int:
     """aq_dtype_t of a torch tensor / dtype / short name."""
-    if isinstance(t, str):
-        return _DT[t]
-    import torch
-    dt = t.dtype if hasattr(t, "data_ptr") else t
-    return {torch.float16: AQ_F16, torch.bfloat16: AQ_BF16, torch.float32: AQ_F32}[dt]
+    dt = getattr(t, "dtype", t)
+    code = _DT.get(dt)
+    if code is None:
+        import torch
+        _DT.update({torch.float16: AQ_F16, torch.bfloat16: AQ_BF16, torch.float32: AQ_F32})
+        code = _DT[dt]
+    return code
 
 
 class Handle:
@@ -347,12 +361,13 @@ def aq_dequant(h: Handle, out, stream=None):
 def aq_linear(h: Handle, x, y, M: int | None = None, stream=None):
     """x: CUDA [M][K] float16/bfloat16; y: CUDA [M][N] of the same dtype, or float32."""
     M = int(x.shape[0]) if M is None else M
-    if dtype_code(y) == AQ_F32:
-        _check(_lib.aq_linear_f32out(h.raw, _ptr(x), _ptr(y), M, dtype_code(x), _stream(stream)), "aq_linear_f32out")
+    xt, yt = dtype_code(x), dtype_code(y)
+    if yt == AQ_F32:
+        _check(_lib.aq_linear_f32out(h.raw, _ptr(x), _ptr(y), M, xt, _stream(stream)), "aq_linear_f32out")
     else:
-        if dtype_code(y) != dtype_code(x):
+        if yt != xt:
             raise AqError(AQ_ERR_INVALID_ARG, "aq_linear: y dtype must equal x dtype (or float32)")
-        _check(_lib.aq_linear(h.raw, _ptr(x), _ptr(y), M, dtype_code(x), _stream(stream)), "aq_linear")
+        _check(_lib.aq_linear(h.raw, _ptr(x), _ptr(y), M, xt, _stream(stream)), "aq_linear")
     return y
 
 
