@@ -12,9 +12,13 @@
 // are zero), P = exp2(S - max) straight from the accumulator registers into the A operand of O += P V.  The warps'
 // running (max, sum, O) are merged in shared memory, each CTA writes one partial per split, and the last CTA of a head to
 // arrive (a ticket after a fence; nobody waits) merges the splits and writes the output.
+// A stack program's step hands it the float32 q, k, v rows: it rotates and rounds them itself, appends the new rows of its
+// positions, and starts copying older rows on the SMs that the decode launch before it leaves first (with a launch of its own
+// for that in between, a step of one 7B token at 1000 positions took 3.8 us longer, of a 2B token 2.6).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <cstring>
 #include <type_traits>
 
 #include "aq_internal.h"
@@ -28,7 +32,9 @@ constexpr int AT_WARPS = 4;
 constexpr int AT_STAGES = 3;
 constexpr int AT_ROW_BYTES = AT_D * 2;
 constexpr int AT_TILE_BYTES = AT_TILE * AT_ROW_BYTES;                  // 8 KB
-constexpr int AT_SMEM = AT_WARPS * AT_STAGES * 2 * AT_TILE_BYTES;      // 192 KB
+constexpr int AT_RING = AT_WARPS * AT_STAGES * 2 * AT_TILE_BYTES;      // 192 KB
+constexpr int AT_Q_PITCH = AT_ROW_BYTES + 16;                          // (rows of q four banks apart)
+constexpr int AT_SMEM = AT_RING + 16 * AT_Q_PITCH;
 constexpr int AT_MAX_SPLITS = 64;
 
 // One ticket per key/value head: zero when the module is loaded, and put back to zero by the CTA that takes the last
@@ -49,6 +55,12 @@ struct AttnArgs {
     int chunk;              // positions per split (a multiple of AT_TILE)
     int out_dtype;          // aq_dtype_t of out
     float scale_log2;       // scale * log2(e)
+    // a stack program's step: the float32 q, k, v rows of the M new tokens, [M][heads][D] each (qf null: q is given as it is and
+    // the caches are complete).  The kernel rotates q and k for their positions, rounds, and appends k and v to the caches.
+    const float* qf;
+    const float* kf;
+    const float* vf;
+    const float2* turn;     // (cosine, sine) of the M tokens' D/2 angles (launch_attn_angles), complete before the kernel before this one
 };
 
 __device__ __forceinline__ void at_cp16(uint32_t dst, const void* src, uint32_t src_bytes) {
@@ -121,25 +133,87 @@ __global__ void __launch_bounds__(AT_WARPS * 32, 1) attn_decode_kernel(const Att
     for (int nd = 0; nd < AT_D / 8; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
     float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // rows g and g + 8: running maximum (log2 domain), sum
 
-    // Launched as a programmatic dependent: the kernel before this one on the stream (the one that rotates q and
-    // appends the new rows, when a stack program runs) may still be at work.  Only the last M rows of the cache and q can
-    // be its output: a CTA whose positions include those rows waits for it before its first copy, the others start
-    // their copies of older rows at once and wait before they read q (and before they write anything).
-    const bool has_new_rows = p1 > a.L - a.M;
-    if (has_new_rows) pdl_wait();
+    // Launched as a programmatic dependent: the kernel before this one on the stream may still be at work.  Only q and the
+    // last M rows of the cache can be its output (or are appended here): a warp whose first tiles lie before those rows
+    // starts its copies at once, the others wait first; all wait before they read q and before they write anything.
+    const int64_t old = a.L - a.M;   // rows that were there before
+    const bool early = p0 + (int64_t)(warp + AT_WARPS * (min(AT_STAGES - 1, my_tiles) - 1) + 1) * AT_TILE <= old;
+    auto first_tiles = [&] {
 #pragma unroll
-    for (int s = 0; s < AT_STAGES - 1; ++s) {
-        if (s < my_tiles) issue(s, s);
-        at_commit();
-    }
-    if (!has_new_rows) pdl_wait();
-    // (while the first tiles are on their way) the query heads of this key/value head as the A operand: row r = head
-    // hk G + r, rows >= G are zero
-    // row r = token r / G, head hk G + r % G of that token; rows >= G M are zero
+        for (int s = 0; s < AT_STAGES - 1; ++s) {
+            if (s < my_tiles) issue(s, s);
+            at_commit();
+        }
+    };
+    if (early) first_tiles();
+    // the query heads of this key/value head as the A operand: row r = token r / G, head hk G + r % G of that token; rows
+    // >= G M are zero
     const int R = a.G * a.M;
     const int tok0 = g / a.G, tok1 = (g + 8) / a.G;
     uint32_t qf[AT_D / 16][4];
-    {
+    if (a.qf != nullptr) {
+        // Thread: pair (i, i + D/2) of rows (and new tokens) sub, sub + 2, ...; everything is loaded before anything is stored
+        const int i = threadIdx.x & (AT_D / 2 - 1), sub = threadIdx.x / (AT_D / 2);
+        auto cast = [](float x) -> uint16_t {
+            if constexpr (BF16) return __bfloat16_as_ushort(__float2bfloat16_rn(x));
+            else return __half_as_ushort(__float2half_rn(x));
+        };
+        auto put = [&](uint16_t* d, float x, float y, const float2& cs) {
+            d[0] = cast(fmaf(x, cs.x, -y * cs.y));
+            d[AT_D / 2] = cast(fmaf(y, cs.x, x * cs.y));
+        };
+        pdl_wait();
+        float2 q2[8], qt[8], k2[4], v2[4], kt[4];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int r = sub + 2 * u, m = r / a.G;
+            if (r < R) {
+                const float* q = a.qf + ((size_t)m * a.H + (size_t)hk * a.G + (r - m * a.G)) * AT_D + i;
+                q2[u] = make_float2(__ldcg(q), __ldcg(q + AT_D / 2));
+                qt[u] = __ldg(a.turn + m * (AT_D / 2) + i);
+            }
+        }
+        auto mine = [&](int m) { return m < a.M && old + m >= p0 && old + m < p1; };   // this CTA's row: nobody else reads or writes it
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int m = sub + 2 * u;
+            if (mine(m)) {
+                const size_t from = ((size_t)m * gridDim.x + hk) * AT_D + i;
+                k2[u] = make_float2(__ldcg(a.kf + from), __ldcg(a.kf + from + AT_D / 2));
+                v2[u] = make_float2(__ldcg(a.vf + from), __ldcg(a.vf + from + AT_D / 2));
+                kt[u] = __ldg(a.turn + m * (AT_D / 2) + i);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int m = sub + 2 * u;
+            if (mine(m)) {
+                const size_t to = ((size_t)hk * a.Lmax + (size_t)(old + m)) * AT_D + i;
+                put(reinterpret_cast<uint16_t*>(const_cast<void*>(a.kc)) + to, k2[u].x, k2[u].y, kt[u]);
+                uint16_t* vd = reinterpret_cast<uint16_t*>(const_cast<void*>(a.vc)) + to;
+                vd[0] = cast(v2[u].x);
+                vd[AT_D / 2] = cast(v2[u].y);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int r = sub + 2 * u;
+            if (r < R) put(reinterpret_cast<uint16_t*>(smem + AT_RING + r * AT_Q_PITCH) + i, q2[u].x, q2[u].y, qt[u]);
+        }
+        if (p1 > old) __threadfence();   // (the copies below read through L2)
+        __syncthreads();
+        const uint8_t* q0 = smem + AT_RING + g * AT_Q_PITCH;
+        const uint8_t* q1 = q0 + 8 * AT_Q_PITCH;
+#pragma unroll
+        for (int ks = 0; ks < AT_D / 16; ++ks) {
+            const int o0 = 2 * (16 * ks + 2 * t);
+            qf[ks][0] = g < R ? *reinterpret_cast<const uint32_t*>(q0 + o0) : 0u;
+            qf[ks][1] = g + 8 < R ? *reinterpret_cast<const uint32_t*>(q1 + o0) : 0u;
+            qf[ks][2] = g < R ? *reinterpret_cast<const uint32_t*>(q0 + o0 + 16) : 0u;
+            qf[ks][3] = g + 8 < R ? *reinterpret_cast<const uint32_t*>(q1 + o0 + 16) : 0u;
+        }
+    } else {
+        pdl_wait();
         const uint16_t* q = reinterpret_cast<const uint16_t*>(a.q);
         const uint16_t* q0 = q + ((int64_t)tok0 * a.H + (int64_t)hk * a.G + (g - tok0 * a.G)) * AT_D;
         const uint16_t* q1 = q + ((int64_t)tok1 * a.H + (int64_t)hk * a.G + (g + 8 - tok1 * a.G)) * AT_D;
@@ -152,6 +226,7 @@ __global__ void __launch_bounds__(AT_WARPS * 32, 1) attn_decode_kernel(const Att
             qf[ks][3] = g + 8 < R ? *reinterpret_cast<const uint32_t*>(q1 + d0 + 8) : 0u;
         }
     }
+    if (!early) first_tiles();
     // a token sees the positions up to its own: token m of M up to L - M + m (rows past the last one: any limit will do)
     const int64_t lim0 = a.L - (a.M - 1 - min(tok0, a.M - 1)), lim1 = a.L - (a.M - 1 - min(tok1, a.M - 1));
     for (int j = 0; j < my_tiles; ++j) {
@@ -347,53 +422,6 @@ __global__ void kv_append_kernel(uint4* kc, uint4* vc, const uint4* k, const uin
     vc[o] = v[idx];
 }
 
-// What a stack program's attention step does with the float32 q, k, v rows of its M new tokens before the attention
-// itself: rotates q and k for their positions, rounds q to the activation type into a staging array [M][H][D], and puts
-// the rounded k and v into rows pos .. pos + M - 1 of the caches.  One CTA of D/2 threads per (token, head).
-template <typename T>
-__global__ void attn_prepare_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, T* __restrict__ q16,
-                                    T* __restrict__ kc, T* __restrict__ vc, int H, int Hkv, int D, int64_t pos, int64_t Lmax, double log2_theta) {
-    const int m = blockIdx.y, hh = blockIdx.x, i = threadIdx.x, half = D / 2;
-    pdl_launch_dependents();   // the attention kernel may set itself up and read older cache rows meanwhile
-    auto cast = [](float x) -> T {
-        if constexpr (std::is_same<T, __half>::value) return __float2half_rn(x);
-        else return __float2bfloat16_rn(x);
-    };
-    if (hh >= H + Hkv) {   // a value head: rounded as it is
-        const int hk = hh - H - Hkv;
-        const float* src = v + ((size_t)m * Hkv + hk) * D;
-        T* dst = vc + ((size_t)hk * Lmax + pos + m) * D;
-        dst[i] = cast(src[i]);
-        dst[i + half] = cast(src[i + half]);
-        return;
-    }
-    const double ang = (double)(pos + m) * exp2(-2.0 * (double)i / (double)D * log2_theta);
-    double sn, cs;
-    sincos(ang, &sn, &cs);
-    const float fc = (float)cs, fs = (float)sn;
-    const bool is_q = hh < H;
-    const float* src = is_q ? q + ((size_t)m * H + hh) * D : k + ((size_t)m * Hkv + (hh - H)) * D;
-    T* dst = is_q ? q16 + ((size_t)m * H + hh) * D : kc + ((size_t)(hh - H) * Lmax + pos + m) * D;
-    const float a = src[i], b = src[i + half];
-    dst[i] = cast(fmaf(a, fc, -b * fs));
-    dst[i + half] = cast(fmaf(b, fc, a * fs));
-}
-
-cudaError_t launch_attn_prepare(const float* q, const float* k, const float* v, void* q16, void* kc, void* vc, int M, int H, int Hkv,
-                                int64_t pos, int64_t Lmax, float theta, aq_dtype_t dt, cudaStream_t s) {
-    const dim3 grid((unsigned)(H + 2 * Hkv), (unsigned)M);
-    const double l2t = log2((double)theta);
-    if (dt == AQ_F16)
-        attn_prepare_kernel<__half><<<grid, AT_D / 2, 0, s>>>(q, k, v, reinterpret_cast<__half*>(q16), reinterpret_cast<__half*>(kc),
-                                                             reinterpret_cast<__half*>(vc), H, Hkv, AT_D, pos, Lmax, l2t);
-    else
-        attn_prepare_kernel<__nv_bfloat16><<<grid, AT_D / 2, 0, s>>>(q, k, v, reinterpret_cast<__nv_bfloat16*>(q16),
-                                                                    reinterpret_cast<__nv_bfloat16*>(kc), reinterpret_cast<__nv_bfloat16*>(vc), H,
-                                                                    Hkv, AT_D, pos, Lmax, l2t);
-    count_launch();
-    return cudaGetLastError();
-}
-
 // ---- host ---------------------------------------------------------------------------------------------------
 static int attn_max_splits(int n_kv) {
     // one CTA per SM fits (its rings take most of the shared memory), so one wave: as many splits as keep the grid
@@ -417,12 +445,10 @@ size_t attn_scratch_bytes(int n_kv) {
     return 256 + (size_t)n_kv * AT_MAX_SPLITS * 16 * 2 * sizeof(float) + (size_t)n_kv * attn_max_splits(n_kv) * 16 * AT_D * sizeof(float) + 256;
 }
 
-cudaError_t launch_attn_decode(const void* q, const void* kc, const void* vc, void* out, int M, int n_heads, int n_kv, int64_t L,
-                               int64_t Lmax, float scale, aq_dtype_t dt, aq_dtype_t out_dt, void* scratch, cudaStream_t s) {
+static cudaError_t launch_attn(AttnArgs& a, int n_heads, int n_kv, int M, int64_t L, int64_t Lmax, float scale, aq_dtype_t dt, aq_dtype_t out_dt,
+                               void* scratch, cudaStream_t s) {
     int splits, chunk;
     attn_geometry(n_kv, L, &splits, &chunk);
-    AttnArgs a;
-    a.q = q; a.kc = kc; a.vc = vc; a.out = out;
     uint8_t* sc = reinterpret_cast<uint8_t*>(scratch);
     a.ml = reinterpret_cast<float*>(sc + 256);
     a.part = reinterpret_cast<float*>(sc + 256 + (size_t)n_kv * AT_MAX_SPLITS * 16 * 2 * sizeof(float));
@@ -442,6 +468,38 @@ cudaError_t launch_attn_decode(const void* q, const void* kc, const void* vc, vo
                              : launch_pdl(attn_decode_kernel<false>, grid, dim3(AT_WARPS * 32), AT_SMEM, s, a);
     count_launch();
     return e;
+}
+
+cudaError_t launch_attn_decode(const void* q, const void* kc, const void* vc, void* out, int M, int n_heads, int n_kv, int64_t L,
+                               int64_t Lmax, float scale, aq_dtype_t dt, aq_dtype_t out_dt, void* scratch, cudaStream_t s) {
+    AttnArgs a;
+    memset(&a, 0, sizeof(a));
+    a.q = q; a.kc = kc; a.vc = vc; a.out = out;
+    return launch_attn(a, n_heads, n_kv, M, L, Lmax, scale, dt, out_dt, scratch, s);
+}
+
+// The rotation angles of positions pos .. pos + M - 1, as rope_kernel forms them: once per pass, for they are the same in every
+// block (formed by the attention kernel, 8 tokens cost 2 us a block).
+__global__ void attn_angles_kernel(float2* turn, int64_t pos, double log2_theta) {
+    const int m = blockIdx.x, i = threadIdx.x;
+    double s, c;
+    sincos((double)(pos + m) * exp2(-2.0 * (double)i / (double)AT_D * log2_theta), &s, &c);
+    turn[m * (AT_D / 2) + i] = make_float2((float)c, (float)s);
+}
+
+cudaError_t launch_attn_angles(void* turn, int M, int64_t pos, float theta, cudaStream_t s) {
+    attn_angles_kernel<<<(unsigned)M, AT_D / 2, 0, s>>>(reinterpret_cast<float2*>(turn), pos, log2((double)theta));
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_attn_step(const float* q, const float* k, const float* v, void* kc, void* vc, float* out, int M, int n_heads, int n_kv,
+                             int64_t pos, int64_t Lmax, const void* turn, float scale, aq_dtype_t dt, void* scratch, cudaStream_t s) {
+    AttnArgs a;
+    memset(&a, 0, sizeof(a));
+    a.qf = q; a.kf = k; a.vf = v; a.kc = kc; a.vc = vc; a.out = out;
+    a.turn = reinterpret_cast<const float2*>(turn);
+    return launch_attn(a, n_heads, n_kv, M, pos + M, Lmax, scale, dt, AQ_F32, scratch, s);
 }
 
 cudaError_t launch_rope(void* x, int n_heads, int D, int64_t pos, float theta, aq_dtype_t dt, cudaStream_t s) {

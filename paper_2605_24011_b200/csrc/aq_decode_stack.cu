@@ -604,6 +604,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
     const int quarter = warp & 3;   // (a warp reaches the TMEM lanes of its quarter only)
     const int M = a.M;
     const u64 wait_ns = a.wait_ns;
+    pdl_launch_dependents();   // (an attention step that follows may read its cache on the SMs this launch leaves first)
 
     if (threadIdx.x == 0) {
         sh.abort_flag = 0;
@@ -1235,6 +1236,36 @@ bool build_decode_tables(const aq_stack_t* p, const StackPlan& plan, int M, int 
     return true;
 }
 
+// What a pass needs before its first launch: x as float32 (groups of eight) and zeros in the packed sums.  One kernel in place of
+// a conversion and a memset: a pass of a small program takes 15 us, and each launch before the big one added 1.5.
+template <bool BF16>
+__global__ void __launch_bounds__(256) begin_pass_kernel(const uint4* __restrict__ x, float4* __restrict__ out, int64_t n8, int rest, uint4* __restrict__ zero, int64_t zero16) {
+    pdl_wait();
+    const int64_t i0 = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
+    for (int64_t i = i0; i < n8; i += step) {
+        const uint4 v = x[i];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float2 p;
+            if constexpr (BF16) p = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[j]));
+            else p = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
+            f[2 * j] = p.x; f[2 * j + 1] = p.y;
+        }
+        out[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
+        out[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+    if (i0 < rest) {   // elements past the last whole group
+        const uint16_t u = reinterpret_cast<const uint16_t*>(x + n8)[i0];
+        float f;
+        if constexpr (BF16) f = __bfloat162float(__ushort_as_bfloat16(u));
+        else f = __half2float(__ushort_as_half(u));
+        reinterpret_cast<float*>(out + 2 * n8)[i0] = f;
+    }
+    for (int64_t i = i0; i < zero16; i += step) zero[i] = make_uint4(0, 0, 0, 0);
+}
+
 template <int MT, bool BF16>
 static cudaError_t launch_ds(const DsArgs& a, int grid, cudaStream_t s) {
     auto kern = decode_stack_kernel<MT, BF16>;
@@ -1270,7 +1301,7 @@ void decode_program_key(const aq_stack_t* p, std::vector<uint8_t>& key) {
 }
 
 int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dtype_t dt, uint8_t* ws, cudaStream_t s,
-                        cudaError_t* err, void* out, int out_buf, bool* wrote_out, int op_first, int op_end, bool clear,
+                        cudaError_t* err, const void* x0, void* out, int out_buf, bool* wrote_out, int op_first, int op_end,
                         const std::vector<uint8_t>* program_key) {
     *err = cudaSuccess;
     *wrote_out = false;
@@ -1363,8 +1394,17 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
         a.out_n = (int64_t)M * p->buf_width[out_buf];
         *wrote_out = true;
     }
-    // the packed sums start from zero (once per pass: a later launch of the same pass reads what the earlier ones left)
-    cudaError_t e = clear ? cudaMemsetAsync(ws + plan.pk_begin, 0, plan.pk_end - plan.pk_begin, s) : cudaSuccess;
+    // once per pass: the input widened, and the packed sums zeroed (a later launch reads what the earlier ones left)
+    cudaError_t e = cudaSuccess;
+    if (x0) {
+        const int64_t n0 = (int64_t)M * p->buf_width[0], n8 = n0 / 8, zero16 = (int64_t)(plan.pk_end - plan.pk_begin) / 16;
+        const unsigned blocks = (unsigned)std::min<int64_t>((std::max(n8, zero16) + 511) / 512, 4 * grid);
+        float4* widened = reinterpret_cast<float4*>(ws + plan.buf_off[0]);
+        uint4* zero = reinterpret_cast<uint4*>(ws + plan.pk_begin);
+        if (dt == AQ_BF16) e = launch_pdl(begin_pass_kernel<true>, dim3(blocks), dim3(256), 0, s, (const uint4*)x0, widened, n8, (int)(n0 - 8 * n8), zero, zero16);
+        else e = launch_pdl(begin_pass_kernel<false>, dim3(blocks), dim3(256), 0, s, (const uint4*)x0, widened, n8, (int)(n0 - 8 * n8), zero, zero16);
+        count_launch();
+    }
     if (e == cudaSuccess) {
         const bool bf = (dt == AQ_BF16);
         if (M == 1) e = bf ? launch_ds<1, true>(a, grid, s) : launch_ds<1, false>(a, grid, s);

@@ -93,9 +93,9 @@ struct StackPlan {
 // whole-program decode (M <= AQ_DECODE_MAX_M) in one persistent kernel: 0 = launched,
 // 1 = the program does not fit that kernel (nothing launched), -1 = CUDA error in *err
 // (out: the caller's rounded copy of buffer out_buf, or null; *wrote_out: the kernel itself writes it; op_first, op_end:
-// the ops of the program this launch runs, whole phases; clear: the packed sums are zeroed first)
+// the ops of the program this launch runs, whole phases; x0: the pass's input, given with its first launch, which widens it and zeroes the packed sums)
 int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dtype_t dt, uint8_t* ws, cudaStream_t s,
-                        cudaError_t* err, void* out, int out_buf, bool* wrote_out, int op_first = 0, int op_end = -1, bool clear = true,
+                        cudaError_t* err, const void* x0, void* out, int out_buf, bool* wrote_out, int op_first = 0, int op_end = -1,
                         const std::vector<uint8_t>* program_key = nullptr);
 void decode_program_key(const aq_stack_t* p, std::vector<uint8_t>& key);   // the program's share of a plan's key
 void decode_stack_forget(aq_handle_t h);   // drops cached device tables that name h
@@ -137,8 +137,11 @@ size_t attn_scratch_bytes(int n_kv);
 cudaError_t launch_attn_decode(const void* q, const void* kc, const void* vc, void* out, int M, int n_heads, int n_kv, int64_t L,
                                int64_t Lmax, float scale, aq_dtype_t dt, aq_dtype_t out_dt, void* scratch, cudaStream_t s);
 cudaError_t launch_rope(void* x, int n_heads, int D, int64_t pos, float theta, aq_dtype_t dt, cudaStream_t s);
-cudaError_t launch_attn_prepare(const float* q, const float* k, const float* v, void* q16, void* kc, void* vc, int M, int H, int Hkv,
-                                int64_t pos, int64_t Lmax, float theta, aq_dtype_t dt, cudaStream_t s);
+// the attention step of a stack program, turn from launch_attn_angles: q [M][n_heads][128], k, v [M][n_kv][128] float32; q and k are rotated for positions
+// pos .. pos + M - 1, k and v are appended to the caches, out [M][n_heads][128] float32
+cudaError_t launch_attn_step(const float* q, const float* k, const float* v, void* kc, void* vc, float* out, int M, int n_heads, int n_kv,
+                             int64_t pos, int64_t Lmax, const void* turn, float scale, aq_dtype_t dt, void* scratch, cudaStream_t s);
+cudaError_t launch_attn_angles(void* turn, int M, int64_t pos, float theta, cudaStream_t s);   // turn: M * 512 bytes
 cudaError_t launch_kv_append(void* kc, void* vc, const void* k, const void* v, int n_kv, int D, int64_t pos, int64_t Lmax, cudaStream_t s);
 
 // memory (aq_memory.cu): device blocks out of a bounded cache (null: no memory left); a copy into pageable host memory, complete

@@ -293,14 +293,15 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
     cudaError_t e = cudaSuccess;
     const bool decode = (M <= AQ_DECODE_MAX_M);
     auto buf = [&](int b) { return reinterpret_cast<float*>(ws + plan.buf_off[b]); };
-    {
+    auto widen = [&] {
         const int64_t n = (int64_t)M * p->buf_width[0];
         widen_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x0, buf(0), n);
         count_launch();
-    }
+    };
+    if (!decode) widen();
     if (decode) {   // one persistent kernel for the whole program, when it fits
         bool wrote_out = false;
-        const int r = launch_decode_stack(p, plan, M, dt, ws, s, &e, out, out_buf, &wrote_out);
+        const int r = launch_decode_stack(p, plan, M, dt, ws, s, &e, x0, out, out_buf, &wrote_out);
         if (r < 0) return e;
         if (r == 0) {
             for (int k = 0; k < p->n_ops; ++k) p->ops[k].w->last_stream = s;
@@ -311,6 +312,7 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
             count_launch();
         }
         if (r == 0) return cudaGetLastError();
+        widen();
         // op by op: the streaming kernel accumulates with red.add, so every output starts at zero (inputs that somebody
         // else has filled are left alone: runs of buffers between them are cleared)
         for (int b = 1; b < p->n_bufs;) {
@@ -462,9 +464,12 @@ aq_status_t aq_stack_forward(const aq_stack_t* prog, const void* x0_dev, void* o
     return AQ_OK;
 }
 
+// Scratch of an attention step: the rotation angles first, common to all steps.
+static size_t angles_end(int M, int n_heads) { return align_up((size_t)M * 256 * std::max(n_heads, 2), 256); }
+
 size_t aq_stack_attn_scratch_bytes(int n_heads, int n_kv_heads, int M) {
     if (n_heads < 1 || n_kv_heads < 1 || n_kv_heads > 64 || M < 1 || M > AQ_DECODE_MAX_M) return 0;
-    return align_up((size_t)M * n_heads * 128 * 2, 256) + attn_scratch_bytes(n_kv_heads);
+    return angles_end(M, n_heads) + attn_scratch_bytes(n_kv_heads);
 }
 
 aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t* attn, int n_attn, int64_t pos, float theta,
@@ -513,11 +518,9 @@ aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t*
     uint8_t* ws = reinterpret_cast<uint8_t*>(workspace_dev);
     auto buf = [&](int b) { return reinterpret_cast<float*>(ws + plan.buf_off[b]); };
     cudaError_t e = cudaSuccess;
-    {
-        const int64_t n = (int64_t)M * prog->buf_width[0];
-        if (dtype == AQ_F16) widen_kernel<__half><<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const __half*)x0_dev, buf(0), n);
-        else widen_kernel<__nv_bfloat16><<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const __nv_bfloat16*)x0_dev, buf(0), n);
-        count_launch();
+    if (n_attn > 0) {
+        e = launch_attn_angles(attn_scratch_dev, M, pos, theta, s);
+        if (e != cudaSuccess) return cuda_fail(e);
     }
     int first = 0;
     bool wrote_out = false;
@@ -527,8 +530,8 @@ aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t*
         const int end = (i < n_attn) ? attn[i].after_op + 1 : prog->n_ops;
         if (end > first) {
             bool w = false;
-            const int r = launch_decode_stack(prog, plan, M, dtype, ws, s, &e, (i == n_attn) ? out_dev : nullptr, out_buf, &w, first, end,
-                                              first == 0, &program_key);
+            const int r = launch_decode_stack(prog, plan, M, dtype, ws, s, &e, first == 0 ? x0_dev : nullptr, (i == n_attn) ? out_dev : nullptr,
+                                              out_buf, &w, first, end, &program_key);
             if (r < 0) return cuda_fail(e);
             if (r > 0) return AQ_ERR_UNSUPPORTED;
             wrote_out = wrote_out || w;
@@ -536,14 +539,9 @@ aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t*
         first = end;
         if (i == n_attn) break;
         const aq_stack_attn_t& t = attn[i];
-        uint8_t* sc = reinterpret_cast<uint8_t*>(attn_scratch_dev);
-        void* q16 = sc;
-        void* asc = sc + align_up((size_t)M * t.n_heads * 128 * 2, 256);
-        e = launch_attn_prepare(buf(t.q_buf), buf(t.k_buf), buf(t.v_buf), q16, t.k_cache_dev, t.v_cache_dev, M, t.n_heads, t.n_kv_heads, pos,
-                                t.L_max, theta, dtype, s);
-        if (e == cudaSuccess)
-            e = launch_attn_decode(q16, t.k_cache_dev, t.v_cache_dev, buf(t.dst_buf), M, t.n_heads, t.n_kv_heads, pos + M, t.L_max,
-                                   0.08838834764831845f, dtype, AQ_F32, asc, s);
+        uint8_t* sc = reinterpret_cast<uint8_t*>(attn_scratch_dev) + angles_end(M, t.n_heads);
+        e = launch_attn_step(buf(t.q_buf), buf(t.k_buf), buf(t.v_buf), t.k_cache_dev, t.v_cache_dev, buf(t.dst_buf), M, t.n_heads, t.n_kv_heads, pos,
+                             t.L_max, attn_scratch_dev, 0.08838834764831845f, dtype, sc, s);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     for (int k = 0; k < prog->n_ops; ++k) prog->ops[k].w->last_stream = s;
