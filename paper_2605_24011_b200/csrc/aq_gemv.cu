@@ -171,7 +171,6 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_rows_kernel(const GemvAr
     __shared__ float sums[8 * 16];   // [token][row of the tile]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_wait();
-    pdl_launch_dependents();
     const int R = blockIdx.x;
     const int KP = (int)(a.n_units / a.NT);
     uint8_t* ring = smem + (size_t)warp * ROWS_STAGES * UB;
@@ -207,6 +206,9 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) gemv_rows_kernel(const GemvAr
         cp_async_commit();
         slot ^= 1;
     }
+    // (here, not at the start: the next linear's CTAs would be dealt to whichever SMs have fewer of this one's, and its time is
+    // that of the fullest SM: 4096 x 4096 at 4 bits 5.3 us a call instead of 4.8)
+    pdl_launch_dependents();
     cp_async_wait<0>();
     __syncthreads();   // sums are zero
     if (warp < KP) unit_commit<MT>(acc, sums, 16, 0, 16, a.M, lane);
@@ -235,25 +237,26 @@ static cudaError_t launch_rows(const GemvArgs& a, cudaStream_t s) {
 
 // True when the row-tile kernel above is the better choice: a warp has few units along k (x is fetched anew for each, and more
 // of it the more tokens there are) and the CTAs are few waves.  Measured, streaming kernel and cast / this, us:
-//   1 token:  2048 x 1024 5.6 / 2.3   4096 x 4096 5.7 / 4.1   16384 x 4096 11.2 / 9.2   2048 x 8192 7.3 / 4.9   512 x 8192 4.7 / 4.8
-//             4096 x 16384, 2 bits 11.3 / 9.7, 4 bits 11.7 / 14.0
-//   4 tokens: 4096 x 4096 6.4 / 6.3   11008 x 4096 10.3 / 9.7   16384 x 4096 12.7 / 13.0   4096 x 8192 8.9 / 10.2
-//   8 tokens: 4096 x 4096 7.0 / 6.6   9000 x 4096 9.9 / 11.5   2048 x 8192 7.0 / 7.6
-static bool rows_kernel_fits(int NT, int KP, int M, int bits) {
+//   1 token:  2048 x 1024 5.7 / 2.2   4096 x 4096, 4 bits 5.8 / 4.8   16384 x 4096, 4 bits 13.0 / 12.0   2048 x 8192 7.3 / 4.8
+//             9000 x 16384, 2 bits 20.4 / 17.5, 3 bits 22.8 / 22.7   4096 x 16384, 4 bits 12.9 / 13.9   512 x 16384 4.9 / 7.3
+//   2 tokens: 4096 x 8192, 4 bits 8.7 / 8.0   9000 x 16384, 4 bits 23.1 / 25.4
+//   4 tokens: 4096 x 4096 6.5 / 5.6   9000 x 4096 9.2 / 8.3   16384 x 4096, 4 bits 14.5 / 15.5   4096 x 8192 8.9 / 9.0
+//   8 tokens: 4096 x 4096 7.0 / 6.5   9000 x 4096 10.0 / 11.3   2048 x 8192 7.0 / 8.2
+static bool rows_kernel_fits(int NT, int KP, int M) {
     const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2);
     if (NT > waves * sm_count() || KP < 2) return false;
     if (KP <= 2 * GEMV_WARPS) return true;
     if (M > 2 || 2 * NT < sm_count()) return false;
-    return KP <= (M == 1 && bits == 2 ? 8 : 4) * GEMV_WARPS;
+    return KP <= (M == 1 ? 8 : 4) * GEMV_WARPS;
 }
 
 // The kernel casts the outputs itself: any number of them from the row-tile kernel, few from the streaming kernel, whose last
 // CTA does it alone (about 0.1 us per 256 outputs; the cast as a launch of its own adds 1 us).
-bool gemv_writes_y(const aq_handle_s* h, int M) { return (int64_t)M * h->N <= 2048 || rows_kernel_fits(h->NT, h->KP, M, h->bits); }
+bool gemv_writes_y(const aq_handle_s* h, int M) { return (int64_t)M * h->N <= 2048 || rows_kernel_fits(h->NT, h->KP, M); }
 
 template <int BITS, bool BF16>
 static cudaError_t launch_mt(const GemvArgs& a, cudaStream_t s) {
-    if (a.y != nullptr && rows_kernel_fits(a.NT, (int)(a.n_units / a.NT), a.M, BITS)) {
+    if (a.y != nullptr && rows_kernel_fits(a.NT, (int)(a.n_units / a.NT), a.M)) {
         if (a.M == 1) return launch_rows<BITS, 1, BF16>(a, s);
         if (a.M == 2) return launch_rows<BITS, 2, BF16>(a, s);
         if (a.M <= 4) return launch_rows<BITS, 4, BF16>(a, s);
