@@ -9,8 +9,11 @@
 // inside binary16's range; a token row that is not comes scaled by a power of
 // two, undone in the epilogue through tok_scale).
 //
-// Bound: tensor cores (dense contraction, 2 M flops per weight).  tcgen05
-// UMMA, 256 weight rows x up to 128 tokens per tile:
+// Bound: by its flops the tensor cores (dense contraction, 2 M flops per weight); in
+// fact, from 128 tokens on, L2: a slab of 256 rows x 128 k x 128 tokens reads 33 KB of
+// tokens and 12 to 20 KB of weights, 270 MB in 40 us (6.7 TB/s) for 11008 x 4096 at 512
+// tokens; with few tokens the chain of latencies from launch to sums (2.7 us), epilogue
+// and adds.  tcgen05 UMMA, 256 weight rows x up to 128 tokens per tile:
 //   A (M side, 2 x 128) = weight rows, dequantised by sixteen warps from the packed
 //                       fragments straight into TMEM (tcgen05.st): two row halves
 //                       of 64 k are a stage of 64 columns, four stages,
