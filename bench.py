@@ -628,9 +628,9 @@ def main():
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
 DECODE_TRAFFIC_BYTES = 8 * (355_717_888 + 4_195_584)
-# gemm_kernel (profiles/gemm_kernel_11008x4096_M512_2bit.md): 21,212,160 + 19,456 bytes of DRAM traffic for one 11008 x 4096
+# gemm_kernel (profiles/gemm_kernel_11008x4096_M512_2bit.md): 21,204,224 + 31,488 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
-PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_212_160 + 19_456) / 16_908_288)
+PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_204_224 + 31_488) / 16_908_288)
 
 
 def prefill_leg(aq, workloads, prog, out_buf, info, peaks, torch, gpu_index=0):

@@ -9,11 +9,15 @@
 // inside binary16's range; a token row that is not comes scaled by a power of
 // two, undone in the epilogue through tok_scale).
 //
-// Bound: by its flops the tensor cores (dense contraction, 2 M flops per weight); in
-// fact, from 128 tokens on, L2: a slab of 256 rows x 128 k x 128 tokens reads 33 KB of
-// tokens and 12 to 20 KB of weights, 270 MB in 40 us (6.7 TB/s) for 11008 x 4096 at 512
-// tokens; with few tokens the chain of latencies from launch to sums (2.7 us), epilogue
-// and adds.  tcgen05 UMMA, 256 weight rows x up to 128 tokens per tile:
+// Bound: by its flops the tensor cores (dense contraction, 2 M flops per weight).  In
+// fact no unit is full: 11008 x 4096 at 512 tokens keeps the tensor pipe 47 % active, L2
+// at 20 % of its rate, issue slots at 38 %; the dequantise warps wait 40 % of their time for
+// instructions to release a stage, and with one instruction in eight the call still takes 37
+// of 48 us, so hand-overs, fill, epilogue and uneven runs (172 tiles on 148 SMs) share the
+// rest.  With few tokens it is the chain of latencies from launch to sums (2.7 us), epilogue
+// and adds.
+//
+// tcgen05 UMMA, 256 weight rows x up to 128 tokens per tile:
 //   A (M side, 2 x 128) = weight rows, dequantised by sixteen warps from the packed
 //                       fragments straight into TMEM (tcgen05.st): two row halves
 //                       of 64 k are a stage of 64 columns, four stages,
