@@ -416,7 +416,8 @@ aq_status_t aq_set_wait_limit_ns(uint64_t ns);
  * aq_debug_decode_hold -- TESTING ONLY.  While on, the tables aq_stack_forward builds for the decode kernel make the
  * first phase that reads another op's output expect one contribution more than will ever arrive, so every CTA's
  * wait for that input runs out (after the limit above) and the time-out path can be exercised on a healthy GPU:
- * nothing traps, faults or spins without bound.  Programs run while it is off are not affected.
+ * nothing traps, faults or spins without bound.  Likewise the prefill GEMM's launches made while it is on never report
+ * a tile as stored, so the runs that add to it give up (after about a second).  Calls made while it is off are not affected.
  */
 void aq_debug_decode_hold(int on);
 

@@ -444,7 +444,10 @@ aq_status_t aq_set_wait_limit_ns(uint64_t ns) {
     return AQ_OK;
 }
 
-void aq_debug_decode_hold(int on) { set_decode_hold(on != 0); }
+void aq_debug_decode_hold(int on) {
+    set_decode_hold(on != 0);
+    set_gemm_hold(on != 0);
+}
 
 void aq_free(aq_handle_t h) {
     if (!handle_ok(h)) return;

@@ -93,11 +93,14 @@ constexpr uint32_t GM_SPIN_LIMIT = 40u * 1000u * 1000u;
 __device__ int g_gemm_status = 0;  // nonzero: a bounded wait ran out (code = which)
 
 // Split tiles without zeroing the output first: the run that holds a tile's last k-slab is the first thing its CTA
-// does; it STORES its sums and then writes the launch's epoch into the tile's flag; the other runs of the tile add
-// theirs once they see it.  Flags are never reset: every launch has its own epoch and takes the next of a few arrays.
+// does; it STORES its sums and then writes the launch's epoch into the tile's flags; the other runs of the tile add
+// theirs once they see it.  One flag per epilogue warp: a warp adds to the rows that the warp of the same TMEM quarter
+// stored, so no warp of a CTA waits for another (a barrier between them would not end when one of them has given up).
+// Flags are never reset: every launch has its own epoch and takes the next of a few arrays.
 constexpr int GM_FLAG_SLOTS = 8;
 constexpr int GM_MAX_TILES = 8192;
-__device__ uint32_t g_tile_flags[GM_FLAG_SLOTS][GM_MAX_TILES];
+__device__ uint32_t g_tile_flags[GM_FLAG_SLOTS][GM_MAX_TILES][GM_EP_WARPS];
+static std::atomic<bool> g_gemm_hold{false};   // testing: launches leave their flags down
 
 constexpr int GM_MAX_OPS = 4;      // matrices that share one input (q|k|v, gate|up) run as one launch
 
@@ -123,6 +126,7 @@ struct GemmArgs {
     int store_first;       // 1: split tiles of matrices without a residual use the store-then-add protocol above
     int flag_slot;
     uint32_t epoch;
+    int hold;              // testing: flags stay down
     const float* tok_scale;    // per token: the power of two its row of x was divided by, or null
     int bounds[GM_MAX_GRID + 1];   // CTA c works on half slabs [bounds[c], bounds[c + 1]) (even numbers)
 };
@@ -326,7 +330,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             const bool whole = (entire && (op.res == nullptr || !a.tma_out)) || (first_mode && sg.s1 == a.n_slabs);
             const bool raise_flag = first_mode && whole && !entire;
             if (first_mode && !whole) {   // the tile's last-slab run has to have stored before anything is added
-                const uint32_t* fl = &g_tile_flags[a.flag_slot][sg.tile];
+                const uint32_t* fl = &g_tile_flags[a.flag_slot][sg.tile][quarter];
                 uint32_t seen = 0, spins = 0;
                 if (lane == 0) {
                     while ((seen = ld_acquire_u32(fl)) != a.epoch) {
@@ -403,12 +407,11 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             if (lane == 0) mbar_arrive(bar_dempty + 8 * buf);   // the next instructions may overwrite the accumulators
             if (raise_flag) {
                 if (lane == 0) {
-                    bulk_wait_all<0>();   // the stores must have landed before the flag goes up
+                    bulk_wait_all<0>();   // this warp's stores must have landed before its flag goes up
                     asm volatile("fence.proxy.async;" ::: "memory");
+                    if (!a.hold) st_release_u32(&g_tile_flags[a.flag_slot][sg.tile][quarter], a.epoch);
                 }
                 __syncwarp();
-                asm volatile("bar.sync 1, %0;" ::"n"(GM_EP_WARPS * 32) : "memory");
-                if (quarter == 0 && lane == 0) st_release_u32(&g_tile_flags[a.flag_slot][sg.tile], a.epoch);
             }
         }
         if (lane == 0) bulk_wait_all<0>();   // this thread's output copies are complete
@@ -607,6 +610,7 @@ cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x
     a.epoch = epoch_counter.fetch_add(1) + 1;
     if (a.epoch == 0) a.epoch = epoch_counter.fetch_add(1) + 1;   // flags start out as zero: never use that value
     a.flag_slot = (int)(a.epoch % GM_FLAG_SLOTS);
+    a.hold = g_gemm_hold.load(std::memory_order_relaxed) ? 1 : 0;
     // What an output holds before the kernel: the residual when there is one (every run then adds to it); zeros
     // when runs add without the store-first protocol; else nothing.  With outs_ready the caller has done this.
     for (int i = 0; i < n && !outs_ready; ++i) {
@@ -719,6 +723,8 @@ bool gemm_outputs_can_be_preset(float* const* outs, const int64_t* ldos, int n) 
         if (ldos[i] % 4 != 0 || (reinterpret_cast<uintptr_t>(outs[i]) & 15u) != 0) return false;
     return true;
 }
+
+void set_gemm_hold(bool on) { g_gemm_hold.store(on, std::memory_order_relaxed); }
 
 int read_gemm_status(bool clear) {
     int v = 0;

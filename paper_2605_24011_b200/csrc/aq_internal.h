@@ -154,5 +154,6 @@ int current_device();               // cudaGetDevice, or -1
 int sm_count();                     // of the current device
 void count_launch(int n = 1);       // process-wide count of this library's kernel launches
 int read_gemm_status(bool clear);   // nonzero: a bounded wait in the GEMM kernel ran out
+void set_gemm_hold(bool on);        // testing: tiles of the GEMM that are stored first are never reported as stored
 
 }  // namespace aq

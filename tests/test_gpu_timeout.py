@@ -62,3 +62,32 @@ def test_bounded_wait_runs_out_and_the_next_call_is_clean(aq, M):
     aq.aq_check()
     check_program(prog, names, ws, M, torch.float16, quant)
     assert bool(torch.isfinite(out.float()).all())
+
+
+def test_prefill_wait_runs_out_and_the_next_call_is_clean(aq):
+    """104 tiles of 256 rows x 128 tokens on about 148 CTAs: many are stored by one run and added to by another, whose
+    epilogue warps give up one by one while the hook is on.  Every CTA has to return all the same."""
+    M, N, K, bits = 512, 6656, 4096, 3
+    W = synth.weights(N, K, 56, outliers=True)
+    h = aq.aq_pack(bits, 32, torch.from_numpy(W).cuda())
+    x = torch.from_numpy(synth.activations(M, K, 57)).to(torch.float16).cuda()
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    aq.aq_linear(h, x, y)
+    aq.aq_check()
+    try:
+        aq.aq_debug_decode_hold(True)
+        t0 = time.time()
+        aq.aq_linear(h, x, y)
+        with pytest.raises(aq.AqError) as err:
+            aq.aq_check()
+        assert err.value.status == aq.AQ_ERR_TIMEOUT
+        assert time.time() - t0 < 10.0
+        aq.aq_check()                                 # the record was cleared: no second report
+    finally:
+        aq.aq_debug_decode_hold(False)
+    y.fill_(float("nan"))
+    aq.aq_linear(h, x, y)
+    aq.aq_check()
+    rows = np.arange(0, M, 37)
+    want, T = O.linear(*O.quantize(W, bits), x[rows].double().cpu().numpy())
+    assert O.linear_excess(y[rows].double().cpu().numpy(), want, T).max() <= 1.0
