@@ -133,11 +133,13 @@ __global__ void __launch_bounds__(AT_WARPS * 32, 1) attn_decode_kernel(const Att
     for (int nd = 0; nd < AT_D / 8; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
     float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // rows g and g + 8: running maximum (log2 domain), sum
 
-    // Launched as a programmatic dependent: the kernel before this one on the stream may still be at work.  Only q and the
-    // last M rows of the cache can be its output (or are appended here): a warp whose first tiles lie before those rows
-    // starts its copies at once, the others wait first; all wait before they read q and before they write anything.
+    // Launched as a programmatic dependent: the kernel before this one on the stream may still be at work.  In a stack
+    // program's step that is the decode launch, which writes no cache: only the last M rows are new (appended here), and a
+    // warp whose first tiles lie before them starts its copies at once.  A standalone call can follow anything, a linear that
+    // has let its successor in and is still storing rows of the cache included, so there every warp waits first.  All wait
+    // before they read q and before they write anything.
     const int64_t old = a.L - a.M;   // rows that were there before
-    const bool early = p0 + (int64_t)(warp + AT_WARPS * (min(AT_STAGES - 1, my_tiles) - 1) + 1) * AT_TILE <= old;
+    const bool early = a.qf != nullptr && p0 + (int64_t)(warp + AT_WARPS * (min(AT_STAGES - 1, my_tiles) - 1) + 1) * AT_TILE <= old;
     auto first_tiles = [&] {
 #pragma unroll
         for (int s = 0; s < AT_STAGES - 1; ++s) {

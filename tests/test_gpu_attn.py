@@ -172,3 +172,29 @@ def test_attention_of_several_new_tokens(aq, name):
         assert np.all(np.isfinite(got))
         tol = (U[name] + 2.0 ** -16) * T + 1e-6
         assert np.all(np.abs(got - ref) <= tol), f"M={M} H={H} Hkv={Hkv} L={L} {name}: worst {np.max(np.abs(got - ref) / tol):.3f}"
+
+
+def test_attention_right_after_a_linear_that_wrote_older_rows(aq):
+    """With one key/value head a linear of 8 tokens may write its values straight into the cache.  It lets its successor in
+    before its stores; an attention of one token that follows directly has to see all eight rows.  Same cache, same kernel,
+    nothing else at work: the second call's output is the first one's bit for bit."""
+    g = np.random.default_rng(60)
+    L, Lmax, K, M = 96, 128, 4096, 8
+    W = torch.from_numpy((g.standard_normal((128, K)) * 0.02).astype(np.float32)).cuda()
+    h = aq.aq_pack(4, 32, W)
+    q = torch.from_numpy(g.standard_normal((8, 128)).astype(np.float32)).half().cuda()
+    kc = torch.from_numpy(g.standard_normal((1, Lmax, 128)).astype(np.float32)).half().cuda()
+    vc = torch.from_numpy(g.standard_normal((1, Lmax, 128)).astype(np.float32)).half().cuda()
+    scratch = torch.empty(aq.aq_attn_scratch_bytes(1), dtype=torch.uint8, device="cuda")
+    out, again = (torch.empty((8, 128), dtype=torch.float32, device="cuda") for _ in range(2))
+    for rep in range(50):
+        x = torch.from_numpy(g.standard_normal((M, K)).astype(np.float32)).half().cuda()
+        vc[0, L - M:L] = 1000.0
+        aq.aq_linear(h, x, vc[0, L - M:L])
+        aq.aq_attn_decode(q, kc, vc, L, out, scratch)
+        torch.cuda.synchronize()
+        assert float(vc[0, :L].abs().max()) < 100.0
+        aq.aq_attn_decode(q, kc, vc, L, again, scratch)
+        torch.cuda.synchronize()
+        assert torch.equal(out, again), rep
+    aq.aq_check()
