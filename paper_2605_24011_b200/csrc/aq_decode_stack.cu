@@ -49,6 +49,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "aq_decode_tc.cuh"
@@ -462,18 +463,23 @@ __device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint3
             tmem_st_16x128(ta, va);
             tmem_st_16x128(ta + (16u << 16), vb);
         } else {
-            uint32_t v[32];
-            auto unpack = [&](const uint8_t* f) {
-                if (bits == 2) dt_unpack1<2, BF16>(f, lane, v);
-                else if (bits == 3) dt_unpack1<3, BF16>(f, lane, v);
-                else dt_unpack1<4, BF16>(f, lane, v);
+            // (the second fragment's words are loaded before the wait: what follows it delays the stage)
+            auto both = [&](auto width) -> bool {
+                constexpr int BITS = decltype(width)::value;
+                LaneCodes<BITS> la, lb;
+                load_lane_codes<BITS>(la, fr, lane);
+                load_lane_codes<BITS>(lb, fr + fb, lane);
+                uint32_t v[32];
+                dt_unpack<BITS, BF16>(la, v);
+                if (!stage_free()) return false;
+                tc_fence_after();
+                tmem_st_16x128(ta, v);
+                dt_unpack<BITS, BF16>(lb, v);
+                tmem_st_16x128(ta + (16u << 16), v);
+                return true;
             };
-            unpack(fr);
-            if (!stage_free()) return;
-            tc_fence_after();
-            tmem_st_16x128(ta, v);
-            unpack(fr + fb);
-            tmem_st_16x128(ta + (16u << 16), v);
+            const bool ok = bits == 2 ? both(std::integral_constant<int, 2>()) : bits == 3 ? both(std::integral_constant<int, 3>()) : both(std::integral_constant<int, 4>());
+            if (!ok) return;
         }
         *reinterpret_cast<uint4*>(&sh.dm[stage][half * DS_FRAGS + quarter * 2 + (lane >> 4)][(lane & 15) * 16]) = dm;
         if (half == 0 && quarter == 0 && lane == 0) sh.sdesc[stage] = d;

@@ -60,3 +60,46 @@ def test_row_tiles(M, dtype, N):
 @pytest.mark.parametrize("M,dtype", [(1, "f16"), (1, "bf16"), (2, "f16"), (6, "bf16")])
 def test_wide_magnitudes(M, dtype, bits):
     _run(M, 512, 96, dtype, (bits,), True)
+
+
+def _emulated(d, m, q, x):
+    """y and sum |x w| of the several-token arithmetic with binary16 activations, rounding where it rounds: the two half sums of
+    a block are joined in binary32, two multiply-adds bring the block into the unit's sum (256 k), units are added in steps of
+    2^-24.  d, m [N][blocks], q [N][K] (codes), x [M][K] (binary64)."""
+    f32 = lambda v: v.astype(np.float32).astype(np.float64)
+    N, K = q.shape
+    M = x.shape[0]
+    total = np.zeros((M, N))
+    for u0 in range(0, K, 256):
+        acc = np.zeros((M, N))
+        for b in range(u0 // 32, (u0 + 256) // 32):
+            s = slice(32 * b, 32 * b + 32)
+            c = f32(x[:, s] @ q[:, s].astype(np.float64).T)
+            sx = f32(x[:, s].sum(1))[:, None]
+            acc = f32(d[:, b] * c + f32(m[:, b] * sx + acc))
+        total += np.round(acc * 2.0 ** 24) * 2.0 ** -24
+    return total
+
+
+@pytest.mark.parametrize("bits", (2, 3, 4))
+@pytest.mark.parametrize("M", (2, 3, 8))
+def test_several_tokens_round_like_binary32(M, bits):
+    """The error against binary64 is that of the binary32 steps (twice their root mean square leaves room for what the
+    tensor core itself drops below a product's last place); codes used as subnormals with many leading zeros lost ten times
+    that."""
+    from paper_2605_24011_b200 import aq
+    N, K = 256, 2048
+    W = synth.weights(N, K, 93, bits)
+    h = aq.aq_pack(bits, 32, torch.from_numpy(W).cuda())
+    d, m, q = O.quantize(W, bits)
+    prog = aq.Program([K, N], [{"w": h, "src": 0, "dst": 1}])
+    x0 = torch.from_numpy(synth.activations(M, K, 94, M)).half().cuda()
+    ws = torch.empty(prog.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+    aq.aq_stack_forward(prog, x0, None, 1, M, ws)
+    aq.aq_check()
+    x = x0.double().cpu().numpy()
+    want, T = O.linear(d, m, q, x)
+    d, m = (np.asarray(v, dtype=np.float64).reshape(N, K // 32) for v in (d, m))
+    rms = lambda y: float(np.sqrt(np.mean(((y - want) / T) ** 2)))
+    got, bound = rms(aq.stack_buffer(prog, ws, M, 1).double().cpu().numpy()), rms(_emulated(d, m, np.asarray(q).reshape(N, K), x))
+    assert got <= 2.0 * bound, f"{got:.2e}, binary32 steps {bound:.2e}"
