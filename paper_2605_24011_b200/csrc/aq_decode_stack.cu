@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
                     const uint32_t sc = dt_fix_scale(mx);
                     dt_stage4_fix(sl, kl, f, sc);
-                    if ((lane & 7) == 0) reinterpret_cast<float2*>(sl + DT_SUMS<1>)[kl >> 5] = make_float2(sum, dt_fix_step(sc));
+                    if ((lane & 7) == 0) reinterpret_cast<float2*>(sl + DT_SUMS<1>)[kl >> 5] = make_float2(sum, dt_fix_step(sc, sum));
                 } else {
                     dt_stage4(sl, m, kl, r);
                     if ((lane & 7) == 0) reinterpret_cast<float*>(sl + DT_SUMS<MT>)[(kl >> 5) * 8 + m] = sum;

@@ -103,3 +103,26 @@ def test_several_tokens_round_like_binary32(M, bits):
     rms = lambda y: float(np.sqrt(np.mean(((y - want) / T) ** 2)))
     got, bound = rms(aq.stack_buffer(prog, ws, M, 1).double().cpu().numpy()), rms(_emulated(d, m, np.asarray(q).reshape(N, K), x))
     assert got <= 2.0 * bound, f"{got:.2e}, binary32 steps {bound:.2e}"
+
+
+@pytest.mark.parametrize("dtype,positive", [("f16", False), ("f16", True), ("bf16", False)])
+@pytest.mark.parametrize("bad", (float("inf"), float("-inf"), float("nan")))
+def test_one_token_with_a_non_finite_element_is_the_first_of_two(bad, dtype, positive):
+    """A sum that an infinite or undefined element has made infinite or undefined leaves the kernel as the largest or the smallest
+    number its packed sums hold: the same one whether a token comes alone or with another (whose arithmetic is the tensor
+    core's own).  `positive`: weights whose codes and minima keep the sign, so that some rows stay infinite."""
+    from paper_2605_24011_b200 import aq
+    N, K = 64, 512
+    W = synth.weights(N, K, 95, int(positive))
+    h = aq.aq_pack(3, 32, torch.from_numpy(np.abs(W) + np.float32(0.01) if positive else W).cuda())
+    prog = aq.Program([K, N], [{"w": h, "src": 0, "dst": 1}])
+    x = torch.ones((2, K), dtype=torch.float16 if dtype == "f16" else torch.bfloat16, device="cuda")
+    x[0, 37] = bad
+    got = []
+    for M in (1, 2):
+        ws = torch.empty(prog.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+        aq.aq_stack_forward(prog, x, None, 1, M, ws)
+        aq.aq_check()
+        got.append(aq.stack_buffer(prog, ws, M, 1)[0].clone())
+    assert torch.equal(got[0], got[1])
+    assert (got[0].abs() > 1e8).all() and (not positive or bad < 0 or bad != bad or (got[0] > 0).any())
