@@ -38,6 +38,17 @@ Cache& cache() {
     return *c;
 }
 
+// `device` is the current one while this lives (the calling thread's own may be another).
+struct OnDevice {
+    int before = -1;
+    bool changed = false;
+    explicit OnDevice(int device) {
+        if (cudaGetDevice(&before) != cudaSuccess) { cudaGetLastError(); before = -1; }
+        if (before != device) changed = cudaSetDevice(device) == cudaSuccess;
+    }
+    ~OnDevice() { if (changed && before >= 0) cudaSetDevice(before); }
+};
+
 }  // namespace
 
 void* device_alloc(size_t bytes, int device) {
@@ -56,6 +67,7 @@ void* device_alloc(size_t bytes, int device) {
             return p;
         }
     }
+    OnDevice here(device);
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
     cudaGetLastError();
@@ -73,12 +85,12 @@ void* device_alloc(size_t bytes, int device) {
 void device_release(void* p, size_t bytes, int device) {
     if (p == nullptr) return;
     bytes = (bytes + 511) / 512 * 512;
-    int current = -1;
-    if (cudaGetDevice(&current) != cudaSuccess) current = -1;
-    if (current != device) cudaSetDevice(device);
-    const bool idle = cudaDeviceSynchronize() == cudaSuccess;   // whatever still uses the block, on any stream
-    if (!idle) cudaGetLastError();
-    if (current >= 0 && current != device) cudaSetDevice(current);
+    bool idle;
+    {
+        OnDevice there(device);
+        idle = cudaDeviceSynchronize() == cudaSuccess;   // whatever still uses the block, on any stream
+        if (!idle) cudaGetLastError();
+    }
     std::vector<void*> out;
     {
         Cache& c = cache();

@@ -1,0 +1,106 @@
+"""Host logic of `csrc/aq_memory.cu` (device blocks out of a bounded cache, copies into pageable memory), compiled with the
+host compiler against a stand-in for the CUDA runtime that knows on which device a block lies and what was asked of it."""
+import os
+import shutil
+import subprocess
+import textwrap
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2605_24011_b200", "csrc")
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host C++ compiler")
+
+FAKE = textwrap.dedent(r"""
+    #pragma once
+    #include <atomic>
+    #include <cstddef>
+    #include <cstdint>
+    #include <cstdio>
+    #include <cstdlib>
+    #include <cstring>
+    #include <map>
+    #include <mutex>
+    typedef struct FakeStream* cudaStream_t;
+    typedef struct FakeEvent* cudaEvent_t;
+    enum cudaError_t { cudaSuccess = 0, cudaErrorMemoryAllocation = 2, cudaErrorUnknown = 999 };
+    enum cudaMemcpyKind { cudaMemcpyDeviceToHost = 2 };
+    constexpr unsigned cudaHostAllocPortable = 1, cudaEventDisableTiming = 2;
+    namespace fake {
+    struct Alloc { int device; size_t bytes; };
+    inline std::mutex m;
+    inline std::map<void*, Alloc> live;         // device blocks the driver has given out
+    inline thread_local int current = 0;
+    inline size_t limit = SIZE_MAX, used = 0;   // device memory
+    inline int mallocs = 0, frees = 0, device_syncs = 0;
+    inline std::atomic<int> stream_syncs{0}, copies{0}, copies_fail_from{1 << 30}, event_syncs_fail_from{1 << 30}, event_syncs{0};
+    inline std::atomic<bool> unsynced{false};   // a copy was issued and its stream has not been waited for since
+    }
+    inline cudaError_t cudaGetDevice(int* d) { *d = fake::current; return cudaSuccess; }
+    inline cudaError_t cudaSetDevice(int d) { fake::current = d; return cudaSuccess; }
+    inline cudaError_t cudaGetLastError() { return cudaSuccess; }
+    inline cudaError_t cudaDeviceSynchronize() { ++fake::device_syncs; return cudaSuccess; }
+    inline cudaError_t cudaMalloc(void** p, size_t n) {
+        std::lock_guard<std::mutex> l(fake::m);
+        if (fake::used + n > fake::limit) return cudaErrorMemoryAllocation;
+        *p = std::malloc(n);
+        fake::live[*p] = {fake::current, n}; fake::used += n; ++fake::mallocs;
+        return cudaSuccess;
+    }
+    inline cudaError_t cudaFree(void* p) {
+        std::lock_guard<std::mutex> l(fake::m);
+        auto it = fake::live.find(p);
+        if (it == fake::live.end()) { std::printf("freed twice\n"); std::exit(1); }
+        fake::used -= it->second.bytes; fake::live.erase(it); ++fake::frees;
+        std::free(p);
+        return cudaSuccess;
+    }
+    inline cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::malloc(n); return cudaSuccess; }
+    inline cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = reinterpret_cast<cudaEvent_t>(std::malloc(1)); return cudaSuccess; }
+    inline cudaError_t cudaEventDestroy(cudaEvent_t e) { std::free(e); return cudaSuccess; }
+    inline cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+    inline cudaError_t cudaEventSynchronize(cudaEvent_t) { return fake::event_syncs++ >= fake::event_syncs_fail_from ? cudaErrorUnknown : cudaSuccess; }
+    inline cudaError_t cudaStreamSynchronize(cudaStream_t) { ++fake::stream_syncs; fake::unsynced = false; return cudaSuccess; }
+    inline cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+        if (fake::copies++ >= fake::copies_fail_from) return cudaErrorUnknown;
+        fake::unsynced = true;
+        std::memcpy(d, s, n);
+        return cudaSuccess;
+    }
+""")
+
+MAIN = r"""
+    #include "aq_memory.cu"
+    namespace aq { int current_device() { int d = 0; cudaGetDevice(&d); return d; } }
+    using namespace aq;
+    #define CHECK(c) do { if (!(c)) { std::printf("FAIL line %d: %s\n", __LINE__, #c); return 1; } } while (0)
+"""
+
+
+def _run(tmp_path, body, flags=()):
+    (tmp_path / "cuda_runtime.h").write_text(FAKE)
+    src = tmp_path / "t.cpp"
+    src.write_text(textwrap.dedent(MAIN) + "int main() {\n" + textwrap.dedent(body) + '\n    std::printf("ok\\n");\n    return 0;\n}\n')
+    exe = tmp_path / "t"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", *flags, "-I", str(tmp_path), "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout + r.stderr
+
+
+def test_a_block_lies_on_the_device_it_was_asked_for(tmp_path):
+    _run(tmp_path, r"""
+        fake::current = 1;
+        void* p = device_alloc(1 << 20, 0);            // a handle of device 0 exported while device 1 is current
+        CHECK(p && fake::live[p].device == 0 && fake::current == 1);
+        device_release(p, 1 << 20, 0);
+        fake::current = 0;
+        void* q = device_alloc(1 << 20, 0);            // the next handle of device 0 may be built on that block
+        CHECK(q && fake::live[q].device == 0);
+        // the retry after the cache has been emptied looks at the device, too
+        void* r = device_alloc(3 << 20, 0);
+        device_release(r, 3 << 20, 0);
+        fake::current = 1;
+        fake::limit = fake::used;
+        void* t = device_alloc(2 << 20, 0);
+        CHECK(t && fake::live[t].device == 0 && fake::current == 1);
+    """)
