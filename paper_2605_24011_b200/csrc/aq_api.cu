@@ -71,12 +71,12 @@ static aq_status_t new_handle(int bits, int block, int64_t N, int64_t K, aq_hand
     h->n_frags = (int64_t)h->NT * h->KP * 2;
     h->dev_bytes = (size_t)h->n_frags * frag_bytes(bits);
     h->frags = nullptr; h->acc = nullptr; h->flags = nullptr; h->last_stream = nullptr;
-    h->big = nullptr; h->big_bytes = 0; h->sb = nullptr;
+    h->big = nullptr; h->big_bytes = 0; h->sb = nullptr; h->sb_held = 0;
     const size_t acc_bytes = (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float);
     // one block: fragments, accumulators, flags (the last two start at zero: see clear_scratch)
     const size_t frag_end = (h->dev_bytes + 255) / 256 * 256, acc_end = frag_end + (acc_bytes + 255) / 256 * 256;
     h->block_bytes = acc_end + 256;
-    h->frags = static_cast<uint8_t*>(device_alloc(h->block_bytes, dev));
+    h->frags = static_cast<uint8_t*>(device_alloc(h->block_bytes, dev, &h->block_held));
     if (!h->frags) { delete h; return AQ_ERR_ALLOC; }
     h->acc = reinterpret_cast<float*>(h->frags + frag_end);
     h->flags = reinterpret_cast<int*>(h->frags + acc_end);
@@ -92,8 +92,8 @@ static cudaError_t clear_scratch(const aq_handle_s* h, cudaStream_t s) {
 
 static void destroy(aq_handle_s* h) {
     device_release(h->big, h->big_bytes, h->device);
-    device_release(h->sb, sb_side_bytes(h), h->device);
-    device_release(h->frags, h->block_bytes, h->device);
+    device_release(h->sb, h->sb_held, h->device);
+    device_release(h->frags, h->block_held, h->device);
     h->magic = 0;
     delete h;
 }
@@ -148,7 +148,7 @@ static aq_status_t new_sb_handle(int bits, int block, int sblock, int64_t N, int
     aq_handle_t h = nullptr;
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
-    h->sb = static_cast<uint8_t*>(device_alloc(sb_side_bytes(h), h->device));
+    h->sb = static_cast<uint8_t*>(device_alloc(sb_side_bytes(h), h->device, &h->sb_held));
     if (!h->sb) { destroy(h); return AQ_ERR_ALLOC; }
     *out = h;
     return AQ_OK;
@@ -183,14 +183,15 @@ aq_status_t aq_import_sb(int bits, int block, int sblock, int64_t N, int64_t K, 
     cudaStream_t s = (cudaStream_t)stream;
     const size_t plain_bytes = (size_t)N * (size_t)(K / 32) * (size_t)(4 + 4 * bits);
     const size_t plain_at = (nbytes + 255) / 256 * 256;
-    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device));
+    size_t tmp_held = 0;
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device, &tmp_held));
     if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, true, s);
     if (e == cudaSuccess) e = launch_import(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    device_release(tmp, plain_at + plain_bytes, h->device);
+    device_release(tmp, tmp_held, h->device);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
     *out = h;
@@ -207,13 +208,14 @@ aq_status_t aq_import(int bits, int block, int64_t N, int64_t K, const void* can
     if (st != AQ_OK) return st;
     if (nbytes != (size_t)N * (size_t)(K / 32) * (size_t)(4 + 4 * bits)) { destroy(h); return AQ_ERR_INVALID_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(nbytes, h->device));
+    size_t tmp_held = 0;
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(nbytes, h->device, &tmp_held));
     if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_import(h, tmp, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    device_release(tmp, nbytes, h->device);
+    device_release(tmp, tmp_held, h->device);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
     h->last_stream = s;
     *out = h;
@@ -234,12 +236,13 @@ aq_status_t aq_export(aq_handle_t h, void* canon_host, size_t cap, size_t* nbyte
     if (nbytes) *nbytes = need;
     if (!canon_host) return nbytes ? AQ_OK : AQ_ERR_INVALID_ARG;
     if (cap < need) return AQ_ERR_INVALID_ARG;
-    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(need, h->device));
+    size_t tmp_held = 0;
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(need, h->device, &tmp_held));
     if (!tmp) return AQ_ERR_ALLOC;
     cudaStream_t s = h->last_stream;
     cudaError_t e = launch_export(h, tmp, s);
     if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
-    device_release(tmp, need, h->device);
+    device_release(tmp, tmp_held, h->device);
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }
@@ -252,13 +255,14 @@ aq_status_t aq_export_sb(aq_handle_t h, void* canon_host, size_t cap, size_t* nb
     if (cap < need) return AQ_ERR_INVALID_ARG;
     const size_t plain_bytes = (size_t)h->N * (size_t)(h->K / 32) * (size_t)(4 + 4 * h->bits);
     const size_t plain_at = (need + 255) / 256 * 256;
-    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device));
+    size_t tmp_held = 0;
+    uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device, &tmp_held));
     if (!tmp) return AQ_ERR_ALLOC;
     cudaStream_t s = h->last_stream;
     cudaError_t e = launch_export(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, false, s);
     if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
-    device_release(tmp, plain_at + plain_bytes, h->device);
+    device_release(tmp, tmp_held, h->device);
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }
@@ -311,9 +315,10 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
         if (need > h->big_bytes) {
             device_release(h->big, h->big_bytes, h->device);   // (waits for whatever still uses the old one)
             h->big_bytes = 0;
-            h->big = static_cast<uint8_t*>(device_alloc(need, h->device));
+            size_t held = 0;
+            h->big = static_cast<uint8_t*>(device_alloc(need, h->device, &held));
             if (!h->big) return AQ_ERR_ALLOC;
-            h->big_bytes = need;
+            h->big_bytes = held;
         }
         float* sums = (ydt == AQ_F32) ? (float*)y_dev : reinterpret_cast<float*>(h->big);
         void* x16 = h->big + out_bytes;

@@ -19,11 +19,13 @@ struct aq_handle_s {
     int KP;            // pair slabs of 256 k
     int64_t n_frags;   // NT * KP * 2
     size_t dev_bytes;  // n_frags * frag_bytes
-    size_t block_bytes;   // of the one device block that holds frags, acc and flags
+    size_t block_bytes;   // of the one device block that holds frags, acc and flags: what they take ...
+    size_t block_held;    // ... and what the block has
     uint8_t* frags;    // DEVICE: fragment layout
     float* acc;        // DEVICE: [AQ_DECODE_MAX_M][NT*16] accumulation scratch, zero between calls
     uint8_t* sb;       // DEVICE: super-block parameters (32 bytes per row and super-block) of a handle made by aq_pack_sb /
                        // aq_import_sb, else null
+    size_t sb_held;
     uint8_t* big;      // DEVICE: scratch of aq_linear with M > AQ_DECODE_MAX_M (float32 sums, binary16 copy of bfloat16
                        // activations, row scales), allocated when the handle first sees such a call and grown on demand
     size_t big_bytes;
@@ -144,10 +146,10 @@ cudaError_t launch_attn_step(const float* q, const float* k, const float* v, voi
 cudaError_t launch_attn_angles(void* turn, int M, int64_t pos, float theta, cudaStream_t s);   // turn: M * 512 bytes
 cudaError_t launch_kv_append(void* kc, void* vc, const void* k, const void* v, int n_kv, int D, int64_t pos, int64_t Lmax, cudaStream_t s);
 
-// memory (aq_memory.cu): device blocks out of a bounded cache (null: no memory left); a copy into pageable host memory, complete
-// when the call returns
-void* device_alloc(size_t bytes, int device);
-void device_release(void* p, size_t bytes, int device);
+// memory (aq_memory.cu): device blocks out of a bounded cache (null: no memory left; *held: the bytes the block really has, which is
+// what it is released with); a copy into pageable host memory, complete when the call returns
+void* device_alloc(size_t bytes, int device, size_t* held);
+void device_release(void* p, size_t held, int device);
 cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t s);
 
 int current_device();               // cudaGetDevice, or -1

@@ -15,7 +15,8 @@ namespace aq {
 namespace {
 
 // ---- device blocks ------------------------------------------------------------------
-// A released block is kept for the next handle of about its size.  Bounded in bytes and number; a block that the next
+// A released block is kept for the next handle of about its size.  Bounded in bytes and number (a block counts with the bytes
+// it was allocated with, however little its last owner asked for); a block that the next
 // few releases have not found a use for goes back to the driver, and all of them do when an allocation fails.  Blocks
 // are idle when they come in (device_release waits for the device, as cudaFree did), so a block may go to any stream.
 struct Block {
@@ -51,8 +52,9 @@ struct OnDevice {
 
 }  // namespace
 
-void* device_alloc(size_t bytes, int device) {
+void* device_alloc(size_t bytes, int device, size_t* held) {
     bytes = (bytes + 511) / 512 * 512;
+    *held = bytes;
     Cache& c = cache();
     {
         std::lock_guard<std::mutex> lock(c.m);
@@ -63,6 +65,7 @@ void* device_alloc(size_t bytes, int device) {
         }
         if (best < c.blocks.size()) {
             void* p = c.blocks[best].p;
+            *held = c.blocks[best].bytes;
             c.blocks.erase(c.blocks.begin() + best);
             return p;
         }
@@ -82,9 +85,8 @@ void* device_alloc(size_t bytes, int device) {
     return nullptr;
 }
 
-void device_release(void* p, size_t bytes, int device) {
+void device_release(void* p, size_t held, int device) {
     if (p == nullptr) return;
-    bytes = (bytes + 511) / 512 * 512;
     bool idle;
     {
         OnDevice there(device);
@@ -96,7 +98,7 @@ void device_release(void* p, size_t bytes, int device) {
         Cache& c = cache();
         std::lock_guard<std::mutex> lock(c.m);
         ++c.clock;
-        if (idle && bytes <= CACHE_BYTES) c.blocks.push_back({p, bytes, device, c.clock});
+        if (idle && held <= CACHE_BYTES) c.blocks.push_back({p, held, device, c.clock});
         else out.push_back(p);
         size_t total = 0;
         for (const Block& b : c.blocks) total += b.bytes;

@@ -90,17 +90,40 @@ def _run(tmp_path, body, flags=()):
 def test_a_block_lies_on_the_device_it_was_asked_for(tmp_path):
     _run(tmp_path, r"""
         fake::current = 1;
-        void* p = device_alloc(1 << 20, 0);            // a handle of device 0 exported while device 1 is current
+        size_t held;
+        void* p = device_alloc(1 << 20, 0, &held);            // a handle of device 0 exported while device 1 is current
         CHECK(p && fake::live[p].device == 0 && fake::current == 1);
-        device_release(p, 1 << 20, 0);
+        device_release(p, held, 0);
         fake::current = 0;
-        void* q = device_alloc(1 << 20, 0);            // the next handle of device 0 may be built on that block
+        void* q = device_alloc(1 << 20, 0, &held);            // the next handle of device 0 may be built on that block
         CHECK(q && fake::live[q].device == 0);
         // the retry after the cache has been emptied looks at the device, too
-        void* r = device_alloc(3 << 20, 0);
-        device_release(r, 3 << 20, 0);
+        void* r = device_alloc(3 << 20, 0, &held);
+        device_release(r, held, 0);
         fake::current = 1;
         fake::limit = fake::used;
-        void* t = device_alloc(2 << 20, 0);
+        void* t = device_alloc(2 << 20, 0, &held);
         CHECK(t && fake::live[t].device == 0 && fake::current == 1);
+    """)
+
+
+def test_a_block_counts_with_the_bytes_it_has(tmp_path):
+    """Ten blocks of 24 MB are handed out again for requests of 20 and 16 MB, two of 40 MB join: what the cache keeps with
+    nothing in use stays within its 256 MB."""
+    _run(tmp_path, r"""
+        void* p[10];
+        size_t held[10];
+        for (size_t s : {24u << 20, 20u << 20, 16u << 20}) {
+            for (int i = 0; i < 10; ++i) {
+                p[i] = device_alloc(s, 0, &held[i]);
+                CHECK(p[i] && held[i] == fake::live[p[i]].bytes && held[i] >= s);
+            }
+            for (int i = 0; i < 10; ++i) device_release(p[i], held[i], 0);
+        }
+        CHECK(fake::mallocs >= 10 && fake::used >= (200u << 20) && fake::used <= (256u << 20));
+        void* q[2];
+        size_t q_held[2];
+        for (int i = 0; i < 2; ++i) q[i] = device_alloc(40u << 20, 0, &q_held[i]);
+        for (int i = 0; i < 2; ++i) device_release(q[i], q_held[i], 0);
+        CHECK(fake::used <= (256u << 20));
     """)
