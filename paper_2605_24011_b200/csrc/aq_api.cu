@@ -20,6 +20,33 @@ aq_status_t cuda_fail(cudaError_t e) {
 
 bool handle_ok(aq_handle_t h) { return h != nullptr && h->magic == AQ_HANDLE_MAGIC; }
 
+bool being_recorded(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); return true; }   // (the legacy stream beside a recording)
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+void handle_used(aq_handle_t h, cudaStream_t s, bool recorded) {
+    if (s != h->last_stream || recorded || s == cudaStreamPerThread) h->elsewhere = true;
+    h->last_stream = s;
+}
+
+static void handle_made(aq_handle_t h, cudaStream_t s) {
+    h->last_stream = s;
+    if (cudaStreamGetId(s, &h->stream_id) != cudaSuccess) { cudaGetLastError(); h->elsewhere = true; }
+    if (s == cudaStreamPerThread || being_recorded(s)) h->elsewhere = true;   // (the former is another stream in every thread)
+}
+
+// Waits for the handle's last stream; true when that was waiting for all uses of its memory: it has been used on the stream
+// that it was made on and on no other (nor on a later stream of the same address), and no graph holds it.
+static bool handle_idle(const aq_handle_s* h) {
+    if (cudaStreamSynchronize(h->last_stream) != cudaSuccess) { cudaGetLastError(); return false; }
+    unsigned long long id = 0;
+    if (h->elsewhere) return false;
+    if (cudaStreamGetId(h->last_stream, &id) != cudaSuccess) { cudaGetLastError(); return false; }
+    return id == h->stream_id;
+}
+
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
@@ -72,6 +99,7 @@ static aq_status_t new_handle(int bits, int block, int64_t N, int64_t K, aq_hand
     h->dev_bytes = (size_t)h->n_frags * frag_bytes(bits);
     h->frags = nullptr; h->acc = nullptr; h->flags = nullptr; h->last_stream = nullptr;
     h->big = nullptr; h->big_bytes = 0; h->sb = nullptr; h->sb_held = 0;
+    h->stream_id = 0; h->elsewhere = false;
     const size_t acc_bytes = (size_t)AQ_DECODE_MAX_M * h->NT * 16 * sizeof(float);
     // one block: fragments, accumulators, flags (the last two start at zero: see clear_scratch)
     const size_t frag_end = (h->dev_bytes + 255) / 256 * 256, acc_end = frag_end + (acc_bytes + 255) / 256 * 256;
@@ -90,10 +118,10 @@ static cudaError_t clear_scratch(const aq_handle_s* h, cudaStream_t s) {
     return cudaMemsetAsync(h->acc, 0, h->block_bytes - (size_t)(reinterpret_cast<uint8_t*>(h->acc) - h->frags), s);
 }
 
-static void destroy(aq_handle_s* h) {
-    device_release(h->big, h->big_bytes, h->device);
-    device_release(h->sb, h->sb_held, h->device);
-    device_release(h->frags, h->block_held, h->device);
+static void destroy(aq_handle_s* h, bool idle = false) {
+    device_release(h->big, h->big_bytes, h->device, idle);
+    device_release(h->sb, h->sb_held, h->device, idle);
+    device_release(h->frags, h->block_held, h->device, idle);
     h->magic = 0;
     delete h;
 }
@@ -113,10 +141,10 @@ aq_status_t aq_pack(int bits, int block, const float* W_dev, int64_t N, int64_t 
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
+    handle_made(h, s);
     cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack(h, W_dev, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
-    h->last_stream = s;
     *out = h;
     return AQ_OK;
 }
@@ -130,10 +158,10 @@ aq_status_t aq_pack_opt(int bits, int block, const float* W_dev, const float* F_
     aq_status_t st = new_handle(bits, block, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
+    handle_made(h, s);
     cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack_opt(h, W_dev, F_dev, rounds, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
-    h->last_stream = s;
     *out = h;
     return AQ_OK;
 }
@@ -163,10 +191,10 @@ aq_status_t aq_pack_sb(int bits, int block, int sblock, const float* W_dev, int6
     aq_status_t st = new_sb_handle(bits, block, sblock, N, K, &h);
     if (st != AQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
+    handle_made(h, s);
     cudaError_t e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_pack_sb(h, W_dev, s);
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
-    h->last_stream = s;
     *out = h;
     return AQ_OK;
 }
@@ -186,14 +214,14 @@ aq_status_t aq_import_sb(int bits, int block, int sblock, int64_t N, int64_t K, 
     size_t tmp_held = 0;
     uint8_t* tmp = static_cast<uint8_t*>(device_alloc(plain_at + plain_bytes, h->device, &tmp_held));
     if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
+    handle_made(h, s);
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, true, s);
     if (e == cudaSuccess) e = launch_import(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    device_release(tmp, tmp_held, h->device);
+    device_release(tmp, tmp_held, h->device, e == cudaSuccess);   // (the stream has been waited for)
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
-    h->last_stream = s;
     *out = h;
     return AQ_OK;
 }
@@ -211,13 +239,13 @@ aq_status_t aq_import(int bits, int block, int64_t N, int64_t K, const void* can
     size_t tmp_held = 0;
     uint8_t* tmp = static_cast<uint8_t*>(device_alloc(nbytes, h->device, &tmp_held));
     if (!tmp) { destroy(h); return AQ_ERR_ALLOC; }
+    handle_made(h, s);
     cudaError_t e = cudaMemcpyAsync(tmp, canon_host, nbytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = clear_scratch(h, s);
     if (e == cudaSuccess) e = launch_import(h, tmp, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    device_release(tmp, tmp_held, h->device);
+    device_release(tmp, tmp_held, h->device, e == cudaSuccess);   // (the stream has been waited for)
     if (e != cudaSuccess) { destroy(h); return cuda_fail(e); }
-    h->last_stream = s;
     *out = h;
     return AQ_OK;
 }
@@ -242,7 +270,7 @@ aq_status_t aq_export(aq_handle_t h, void* canon_host, size_t cap, size_t* nbyte
     cudaStream_t s = h->last_stream;
     cudaError_t e = launch_export(h, tmp, s);
     if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
-    device_release(tmp, tmp_held, h->device);
+    device_release(tmp, tmp_held, h->device, e == cudaSuccess);   // (the stream has been waited for)
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }
@@ -262,7 +290,7 @@ aq_status_t aq_export_sb(aq_handle_t h, void* canon_host, size_t cap, size_t* nb
     cudaError_t e = launch_export(h, tmp + plain_at, s);
     if (e == cudaSuccess) e = launch_sb_records(h, tmp, tmp + plain_at, false, s);
     if (e == cudaSuccess) e = copy_to_host(canon_host, tmp, need, s);
-    device_release(tmp, tmp_held, h->device);
+    device_release(tmp, tmp_held, h->device, e == cudaSuccess);   // (the stream has been waited for)
     if (e != cudaSuccess) return cuda_fail(e);
     return range_status(h);
 }
@@ -283,9 +311,9 @@ aq_status_t aq_dequant(aq_handle_t h, void* out_dev, aq_dtype_t out_dtype, aq_st
     if (!handle_ok(h) || !out_dev || !aligned16(out_dev)) return AQ_ERR_INVALID_ARG;
     if (out_dtype != AQ_F16 && out_dtype != AQ_BF16 && out_dtype != AQ_F32) return AQ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    handle_used(h, s, being_recorded(s));
     cudaError_t e = launch_dequant(h, out_dev, out_dtype, s);
     if (e != cudaSuccess) return cuda_fail(e);
-    h->last_stream = s;
     return AQ_OK;
 }
 
@@ -295,6 +323,7 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
     if (M < 1 || M > AQ_MAX_M) return AQ_ERR_INVALID_ARG;
     if (xdt != AQ_F16 && xdt != AQ_BF16) return (xdt == AQ_F32) ? AQ_ERR_UNSUPPORTED : AQ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    handle_used(h, s, being_recorded(s));
     cudaError_t e;
     if (M <= AQ_DECODE_MAX_M) {
         const int64_t ld = (int64_t)h->NT * 16;
@@ -313,7 +342,8 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
         const size_t rs_bytes = (xdt == AQ_BF16) ? up((size_t)M * sizeof(float)) : 0;
         const size_t need = out_bytes + x16_bytes + rs_bytes;
         if (need > h->big_bytes) {
-            device_release(h->big, h->big_bytes, h->device);   // (waits for whatever still uses the old one)
+            if (h->big) device_release(h->big, h->big_bytes, h->device, handle_idle(h));
+            h->big = nullptr;
             h->big_bytes = 0;
             size_t held = 0;
             h->big = static_cast<uint8_t*>(device_alloc(need, h->device, &held));
@@ -331,7 +361,6 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
         if (e == cudaSuccess && ydt != AQ_F32) e = launch_finalize(sums, nullptr, h->N, y_dev, ydt, M, h->N, s);
     }
     if (e != cudaSuccess) return cuda_fail(e);
-    h->last_stream = s;
     return AQ_OK;
 }
 
@@ -456,9 +485,9 @@ void aq_debug_decode_hold(int on) {
 
 void aq_free(aq_handle_t h) {
     if (!handle_ok(h)) return;
-    cudaStreamSynchronize(h->last_stream);
+    const bool idle = handle_idle(h);
     decode_stack_forget(h);
-    destroy(h);
+    destroy(h, idle);
 }
 
 const char* aq_status_string(aq_status_t s) {

@@ -31,6 +31,8 @@ struct aq_handle_s {
     size_t big_bytes;
     int* flags;        // DEVICE: bit 0 = range error seen while packing
     cudaStream_t last_stream;
+    unsigned long long stream_id;   // of the stream the handle was made on
+    bool elsewhere;    // used on another stream as well, or recorded into a graph: waiting for last_stream is not waiting for all of its uses
 };
 
 namespace aq {
@@ -38,6 +40,8 @@ namespace aq {
 // status helpers (aq_api.cu)
 aq_status_t cuda_fail(cudaError_t e);
 bool handle_ok(aq_handle_t h);
+bool being_recorded(cudaStream_t s);                              // into a CUDA graph
+void handle_used(aq_handle_t h, cudaStream_t s, bool recorded);   // before a call's first launch that touches the handle's memory
 
 // launchers (each checks nothing: arguments are validated by the API layer)
 cudaError_t launch_pack(const aq_handle_s* h, const float* W, cudaStream_t s);
@@ -147,9 +151,10 @@ cudaError_t launch_attn_angles(void* turn, int M, int64_t pos, float theta, cuda
 cudaError_t launch_kv_append(void* kc, void* vc, const void* k, const void* v, int n_kv, int D, int64_t pos, int64_t Lmax, cudaStream_t s);
 
 // memory (aq_memory.cu): device blocks out of a bounded cache (null: no memory left; *held: the bytes the block really has, which is
-// what it is released with); a copy into pageable host memory, complete when the call returns
+// what it is released with; idle: nothing on the device uses it any more); a copy into pageable host memory, complete when the
+// call returns
 void* device_alloc(size_t bytes, int device, size_t* held);
-void device_release(void* p, size_t held, int device);
+void device_release(void* p, size_t held, int device, bool idle);
 cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t s);
 
 int current_device();               // cudaGetDevice, or -1

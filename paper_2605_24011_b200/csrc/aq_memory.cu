@@ -17,8 +17,9 @@ namespace {
 // ---- device blocks ------------------------------------------------------------------
 // A released block is kept for the next handle of about its size.  Bounded in bytes and number (a block counts with the bytes
 // it was allocated with, however little its last owner asked for); a block that the next
-// few releases have not found a use for goes back to the driver, and all of them do when an allocation fails.  Blocks
-// are idle when they come in (device_release waits for the device, as cudaFree did), so a block may go to any stream.
+// few releases have not found a use for goes back to the driver, and all of them do when an allocation fails.  Only idle
+// blocks come in, so that a block may go to any stream; of the others cudaFree takes care, which waits for the device.  (The
+// cache does not: a wait for the whole device ends every recording of a graph on it, another thread's included.)
 struct Block {
     void* p;
     size_t bytes;
@@ -85,14 +86,8 @@ void* device_alloc(size_t bytes, int device, size_t* held) {
     return nullptr;
 }
 
-void device_release(void* p, size_t held, int device) {
+void device_release(void* p, size_t held, int device, bool idle) {
     if (p == nullptr) return;
-    bool idle;
-    {
-        OnDevice there(device);
-        idle = cudaDeviceSynchronize() == cudaSuccess;   // whatever still uses the block, on any stream
-        if (!idle) cudaGetLastError();
-    }
     std::vector<void*> out;
     {
         Cache& c = cache();

@@ -46,11 +46,11 @@ extern "C" aq_status_t aq_linear_noalloc(aq_handle_t h, const void* x_dev, void*
     cudaError_t e = scratch_for_current_device(&scratch);
     if (e != cudaSuccess) return cuda_fail(e);
     cudaStream_t s = (cudaStream_t)stream;
+    handle_used(h, s, being_recorded(s));
     // the array keeps whatever the last call left: the sums must start from zero
     e = cudaMemsetAsync(scratch, 0, (size_t)M * ld * sizeof(float), s);
     if (e == cudaSuccess) e = launch_gemv(h, x_dev, xy_dtype, M, scratch, ld, s);
     if (e == cudaSuccess) e = launch_finalize(scratch, nullptr, ld, y_dev, xy_dtype, M, h->N, s);
     if (e != cudaSuccess) return cuda_fail(e);
-    h->last_stream = s;
     return AQ_OK;
 }

@@ -287,10 +287,16 @@ __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __res
     if (threadIdx.x == 0) scale[m] = sc;
 }
 
+static void program_used(const aq_stack_t* p, cudaStream_t s) {
+    const bool recorded = being_recorded(s);
+    for (int k = 0; k < p->n_ops; ++k) handle_used(p->ops[k].w, s, recorded);
+}
+
 template <typename T>
 static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T* x0, T* out, int out_buf, int M,
                              aq_dtype_t dt, uint8_t* ws, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
+    program_used(p, s);
     const bool decode = (M <= AQ_DECODE_MAX_M);
     auto buf = [&](int b) { return reinterpret_cast<float*>(ws + plan.buf_off[b]); };
     auto widen = [&] {
@@ -303,9 +309,6 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
         bool wrote_out = false;
         const int r = launch_decode_stack(p, plan, M, dt, ws, s, &e, x0, out, out_buf, &wrote_out);
         if (r < 0) return e;
-        if (r == 0) {
-            for (int k = 0; k < p->n_ops; ++k) p->ops[k].w->last_stream = s;
-        }
         if (r == 0 && out && !wrote_out) {
             const int64_t n = (int64_t)M * p->buf_width[out_buf];
             narrow_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(buf(out_buf), out, n);
@@ -388,7 +391,6 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
                 }
                 e = launch_gemv(o.w, stage, dt, M, buf(o.dst), N, s);
                 if (e != cudaSuccess) return e;
-                o.w->last_stream = s;
                 ++j;
             } else {   // the matrices of a phase read the same x: up to AQ_GEMM_MAX_GROUP of them per launch
                 const aq_handle_s* hs[AQ_GEMM_MAX_GROUP];
@@ -400,7 +402,6 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
                     const aq_stack_op_t& o = p->ops[j];
                     hs[n] = o.w; outs[n] = buf(o.dst); ldos[n] = p->buf_width[o.dst];
                     ress[n] = (o.out_op == AQ_OUT_ADD) ? buf(o.res) : nullptr;
-                    o.w->last_stream = s;
                     ++n; ++j;
                 }
                 if (dt == AQ_BF16)
@@ -518,6 +519,7 @@ aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t*
     uint8_t* ws = reinterpret_cast<uint8_t*>(workspace_dev);
     auto buf = [&](int b) { return reinterpret_cast<float*>(ws + plan.buf_off[b]); };
     cudaError_t e = cudaSuccess;
+    program_used(prog, s);
     if (n_attn > 0) {
         e = launch_attn_angles(attn_scratch_dev, M, pos, theta, s);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -544,7 +546,6 @@ aq_status_t aq_stack_forward_attn(const aq_stack_t* prog, const aq_stack_attn_t*
                              t.L_max, attn_scratch_dev, 0.08838834764831845f, dtype, sc, s);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    for (int k = 0; k < prog->n_ops; ++k) prog->ops[k].w->last_stream = s;
     if (out_dev && !wrote_out) {
         const int64_t n = (int64_t)M * prog->buf_width[out_buf];
         if (dtype == AQ_F16) narrow_kernel<__half><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(buf(out_buf), (__half*)out_dev, n);

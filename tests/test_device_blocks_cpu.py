@@ -93,13 +93,13 @@ def test_a_block_lies_on_the_device_it_was_asked_for(tmp_path):
         size_t held;
         void* p = device_alloc(1 << 20, 0, &held);            // a handle of device 0 exported while device 1 is current
         CHECK(p && fake::live[p].device == 0 && fake::current == 1);
-        device_release(p, held, 0);
+        device_release(p, held, 0, true);
         fake::current = 0;
         void* q = device_alloc(1 << 20, 0, &held);            // the next handle of device 0 may be built on that block
         CHECK(q && fake::live[q].device == 0);
         // the retry after the cache has been emptied looks at the device, too
         void* r = device_alloc(3 << 20, 0, &held);
-        device_release(r, held, 0);
+        device_release(r, held, 0, true);
         fake::current = 1;
         fake::limit = fake::used;
         void* t = device_alloc(2 << 20, 0, &held);
@@ -118,12 +118,26 @@ def test_a_block_counts_with_the_bytes_it_has(tmp_path):
                 p[i] = device_alloc(s, 0, &held[i]);
                 CHECK(p[i] && held[i] == fake::live[p[i]].bytes && held[i] >= s);
             }
-            for (int i = 0; i < 10; ++i) device_release(p[i], held[i], 0);
+            for (int i = 0; i < 10; ++i) device_release(p[i], held[i], 0, true);
         }
         CHECK(fake::mallocs >= 10 && fake::used >= (200u << 20) && fake::used <= (256u << 20));
         void* q[2];
         size_t q_held[2];
         for (int i = 0; i < 2; ++i) q[i] = device_alloc(40u << 20, 0, &q_held[i]);
-        for (int i = 0; i < 2; ++i) device_release(q[i], q_held[i], 0);
+        for (int i = 0; i < 2; ++i) device_release(q[i], q_held[i], 0, true);
         CHECK(fake::used <= (256u << 20));
+    """)
+
+
+def test_a_busy_block_goes_to_the_driver_and_the_device_is_not_waited_for(tmp_path):
+    _run(tmp_path, r"""
+        size_t held;
+        void* p = device_alloc(1 << 20, 0, &held);
+        device_release(p, held, 0, false);
+        CHECK(fake::frees == 1);
+        p = device_alloc(1 << 20, 0, &held);
+        CHECK(fake::mallocs == 2);
+        device_release(p, held, 0, true);
+        CHECK(device_alloc(1 << 20, 0, &held) == p && fake::mallocs == 2);
+        CHECK(fake::device_syncs == 0);
     """)

@@ -48,3 +48,69 @@ def test_recycled_blocks_and_threads():
     for t in threads:
         t.join()
     assert not wrong
+
+
+def test_another_threads_recording_survives_a_freed_handle():
+    """A CUDA graph is being recorded (thread-local rules: what other threads allocate and free is their own affair) while a
+    second thread quantises, exports and frees, handles that it has computed with among them."""
+    from paper_2605_24011_b200 import aq
+    W, want = _case(256, 512, 3, 7)
+    aq.aq_export(aq.aq_pack(3, 32, W))                # (set-up that happens once is done)
+    x = torch.zeros((1, 512), dtype=torch.float16, device="cuda")
+    y = torch.empty((1, 256), dtype=torch.float16, device="cuda")
+    a = torch.zeros(1024, device="cuda")
+    side, errors = torch.cuda.Stream(), []
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            for use in (False, True):
+                h = aq.aq_pack(3, 32, W, stream=side)
+                if use:
+                    aq.aq_linear(h, x, y, stream=side)
+                assert np.array_equal(aq.aq_export(h), want)
+                h.free()
+        except Exception as e:                        # an assertion, too, has to reach the test's thread
+            errors.append(e)
+
+    aq.aq_linear(aq.aq_pack(3, 32, W), x, y)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        a.add_(1.0)
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        a.add_(1.0)
+    assert not errors, errors
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(a[0]) == 2.0
+
+
+def test_blocks_of_handles_used_on_two_streams_are_not_handed_on_early():
+    """A handle made on one stream, at work on another, freed at once: its memory is not another handle's while the work
+    lasts, whatever its last stream is."""
+    from paper_2605_24011_b200 import aq
+    N, K = 4096, 4096
+    W = torch.from_numpy(synth.weights(N, K, 96)).cuda()
+    x = torch.from_numpy(synth.activations(64, K, 96)).half().cuda()
+    want = torch.empty((64, N), dtype=torch.float32, device="cuda")
+    aq.aq_linear(aq.aq_pack(2, 32, W), x, want)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    y = torch.empty_like(want)
+    torch.cuda.synchronize()
+    for rep in range(10):
+        h = aq.aq_pack(2, 32, W, stream=s1)
+        s2.wait_stream(s1)
+        for _ in range(20):
+            aq.aq_linear(h, x, y, stream=s2)
+        aq.aq_info(h)                                 # (waits for s2, then the last stream is s1 again)
+        for _ in range(20):
+            aq.aq_linear(h, x, y, stream=s2)
+        aq.aq_dequant(h, torch.empty((N, K), dtype=torch.float16, device="cuda"), stream=s1)
+        h.free()
+        g = aq.aq_pack(4, 32, W * 3.0, stream=s1)     # would write over the other's codes
+        torch.cuda.synchronize()
+        g.free()
+        assert (y - want).abs().max().item() <= 1e-3 * want.abs().max().item(), rep
