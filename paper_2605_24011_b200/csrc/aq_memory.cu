@@ -5,8 +5,9 @@
 #include <atomic>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <thread>
-#include <vector>
+#include <utility>
 
 #include "aq_internal.h"
 
@@ -30,13 +31,22 @@ constexpr size_t CACHE_BYTES = 256u << 20;
 constexpr size_t CACHE_BLOCKS = 16;
 constexpr uint64_t CACHE_AGE = 16;      // releases
 
+// (no container: nothing here may throw, the callers are C entry points)
 struct Cache {
     std::mutex m;
-    std::vector<Block> blocks;
+    Block blocks[CACHE_BLOCKS + 1];     // in the order of their release
+    size_t n = 0;
     uint64_t clock = 0;
+    Block take(size_t i) {
+        const Block b = blocks[i];
+        std::copy(blocks + i + 1, blocks + n, blocks + i);
+        --n;
+        return b;
+    }
 };
 Cache& cache() {
-    static Cache* c = new Cache;        // (outlives every handle: an interpreter may free some while it exits)
+    alignas(Cache) static unsigned char memory[sizeof(Cache)];
+    static Cache* c = new (memory) Cache;   // (outlives every handle: an interpreter may free some while it exits)
     return *c;
 }
 
@@ -59,58 +69,59 @@ void* device_alloc(size_t bytes, int device, size_t* held) {
     Cache& c = cache();
     {
         std::lock_guard<std::mutex> lock(c.m);
-        size_t best = c.blocks.size();
-        for (size_t i = 0; i < c.blocks.size(); ++i) {
+        size_t best = c.n;
+        for (size_t i = 0; i < c.n; ++i) {
             const Block& b = c.blocks[i];
-            if (b.device == device && b.bytes >= bytes && b.bytes <= bytes + bytes / 4 && (best == c.blocks.size() || b.bytes < c.blocks[best].bytes)) best = i;
+            if (b.device == device && b.bytes >= bytes && b.bytes <= bytes + bytes / 4 && (best == c.n || b.bytes < c.blocks[best].bytes)) best = i;
         }
-        if (best < c.blocks.size()) {
-            void* p = c.blocks[best].p;
-            *held = c.blocks[best].bytes;
-            c.blocks.erase(c.blocks.begin() + best);
-            return p;
+        if (best < c.n) {
+            const Block b = c.take(best);
+            *held = b.bytes;
+            return b.p;
         }
     }
     OnDevice here(device);
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
     cudaGetLastError();
-    std::vector<Block> all;
+    Block all[CACHE_BLOCKS + 1];
+    size_t n = 0;
     {
         std::lock_guard<std::mutex> lock(c.m);
-        all.swap(c.blocks);
+        std::copy(c.blocks, c.blocks + c.n, all);
+        std::swap(n, c.n);
     }
-    for (const Block& b : all) cudaFree(b.p);
-    if (!all.empty() && cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    for (size_t i = 0; i < n; ++i) cudaFree(all[i].p);
+    if (n > 0 && cudaMalloc(&p, bytes) == cudaSuccess) return p;
     cudaGetLastError();
     return nullptr;
 }
 
 void device_release(void* p, size_t held, int device, bool idle) {
     if (p == nullptr) return;
-    std::vector<void*> out;
+    void* out[CACHE_BLOCKS + 2];
+    size_t n_out = 0;
     {
         Cache& c = cache();
         std::lock_guard<std::mutex> lock(c.m);
         ++c.clock;
-        if (idle && held <= CACHE_BYTES) c.blocks.push_back({p, held, device, c.clock});
-        else out.push_back(p);
+        if (idle && held <= CACHE_BYTES) c.blocks[c.n++] = {p, held, device, c.clock};
+        else out[n_out++] = p;
         size_t total = 0;
-        for (const Block& b : c.blocks) total += b.bytes;
-        // the oldest first: blocks are in the order of their release
-        while (!c.blocks.empty() && (total > CACHE_BYTES || c.blocks.size() > CACHE_BLOCKS || c.blocks.front().stamp + CACHE_AGE < c.clock)) {
-            total -= c.blocks.front().bytes;
-            out.push_back(c.blocks.front().p);
-            c.blocks.erase(c.blocks.begin());
+        for (size_t i = 0; i < c.n; ++i) total += c.blocks[i].bytes;
+        while (c.n > 0 && (total > CACHE_BYTES || c.n > CACHE_BLOCKS || c.blocks[0].stamp + CACHE_AGE < c.clock)) {   // the oldest first
+            total -= c.blocks[0].bytes;
+            out[n_out++] = c.take(0).p;
         }
     }
-    for (void* q : out) cudaFree(q);
+    for (size_t i = 0; i < n_out; ++i) cudaFree(out[i]);
 }
 
 // ---- device -> pageable host ----------------------------------------------------------
 namespace {
 constexpr size_t CHUNK = 1u << 20;
 constexpr int SLOTS = 8;                // 8 MB of pinned memory, kept
+constexpr int MAX_THREADS = 4;
 std::mutex g_stage_mutex;
 uint8_t* g_stage = nullptr;
 }  // namespace
@@ -135,11 +146,10 @@ cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t
     if (staged) {
         const int device = current_device();
         const unsigned cores = std::thread::hardware_concurrency();
-        const int n_threads = cores >= 8 ? 4 : cores >= 4 ? 2 : 1;
+        const int n_threads = cores >= 8 ? MAX_THREADS : cores >= 4 ? 2 : 1;   // (a divisor of SLOTS: a slot is always the same thread's)
         std::atomic<size_t> issued{0};
+        std::atomic<size_t> emptied[SLOTS] = {};      // chunks of the slot so far
         std::atomic<bool> failed{false};
-        std::vector<std::atomic<uint8_t>> done(n);
-        for (auto& d : done) d.store(0, std::memory_order_relaxed);
         auto empty_chunks = [&](size_t first) {
             cudaSetDevice(device);
             for (size_t i = first; i < n; i += (size_t)n_threads) {
@@ -147,14 +157,18 @@ cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t
                     if (failed.load(std::memory_order_relaxed)) return;
                 if (cudaEventSynchronize(ev[i % SLOTS]) != cudaSuccess) { failed.store(true); return; }
                 std::memcpy(static_cast<uint8_t*>(host) + i * CHUNK, g_stage + (i % SLOTS) * CHUNK, std::min(CHUNK, bytes - i * CHUNK));
-                done[i].store(1, std::memory_order_release);
+                emptied[i % SLOTS].fetch_add(1, std::memory_order_release);
             }
         };
-        std::vector<std::thread> threads;
-        for (int t = 0; t < n_threads; ++t) threads.emplace_back(empty_chunks, (size_t)t);
-        for (size_t i = 0; i < n && err == cudaSuccess; ++i) {
-            if (i >= SLOTS)
-                while (!done[i - SLOTS].load(std::memory_order_acquire) && !failed.load(std::memory_order_relaxed)) std::this_thread::yield();
+        std::thread threads[MAX_THREADS];
+        try {
+            for (int t = 0; t < n_threads; ++t) threads[t] = std::thread(empty_chunks, (size_t)t);
+        } catch (...) {   // the system has no thread to give: the ordinary copy below
+            staged = false;
+            failed.store(true);
+        }
+        for (size_t i = 0; i < n && staged && err == cudaSuccess; ++i) {
+            while (emptied[i % SLOTS].load(std::memory_order_acquire) < i / SLOTS && !failed.load(std::memory_order_relaxed)) std::this_thread::yield();
             if (failed.load(std::memory_order_relaxed)) break;
             err = cudaMemcpyAsync(g_stage + (i % SLOTS) * CHUNK, static_cast<const uint8_t*>(dev) + i * CHUNK, std::min(CHUNK, bytes - i * CHUNK),
                                   cudaMemcpyDeviceToHost, s);
@@ -162,9 +176,11 @@ cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t
             if (err == cudaSuccess) issued.store(i + 1, std::memory_order_release);
         }
         if (err != cudaSuccess) failed.store(true);
-        for (std::thread& t : threads) t.join();
-        if (err == cudaSuccess && failed.load()) { err = cudaGetLastError(); if (err == cudaSuccess) err = cudaErrorUnknown; }
-    } else {
+        for (std::thread& t : threads)
+            if (t.joinable()) t.join();
+        if (staged && err == cudaSuccess && failed.load()) { err = cudaGetLastError(); if (err == cudaSuccess) err = cudaErrorUnknown; }
+    }
+    if (!staged) {
         err = cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, s);
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     }

@@ -77,12 +77,12 @@ MAIN = r"""
 """
 
 
-def _run(tmp_path, body, flags=()):
+def _run(tmp_path, body, before=""):
     (tmp_path / "cuda_runtime.h").write_text(FAKE)
     src = tmp_path / "t.cpp"
-    src.write_text(textwrap.dedent(MAIN) + "int main() {\n" + textwrap.dedent(body) + '\n    std::printf("ok\\n");\n    return 0;\n}\n')
+    src.write_text(textwrap.dedent(MAIN) + textwrap.dedent(before) + "int main() {\n" + textwrap.dedent(body) + '\n    std::printf("ok\\n");\n    return 0;\n}\n')
     exe = tmp_path / "t"
-    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", *flags, "-I", str(tmp_path), "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", str(tmp_path), "-I", CSRC, str(src), "-o", str(exe), "-ldl"], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout + r.stderr
 
@@ -141,3 +141,33 @@ def test_a_busy_block_goes_to_the_driver_and_the_device_is_not_waited_for(tmp_pa
         CHECK(device_alloc(1 << 20, 0, &held) == p && fake::mallocs == 2);
         CHECK(fake::device_syncs == 0);
     """)
+
+
+THREADS = r"""
+    #include <dlfcn.h>
+    #include <errno.h>
+    #include <pthread.h>
+    static int threads_left = 1 << 30;              // what the system still gives
+    extern "C" int pthread_create(pthread_t* t, const pthread_attr_t* a, void* (*f)(void*), void* x) {
+        static auto real = reinterpret_cast<int (*)(pthread_t*, const pthread_attr_t*, void* (*)(void*), void*)>(dlsym(RTLD_NEXT, "pthread_create"));
+        return threads_left-- > 0 ? real(t, a, f, x) : EAGAIN;
+    }
+    #include <vector>
+    static std::vector<uint8_t> bytes_of(size_t n) {
+        std::vector<uint8_t> v(n);
+        for (size_t i = 0; i < n; ++i) v[i] = (uint8_t)(i * 2654435761u >> 13);
+        return v;
+    }
+"""
+
+
+def test_a_copy_without_threads_is_an_ordinary_copy(tmp_path):
+    """The system refuses the first or a later helper thread: nothing is thrown out of the call, every byte arrives."""
+    _run(tmp_path, r"""
+        const auto from = bytes_of((21u << 20) + 5);
+        for (int given = 0; given <= 4; ++given) {
+            threads_left = given;
+            std::vector<uint8_t> to(from.size(), 0);
+            CHECK(aq::copy_to_host(to.data(), from.data(), from.size(), nullptr) == cudaSuccess && to == from);
+        }
+    """, before=THREADS)
