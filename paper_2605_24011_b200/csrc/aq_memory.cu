@@ -153,8 +153,10 @@ cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t
         auto empty_chunks = [&](size_t first) {
             cudaSetDevice(device);
             for (size_t i = first; i < n; i += (size_t)n_threads) {
-                while (issued.load(std::memory_order_acquire) <= i)
+                while (issued.load(std::memory_order_acquire) <= i) {
                     if (failed.load(std::memory_order_relaxed)) return;
+                    std::this_thread::yield();
+                }
                 if (cudaEventSynchronize(ev[i % SLOTS]) != cudaSuccess) { failed.store(true); return; }
                 std::memcpy(static_cast<uint8_t*>(host) + i * CHUNK, g_stage + (i % SLOTS) * CHUNK, std::min(CHUNK, bytes - i * CHUNK));
                 emptied[i % SLOTS].fetch_add(1, std::memory_order_release);
@@ -178,6 +180,7 @@ cudaError_t copy_to_host(void* host, const void* dev, size_t bytes, cudaStream_t
         if (err != cudaSuccess) failed.store(true);
         for (std::thread& t : threads)
             if (t.joinable()) t.join();
+        if (failed.load()) cudaStreamSynchronize(s);   // chunks that were issued may be on their way into the ring, the next copy's
         if (staged && err == cudaSuccess && failed.load()) { err = cudaGetLastError(); if (err == cudaSuccess) err = cudaErrorUnknown; }
     }
     if (!staged) {

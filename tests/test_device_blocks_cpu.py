@@ -171,3 +171,24 @@ def test_a_copy_without_threads_is_an_ordinary_copy(tmp_path):
             CHECK(aq::copy_to_host(to.data(), from.data(), from.size(), nullptr) == cudaSuccess && to == from);
         }
     """, before=THREADS)
+
+
+def test_a_failed_copy_leaves_nothing_in_flight(tmp_path):
+    """A chunk cannot be issued, or a helper's wait fails: the error is reported, and the ring is given up only after the
+    stream has been waited for."""
+    _run(tmp_path, r"""
+        const auto from = bytes_of(21u << 20);
+        std::vector<uint8_t> to(from.size());
+        for (int at : {1, 7, 12, 20}) {
+            fake::copies = 0; fake::copies_fail_from = at;
+            CHECK(aq::copy_to_host(to.data(), from.data(), from.size(), nullptr) != cudaSuccess && !fake::unsynced);
+        }
+        fake::copies_fail_from = 1 << 30;
+        for (int at : {0, 3, 15}) {
+            fake::event_syncs = 0; fake::event_syncs_fail_from = at;
+            CHECK(aq::copy_to_host(to.data(), from.data(), from.size(), nullptr) != cudaSuccess && !fake::unsynced);
+        }
+        fake::event_syncs_fail_from = 1 << 30;
+        std::fill(to.begin(), to.end(), 0);
+        CHECK(aq::copy_to_host(to.data(), from.data(), from.size(), nullptr) == cudaSuccess && to == from);
+    """, before=THREADS)
