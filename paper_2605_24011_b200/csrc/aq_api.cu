@@ -14,6 +14,7 @@ namespace aq {
 static thread_local char g_last_err[256] = "";
 
 aq_status_t cuda_fail(cudaError_t e) {
+    cudaGetLastError();   // reported once: the runtime would keep a failed launch's error for the next call that asks
     snprintf(g_last_err, sizeof(g_last_err), "%s: %s", cudaGetErrorName(e), cudaGetErrorString(e));
     return AQ_ERR_CUDA;
 }

@@ -60,3 +60,29 @@ def test_replayed_stack_matches_oracle(aq, M, dtype):
         check_program(prog, names, ws, M, tdt, quant)
         assert torch.equal(aq.stack_buffer(prog, ws, M, 0), x_new.float())
         assert torch.equal(out, aq.stack_buffer(prog, ws, M, out_buf).to(tdt))
+
+
+@pytest.mark.parametrize("M", (1, 16))
+def test_a_refused_launch_is_reported_once(aq, M):
+    """The legacy stream may not be used beside the recording of a blocking stream: the call is refused with an error, and
+    the next call, which is a good one, does not report it again."""
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    N, K = 256, 512
+    W = synth.weights(N, K, 43)
+    h = aq.aq_pack(3, 32, torch.from_numpy(W).cuda())
+    x = torch.zeros((M, K), dtype=torch.float16, device="cuda")
+    y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    out = torch.empty((N, K), dtype=torch.float16, device="cuda")
+    aq.aq_linear(h, x, y)
+    torch.cuda.synchronize()
+    err, s = rt.cudaStreamCreateWithFlags(0)
+    assert err == rt.cudaError_t.cudaSuccess
+    assert rt.cudaStreamBeginCapture(s, rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal)[0] == rt.cudaError_t.cudaSuccess
+    refused = aq.raw_lib().aq_linear(h.raw, x.data_ptr(), y.data_ptr(), M, aq.AQ_F16, None)
+    rt.cudaStreamEndCapture(s)
+    rt.cudaGetLastError()                            # (this binding's own copy of the runtime)
+    assert refused == aq.AQ_ERR_CUDA
+    aq.aq_dequant(h, out, stream=torch.cuda.Stream())
+    torch.cuda.synchronize()
+    assert np.array_equal(out.view(torch.int16).cpu().numpy().view(np.uint16), O.dequant(*O.quantize(W, 3), "f16"))
+    rt.cudaStreamDestroy(s)
