@@ -251,8 +251,11 @@ aq_status_t aq_dequant(aq_handle_t h, void* out_dev, aq_dtype_t out_dtype, aq_st
  * to binary16 first, which is exact inside binary16's range; a token row with a magnitude of 2^15 or more is scaled
  * by a power of two and scaled back after the sum).  Calls on one handle must be ordered on a stream (the handle
  * owns accumulation scratch that concurrent calls would share).  With M > AQ_DECODE_MAX_M the handle allocates
- * further scratch (float32 sums, the widened activations) the first time it sees such a call and again when a
- * later call needs more; calls in between allocate nothing.
+ * further scratch (the activations in the tensor cores' order, for half-precision outputs float32 sums) the first time it
+ * sees such a call and again when a later call needs more; calls in between allocate nothing.
+ * CUDA graphs: the call may be recorded and replayed.  With M > AQ_DECODE_MAX_M the graph uses the handle's scratch if an
+ * earlier call has made it large enough -- a later call that needs more replaces it and invalidates the graph -- and
+ * else holds scratch of its own.
  */
 aq_status_t aq_linear(aq_handle_t h, const void* x_dev, void* y_dev, int M,
                       aq_dtype_t xy_dtype, aq_stream_t stream);

@@ -324,7 +324,8 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
     if (M < 1 || M > AQ_MAX_M) return AQ_ERR_INVALID_ARG;
     if (xdt != AQ_F16 && xdt != AQ_BF16) return (xdt == AQ_F32) ? AQ_ERR_UNSUPPORTED : AQ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    handle_used(h, s, being_recorded(s));
+    const bool recorded = being_recorded(s);
+    handle_used(h, s, recorded);
     cudaError_t e;
     if (M <= AQ_DECODE_MAX_M) {
         const int64_t ld = (int64_t)h->NT * 16;
@@ -336,13 +337,19 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
         }
     } else {
         // scratch owned by the handle: float32 sums when the output is half precision, the activations in operand order,
-        // for bfloat16 with row scales; allocated on the first such call and when a later one needs more
+        // for bfloat16 with row scales; allocated on the first such call and when a later one needs more.  A call that is being
+        // recorded cannot allocate that: the graph then gets scratch of its own, between an allocation and a free node.
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
         const size_t out_bytes = (ydt == AQ_F32) ? 0 : up((size_t)M * h->N * sizeof(float));
         const size_t x16_bytes = up((size_t)M * h->K * 2);
         const size_t rs_bytes = (xdt == AQ_BF16) ? up((size_t)M * sizeof(float)) : 0;
         const size_t need = out_bytes + x16_bytes + rs_bytes;
-        if (need > h->big_bytes) {
+        uint8_t* big = h->big;
+        const bool graph_owned = recorded && need > h->big_bytes;
+        if (graph_owned) {
+            e = cudaMallocAsync(reinterpret_cast<void**>(&big), need, s);
+            if (e != cudaSuccess) return cuda_fail(e);
+        } else if (need > h->big_bytes) {
             if (h->big) device_release(h->big, h->big_bytes, h->device, handle_idle(h));
             h->big = nullptr;
             h->big_bytes = 0;
@@ -350,16 +357,21 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
             h->big = static_cast<uint8_t*>(device_alloc(need, h->device, &held));
             if (!h->big) return AQ_ERR_ALLOC;
             h->big_bytes = held;
+            big = h->big;
         }
-        float* sums = (ydt == AQ_F32) ? (float*)y_dev : reinterpret_cast<float*>(h->big);
-        void* x16 = h->big + out_bytes;
-        float* rs = (xdt == AQ_BF16) ? reinterpret_cast<float*>(h->big + out_bytes + x16_bytes) : nullptr;
+        float* sums = (ydt == AQ_F32) ? (float*)y_dev : reinterpret_cast<float*>(big);
+        void* x16 = big + out_bytes;
+        float* rs = (xdt == AQ_BF16) ? reinterpret_cast<float*>(big + out_bytes + x16_bytes) : nullptr;
         const aq_handle_s* hc = h;
         const int64_t ldo = h->N;
         const bool preset = !gemm_stores_first(&hc, 1, M, s) && gemm_outputs_can_be_preset(&sums, &ldo, 1);
         e = launch_operand_rows(x_dev, xdt, x16, rs, M, h->K, preset ? sums : nullptr, h->N, s);
         if (e == cudaSuccess) e = launch_gemm(h, x16, rs, M, sums, h->N, preset, s);
         if (e == cudaSuccess && ydt != AQ_F32) e = launch_finalize(sums, nullptr, h->N, y_dev, ydt, M, h->N, s);
+        if (graph_owned) {
+            const cudaError_t freed = cudaFreeAsync(big, s);
+            if (e == cudaSuccess) e = freed;
+        }
     }
     if (e != cudaSuccess) return cuda_fail(e);
     return AQ_OK;

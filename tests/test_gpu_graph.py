@@ -86,3 +86,35 @@ def test_a_refused_launch_is_reported_once(aq, M):
     torch.cuda.synchronize()
     assert np.array_equal(out.view(torch.int16).cpu().numpy().view(np.uint16), O.dequant(*O.quantize(W, 3), "f16"))
     rt.cudaStreamDestroy(s)
+
+
+@pytest.mark.parametrize("seen", (0, 12, 40))
+@pytest.mark.parametrize("dtype,out", [("f16", "f32"), ("f16", "f16"), ("bf16", "bf16")])
+def test_replayed_prefill_linear_matches_oracle(aq, dtype, out, seen):
+    """A linear of 33 tokens, recorded as the handle's first call of more than 8, after one that needed less scratch, and after
+    one that needed more."""
+    N, K, M, bits = 272, 288, 33, 3
+    tdt = {"f16": torch.float16, "bf16": torch.bfloat16, "f32": torch.float32}
+    W = synth.weights(N, K, 44)
+    h = aq.aq_pack(bits, 32, torch.from_numpy(W).cuda())
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    x = torch.zeros((M, K), dtype=tdt[dtype], device="cuda")
+    y = torch.empty((M, N), dtype=tdt[out], device="cuda")
+    with torch.cuda.stream(stream):
+        aq.aq_linear(h, x[:1], y[:1])
+        if seen:
+            aq.aq_linear(h, torch.zeros((seen, K), dtype=tdt[dtype], device="cuda"), torch.empty((seen, N), dtype=tdt[out], device="cuda"))
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            aq.aq_linear(h, x, y)
+    for rep in range(3):
+        x.copy_(torch.from_numpy(synth.activations(M, K, 45 + rep)).to(tdt[dtype]))
+        y.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        aq.aq_check()
+        want, T = O.linear(*O.quantize(W, bits), x.double().cpu().numpy())
+        u = {"f32": 0.0, "f16": 2.0 ** -11, "bf16": 2.0 ** -8}[out]      # the output's own rounding
+        assert np.all(np.abs(y.double().cpu().numpy() - want) <= 2e-3 * T + 1e-5 + u * np.abs(want))
+    del graph
