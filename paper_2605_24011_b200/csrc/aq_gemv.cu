@@ -282,30 +282,40 @@ cudaError_t launch_gemv(const aq_handle_s* h, const void* x, aq_dtype_t xdt, int
     }
 }
 
-// y = cast(acc) for the first N columns of each row, then acc = 0.  Four elements per thread; blockIdx.y is the row.
+// y = cast(acc) for the first N columns of each row, then acc = 0.  A CTA takes 1024 columns of a row (blockIdx.y): four
+// neighbouring elements per thread where both rows stay aligned to that, else four elements 256 apart, so that a warp's
+// accesses stay side by side (5003 x 4000 at 5 tokens, with the linear: 10.4 us with neighbours, 8.6 so).
 template <typename T>
 __global__ void __launch_bounds__(256) finalize_kernel(const float* __restrict__ acc_in, float* __restrict__ acc_zero, int64_t ld, T* __restrict__ y, int64_t N) {
     pdl_wait();   // the sums are the predecessor's output
-    const int64_t m = blockIdx.y, n = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
-    if (n >= N) return;
-    const float* a = acc_in + m * ld + n;
-    T* o = y + m * N + n;
+    const int64_t m = blockIdx.y, n0 = (int64_t)blockIdx.x * 1024;
     auto cast = [](float v) -> T {
         if constexpr (std::is_same<T, __half>::value) return __float2half_rn(v);
         else if constexpr (std::is_same<T, __nv_bfloat16>::value) return __float2bfloat16_rn(v);
         else return v;
     };
-    if (((ld | N) & 3) == 0) {   // (rows of both stay aligned to four elements)
-        const float4 v = *reinterpret_cast<const float4*>(a);
+    if (((ld | N) & 3) == 0) {
+        const int64_t n = n0 + threadIdx.x * 4;
+        if (n >= N) return;
+        const float4 v = *reinterpret_cast<const float4*>(acc_in + m * ld + n);
         struct __align__(4 * sizeof(T)) Four { T t[4]; } r;
         r.t[0] = cast(v.x); r.t[1] = cast(v.y); r.t[2] = cast(v.z); r.t[3] = cast(v.w);
-        *reinterpret_cast<Four*>(o) = r;
+        *reinterpret_cast<Four*>(y + m * N + n) = r;
         if (acc_zero) *reinterpret_cast<float4*>(acc_zero + m * ld + n) = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
-    for (int i = 0; i < 4 && n + i < N; ++i) {
-        o[i] = cast(a[i]);
-        if (acc_zero) acc_zero[m * ld + n + i] = 0.f;
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t n = n0 + i * 256 + threadIdx.x;
+        v[i] = n < N ? acc_in[m * ld + n] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t n = n0 + i * 256 + threadIdx.x;
+        if (n >= N) break;
+        y[m * N + n] = cast(v[i]);
+        if (acc_zero) acc_zero[m * ld + n] = 0.f;
     }
 }
 
