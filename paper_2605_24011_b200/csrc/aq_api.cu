@@ -340,7 +340,12 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
         // for bfloat16 with row scales; allocated on the first such call and when a later one needs more.  A call that is being
         // recorded cannot allocate that: the graph then gets scratch of its own, between an allocation and a free node.
         auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-        const size_t out_bytes = (ydt == AQ_F32) ? 0 : up((size_t)M * h->N * sizeof(float));
+        // The sums' rows are padded to four floats, what the GEMM's tensor copies and presets want; float32 outputs whose rows are
+        // not that long are written from such sums, too (2595 x 2016 at 627 tokens 72 us with unpadded
+        // rows, 19 so; 990 x 192 at 127 tokens 37 / 9.4).
+        const int64_t ldo = (h->N + 3) / 4 * 4;
+        const bool direct = ydt == AQ_F32 && ldo == h->N;
+        const size_t out_bytes = direct ? 0 : up((size_t)M * ldo * sizeof(float));
         const size_t x16_bytes = up((size_t)M * h->K * 2);
         const size_t rs_bytes = (xdt == AQ_BF16) ? up((size_t)M * sizeof(float)) : 0;
         const size_t need = out_bytes + x16_bytes + rs_bytes;
@@ -359,15 +364,14 @@ static aq_status_t linear_common(aq_handle_t h, const void* x_dev, void* y_dev, 
             h->big_bytes = held;
             big = h->big;
         }
-        float* sums = (ydt == AQ_F32) ? (float*)y_dev : reinterpret_cast<float*>(big);
+        float* sums = direct ? (float*)y_dev : reinterpret_cast<float*>(big);
         void* x16 = big + out_bytes;
         float* rs = (xdt == AQ_BF16) ? reinterpret_cast<float*>(big + out_bytes + x16_bytes) : nullptr;
         const aq_handle_s* hc = h;
-        const int64_t ldo = h->N;
         const bool preset = !gemm_stores_first(&hc, 1, M, s) && gemm_outputs_can_be_preset(&sums, &ldo, 1);
-        e = launch_operand_rows(x_dev, xdt, x16, rs, M, h->K, preset ? sums : nullptr, h->N, s);
-        if (e == cudaSuccess) e = launch_gemm(h, x16, rs, M, sums, h->N, preset, s);
-        if (e == cudaSuccess && ydt != AQ_F32) e = launch_finalize(sums, nullptr, h->N, y_dev, ydt, M, h->N, s);
+        e = launch_operand_rows(x_dev, xdt, x16, rs, M, h->K, preset ? sums : nullptr, ldo, s);
+        if (e == cudaSuccess) e = launch_gemm(h, x16, rs, M, sums, ldo, preset, s);
+        if (e == cudaSuccess && !direct) e = launch_finalize(sums, nullptr, ldo, y_dev, ydt, M, h->N, s);
         if (graph_owned) {
             const cudaError_t freed = cudaFreeAsync(big, s);
             if (e == cudaSuccess) e = freed;
