@@ -374,17 +374,24 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
                     }
                 } else {
                     const int64_t n = (int64_t)n0 + lane;
+                    const int left = min(sg.w - c0, a.M - tok0 - c0);   // tokens of the chunk
                     if (n < op.N) {
+                        const int64_t at = (int64_t)(tok0 + c0) * op.ldo + n;
+                        float* o = op.out + at;
+                        if (add_res) {
+                            const float* r = op.res + at;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const int tok = tok0 + c0 + j;
-                            if (c0 + j < sg.w && tok < a.M) {
-                                const int64_t o = (int64_t)tok * op.ldo + n;
-                                float val = __uint_as_float(v[j]);
-                                if (add_res) val += __ldg(op.res + o);
-                                if (whole) op.out[o] = val;
-                                else atomicAdd(op.out + o, val);
-                            }
+                            for (int j = 0; j < 32; ++j, r += op.ldo)
+                                if (j < left) v[j] = __float_as_uint(__uint_as_float(v[j]) + __ldg(r));
+                        }
+                        if (whole) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j, o += op.ldo)
+                                if (j < left) *o = __uint_as_float(v[j]);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j, o += op.ldo)
+                                if (j < left) atomicAdd(o, __uint_as_float(v[j]));
                         }
                     }
                 }
