@@ -236,17 +236,21 @@ static cudaError_t launch_rows(const GemvArgs& a, cudaStream_t s) {
 }
 
 // True when the row-tile kernel above is the better choice: a warp has few units along k (x is fetched anew for each, and more
-// of it the more tokens there are) and the CTAs are few waves.  Measured, streaming kernel and cast / this, us:
-//   1 token:  2048 x 1024 5.7 / 2.2   4096 x 4096, 4 bits 5.8 / 4.8   16384 x 4096, 4 bits 13.0 / 12.0   2048 x 8192 7.3 / 4.8
-//             9000 x 16384, 2 bits 20.4 / 17.5, 3 bits 22.8 / 22.7   4096 x 16384, 4 bits 12.9 / 13.9   512 x 16384 4.9 / 7.3
-//   2 tokens: 4096 x 8192, 4 bits 8.7 / 8.0   9000 x 16384, 4 bits 23.1 / 25.4
-//   4 tokens: 4096 x 4096 6.5 / 5.6   9000 x 4096 9.2 / 8.3   16384 x 4096, 4 bits 14.5 / 15.5   4096 x 8192 8.9 / 9.0
-//   8 tokens: 4096 x 4096 7.0 / 6.5   9000 x 4096 10.0 / 11.3   2048 x 8192 7.0 / 8.2
+// of it the more tokens there are) and the CTAs are few waves.  Measured over 8 to 1184 row tiles x 512 to 16384 columns at 2
+// and 4 bits (binary16 in and out, three matrices in turn, 24 calls in a graph), this kernel / the streaming kernel and its cast,
+// us at 4 bits:
+//   1 token:  74 tiles, 8192 columns 4.8 / 5.9    148, 8192 5.2 / 5.5    256, 16384 12.5 / 11.4    400, 16384 15.2 / 16.5
+//   2 tokens: 74 tiles, 6144 columns 4.7 / 4.3    148, 6144 5.2 / 5.3    400, 8192 10.0 / 11.3
+//   4 tokens: 148 tiles, 4096 columns 0.86 of it, 6144 0.94, 8192 1.04    740, 2048 0.88, 4096 1.0    1024, 1024 1.0, 4096 1.04 to 1.09
+//   8 tokens: 296 tiles, 4096 columns 0.95 of it, 6144 1.0    400, 1024 1.0, 4096 1.35    74, 4096 1.03
+// Called one by one from the host the streaming kernel's second launch counts for more: 97 tiles, 9472 columns, 1 token 5.6 / 7.4,
+// 117, 11328 6.8 / 9.0, 293, 12672 9.6 / 11.6; but 154, 15392 11.2 / 9.1, 171, 14624 10.4 / 9.0.
 static bool rows_kernel_fits(int NT, int KP, int M) {
-    const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2);
-    if (NT > waves * sm_count() || KP < 2) return false;
+    const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2), sms = sm_count();
+    if (NT > waves * sms || KP < 2) return false;
     if (KP <= 2 * GEMV_WARPS) return true;
-    if (M > 2 || 2 * NT < sm_count()) return false;
+    if (M > 2 || 2 * NT < sms) return false;
+    if (M == 1 && KP > 7 * GEMV_WARPS && NT > sms && NT <= 2 * sms) return false;   // (one to two waves of the longest rows)
     return KP <= (M == 1 ? 8 : 4) * GEMV_WARPS;
 }
 

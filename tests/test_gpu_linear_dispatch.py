@@ -26,3 +26,8 @@ def test_dispatch_edges(N, K, bits, M):
         want, T = O.linear(*O.quantize(W, bits), x.double().cpu().numpy())
         assert O.linear_excess(y.double().cpu().numpy(), want, T).max() <= 1.0   # the library's bound of the exact product
     h.free()
+
+
+@pytest.mark.parametrize("N,K,bits,M", [(2368, 14368, 2, 1), (2369, 14336, 2, 1), (2369, 14368, 4, 1), (4736, 14368, 3, 1), (4737, 14368, 2, 1)])
+def test_dispatch_edges_of_long_rows(N, K, bits, M):
+    test_dispatch_edges(N, K, bits, M)
