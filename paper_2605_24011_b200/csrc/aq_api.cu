@@ -93,7 +93,7 @@ static aq_status_t new_handle(int bits, int block, int64_t N, int64_t K, aq_hand
     aq_handle_s* h = new (std::nothrow) aq_handle_s();
     if (!h) return AQ_ERR_ALLOC;
     h->magic = AQ_HANDLE_MAGIC;
-    h->bits = bits; h->device = dev; h->N = N; h->K = K;
+    h->bits = bits; h->device = dev; h->sms = sm_count(); h->N = N; h->K = K;
     h->NT = (int)((N + 15) / 16);
     h->KP = (int)((K + 255) / 256);
     h->n_frags = (int64_t)h->NT * h->KP * 2;

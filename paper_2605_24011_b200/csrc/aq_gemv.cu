@@ -29,6 +29,7 @@ struct GemvArgs {
     int64_t N;          // true N: rows >= N are padding and are not written
     int NT;
     int M;
+    int sms;
     // when y is given the last CTA to finish casts the sums into y[m][n] and zeroes them again (one launch per linear)
     void* y;
     int ydt;
@@ -150,7 +151,7 @@ static cudaError_t launch_one(const GemvArgs& a, cudaStream_t s) {
         if (rc != 0) return rc < 0 ? cudaErrorInvalidDevice : (cudaError_t)rc;
     }
     const int64_t warps_wanted = a.n_units;
-    int grid = 2 * sm_count();
+    int grid = 2 * a.sms;
     const int64_t need = (warps_wanted + GEMV_WARPS - 1) / GEMV_WARPS;
     if (need < grid) grid = (int)need;
     const cudaError_t e = launch_pdl(kern, dim3((unsigned)grid), dim3(GEMV_WARPS * 32), SMEM, s, a);
@@ -245,8 +246,8 @@ static cudaError_t launch_rows(const GemvArgs& a, cudaStream_t s) {
 //   8 tokens: 296 tiles, 4096 columns 0.95 of it, 6144 1.0    400, 1024 1.0, 4096 1.35    74, 4096 1.03
 // Called one by one from the host the streaming kernel's second launch counts for more: 97 tiles, 9472 columns, 1 token 5.6 / 7.4,
 // 117, 11328 6.8 / 9.0, 293, 12672 9.6 / 11.6; but 154, 15392 11.2 / 9.1, 171, 14624 10.4 / 9.0.
-static bool rows_kernel_fits(int NT, int KP, int M) {
-    const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2), sms = sm_count();
+static bool rows_kernel_fits(int NT, int KP, int M, int sms) {
+    const int waves = M <= 2 ? 8 : (M <= 4 ? 5 : 2);
     if (NT > waves * sms || KP < 2) return false;
     if (KP <= 2 * GEMV_WARPS) return true;
     if (M > 2 || 2 * NT < sms) return false;
@@ -256,11 +257,11 @@ static bool rows_kernel_fits(int NT, int KP, int M) {
 
 // The kernel casts the outputs itself: any number of them from the row-tile kernel, few from the streaming kernel, whose last
 // CTA does it alone (about 0.1 us per 256 outputs; the cast as a launch of its own adds 1 us).
-bool gemv_writes_y(const aq_handle_s* h, int M) { return (int64_t)M * h->N <= 2048 || rows_kernel_fits(h->NT, h->KP, M); }
+bool gemv_writes_y(const aq_handle_s* h, int M) { return (int64_t)M * h->N <= 2048 || rows_kernel_fits(h->NT, h->KP, M, h->sms); }
 
 template <int BITS, bool BF16>
 static cudaError_t launch_mt(const GemvArgs& a, cudaStream_t s) {
-    if (a.y != nullptr && rows_kernel_fits(a.NT, (int)(a.n_units / a.NT), a.M)) {
+    if (a.y != nullptr && rows_kernel_fits(a.NT, (int)(a.n_units / a.NT), a.M, a.sms)) {
         if (a.M == 1) return launch_rows<BITS, 1, BF16>(a, s);
         if (a.M == 2) return launch_rows<BITS, 2, BF16>(a, s);
         if (a.M <= 4) return launch_rows<BITS, 4, BF16>(a, s);
@@ -277,7 +278,7 @@ cudaError_t launch_gemv(const aq_handle_s* h, const void* x, aq_dtype_t xdt, int
     GemvArgs a;
     a.y = y_fused; a.ydt = (int)ydt; a.ticket = reinterpret_cast<unsigned int*>(h->flags) + 16;
     a.frags = h->frags; a.x = x; a.acc = acc; a.K = h->K; a.ldacc = ldacc;
-    a.n_units = (int64_t)h->KP * h->NT; a.NT = h->NT; a.M = M; a.N = h->N;
+    a.n_units = (int64_t)h->KP * h->NT; a.NT = h->NT; a.M = M; a.N = h->N; a.sms = h->sms;
     const bool bf = (xdt == AQ_BF16);
     switch (h->bits) {
         case 2: return bf ? launch_mt<2, true>(a, s) : launch_mt<2, false>(a, s);

@@ -14,6 +14,7 @@ struct aq_handle_s {
     uint32_t magic;
     int bits;
     int device;
+    int sms;           // SMs of the device (asking the runtime takes as long as its other share of a short call's checks)
     int64_t N, K;
     int NT;            // row tiles of 16
     int KP;            // pair slabs of 256 k
