@@ -550,7 +550,7 @@ static void cached_runs(long long total, long long c1, int grid, int* bounds) {
     Entry e;
     memset(&e, 0, sizeof(e));
     e.total = total; e.c1 = c1; e.grid = grid;
-    cut_runs(total, 0, 2, c1, grid, e.bounds);
+    cut_runs(total, c1, grid, e.bounds);
     memcpy(bounds, e.bounds, sizeof(e.bounds));
     if (entries.size() >= 64) entries.erase(entries.begin());
     entries.push_back(e);

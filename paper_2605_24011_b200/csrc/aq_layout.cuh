@@ -62,16 +62,6 @@ __host__ __device__ inline int slot_word_offset(int bits, int s, int widx) {
     return widx < 4 ? 256 + s * 16 + widx * 4 : 256 + 512 + s * 8 + (widx - 4) * 4;
 }
 
-// One code bit's home: byte offset of a 32-bit word inside the fragment and the
-// bit position in it.  r in 0..15, kk in 0..127, tb = bit of the code.
-__host__ __device__ inline void code_bit_home(int bits, int r, int kk, int tb, int& word_off, int& bitpos) {
-    const int j = kk >> 5, e = kk & 31, t = e >> 3, c = e & 7;
-    const int g = r & 7, hi = r >> 3;
-    int widx;
-    slot_bit_home(bits, j, hi, c, tb, widx, bitpos);
-    word_off = slot_word_offset(bits, g * 4 + t, widx);
-}
-
 // ---- register-level extraction -------------------------------------------
 // A lane's code words for one fragment.
 template <int BITS> struct LaneCodes { uint32_t w[2 * BITS]; };

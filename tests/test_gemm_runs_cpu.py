@@ -1,4 +1,4 @@
-"""Host logic of the prefill GEMM's scheduler: `csrc/aq_gemm_runs.h` (how the (row tile, token super-tile, k-slab)
+"""Host logic of the prefill GEMM's scheduler: `csrc/aq_gemm_runs.h` (how the (row tile, token tile, half k-slab)
 work is cut into one contiguous run per CTA), compiled with the host compiler alone and driven from a small C++
 program.  Checked for many shapes: the bounds partition the work (ascending, even, first 0, last total), the run that
 holds a tile's last slab starts inside that tile or covers the tile whole (what the store-first protocol of the kernel
@@ -21,29 +21,23 @@ SRC = textwrap.dedent(r"""
     using namespace aq;
     #define CHECK(c) do { if (!(c)) { std::printf("FAIL line %d: %s (n_slabs %lld R %lld M %d grid %d)\n", __LINE__, #c, n_slabs, R, M, grid); return 1; } } while (0)
 
-    // the same derivation of the tile structure as the launcher's
+    // the same derivation of the tile structure as the launcher's: tiles of 256 rows x up to 128 tokens, half slabs
     static int one(long long n_slabs, long long R, int M, int grid) {
-        long long n_st, n2;
-        if (M > 256) { n_st = (M + 511) / 512; n2 = (M - 512 * (n_st - 1) > 256) ? n_st : n_st - 1; }
-        else { n_st = 1; n2 = 0; }
-        const long long c2 = 2 * n_slabs, c1 = n_slabs, n_two = n2 * R;
-        const long long total = n_slabs * R * (2 * n2 + (n_st - n2));
+        const long long n_st = (M + 127) / 128, c1 = 2 * n_slabs, total = R * n_st * c1;
         if (total / 2 < grid) grid = (int)(total / 2);
         if (grid < 1) return 0;
         std::vector<int> b(grid + 1, -1);
-        cut_runs(total, n_two, c2, c1, grid, b.data());
+        cut_runs(total, c1, grid, b.data());
         CHECK(b[0] == 0 && b[grid] == total);
         long long worst = 0;
         for (int c = 0; c < grid; ++c) {
             CHECK(b[c] <= b[c + 1] && b[c] % 2 == 0);
-            worst = std::max(worst, run_cost(b[c], b[c + 1], n_two, c2, c1));
+            worst = std::max(worst, run_cost(b[c], b[c + 1], c1));
         }
         // a run that contains a tile's last unit and does not start inside that tile covers the tile whole
-        const long long reg2 = n_two * c2;
         for (int c = 0; c < grid; ++c) {
             for (long long pos = b[c]; pos < b[c + 1];) {
-                const long long ts = pos < reg2 ? pos / c2 * c2 : reg2 + (pos - reg2) / c1 * c1;
-                const long long te = ts + (pos < reg2 ? c2 : c1);
+                const long long ts = pos / c1 * c1, te = ts + c1;
                 if (te <= b[c + 1] && ts < b[c]) CHECK(pos == b[c]);          // the tile's tail: first thing of the run
                 pos = std::min<long long>(te, b[c + 1]);
             }
@@ -52,11 +46,11 @@ SRC = textwrap.dedent(r"""
         long long worst_equal = 0;
         for (int c = 0; c < grid; ++c) {
             const long long lo = (total * c / grid) & ~1LL, hi = (c + 1 == grid) ? total : ((total * (c + 1) / grid) & ~1LL);
-            worst_equal = std::max(worst_equal, run_cost(lo, hi, n_two, c2, c1));
+            worst_equal = std::max(worst_equal, run_cost(lo, hi, c1));
         }
         CHECK(worst <= worst_equal);
         // and no run costs more than the work spread evenly plus what one tile and its pieces can add
-        CHECK(worst <= total / grid + c2 + 4 * GM_SEG_COST + 2 || worst <= worst_equal);
+        CHECK(worst <= total / grid + c1 + 4 * GM_SEG_COST + 2 || worst <= worst_equal);
         return 0;
     }
 
@@ -67,7 +61,7 @@ SRC = textwrap.dedent(r"""
         const int grids[] = {1, 7, 132, 148, 160, 192};
         int n = 0;
         for (int M : Ms) for (long long K : Ks) for (long long N : Ns) for (int g : grids) {
-            const long long n_slabs = (K + 255) / 256 * 2, R = (N + 127) / 128;
+            const long long n_slabs = (K + 255) / 256 * 2, R = (N + 255) / 256;
             if (n_slabs * R * 16 > 2000000000LL) continue;
             if (one(n_slabs, R, M, g)) return 1;
             ++n;
