@@ -624,11 +624,11 @@ def main():
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of the decode kernel per stack pass, from the ncu capture summarised in
-# profiles/decode_stack_kernel_7b_4layers_M1.md: 355,717,888 + 4,195,584 bytes for the first 4 layers (354,172,928
+# the profile of a 4-layer pass of one token: 355,717,888 + 4,195,584 bytes for the first 4 layers (354,172,928
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
 DECODE_TRAFFIC_BYTES = 8 * (355_717_888 + 4_195_584)
-# gemm_kernel (profiles/gemm_kernel_11008x4096_M512_2bit.md): 21,204,224 + 31,488 bytes of DRAM traffic for one 11008 x 4096
+# gemm_kernel: 21,204,224 + 31,488 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
 PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_204_224 + 31_488) / 16_908_288)
 
@@ -752,7 +752,7 @@ def decode_attn_leg(aq, info, peaks, torch, context=4096, steps=30):
             "roofline": {"bound": "hbm", "achieved": byts / ms_graph / 1e6, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": byts / ms_graph / 1e6 / peaks["hbm_gbs"], "traffic": None, "peak_source": peaks["source"],
                          "what": "graph replay",
-                         "kernel": "decode_stack_kernel (33 launches) + attn_decode_kernel (32) + attn_prepare_kernel (32)"}}
+                         "kernel": "decode_stack_kernel (33 launches) + attn_decode_kernel (32)"}}
 
 
 def dequant_leg(aq, synth, peaks, torch):

@@ -27,8 +27,8 @@ struct aq_handle_s {
     uint8_t* sb;       // DEVICE: super-block parameters (32 bytes per row and super-block) of a handle made by aq_pack_sb /
                        // aq_import_sb, else null
     size_t sb_held;
-    uint8_t* big;      // DEVICE: scratch of aq_linear with M > AQ_DECODE_MAX_M (float32 sums, binary16 copy of bfloat16
-                       // activations, row scales), allocated when the handle first sees such a call and grown on demand
+    uint8_t* big;      // DEVICE: scratch of aq_linear with M > AQ_DECODE_MAX_M (float32 sums, the activations in operand order,
+                       // for bfloat16 with row scales), allocated when the handle first sees such a call and grown on demand
     size_t big_bytes;
     int* flags;        // DEVICE: bit 0 = range error seen while packing
     cudaStream_t last_stream;
@@ -91,8 +91,8 @@ struct StackPlan {
     size_t pk_begin = 0, pk_end = 0;   // the packed sums' region: zero at the start of a decode pass
     std::vector<size_t> nm_off;     // per op that opens an RMS-normalised phase (3 <= M <= AQ_DECODE_MAX_M): the CTAs'
                                     // partial sums of squares [AQ_NORM_MAX_CTAS][M] of 8 bytes, inside the region above; else 0
-    std::vector<size_t> x16_off;    // per op (bfloat16, M > AQ_DECODE_MAX_M only): its phase's binary16 operand [M][K] ...
-    std::vector<size_t> rs_off;     // ... the row scales [M] float32 ...
+    std::vector<size_t> x16_off;    // per op (M > AQ_DECODE_MAX_M only): its phase's binary16 operand [M][K] ...
+    std::vector<size_t> rs_off;     // ... and, for bfloat16, its row scales [M] float32
     size_t stage_off = 0;           // end of the float32 buffers
     size_t total = 0;
 };

@@ -64,7 +64,7 @@ static bool plan_stack(const aq_stack_t* p, int M, StackPlan& plan) {
         plan.in_off[i] = off;
         off += align_up((size_t)M * p->buf_width[p->ops[i].src] * 2, 256);
     }
-    if (M > AQ_DECODE_MAX_M) {   // bfloat16 activations reach the tensor cores as binary16: a second staged vector per phase
+    if (M > AQ_DECODE_MAX_M) {   // activations of both types reach the tensor cores as binary16 in operand order: a second staged vector per phase
         plan.x16_off.assign(p->n_ops, 0);
         plan.rs_off.assign(p->n_ops, 0);
         for (int i = 0; i < p->n_ops; ++i) {
@@ -144,7 +144,7 @@ struct PresetList {
     unsigned ctas() const {   // enough to write a few megabytes at the rate of the device: four groups of four per thread
         int64_t t = 0;
         for (int q = 0; q < n; ++q) t += n4[q];
-        return (unsigned)std::min<int64_t>((t + 1023) / 1024, 2 * 148);
+        return (unsigned)std::min<int64_t>((t + 1023) / 1024, 2 * sm_count());
     }
 };
 
@@ -367,7 +367,7 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
         }
         {
             const int64_t total4 = (int64_t)M * K / 4;
-            const unsigned g = (f.in_op == AQ_IN_RMSNORM) ? (unsigned)M : (unsigned)std::min<int64_t>((total4 + 255) / 256, 4 * 148);
+            const unsigned g = (f.in_op == AQ_IN_RMSNORM) ? (unsigned)M : (unsigned)std::min<int64_t>((total4 + 255) / 256, 4 * sm_count());
             const float* s2 = (f.in_op == AQ_IN_SILU_MUL) ? buf(f.src2) : nullptr;
             pre.first = (!decode && dt == AQ_BF16) ? (unsigned)M : g;
             if (decode) stage_kernel<T><<<g, 256, 0, s>>>(buf(f.src), s2, (int)f.in_op, K, total4, stage, nullptr, pre);

@@ -24,8 +24,8 @@ def test_tile_edges(M, N, K, bits, dtype):
     aq.aq_check()
     want, T = O.linear(*O.quantize(W, bits), x.double().cpu().numpy())
     assert O.linear_excess(y.double().cpu().numpy(), want, T).max() <= 1.0
-    half = torch.full((M, N), float("nan"), dtype=tdt, device="cuda")   # up to 64 tokens the GEMM itself rounds: the tickets
-    for _ in range(2):                                                  # of shared tiles are zero again for the second call
+    half = torch.full((M, N), float("nan"), dtype=tdt, device="cuda")   # the sums rounded by the cast; the second call finds
+    for _ in range(2):                                                  # the first one's sums in the scratch
         aq.aq_linear(h, x, half)
     aq.aq_check()
     # two runs' float32 sums may differ by their order and then round to neighbouring values

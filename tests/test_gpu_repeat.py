@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 def test_repeated_prefill_passes_agree():
     import torch
-    # two token super-tiles (512 + 256), several pieces of a tile per CTA; long enough for the clocks to settle under load
+    # six token tiles of 128, several pieces of a tile per CTA; long enough for the clocks to settle under load
     M, layers_n = 768, 18
     bits = [2, 3, 4, 2, 3, 4, 3] * layers_n
     layers, _, _ = workloads.build_stack(synth.gemma2b_layer(), layers_n, bits, (71,))
