@@ -30,16 +30,20 @@ def test_recycled_blocks_and_threads():
     cases = [(1200 + 16 * i, 4096, b) for i in range(3) for b in (2, 3, 4)]
     data = [_case(N, K, b, i) for i, (N, K, b) in enumerate(cases)]
     torch.cuda.synchronize()
-    wrong = []
+    wrong, done = [], []
 
     def work(order):
-        s = torch.cuda.Stream()
-        with torch.cuda.stream(s):
-            for i in order:
-                h = aq.aq_pack(cases[i][2], 32, data[i][0])
-                if not np.array_equal(aq.aq_export(h), data[i][1]):
-                    wrong.append(i)
-                h.free()
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                for i in order:
+                    h = aq.aq_pack(cases[i][2], 32, data[i][0])
+                    if not np.array_equal(aq.aq_export(h), data[i][1]):
+                        wrong.append(i)
+                    h.free()
+                    done.append(i)
+        except Exception as e:                        # (an exception that ends a thread ends nothing else)
+            wrong.append(e)
 
     n = len(cases)
     threads = [threading.Thread(target=work, args=([(5 * k + 2 * t) % n for k in range(2 * n)],)) for t in range(3)]
@@ -47,7 +51,36 @@ def test_recycled_blocks_and_threads():
         t.start()
     for t in threads:
         t.join()
-    assert not wrong
+    assert not wrong, wrong
+    assert len(done) == 3 * 2 * n
+
+
+def test_exports_that_go_round_the_ring():
+    """22.5 MB and 9.0 MB through eight chunks of 1 MB, with ragged last chunks; then from two threads at once, one of which
+    gets the ring and the other an ordinary copy."""
+    from paper_2605_24011_b200 import aq
+    cases = [(11008, 4096, 3), (2305, 6272, 4)]
+    data = [_case(N, K, b, 8) for N, K, b in cases]
+    handles = [aq.aq_pack(b, 32, W) for (_, _, b), (W, _) in zip(cases, data)]
+    for h, (_, want) in zip(handles, data):
+        assert np.array_equal(aq.aq_export(h), want)
+    wrong, done = [], []
+
+    def work(i):
+        try:
+            for _ in range(6):
+                if not np.array_equal(aq.aq_export(handles[i]), data[i][1]):
+                    wrong.append(i)
+                done.append(i)
+        except Exception as e:
+            wrong.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in (0, 0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong and len(done) == 18, wrong
 
 
 def test_another_threads_recording_survives_a_freed_handle():
