@@ -6,8 +6,10 @@
 namespace aq {
 
 constexpr int GM_MAX_GRID = 192;   // CTAs of one launch (one per SM)
-// What ending one piece of a tile costs a CTA (accumulator drain, epilogue, refilling the pipeline), in units of one
-// slab-accumulator of MMA work (measured: about 8 us against 0.88 us); the runs are cut so that work + pieces balance.
+// What ending one piece of a tile costs a CTA (accumulators drained, epilogue, adds of a shared tile), in half slabs of 64 k:
+// the runs are cut so that work + pieces balance.  Set by time: over 90 shapes of 9 to 1024 tokens, against 9, a cost of 1
+// takes 1.03 to 1.04 of the time, 2 1.01 to 1.04, 3 1.00 to 1.02, 4 to 14 0.99 to 1.015; eight 7B layers at 200 tokens 1191,
+// 1156, 1139, 1136, 1133 (6), 1131 (9), 1135 us (14).
 constexpr int GM_SEG_COST = 9;
 
 // Cuts [0, total) into `grid` contiguous runs with even bounds (bounds[0] = 0 .. bounds[grid] = total).  The work is a
