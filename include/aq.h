@@ -339,6 +339,8 @@ size_t aq_stack_workspace_bytes(const aq_stack_t* prog, int M);
  *                   afterwards buffer b is float32 [M][width[b]] at byte
  *                   offset aq_stack_buffer_offset(prog, M, b): every op's
  *                   input and output stay readable for per-op checks
+ * Accuracy for M <= AQ_DECODE_MAX_M: exact products, binary32 sums over 256 columns, steps of 2^-24 between them; with
+ * M = 1 an activation enters the products off by at most 2^-26 of the largest magnitude in its block of 32.
  * CUDA graphs: the call may be recorded into a graph (stream capture) and
  * replayed.  For M <= AQ_DECODE_MAX_M make one eager call with the same
  * program, M, dtype and workspace on that device first: it builds the device

@@ -10,10 +10,12 @@
 //   D  = sums in TMEM, read back one row per lane; the block scales need a sum per block.
 //
 // One token (kind::i8, exact integers).  Every byte of an A register is a code times 2^pos (pos 0 or 2 for the first group
-// of a block's slot, 4 or 6 for the second).  x enters as a block-wise fixed-point number of 31 bits (relative to the
-// largest magnitude of its block of 32; a binary16 or bfloat16 value is exact unless it is 2^19 times smaller than
-// that one, and then off by at most 2^-31 of it) in four signed bytes; the elements that meet second groups are scaled down
-// by 16.  B = four byte planes of a block in four rows: a chunk of 16 k is 128 bytes, 4 rows of data and 4 of zeros.  The
+// of a block's slot, 4 or 6 for the second).  x enters as a block-wise fixed-point number in four signed bytes: scaled by the
+// power of two that brings the largest magnitude of its block of 32 into [2^29, 2^30), the elements that meet second groups
+// by 2^-4 of that.  So an element is off by at most 2^-30 of that magnitude in a first group and 2^-26 in a second, and
+// a binary16 value is exact unless it is 2^19 / 2^15 times smaller (bfloat16: 2^22 / 2^18).  (Blocks below 2^-93, which only
+// bfloat16 has: steps of 2^-123 / 2^-119.)  That is below what binary32 sums of the block's products lose, unless the largest
+// element meets a weight that decodes to 0.  B = four byte planes of a block in four rows: a chunk of 16 k is 128 bytes, 4 rows of data and 4 of zeros.  The
 // instruction of an odd block reads its chunks through a window moved down by 64 bytes, so the planes land in rows 4..7:
 // two blocks share one accumulator of 8 columns [block parity][plane].
 //

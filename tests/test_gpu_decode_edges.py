@@ -126,3 +126,38 @@ def test_one_token_with_a_non_finite_element_is_the_first_of_two(bad, dtype, pos
         got.append(aq.stack_buffer(prog, ws, M, 1)[0].clone())
     assert torch.equal(got[0], got[1])
     assert (got[0].abs() > 1e8).all() and (not positive or bad < 0 or bad != bad or (got[0] > 0).any())
+
+
+@pytest.mark.parametrize("bits", (2, 3, 4))
+@pytest.mark.parametrize("dtype", ("f16", "bf16"))
+def test_one_token_with_an_outlier_that_meets_a_zero_weight(dtype, bits):
+    """An activation of one token is a fixed-point number relative to the largest of its block: off by at most 2^-30 of it in
+    the first groups (k mod 8 below 4) and 2^-26 in the second.  The outlier sits in a first group, where the weight decodes to
+    0, and the small values in second groups only, so nothing hides those steps."""
+    from paper_2605_24011_b200 import aq
+    N, K = 96, 1024
+    k = np.arange(K)
+    W = np.abs(synth.weights(N, K, 96, bits)) + np.float32(0.01)
+    W[:, k % 32 == 0] = 0.0
+    x = synth.activations(1, K, 97) * np.float32(2.0 ** -8)
+    x[:, k % 8 < 4] = 0.0
+    x[:, k % 32 == 0] = 60000.0
+    x0 = torch.from_numpy(x).to(torch.float16 if dtype == "f16" else torch.bfloat16).cuda()
+    h = aq.aq_pack(bits, 32, torch.from_numpy(W).cuda())
+    prog = aq.Program([K, N], [{"w": h, "src": 0, "dst": 1}])
+    ws = torch.empty(prog.workspace_bytes(1), dtype=torch.uint8, device="cuda")
+    aq.aq_stack_forward(prog, x0, None, 1, 1, ws)
+    aq.aq_check()
+    x = x0.double().cpu().numpy()
+    d, m, q = O.quantize(W, bits)
+    want, T = O.linear(d, m, q, x)
+    d, m, q = (np.asarray(v, dtype=np.float64).reshape(N, K // 32, -1) for v in (d, m, q))
+    xb = x.reshape(K // 32, 32)
+    step = np.where(np.arange(32) % 8 < 4, 2.0 ** -30, 2.0 ** -26)
+    fixed = (d[:, :, 0] * (q * step).sum(2) * np.abs(xb).max(1)).sum(1)
+    # binary32: a handful of roundings of a block's two terms, then of the sums along k; 2^-25 per 256 columns when units are added
+    terms = (np.abs(d[:, :, 0] * (q * xb).sum(2)) + np.abs(m[:, :, 0] * xb.sum(1))).sum(1)
+    bound = fixed + 2.0 ** -21 * (terms + T[0]) + K / 256 * 2.0 ** -25
+    err = np.abs(aq.stack_buffer(prog, ws, 1, 1).double().cpu().numpy()[0] - want[0])
+    assert np.all(err <= bound), float((err / bound).max())
+    assert fixed.max() > 10 * (bound - fixed).max()      # (the steps are what is tested)
