@@ -426,7 +426,7 @@ aq_status_t aq_set_wait_limit_ns(uint64_t ns);
  */
 void aq_debug_decode_hold(int on);
 
-/* Releases the handle and its device memory (synchronises its last stream).  Up to 256 MB of released blocks per process are
+/* Releases the handle and its device memory (synchronises its last stream); graphs recorded with it are invalid then.  Up to 256 MB of released blocks per process are
  * kept for the next handles of about their size; they go back to the driver when later releases have not found a use for
  * them, or when an allocation of this library fails. */
 void aq_free(aq_handle_t h);
