@@ -624,13 +624,13 @@ def main():
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of the decode kernel per stack pass, from the ncu capture summarised in
-# the profile of a 4-layer pass of one token: 355,717,888 + 4,195,584 bytes for the first 4 layers (354,172,928
+# the profile of a 4-layer pass of one token: 355,696,384 + 4,406,784 bytes for the first 4 layers (354,172,928
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
-DECODE_TRAFFIC_BYTES = 8 * (355_717_888 + 4_195_584)
-# gemm_kernel: 21,204,224 + 31,488 bytes of DRAM traffic for one 11008 x 4096
+DECODE_TRAFFIC_BYTES = 8 * (355_696_384 + 4_406_784)
+# gemm_kernel: 21,203,456 + 4,608 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
-PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_204_224 + 31_488) / 16_908_288)
+PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_456 + 4_608) / 16_908_288)
 
 
 def prefill_leg(aq, workloads, prog, out_buf, info, peaks, torch, gpu_index=0):
@@ -702,7 +702,7 @@ def attn_leg(aq, peaks, torch):
         gbs = per / us / 1e3
         out[f"L{L}"] = {"us_per_call": us, "gbs": gbs,
                         "roofline": {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
-                                     "traffic": 67_175_680 + 434_688 if L == 4096 else None, "peak_source": peaks["source"],
+                                     "traffic": 67_196_672 + 469_760 if L == 4096 else None, "peak_source": peaks["source"],
                                      "kernel": "attn_decode_kernel"}}
         del caches
     return out
