@@ -13,12 +13,12 @@
 //       - the feeder (one thread) keeps a ring of bulk copies (cp.async.bulk +
 //         mbarrier, L2 evict-first) full;
 //       - eight unpack warps turn codes into tensor-core operands in TMEM, in two
-//         to five stages.  Neither depends on any activation: they run ahead
+//         or five stages.  Neither depends on any activation: they run ahead
 //         across op and phase boundaries, so a phase starts with its first units
 //         waiting in TMEM;
 //       - the issuer (one thread) starts a unit's tensor-core instructions;
-//       - eight collect warps form a phase's input, read the units' sums back,
-//         apply scales and minima and add the rows up in memory;
+//       - eight collect warps (twelve from three tokens on) form a phase's input, read
+//         the units' sums back, apply scales and minima and add the rows up in memory;
 //       - two record warps write the caller's copies of a phase's input.
 //     Four warps that each did all of this in turn, step after step, needed 1404
 //     us for a 7B-shaped pass of one token (software-pipelined: 1398); the roles
@@ -38,8 +38,15 @@
 //
 // What bounds it now (7B shapes, one token): between two boundaries a unit takes
 // 304 ns per SM, HBM's rate is 323; a boundary costs 3.3 us, of which the ring
-// (160 KB per SM, 3.6 us of HBM) hides the weights' part.  With 8 tokens a unit
-// takes 0.8 us (applying block scales to 8 columns and 1024 red.adds per unit).
+// (160 KB per SM, 3.6 us of HBM) hides the weights' part.  With 8 tokens the collect
+// warps set the pace: a team of four takes 1.7 us per unit, 0.7 to read the sums and
+// apply the block scales and 1 for 1024 red.adds, and a boundary costs about 9 us, most
+// of it the wait for the slowest CTA and the exchange of row norms.  Two teams, with A
+// kept until the sums were read and one multiply-add per value, took 2304 us for a 7B-shaped
+// pass, three teams with operand and sums released on their own 2090 (M = 4 with
+// instrumentation 447 -> 383 thousand cycles for four layers, M = 2 no difference).  Neither
+// the L2 rate of the adds (204 ns per 1024 of them with every SM adding) nor the polls
+// (pauses of 32 to 250 ns in them changed nothing) is the limit.
 //
 // Every wait is bounded: when one runs out the kernel raises a status word,
 // gives copies in flight time to land and returns.
@@ -60,25 +67,61 @@ namespace aq {
 typedef unsigned long long u64;
 
 // Warps by role (a warp reaches the TMEM lanes of its quarter only: unpack and collect teams start at multiples of four).
-// At most five warps per scheduler leave 96 registers per thread.
 constexpr int DS_UNPACK_WARPS = 8;          // two teams of four: one per half (128 k) of a unit
-constexpr int DS_COLLECT_WARPS = 8;         // two teams of four, taking units in turn
 constexpr int DS_RECORD_WARPS = 2;
-constexpr int DS_COLLECT0 = DS_UNPACK_WARPS, DS_ISSUER = DS_COLLECT0 + DS_COLLECT_WARPS, DS_FEEDER = DS_ISSUER + 1, DS_RECORD0 = DS_FEEDER + 1;
-constexpr int DS_WARPS = DS_RECORD0 + DS_RECORD_WARPS;
-constexpr int DS_THREADS = DS_WARPS * 32;
-constexpr int DS_CTHREADS = DS_COLLECT_WARPS * 32;
+// Collect warps: teams of four that take the units in turn.  One token: two teams.  Several tokens: a unit costs its team four
+// times as many instructions, so there are three, and the roles get registers by what they need.
+template <int MT> struct DsRoles {
+    static constexpr int COLLECT_WARPS = MT <= 2 ? 8 : 12, TEAMS = COLLECT_WARPS / 4, CTHREADS = COLLECT_WARPS * 32;
+    static constexpr int COLLECT0 = DS_UNPACK_WARPS, ISSUER = COLLECT0 + COLLECT_WARPS, FEEDER = ISSUER + 1, RECORD0 = FEEDER + 1;
+    static constexpr int WARPS = RECORD0 + DS_RECORD_WARPS, THREADS = WARPS * 32;
+    static constexpr bool SHARES = MT > 2;      // registers per thread: 80 at the launch, then
+    static constexpr int REGS_UNPACK = 56, REGS_COLLECT = 104, REGS_OTHER = 56;
+    static_assert(!SHARES || (DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80 && WARPS % 4 == 0), "the roles' registers fit");
+};
+constexpr int DS_MAX_COLLECT_WARPS = 12;
 constexpr int DS_FRAGS = 8;                 // 16-row tiles of a unit
 constexpr int DS_QUEUE = 16;                // units in flight at most
 constexpr int DS_RING_BYTES = 160 * 1024;   // packed units in flight
 constexpr int DS_MAX_SLOTS = 6;             // staged slabs per phase per CTA
 constexpr int DS_XS_BYTES = DS_MAX_SLOTS * dt_slab_bytes(AQ_DECODE_MAX_M);
-// A unit's operands and sums in TMEM: A of both halves, D of both halves.
+// A unit's operands and sums in TMEM, A of both halves and D of both halves, and what goes with it (descriptor, scales, the
+// barrier that says they are there).  One token: five stages of both, refilled once the sums have been read.  Several tokens:
+// reading the sums takes longer than anything else, so A (two stages) is refilled as soon as the instructions have read it
+// and D (two as well) is written again once the sums have been read; unit n + 4 is not unpacked before unit n + 2 was issued,
+// which waited for the sums of unit n.
 template <int MT> struct DsStage {
-    static constexpr int COLS = 2 * (DtShape<MT>::A_COLS + DtShape<MT>::D_COLS);   // 96 / 256
-    static constexpr int N = 512 / COLS;                                           // 5 / 2 stages
+    static constexpr int A_COLS = 2 * DtShape<MT>::A_COLS, D_COLS = 2 * DtShape<MT>::D_COLS;   // 64 + 32 / 128 + 128
+    static constexpr bool SPLIT = MT > 1;
+    static constexpr int A = SPLIT ? 2 : 5, D = SPLIT ? 2 : 5, META = SPLIT ? 4 : 5;
+    static_assert(A * A_COLS + D * D_COLS <= 512 && META <= A + D, "fits TMEM; see above");
+    // first columns of stages (one token: a stage's sums lie behind its operand, one address serves both)
+    __device__ static __forceinline__ uint32_t a_col(uint32_t s) { return s * (SPLIT ? A_COLS : A_COLS + D_COLS); }
+    __device__ static __forceinline__ uint32_t d_col(uint32_t s) { return SPLIT ? A * A_COLS + s * D_COLS : a_col(s) + A_COLS; }
 };
 constexpr int DS_MAX_STAGES = 5;
+// A slot of a ring and how often the ring has gone round.
+template <int N> struct DsRing {
+    uint32_t at = 0, use = 0;
+    __device__ __forceinline__ void next() { if (++at == N) { at = 0; ++use; } }
+};
+// Where the next unit lies: its A stage, D stage and what goes with it (one token: all the same).
+template <int MT> struct DsPlace {
+    DsRing<DsStage<MT>::A> ra;
+    DsRing<DsStage<MT>::D> rd;
+    DsRing<DsStage<MT>::META> rm;
+    __device__ __forceinline__ const auto& a() const { return ra; }
+    __device__ __forceinline__ const auto& d() const { return rd; }
+    __device__ __forceinline__ const auto& m() const { return rm; }
+    __device__ __forceinline__ void next() { ra.next(); rd.next(); rm.next(); }
+};
+template <> struct DsPlace<1> {
+    DsRing<DsStage<1>::A> r;
+    __device__ __forceinline__ const auto& a() const { return r; }
+    __device__ __forceinline__ const auto& d() const { return r; }
+    __device__ __forceinline__ const auto& m() const { return r; }
+    __device__ __forceinline__ void next() { r.next(); }
+};
 constexpr int DS_MAX_PHASE_OPS = 8;
 constexpr int DS_RMS_HOLD = 4;              // groups of four elements per thread kept in registers by the one-token RMS path
 // Several tokens: up to this many elements (M K) every CTA reads the rows whole for the row norms, above it the norms come from
@@ -233,10 +276,12 @@ __device__ __forceinline__ bool ds_warp_wait(uint32_t bar, uint32_t parity, u64 
     return __all_sync(0xffffffffu, ds_mbar_wait(bar, parity, wait_ns, abort_flag));
 }
 // Barrier among the collect warps only.
-__device__ __forceinline__ void ds_collect_sync() { asm volatile("bar.sync 1, %0;" ::"n"(DS_CTHREADS) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void ds_collect_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
 // The same barrier, returning the OR of `flag` over all collect threads: every thread gets the same answer, so a
 // decision to leave the phase loop is taken by all warps or by none (a flag read after a plain barrier could change
 // between two threads' reads).
+template <int THREADS>
 __device__ __forceinline__ bool ds_collect_sync_or(int flag) {
     uint32_t r;
     asm volatile(
@@ -244,7 +289,7 @@ __device__ __forceinline__ bool ds_collect_sync_or(int flag) {
         "setp.ne.u32 q, %1, 0;\n\t"
         "bar.red.or.pred p, 1, %2, q;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(r) : "r"(flag), "n"(DS_CTHREADS) : "memory");
+        : "=r"(r) : "r"(flag), "n"(THREADS) : "memory");
     return r != 0;
 }
 
@@ -347,7 +392,7 @@ struct DsShared {
     alignas(8) uint64_t taken[DS_MAX_STAGES];    // its sums have been read
     alignas(8) uint64_t rec_bar[DS_RECS];
     uint32_t qsize[DS_QUEUE];               // (the feeder's) ring bytes of the units in flight
-    float red[AQ_DECODE_MAX_M][DS_COLLECT_WARPS];
+    float red[AQ_DECODE_MAX_M][DS_MAX_COLLECT_WARPS];
     float scale[DS_RECS][AQ_DECODE_MAX_M];  // row scales of the phases (1 / rms)
     uint32_t tmem;
     int xphase;                             // phases whose input is staged
@@ -360,6 +405,21 @@ static_assert(sizeof(DsShared) <= 227 * 1024, "fits an SM");
 template <int MT>
 __device__ __forceinline__ void ds_commit(const float (&acc)[MT], u64* out, const void* res, bool res_plain, int row, int N, int M) {
     if (row >= N) return;
+    if constexpr (MT > 1) {
+        // (what a sum costs here, times 1024 per unit, is a third of the collect warps' instructions: the limits are looked at
+        // once for all tokens)
+        float mx = 0.f;
+        bool clean = true;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) { mx = fmaxf(mx, fabsf(acc[m])); clean = clean && acc[m] == acc[m]; }
+        if (res == nullptr && clean && mx < DS_FIX_MAX) {
+            u64* p = out + row;
+#pragma unroll
+            for (int m = 0; m < MT; ++m, p += N)
+                if (m < M) ds_red_add(p, ((u64)__float2ll_rn(acc[m] * DS_FIX_ONE) << DS_CNT_BITS) + 1ull);
+            return;
+        }
+    }
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
         if (m >= M) break;
@@ -440,7 +500,7 @@ template <int MT, bool BF16>
 __device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint32_t tmem, int half, int quarter, int lane) {
     using ST = DsStage<MT>;
     using SH = DtShape<MT>;
-    uint32_t stage = 0, use = 0;   // TMEM stage and how often the stages have gone round
+    DsPlace<MT> at;
     for (uint32_t n = 0;; ++n) {
         const uint32_t e = n % DS_QUEUE;
         if (!ds_warp_wait(ds_smem(&sh.full[e]), (n / DS_QUEUE) & 1u, wait_ns, &sh.abort_flag)) return;
@@ -450,9 +510,14 @@ __device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint3
         // (row tiles past the matrix's last one: whatever lies there; their rows are not written)
         const uint8_t* fr = sh.ring + (d.w & 0xFFFFFu) + (half ? (d.w >> 20) << 8 : 0u) + (uint32_t)(quarter * 2 * fb);
         const uint4 dm = *reinterpret_cast<const uint4*>(fr + (lane >> 4) * fb + (lane & 15) * 16);
-        const uint32_t ta = tmem + stage * ST::COLS + (uint32_t)(half * SH::A_COLS) + ((uint32_t)(quarter * 32) << 16);
-        // the stage is free once its last unit's sums have been read
-        auto stage_free = [&]() { return use == 0 || ds_warp_wait(ds_smem(&sh.taken[stage]), (use - 1) & 1u, wait_ns, &sh.abort_flag); };
+        const uint32_t ta = tmem + ST::a_col(at.a().at) + (uint32_t)(half * SH::A_COLS) + ((uint32_t)(quarter * 32) << 16);
+        // the stage is free once its last unit's instructions have completed (one token: and its sums have been read)
+        auto stage_free = [&]() {
+            if (at.a().use == 0) return true;
+            if constexpr (!ST::SPLIT) return ds_warp_wait(ds_smem(&sh.taken[at.a().at]), (at.a().use - 1) & 1u, wait_ns, &sh.abort_flag);
+            const uint32_t before = n - ST::A;   // the unit that had the stage
+            return ds_warp_wait(ds_smem(&sh.done[before % ST::D]), (before / ST::D) & 1u, wait_ns, &sh.abort_flag);
+        };
         if constexpr (MT == 1) {
             uint32_t va[16], vb[16];
             if (bits == 2) dt_unpack2<2>(fr, lane, va, vb);
@@ -481,16 +546,16 @@ __device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint3
             const bool ok = bits == 2 ? both(std::integral_constant<int, 2>()) : bits == 3 ? both(std::integral_constant<int, 3>()) : both(std::integral_constant<int, 4>());
             if (!ok) return;
         }
-        *reinterpret_cast<uint4*>(&sh.dm[stage][half * DS_FRAGS + quarter * 2 + (lane >> 4)][(lane & 15) * 16]) = dm;
-        if (half == 0 && quarter == 0 && lane == 0) sh.sdesc[stage] = d;
+        *reinterpret_cast<uint4*>(&sh.dm[at.m().at][half * DS_FRAGS + quarter * 2 + (lane >> 4)][(lane & 15) * 16]) = dm;
+        if (half == 0 && quarter == 0 && lane == 0) sh.sdesc[at.m().at] = d;
         tmem_st_wait();          // (everything read from the ring has been used: the slot may be refilled)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
             ds_mbar_arrive(ds_smem(&sh.empty[e]));
-            ds_mbar_arrive(ds_smem(&sh.stored[stage]));
+            ds_mbar_arrive(ds_smem(&sh.stored[at.m().at]));
         }
-        if (++stage == ST::N) { stage = 0; ++use; }
+        at.next();
     }
 }
 
@@ -518,26 +583,29 @@ __device__ __forceinline__ int ds_wait_count(const int* count, int value, u64 wa
 template <int MT, bool BF16>
 __device__ __forceinline__ void ds_issue_units(DsShared& sh, const DsArgs& a, uint32_t tmem) {
     using ST = DsStage<MT>;
-    uint32_t stage = 0, use = 0;
+    DsPlace<MT> at;
     int ready = 0;   // phases whose input is staged
     const uint32_t zlow = ds_smem(sh.zlow), zhigh = ds_smem(sh.zhigh), xs = ds_smem(sh.xs);
     for (int left = a.unit_total[blockIdx.x]; left > 0; --left) {
-        if (!ds_warp_wait(ds_smem(&sh.stored[stage]), use & 1u, 2 * a.wait_ns, &sh.abort_flag)) return;
-        const uint2 d = *reinterpret_cast<const uint2*>(&sh.sdesc[stage]);
+        if (!ds_warp_wait(ds_smem(&sh.stored[at.m().at]), at.m().use & 1u, 2 * a.wait_ns, &sh.abort_flag)) return;
+        if (ST::SPLIT && at.d().use > 0 && !ds_warp_wait(ds_smem(&sh.taken[at.d().at]), (at.d().use - 1) & 1u, 2 * a.wait_ns, &sh.abort_flag)) return;
+        const uint2 d = *reinterpret_cast<const uint2*>(&sh.sdesc[at.m().at]);
         const int ph = (int)(d.x >> DS_DESC_PHASE_SHIFT);
         if (ready <= ph) {
             ready = ds_wait_count(&sh.xphase, ph, 2 * a.wait_ns, &sh.abort_flag);
             if (ready <= ph) return;
         }
         const uint32_t x = __shfl_sync(0xffffffffu, xs + d.y, 0);
-        const uint32_t t0 = __shfl_sync(0xffffffffu, tmem + stage * ST::COLS, 0);
+        const uint32_t ta = __shfl_sync(0xffffffffu, tmem + ST::a_col(at.a().at), 0);
+        uint32_t td = ta + ST::A_COLS;
+        if constexpr (ST::SPLIT) td = __shfl_sync(0xffffffffu, tmem + ST::d_col(at.d().at), 0);
         tc_fence_after();
         if (elect_one()) {
-            dt_issue<MT, BF16>(t0, t0 + 2 * DtShape<MT>::A_COLS, x, zlow, zhigh);
-            umma_commit(ds_smem(&sh.done[stage]));
+            dt_issue<MT, BF16>(ta, td, x, zlow, zhigh);
+            umma_commit(ds_smem(&sh.done[at.d().at]));
         }
         __syncwarp();
-        if (++stage == ST::N) { stage = 0; ++use; }
+        at.next();
     }
 }
 
@@ -602,8 +670,9 @@ __device__ __forceinline__ void ds_record(DsShared& sh, const DsArgs& a, int rw,
 
 // ---- the kernel ---------------------------------------------------------------------
 template <int MT, bool BF16>
-__global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArgs a) {
+__global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(const DsArgs a) {
     using ST = DsStage<MT>;
+    using RO = DsRoles<MT>;
     extern __shared__ __align__(128) uint8_t ds_smem_raw[];
     DsShared& sh = *reinterpret_cast<DsShared*>(ds_smem_raw);
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -637,7 +706,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
     }
     // the slabs keep zeros everywhere but in the elements the stagers rewrite every phase (rows of absent tokens; one
     // token: every row but the first)
-    for (int i = threadIdx.x; i < (DS_XS_BYTES + 2 * DT_ZERO_BYTES) / 16; i += DS_THREADS)
+    for (int i = threadIdx.x; i < (DS_XS_BYTES + 2 * DT_ZERO_BYTES) / 16; i += RO::THREADS)
         reinterpret_cast<uint4*>(sh.zlow)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -647,17 +716,22 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
     const uint32_t tmem = sh.tmem;
 
     if (warp < DS_UNPACK_WARPS) {
+        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_UNPACK));
         ds_unpack_units<MT, BF16>(sh, wait_ns, tmem, warp >> 2, quarter, lane);
-    } else if (warp == DS_ISSUER) {
+    } else if (warp == RO::ISSUER) {
+        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
         ds_issue_units<MT, BF16>(sh, a, tmem);
-    } else if (warp == DS_FEEDER) {
+    } else if (warp == RO::FEEDER) {
+        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
         if (lane == 0) ds_feed(sh, a);
         __syncwarp();
-    } else if (warp >= DS_RECORD0) {
-        ds_record<BF16>(sh, a, warp - DS_RECORD0, lane);
+    } else if (warp >= RO::RECORD0) {
+        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
+        ds_record<BF16>(sh, a, warp - RO::RECORD0, lane);
     } else {
+    if constexpr (RO::SHARES) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RO::REGS_COLLECT));
     // ================= collect warps =================
-    const int ctid = (int)threadIdx.x - DS_COLLECT0 * 32, cwarp = warp - DS_COLLECT0;
+    const int ctid = (int)threadIdx.x - RO::COLLECT0 * 32, cwarp = warp - RO::COLLECT0;
     auto fetch_record = [&](int q) {   // the phase's record and this CTA's tables for it, on one barrier
         const uint32_t bar = ds_smem(&sh.rec_bar[q % DS_RECS]);
         uint64_t pol_keep;
@@ -670,7 +744,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
         if (a.n_phases > 0) fetch_record(0);
         if (a.n_phases > 1) fetch_record(1);
     }
-    uint32_t stage = 0, use = 0;       // TMEM stage of the next unit, and how often the stages have gone round
+    DsPlace<MT> at;                    // of the next unit
     uint32_t turn = 0;                 // the team whose unit that is
 
 #pragma unroll 1
@@ -687,7 +761,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
             if (lane == 0) fetch_record(ph + 2);
         }
         // every warp is through with phase ph - 1: the staged slabs are free
-        if (ds_collect_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
+        if (ds_collect_sync_or<RO::CTHREADS>(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
 
         // -- form the rounded input vector for the slabs this CTA reads --
         {
@@ -718,7 +792,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                     if ((lane & 7) == 0) reinterpret_cast<float*>(sl + DT_SUMS<MT>)[(kl >> 5) * 8 + m] = sum;
                 }
             };
-            if (P.in_op == AQ_IN_RMSNORM && MT == 1 && q4 <= DS_RMS_HOLD * DS_CTHREADS) {
+            if (P.in_op == AQ_IN_RMSNORM && MT == 1 && q4 <= DS_RMS_HOLD * RO::CTHREADS) {
                 // one token, row held in registers: one trip to L2 once the row is complete (all of a thread's readings
                 // go out together and are repeated together until every one of them is complete)
                 float4 v[DS_RMS_HOLD];
@@ -731,12 +805,12 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                         bool ready = true;
 #pragma unroll
                         for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                            const int i4 = ctid + n * DS_CTHREADS;
+                            const int i4 = ctid + n * RO::CTHREADS;
                             if (i4 < q4) ds_ld_quad(P.src + 4 * (int64_t)i4, q[n]);
                         }
 #pragma unroll
                         for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                            const int i4 = ctid + n * DS_CTHREADS;
+                            const int i4 = ctid + n * RO::CTHREADS;
                             if (i4 < q4) ready = ready && ds_quad_ready(q[n], expect);
                         }
                         if (ready || pat.over(sh, wait_ns)) break;
@@ -744,13 +818,13 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                     const bool failed = *reinterpret_cast<volatile int*>(&sh.abort_flag) != 0;
 #pragma unroll
                     for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                        const int i4 = ctid + n * DS_CTHREADS;
+                        const int i4 = ctid + n * RO::CTHREADS;
                         v[n] = (i4 < q4 && !failed) ? ds_quad_value(q[n]) : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 } else {
 #pragma unroll
                     for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                        const int i4 = ctid + n * DS_CTHREADS;
+                        const int i4 = ctid + n * RO::CTHREADS;
                         v[n] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (i4 < q4) v[n] = __ldcg(reinterpret_cast<const float4*>(P.src_f) + i4);
                     }
@@ -765,16 +839,16 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
 #pragma unroll
                 for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
                 if (lane == 0) sh.red[0][cwarp] = ss;
-                ds_collect_sync();
+                ds_collect_sync<RO::CTHREADS>();
                 float tot = 0.f;
 #pragma unroll
-                for (int w = 0; w < DS_COLLECT_WARPS; ++w) tot += sh.red[0][w];
+                for (int w = 0; w < RO::COLLECT_WARPS; ++w) tot += sh.red[0][w];
                 const float scale = rsqrtf(tot / (float)P.K + 1e-6f);
                 if (ctid == 0) sh.scale[pb][0] = scale;
 #pragma unroll
                 for (int n = 0; n < DS_RMS_HOLD; ++n) {
-                    const int i4 = ctid + n * DS_CTHREADS;
-                    if (n * DS_CTHREADS < q4) {   // the same for every thread: warps stay whole
+                    const int i4 = ctid + n * RO::CTHREADS;
+                    if (n * RO::CTHREADS < q4) {   // the same for every thread: warps stay whole
                         const int slab = i4 >> 6;   // (a warp's 32 groups are half a slab)
                         int sl = -1;
 #pragma unroll
@@ -823,7 +897,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                         for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
                         if (lane == 0) sh.scale[pb][cwarp] = rsqrtf(tot / (float)P.K + 1e-6f);
                     }
-                    ds_collect_sync();
+                    ds_collect_sync<RO::CTHREADS>();
                     normed = true;
                 }
                 }
@@ -831,7 +905,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                     if constexpr (MT < 4) {
                         for (int m = 0; m < M; ++m) {
                             float ss = 0.f;
-                            for (int i = ctid; i < q4; i += DS_CTHREADS) {
+                            for (int i = ctid; i < q4; i += RO::CTHREADS) {
                                 const float4 v = ds_source4(sh, P.src, P.src_f, expect, (int64_t)m * P.K + 4 * (int64_t)i, wait_ns, pat);
                                 ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
                             }
@@ -845,7 +919,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                         for (int m = 0; m < M; m += 2) {
                             float ss[2] = {0.f, 0.f};
                             const bool second = m + 1 < M;
-                            for (int i = ctid; i < q4; i += DS_CTHREADS) {
+                            for (int i = ctid; i < q4; i += RO::CTHREADS) {
                                 const int64_t o = (int64_t)m * P.K + 4 * (int64_t)i;
                                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
                                 if (P.src == nullptr) {
@@ -874,26 +948,26 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                             }
                         }
                     }
-                    ds_collect_sync();
+                    ds_collect_sync<RO::CTHREADS>();
                     if (ctid < M) {
                         float tot = 0.f;
 #pragma unroll
-                        for (int w = 0; w < DS_COLLECT_WARPS; ++w) tot += sh.red[ctid][w];
+                        for (int w = 0; w < RO::COLLECT_WARPS; ++w) tot += sh.red[ctid][w];
                         sh.scale[pb][ctid] = rsqrtf(tot / (float)P.K + 1e-6f);
                     }
-                    ds_collect_sync();
+                    ds_collect_sync<RO::CTHREADS>();
                 }
                 // half a slab of one token (32 groups) per warp and item, NB items in flight
                 constexpr int NB = MT == 1 ? 1 : 2;
                 const int n_items = 2 * n_slots * M;
                 const uint32_t by_m = (65536u + (uint32_t)M - 1) / (uint32_t)M;   // (v * by_m) >> 16 = v / M for v < 64
                 const bool two = (P.in_op == AQ_IN_SILU_MUL), rms = (P.in_op == AQ_IN_RMSNORM);
-                for (int it0 = cwarp; it0 < n_items; it0 += NB * DS_COLLECT_WARPS) {
+                for (int it0 = cwarp; it0 < n_items; it0 += NB * RO::COLLECT_WARPS) {
                     int slot[NB], m[NB], i4[NB];
                     bool on[NB];
 #pragma unroll
                     for (int n = 0; n < NB; ++n) {
-                        const int it = it0 + n * DS_COLLECT_WARPS, v = it >> 1;
+                        const int it = it0 + n * RO::COLLECT_WARPS, v = it >> 1;
                         slot[n] = (int)(((uint32_t)v * by_m) >> 16);
                         m[n] = v - slot[n] * M;
                         i4[n] = 0; on[n] = false;
@@ -930,7 +1004,7 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                     __syncwarp();
 #pragma unroll
                     for (int n = 0; n < NB; ++n) {
-                        if (it0 + n * DS_COLLECT_WARPS >= n_items) break;
+                        if (it0 + n * RO::COLLECT_WARPS >= n_items) break;
                         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (on[n] && ready) {
                             v = P.src ? ds_quad_value(qa[n]) : s[n];
@@ -949,25 +1023,25 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
             }
         }
         fence_async_smem();   // (the tensor core reads the slabs through the asynchronous proxy)
-        if (ds_collect_sync_or(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
+        if (ds_collect_sync_or<RO::CTHREADS>(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
         if (ctid == 0) asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(ds_smem(&sh.xphase)), "r"(ph + 1) : "memory");
 
-        // -- the sums of the phase's units, the two teams taking turns --
+        // -- the sums of the phase's units, the teams taking turns --
         const int total = C.total;
         bool ok = true;
 #pragma unroll 1
         for (int i = 0; i < total && ok; ++i) {
             if (turn == (uint32_t)(cwarp >> 2)) {
-                ok = ds_warp_wait(ds_smem(&sh.stored[stage]), use & 1u, wait_ns, &sh.abort_flag) &&
-                     ds_warp_wait(ds_smem(&sh.done[stage]), use & 1u, wait_ns, &sh.abort_flag);
+                ok = ds_warp_wait(ds_smem(&sh.stored[at.m().at]), at.m().use & 1u, wait_ns, &sh.abort_flag) &&
+                     ds_warp_wait(ds_smem(&sh.done[at.d().at]), at.d().use & 1u, wait_ns, &sh.abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                const uint4 d = sh.sdesc[stage];
+                const uint4 d = sh.sdesc[at.m().at];
                 const int bits = (int)(d.x >> DS_DESC_BITS_SHIFT) & 7;
                 const float* sums = reinterpret_cast<const float*>(sh.xs + d.y + DT_SUMS<MT>);
-                const uint8_t* dmp = &sh.dm[stage][quarter * 2 + (lane >> 4)][(lane & 15) * 16];
+                const uint8_t* dmp = &sh.dm[at.m().at][quarter * 2 + (lane >> 4)][(lane & 15) * 16];
                 const uint4 dm0 = *reinterpret_cast<const uint4*>(dmp), dm1 = *reinterpret_cast<const uint4*>(dmp + DS_FRAGS * SCALE_BYTES);
-                const uint32_t td = tmem + stage * ST::COLS + 2 * DtShape<MT>::A_COLS + ((uint32_t)(quarter * 32) << 16);
+                const uint32_t td = tmem + ST::d_col(at.d().at) + ((uint32_t)(quarter * 32) << 16);
                 float acc[MT];
 #pragma unroll
                 for (int m = 0; m < MT; ++m) acc[m] = 0.f;
@@ -976,19 +1050,20 @@ __global__ void __launch_bounds__(DS_THREADS, 1) decode_stack_kernel(const DsArg
                 else dt_collect<4, MT, BF16>(td, dm0, dm1, sums, acc);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ds_mbar_arrive(ds_smem(&sh.taken[stage]));
+                if (lane == 0) ds_mbar_arrive(ds_smem(&sh.taken[at.d().at]));
                 const DsOp& op = P.ops[d.x & (DS_MAX_PHASE_OPS - 1)];
                 ds_commit<MT>(acc, op.dst, (d.x & DS_DESC_FIRST) ? op.res : nullptr, op.res_plain != 0, (int)d.z * DT_ROWS + quarter * 32 + lane, op.N, M);
             }
-            turn ^= 1u;
-            if (++stage == ST::N) { stage = 0; ++use; }
+            if constexpr (RO::TEAMS == 2) turn ^= 1u;
+            else turn = turn + 1 == RO::TEAMS ? 0u : turn + 1;
+            at.next();
         }
     }
 
     // -- buffers no phase reads (and the last outputs): float32 copies for the caller, one chunk per warp --
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag) == 0) {
 #pragma unroll 1
-        for (int e = (int)blockIdx.x * DS_COLLECT_WARPS + cwarp; e < a.n_tails; e += (int)gridDim.x * DS_COLLECT_WARPS) {
+        for (int e = (int)blockIdx.x * RO::COLLECT_WARPS + cwarp; e < a.n_tails; e += (int)gridDim.x * RO::COLLECT_WARPS) {
             const DsTail T = a.tails[e];
             bool ok = true;
             for (int i = lane * 4; i < T.n && ok; i += 128) {      // n is a multiple of 4
@@ -1281,7 +1356,7 @@ static cudaError_t launch_ds(const DsArgs& a, int grid, cudaStream_t s) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsShared));
             if (e != cudaSuccess) return (int)e;
             int per_sm = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DS_THREADS, sizeof(DsShared));
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DsRoles<MT>::THREADS, sizeof(DsShared));
             if (e != cudaSuccess) return (int)e;
             return per_sm < 1 ? (int)cudaErrorCooperativeLaunchTooLarge : 0;
         });
@@ -1289,7 +1364,7 @@ static cudaError_t launch_ds(const DsArgs& a, int grid, cudaStream_t s) {
     }
     DsArgs args = a;
     void* params[1] = {&args};
-    cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3((unsigned)grid), dim3(DS_THREADS), params,
+    cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3((unsigned)grid), dim3(DsRoles<MT>::THREADS), params,
                                                 sizeof(DsShared), s);
     if (e == cudaSuccess) count_launch();
     return e;

@@ -25,7 +25,8 @@
 // B: a chunk of 8 k is 128 bytes, row = token.  Instruction f = 2 j + h (block j, half h of it) reads chunks 2 f and
 // 2 f + 1; element 2 t + e of chunk 2 f + c is x[32 j + 8 t + 4 h + 2 c + e].  One accumulator of 16 columns per block:
 // columns 0..7 are the tokens' sums of half 0 (the second group of eight B rows is then a region of zeros), 8..15
-// those of half 1 (the first group is); they are joined when they are read.
+// those of half 1 (the first group is); they are joined when they are read.  (Joined by the tensor core, which leaves half the
+// columns to be read, sums come out up to 1.08 times further from 64 bits for normal activations, 1.5 for heavy-tailed ones.)
 //
 // Why tcgen05 with so few tokens: with A in TMEM a 128 x 8 x 32 byte or 128 x 16 x 16 half-word instruction takes 8.4 / 9.6
 // cycles of the tensor pipe (measured), 8.4 / 19 per 4096 weights, against 117 for the same weights as mma.sync, and one
@@ -77,11 +78,28 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, int (&v)[16]) {
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
                    "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(taddr) : "memory");
 }
-
 __device__ __forceinline__ void tmem_ld16f(uint32_t taddr, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]),
                    "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]) : "r"(taddr) : "memory");
+}
+// two binary32 numbers in a register pair, and a multiply-add on both
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
 // K-major without swizzle: core matrices of 8 rows x 16 bytes, `lbo` apart along K, `sbo` apart along the rows.
@@ -226,32 +244,54 @@ __device__ __forceinline__ void dt_collect(uint32_t tmem_d, const uint4& dm0, co
         }
         acc[0] += part[0] + part[1];
     } else {
-        // (joined first: a block enters the running sum with two roundings at its size, not three)
         auto unpos = [](int j) -> float { return BF16 ? 1.f : (float)(1u << (24 - SlotWords<BITS>::pos(j, 1))); };   // a code's power of two
-        float v[2][2 * MT];   // [buffer][half of the block][token]: the next block's sums are on their way meanwhile
-        auto load = [&](int j, float (&b)[2 * MT]) {
-            if constexpr (MT == 2) { tmem_ld2(tmem_d + 16 * j, b); tmem_ld2(tmem_d + 16 * j + 8, b + MT); }
-            else if constexpr (MT == 4) { tmem_ld4(tmem_d + 16 * j, b); tmem_ld4(tmem_d + 16 * j + 8, b + MT); }
-            else tmem_ld16f(tmem_d + 16 * j, b);
+        // BB blocks at a time, [block][half][token]; the next ones' sums are on their way meanwhile
+        constexpr int BB = MT == 8 ? 1 : 2;
+        float v[2][BB * 2 * MT];
+        auto load = [&](int j, float* b) {
+#pragma unroll
+            for (int i = 0; i < BB; ++i) {
+                const uint32_t t = tmem_d + 16 * (j + i);
+                if constexpr (MT == 2) { tmem_ld2(t, b + 4 * i); tmem_ld2(t + 8, b + 4 * i + 2); }
+                else if constexpr (MT == 4) { tmem_ld4(t, b + 8 * i); tmem_ld4(t + 8, b + 8 * i + 4); }
+                else tmem_ld16f(t, b);
+            }
         };
+        f32x2 a[MT / 2];   // token pairs: one multiply-add instruction for two
+#pragma unroll
+        for (int m = 0; m < MT / 2; ++m) a[m] = pair2(acc[2 * m], acc[2 * m + 1]);
         load(0, v[0]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float (&b)[2 * MT] = v[j & 1];
+        for (int j = 0; j < 8; j += BB) {
+            float (&b)[BB * 2 * MT] = v[(j / BB) & 1];
             tmem_ld_wait();
 #pragma unroll
-            for (int m = 0; m < 2 * MT; ++m) asm volatile("" : "+f"(b[m]));
-            if (j + 1 < 8) load(j + 1, v[(j + 1) & 1]);
-            const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
-            const float mp = BF16 ? fmaf(-128.f, p.x, p.y) : p.y;
-            const float d = p.x * unpos(j & 3);   // (exact: a power of two)
+            for (int m = 0; m < BB * 2 * MT; ++m) asm volatile("" : "+f"(b[m]));
+            if (j + BB < 8) load(j + BB, v[(j / BB + 1) & 1]);
 #pragma unroll
-            for (int m = 0; m < MT; m += 2) {
-                const float2 x2 = *reinterpret_cast<const float2*>(sums + 8 * j + m);
-                acc[m] = fmaf(d, b[m] + b[MT + m], fmaf(mp, x2.x, acc[m]));
-                acc[m + 1] = fmaf(d, b[m + 1] + b[MT + m + 1], fmaf(mp, x2.y, acc[m + 1]));
+            for (int i = 0; i < BB; ++i) {
+                const float2 p = __half22float2(*reinterpret_cast<const __half2*>(&w[j + i]));
+                const float mp = BF16 ? fmaf(-128.f, p.x, p.y) : p.y;
+                const float d = p.x * unpos((j + i) & 3);   // (exact: a power of two)
+                const f32x2 m2 = pair2(mp, mp), d2 = pair2(d, d);
+                f32x2 x2[MT / 2];
+                if constexpr (MT == 2) x2[0] = *reinterpret_cast<const f32x2*>(sums + 8 * (j + i));
+                else {
+#pragma unroll
+                    for (int m = 0; m < MT / 2; m += 2) {
+                        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(sums + 8 * (j + i) + 2 * m);
+                        x2[m] = q.x; x2[m + 1] = q.y;
+                    }
+                }
+#pragma unroll
+                for (int m = 0; m < MT / 2; ++m) {   // (joined first: a block enters the running sum with two roundings at its size, not three)
+                    const float* h = b + 2 * MT * i + 2 * m;
+                    a[m] = fma2(d2, add2(pair2(h[0], h[1]), pair2(h[MT], h[MT + 1])), fma2(m2, x2[m], a[m]));
+                }
             }
         }
+#pragma unroll
+        for (int m = 0; m < MT / 2; ++m) unpair2(a[m], acc[2 * m], acc[2 * m + 1]);
     }
 }
 
