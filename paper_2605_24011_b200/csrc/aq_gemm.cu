@@ -34,7 +34,13 @@
 // 18 of a 300M expert at 50 tokens 931 / 678 us, one 11008 x 4096 matrix at 200 tokens
 // 49.2 / 30.8 us (with the zeroing rule at gemm_stores_first and the cast by finalize_kernel).
 //
-// One persistent CTA per SM.  The work -- (row tile, token tile, 128-k slab)
+// Large products run on CTA pairs (tcgen05 cta_group::2, one instruction over 256 rows and up to 256 tokens; each CTA
+// dequantises its 128 rows and holds half of the tokens): half the dequantisation, half the packed bytes and half the
+// operand reads from shared memory per flop.  In an instrumented copy 64 k of a tile (512 cycles of instructions) take 595
+// cycles instead of 880, yet a pass gains 3 to 4 % only: the chip is at its power limit by then (22016 x 4096 at 512 tokens in a
+// loop: 987 W, 1.66 GHz of 1.97; cuBLAS 993 W at 1.34), so it is the energy of dequantising, moving and adding that counts.  Deeper rings (4 to 7 token slots, 4 to 7 epilogue chunks per warp) change nothing.
+//
+// One persistent CTA, or pair, per SM (or two).  The work -- (row tile, token tile, 128-k slab)
 // triples -- is cut into contiguous runs, one per CTA, balanced for slabs plus a
 // fixed cost per piece of a tile; a run that covers a tile's whole K stores its
 // sums, any other run adds them (reduce-add copies; see the store-first protocol
@@ -47,6 +53,7 @@
 // wait is bounded; when one runs out the CTA raises a status word, drains and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <mutex>
@@ -60,34 +67,37 @@
 
 namespace aq {
 
-constexpr int GM_ROWS = 256;       // weight rows per tile: two instructions' worth
+constexpr int GM_ROWS = 256;       // weight rows per tile: two instructions of one CTA, or one instruction of a CTA pair
 constexpr int GM_FRAGS = GM_ROWS / ROWS;
 constexpr int GM_KSTAGE = 64;      // k per stage (one 128-byte swizzle atom of 16-bit elements)
-constexpr int GM_ASTAGES = 4;      // dequantised stages in TMEM
-constexpr int GM_ACOLS = 64;       // TMEM columns of one: [row half][32]
-constexpr int GM_ACOL0 = 256;      // the first of them; D lies below
-constexpr int GM_BSLOTS = 5;       // token ring: up to 128 tokens x 64 k = 16 KB each
+constexpr int GM_ACOL0 = 256;      // first TMEM column of the dequantised stages; D lies below
 constexpr int GM_PSTAGES = 4;      // packed-fragment ring (one k-slab of 128 per slot)
-// Dequantise warps: two groups of eight take the k-slabs in turn, two fragments per warp (with one group of sixteen a slab took
-// as long as one warp's chain of waits).  Both rings have an even number of slots per group, so a group meets every use of the
-// slots it works on (a barrier only tells a phase from the one before it).
-constexpr int GM_DQ_GROUPS = 2, GM_DQ_GROUP = 8;
-constexpr int GM_DQ_WARPS = GM_DQ_GROUPS * GM_DQ_GROUP;
-static_assert(GM_ASTAGES == 2 * GM_DQ_GROUPS && GM_PSTAGES % GM_DQ_GROUPS == 0, "slots belong to groups");
-constexpr int GM_EP_WARPS = 4;
+constexpr int GM_DQ_WARPS = 16, GM_EP_WARPS = 4;
 constexpr int GM_EP0 = GM_DQ_WARPS, GM_TMA = GM_EP0 + GM_EP_WARPS, GM_MMA = GM_TMA + 1, GM_PACKED = GM_MMA + 1;
 constexpr int GM_WARPS = 24;       // (one idle: registers are dealt to groups of four)
 constexpr int GM_THREADS = GM_WARPS * 32;
 // Registers per thread by role, out of the 80 the block is launched with
 constexpr int GM_REGS = 80, GM_REGS_DQ = 72, GM_REGS_EP = 128, GM_REGS_OTHER = 64;
 static_assert(GM_DQ_WARPS * GM_REGS_DQ + GM_EP_WARPS * GM_REGS_EP + 4 * GM_REGS_OTHER <= GM_WARPS * GM_REGS && GM_THREADS * GM_REGS <= 65536, "the roles' registers fit");
-constexpr int GM_MAX_TN = 128;     // tokens per tile (UMMA N)
-constexpr int GM_B_BYTES = GM_MAX_TN * 128;
-constexpr int GM_P_BYTES = GM_FRAGS * frag_bytes(4);   // packed fragments of one slab (largest width)
-constexpr int GM_CHUNKS = 4;       // epilogue chunks per warp
-constexpr int GM_STG_BYTES = GM_EP_WARPS * GM_CHUNKS * 4096;
-constexpr int GM_SMEM = 1024 + GM_BSLOTS * GM_B_BYTES + GM_PSTAGES * GM_P_BYTES + GM_STG_BYTES + 512;
-static_assert(GM_SMEM <= 227 * 1024, "fits an SM");
+
+// What depends on whether a tile belongs to one CTA or to a pair of them.
+template <bool PAIR> struct Tile {
+    static constexpr int FRAGS = PAIR ? GM_FRAGS / 2 : GM_FRAGS;   // 16-row tiles a CTA dequantises
+    static constexpr int MAX_TN = PAIR ? 256 : 128;                // tokens per tile (UMMA N)
+    static constexpr int B_BYTES = 128 * 128;                      // token slot: 128 tokens x 64 k (of a pair each CTA holds half of the tile's tokens)
+    static constexpr int B_SLOTS = PAIR ? 7 : 5;
+    static constexpr int P_BYTES = FRAGS * frag_bytes(4);          // packed fragments of one slab (largest width)
+    // Dequantise warps: groups take the k-slabs in turn, two fragments per warp (with one group of sixteen a slab took as long
+    // as one warp's chain of waits).  Both rings have whole numbers of slots per group, so a group meets every use of the
+    // slots it works on (a barrier only tells a phase from the one before it).
+    static constexpr int DQ_GROUP = FRAGS / 2, DQ_GROUPS = GM_DQ_WARPS / DQ_GROUP;
+    static constexpr int A_STAGES = 2 * DQ_GROUPS;                 // dequantised stages in TMEM
+    static constexpr int A_COLS = FRAGS * 4;                       // TMEM columns of one: [row half][32]
+    static constexpr int CHUNKS = 4;                    // epilogue chunks per warp
+    static constexpr int STG_BYTES = GM_EP_WARPS * CHUNKS * 4096;
+    static constexpr int SMEM = 1024 + B_SLOTS * B_BYTES + GM_PSTAGES * P_BYTES + STG_BYTES + 512;
+    static_assert(GM_PSTAGES % DQ_GROUPS == 0 && GM_ACOL0 + A_STAGES * A_COLS <= 512 && SMEM <= 227 * 1024, "slots belong to groups; fits an SM");
+};
 constexpr uint32_t GM_SPIN_LIMIT = 40u * 1000u * 1000u;
 
 __device__ int g_gemm_status = 0;  // nonzero: a bounded wait ran out (code = which)
@@ -99,7 +109,7 @@ __device__ int g_gemm_status = 0;  // nonzero: a bounded wait ran out (code = wh
 // Flags are never reset: every launch has its own epoch and takes the next of a few arrays.
 constexpr int GM_FLAG_SLOTS = 8;
 constexpr int GM_MAX_TILES = 8192;
-__device__ uint32_t g_tile_flags[GM_FLAG_SLOTS][GM_MAX_TILES][GM_EP_WARPS];
+__device__ uint32_t g_tile_flags[GM_FLAG_SLOTS][GM_MAX_TILES][2 * GM_EP_WARPS];   // (the second half: the odd CTA of a pair)
 static std::atomic<bool> g_gemm_hold{false};   // testing: launches leave their flags down
 
 constexpr int GM_MAX_OPS = 4;      // matrices that share one input (q|k|v, gate|up) run as one launch
@@ -128,7 +138,7 @@ struct GemmArgs {
     uint32_t epoch;
     int hold;              // testing: flags stay down
     const float* tok_scale;    // per token: the power of two its row of x was divided by, or null
-    int bounds[GM_MAX_GRID + 1];   // CTA c works on half slabs [bounds[c], bounds[c + 1]) (even numbers)
+    int bounds[GM_MAX_GRID + 1];   // CTA (or pair) c works on half slabs [bounds[c], bounds[c + 1]) (even numbers)
 };
 
 struct GemmOutMaps { CUtensorMap m[GM_MAX_OPS]; };
@@ -137,12 +147,13 @@ struct GemmOutMaps { CUtensorMap m[GM_MAX_OPS]; };
 struct GemmSeg {
     int op, rt, st, s0, s1;   // rt: row tile inside matrix op
     int tile;                 // index of the tile in the launch
-    int w;                    // its tokens, rounded up to 16
-    int n_rt;                 // its 16-row tiles (1..16)
+    int w;                    // its tokens, rounded up to 16 (a pair: 32)
+    int n_rt;                 // the CTA's 16-row tiles (1..16; of a pair 0..8)
 };
 
 // Tiles are ordered by matrix, row tile, token tile: a CTA that goes on to the next token tile finds the packed rows in L2.
-__device__ __forceinline__ bool gemm_next_seg(int& pos, int hi, const GemmArgs& a, GemmSeg& sg) {
+template <bool PAIR>
+__device__ __forceinline__ bool gemm_next_seg(int& pos, int hi, const GemmArgs& a, int rank, GemmSeg& sg) {
     if (pos >= hi) return false;
     const int c1 = 2 * a.n_slabs;
     const int t = pos / c1, end = min(hi, (t + 1) * c1);
@@ -154,12 +165,19 @@ __device__ __forceinline__ bool gemm_next_seg(int& pos, int hi, const GemmArgs& 
     sg.op = 0;
     while (sg.op + 1 < a.n_ops && r >= a.op[sg.op].R) { r -= a.op[sg.op].R; ++sg.op; }
     sg.rt = r;
-    sg.w = min(a.tn, (a.M - sg.st * a.tn + 15) & ~15);
-    sg.n_rt = min(GM_FRAGS, a.op[sg.op].NT - r * GM_FRAGS);
+    sg.w = min(a.tn, (a.M - sg.st * a.tn + (PAIR ? 31 : 15)) & ~(PAIR ? 31 : 15));
+    sg.n_rt = max(0, min(Tile<PAIR>::FRAGS, a.op[sg.op].NT - r * GM_FRAGS - rank * Tile<PAIR>::FRAGS));
     return true;
 }
 
-// Bounded wait.  Returns false when the limit ran out or another role gave up.
+template <bool PAIR>
+__device__ __forceinline__ void give_up(volatile int* abort_flag, int code) {
+    *abort_flag = 1;
+    if constexpr (PAIR) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32((const void*)abort_flag), cluster_rank() ^ 1u)), "r"(1) : "memory");
+    atomicCAS(&g_gemm_status, 0, code);
+}
+// Bounded wait.  Returns false when the limit ran out or another role (of either CTA of a pair) gave up.
+template <bool PAIR>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code) {
     for (uint32_t i = 0; i < GM_SPIN_LIMIT; ++i) {
         if (mbar_try(bar, parity)) return true;
@@ -168,12 +186,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             if (*abort_flag) return false;
         }
     }
-    *abort_flag = 1;
-    atomicCAS(&g_gemm_status, 0, code);
+    give_up<PAIR>(abort_flag, code);
     return false;
 }
+template <bool PAIR>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, code));
+    return __all_sync(0xffffffffu, mbar_wait<PAIR>(bar, parity, abort_flag, code));
+}
+// Arrive on a barrier of the CTA that issues the instructions: given as a cluster address for a pair, as a local one otherwise.
+template <bool PAIR>
+__device__ __forceinline__ void arrive_issuer(uint32_t bar) {
+    if constexpr (PAIR) mbar_arrive_cluster(bar);
+    else mbar_arrive(bar);
+}
+// Barriers of the CTA, or of both CTAs of the pair, count the instructions issued so far.
+template <bool PAIR>
+__device__ __forceinline__ void commit_all(uint32_t bar) {
+    if constexpr (PAIR) umma_commit_both(bar);
+    else umma_commit(bar);
 }
 
 // Pair (codes 2i, 2i + 1) of block j, row half hi as two dequantised weights.  The codes are OR-ed, where they lie, into the
@@ -192,7 +222,7 @@ __device__ __forceinline__ uint32_t dequant_pair(const InPlace<BITS>& ip, int f,
 // One dequantise warp's share of a k-slab: two neighbouring fragments (32 rows x 128 k) as lanes of two A stages.  n_have of
 // them exist (past the end of the matrix nothing is written: those rows of D are not stored).  Returns false when a wait
 // ran out.
-template <int BITS>
+template <int BITS, bool PAIR>
 __device__ __forceinline__ bool dequant_slab(const uint8_t* frags, int n_have, int lane, uint32_t tmem_a, uint32_t bar_pempty_slot,
                                              uint32_t bar_aempty, uint32_t bar_afull, uint32_t parity, volatile int* abort_flag) {
     const int g = lane >> 2;
@@ -208,7 +238,7 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* frags, int n_have, i
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        if (!mbar_wait_warp(bar_aempty + 8 * h, parity ^ 1, abort_flag, 6)) return false;
+        if (!mbar_wait_warp<PAIR>(bar_aempty + 8 * h, parity ^ 1, abort_flag, 6)) return false;
         tc_fence_after();
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -220,7 +250,7 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* frags, int n_have, i
             for (int f = 0; f < 4; ++f)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) v[4 * f + r] = dequant_pair<BITS>(ip, 4 * h + f, r, dm[r & 1][2 * h + (f >> 1)]);
-            if (i < n_have) tmem_st_16x128(tmem_a + h * GM_ACOLS + ((uint32_t)(i * 16) << 16), v);
+            if (i < n_have) tmem_st_16x128(tmem_a + h * Tile<PAIR>::A_COLS + ((uint32_t)(i * 16) << 16), v);
             else if (h == 1 && i == 0) asm volatile("" ::"r"(v[0]));
         }
         if (h == 1) {
@@ -233,42 +263,55 @@ __device__ __forceinline__ bool dequant_slab(const uint8_t* frags, int n_have, i
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_afull + 8 * h);
+        if (lane == 0) arrive_issuer<PAIR>(bar_afull + 8 * h);
     }
     return true;
 }
 
+template <bool PAIR>
 __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ GemmOutMaps tmap_out, const __grid_constant__ GemmArgs a) {
+    using T = Tile<PAIR>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* sB = smem;
-    uint8_t* sP = sB + GM_BSLOTS * GM_B_BYTES;
-    uint8_t* sC = sP + GM_PSTAGES * GM_P_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sC + GM_STG_BYTES);
-    const uint32_t bar_afull = smem_u32(bars), bar_aempty = bar_afull + 8 * GM_ASTAGES;
-    const uint32_t bar_bfull = bar_aempty + 8 * GM_ASTAGES, bar_bempty = bar_bfull + 8 * GM_BSLOTS;
-    const uint32_t bar_pfull = bar_bempty + 8 * GM_BSLOTS, bar_pempty = bar_pfull + 8 * GM_PSTAGES;
+    uint8_t* sP = sB + T::B_SLOTS * T::B_BYTES;
+    uint8_t* sC = sP + GM_PSTAGES * T::P_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sC + T::STG_BYTES);
+    const uint32_t bar_afull = smem_u32(bars), bar_aempty = bar_afull + 8 * T::A_STAGES;
+    const uint32_t bar_bfull = bar_aempty + 8 * T::A_STAGES, bar_bempty = bar_bfull + 8 * T::B_SLOTS;
+    const uint32_t bar_pfull = bar_bempty + 8 * T::B_SLOTS, bar_pempty = bar_pfull + 8 * GM_PSTAGES;
     const uint32_t bar_dfull = bar_pempty + 8 * GM_PSTAGES, bar_dempty = bar_dfull + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * GM_ASTAGES + 2 * GM_BSLOTS + 2 * GM_PSTAGES + 4);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * T::A_STAGES + 2 * T::B_SLOTS + 2 * GM_PSTAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int n_buf = a.tn <= 64 ? 2 : 1, d_cols = a.tn <= 64 ? 64 : 128;   // sets of accumulators, columns of a row half
+    // Of a pair both CTAs take rows (rank 0 the first 128 of the tile) and half of the tokens; rank 0 issues the instructions,
+    // and its afull, bfull and dempty collect both CTAs' arrivals.
+    const int rank = PAIR ? (int)cluster_rank() : 0, run = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    // sets of accumulators (128 columns each, where two fit), columns of a row half
+    const int n_buf = a.tn <= T::MAX_TN / 2 ? 2 : 1, d_cols = a.tn <= 64 ? 64 : 128;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < GM_ASTAGES; ++s) { mbar_init(bar_afull + 8 * s, GM_DQ_GROUP); mbar_init(bar_aempty + 8 * s, 1); }
-        for (int s = 0; s < GM_BSLOTS; ++s) { mbar_init(bar_bfull + 8 * s, 1); mbar_init(bar_bempty + 8 * s, 1); }
-        for (int s = 0; s < GM_PSTAGES; ++s) { mbar_init(bar_pfull + 8 * s, 1); mbar_init(bar_pempty + 8 * s, GM_DQ_GROUP); }
-        for (int s = 0; s < 2; ++s) { mbar_init(bar_dfull + 8 * s, 1); mbar_init(bar_dempty + 8 * s, GM_EP_WARPS); }
+        constexpr int N = PAIR ? 2 : 1;
+        for (int s = 0; s < T::A_STAGES; ++s) { mbar_init(bar_afull + 8 * s, N * T::DQ_GROUP); mbar_init(bar_aempty + 8 * s, 1); }
+        for (int s = 0; s < T::B_SLOTS; ++s) { mbar_init(bar_bfull + 8 * s, 1); mbar_init(bar_bempty + 8 * s, 1); }
+        for (int s = 0; s < GM_PSTAGES; ++s) { mbar_init(bar_pfull + 8 * s, 1); mbar_init(bar_pempty + 8 * s, T::DQ_GROUP); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_dfull + 8 * s, 1); mbar_init(bar_dempty + 8 * s, N * GM_EP_WARPS); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == GM_TMA) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(512) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(512) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(512) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();   // the partner's barriers exist before anything is counted on them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // The packed weights never change, so their copies and the dequantisation start at once, under the tail of the
@@ -276,40 +319,41 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
     pdl_launch_dependents();
 
     GemmSeg sg;
-    int pos = a.bounds[blockIdx.x];
-    const int run_hi = a.bounds[blockIdx.x + 1];
+    int pos = a.bounds[run];
+    const int run_hi = a.bounds[run + 1];
 
     if (warp < GM_DQ_WARPS) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GM_REGS_DQ));
         // ---------------- dequantise ------------------------------------------------------------------
         // TMEM lanes 32 quarter .. + 31 of row half rh: fragments 8 rh + 2 quarter and the next of the tile
-        const int quarter = warp & 3, rh = (warp >> 2) & 1, group = warp >> 3, ft = 8 * rh + 2 * quarter;
-        const uint32_t tmem_a = tmem_base + GM_ACOL0 + (uint32_t)(group * 2 * GM_ACOLS + rh * 32) + ((uint32_t)(quarter * 32) << 16);
+        const int quarter = warp & 3, rh = PAIR ? 0 : (warp >> 2) & 1, group = warp / T::DQ_GROUP, ft = 8 * rh + 2 * quarter;
+        const uint32_t tmem_a = tmem_base + GM_ACOL0 + (uint32_t)(group * 2 * T::A_COLS + rh * 32) + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t ae = bar_aempty + 16 * group, af = PAIR ? cluster_map(bar_afull + 16 * group, 0) : bar_afull + 16 * group;
         uint32_t n = 0;   // slabs of the run so far
         bool ok = true;
-        while (ok && gemm_next_seg(pos, run_hi, a, sg)) {
+        while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
             const int bits = a.op[sg.op].bits;
             const int n_have = min(2, sg.n_rt - ft);
             for (int s = sg.s0; s < sg.s1 && ok; ++s, ++n) {
-                if ((int)(n & 1) != group) continue;
-                const uint32_t ps = n % GM_PSTAGES, parity = (n / GM_DQ_GROUPS) & 1;   // (of the group's two A stages)
-                ok = mbar_wait_warp(bar_pfull + 8 * ps, (n / GM_PSTAGES) & 1, abort_flag, 5);
+                if ((int)(n % T::DQ_GROUPS) != group) continue;
+                const uint32_t ps = n % GM_PSTAGES, parity = (n / T::DQ_GROUPS) & 1;   // (of the group's two A stages)
+                ok = mbar_wait_warp<PAIR>(bar_pfull + 8 * ps, (n / GM_PSTAGES) & 1, abort_flag, 5);
                 if (!ok) break;
-                const uint8_t* frags = sP + ps * GM_P_BYTES + ft * frag_bytes(bits);
-                const uint32_t ae = bar_aempty + 16 * group, af = bar_afull + 16 * group;
-                if (bits == 2) ok = dequant_slab<2>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
-                else if (bits == 3) ok = dequant_slab<3>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
-                else ok = dequant_slab<4>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
+                const uint8_t* frags = sP + ps * T::P_BYTES + ft * frag_bytes(bits);
+                if (bits == 2) ok = dequant_slab<2, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
+                else if (bits == 3) ok = dequant_slab<3, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
+                else ok = dequant_slab<4, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
             }
         }
     } else if (warp < GM_TMA) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GM_REGS_EP));
         // ---------------- epilogue: TMEM lane quarter (warp & 3) -> out[token][row] -------------------------------
         const int quarter = warp & 3;
-        float* stg = reinterpret_cast<float*>(sC + quarter * GM_CHUNKS * 4096);
+        const uint32_t dempty = PAIR ? cluster_map(bar_dempty, 0) : bar_dempty;
+        float* stg = reinterpret_cast<float*>(sC + quarter * T::CHUNKS * 4096);
         uint32_t segc = 0, n_chunks = 0;
         bool ok = true;
-        while (ok && gemm_next_seg(pos, run_hi, a, sg)) {
+        while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
             const GemmOp& op = a.op[sg.op];
             const uint32_t buf = n_buf == 2 ? (segc & 1u) : 0u, use = n_buf == 2 ? (segc >> 1) : segc;
             ++segc;
@@ -318,10 +362,10 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             bool scaled = false;
             if (a.tok_scale != nullptr) {
 #pragma unroll
-                for (int i = 0; i < GM_MAX_TN / 32; ++i) scaled |= __ldcg(a.tok_scale + min(sg.st * a.tn + 32 * i + lane, a.M - 1)) != 1.f;
+                for (int i = 0; i < T::MAX_TN / 32; ++i) scaled |= __ldcg(a.tok_scale + min(sg.st * a.tn + 32 * i + lane, a.M - 1)) != 1.f;
                 scaled = __any_sync(0xffffffffu, scaled);
             }
-            ok = mbar_wait_warp(bar_dfull + 8 * buf, use & 1, abort_flag, 7);
+            ok = mbar_wait_warp<PAIR>(bar_dfull + 8 * buf, use & 1, abort_flag, 7);
             if (!ok) break;
             tc_fence_after();
             // with a residual the launcher has copied it into out: every run then adds on top of it
@@ -330,14 +374,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             const bool whole = (entire && (op.res == nullptr || !a.tma_out)) || (first_mode && sg.s1 == a.n_slabs);
             const bool raise_flag = first_mode && whole && !entire;
             if (first_mode && !whole) {   // the tile's last-slab run has to have stored before anything is added
-                const uint32_t* fl = &g_tile_flags[a.flag_slot][sg.tile][quarter];
+                const uint32_t* fl = &g_tile_flags[a.flag_slot][sg.tile][rank * GM_EP_WARPS + quarter];
                 uint32_t seen = 0, spins = 0;
                 if (lane == 0) {
                     while ((seen = ld_acquire_u32(fl)) != a.epoch) {
                         if (++spins > (1u << 22) || *abort_flag) break;
                         __nanosleep(100);
                     }
-                    if (seen != a.epoch) { *abort_flag = 1; atomicCAS(&g_gemm_status, 0, 8); }
+                    if (seen != a.epoch) give_up<PAIR>(abort_flag, 8);
                     asm volatile("fence.proxy.async;" ::: "memory");   // (the additions below go through the asynchronous proxy)
                 }
                 seen = __shfl_sync(0xffffffffu, seen, 0);
@@ -346,23 +390,23 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             }
             const bool add_res = (op.res != nullptr && sg.s0 == 0 && !a.tma_out);
             const CUtensorMap* tmo = &tmap_out.m[sg.op];
-            const int tok0 = sg.st * a.tn, halves = sg.n_rt > 8 ? 2 : 1;
+            const int tok0 = sg.st * a.tn, halves = PAIR ? (sg.n_rt > 0 ? 1 : 0) : sg.n_rt > 8 ? 2 : 1;
             const uint32_t td = tmem_base + buf * 128u + ((uint32_t)(quarter * 32) << 16);
             const int n_cc = (sg.w + 31) / 32, n_all = halves * n_cc;
             auto column = [&](int c) -> uint32_t { const int rh = c >= n_cc ? 1 : 0; return td + (uint32_t)(rh * d_cols + (c - rh * n_cc) * 32); };
             auto emit = [&](uint32_t (&v)[32], int c) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) asm volatile("" : "+r"(v[j]));   // (read only after the wait)
-                const int rh = c >= n_cc ? 1 : 0, c0 = (c - rh * n_cc) * 32, n0 = sg.rt * GM_ROWS + rh * 128 + quarter * 32;
+                const int rh = c >= n_cc ? 1 : 0, c0 = (c - rh * n_cc) * 32, n0 = sg.rt * GM_ROWS + (PAIR ? rank : rh) * 128 + quarter * 32;
                 if (scaled) {
                     const float sc = __ldcg(a.tok_scale + min(tok0 + c0 + lane, a.M - 1));
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * __shfl_sync(0xffffffffu, sc, j));
                 }
                 if (a.tma_out) {
-                    if (lane == 0) bulk_wait_read<GM_CHUNKS - 1>();   // the copy that last read this chunk has left shared memory
+                    if (lane == 0) bulk_wait_read<T::CHUNKS - 1>();   // the copy that last read this chunk has left shared memory
                     __syncwarp();
-                    float* chunk = stg + (n_chunks++ % GM_CHUNKS) * 1024;      // [32 tokens][32 rows]
+                    float* chunk = stg + (n_chunks++ % T::CHUNKS) * 1024;      // [32 tokens][32 rows]
 #pragma unroll
                     for (int j = 0; j < 32; ++j) chunk[j * 32 + lane] = __uint_as_float(v[j]);
                     fence_async_smem();
@@ -398,7 +442,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             };
             // two register sets: the TMEM load of the next 32 columns is in flight while this one is staged
             uint32_t va[32], vb[32];
-            tmem_ld32(column(0), va);
+            if (n_all > 0) tmem_ld32(column(0), va);
             for (int c = 0; c < n_all; c += 2) {
                 tmem_ld_wait();
                 if (c + 1 < n_all) tmem_ld32(column(c + 1), vb);
@@ -411,12 +455,12 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_dempty + 8 * buf);   // the next instructions may overwrite the accumulators
+            if (lane == 0) arrive_issuer<PAIR>(dempty + 8 * buf);   // the next instructions may overwrite the accumulators
             if (raise_flag) {
                 if (lane == 0) {
                     bulk_wait_all<0>();   // this warp's stores must have landed before its flag goes up
                     asm volatile("fence.proxy.async;" ::: "memory");
-                    if (!a.hold) st_release_u32(&g_tile_flags[a.flag_slot][sg.tile][quarter], a.epoch);
+                    if (!a.hold) st_release_u32(&g_tile_flags[a.flag_slot][sg.tile][rank * GM_EP_WARPS + quarter], a.epoch);
                 }
                 __syncwarp();
             }
@@ -430,14 +474,16 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
         if (lane == 0) {
             uint32_t bi = 0;
             bool ok = true;
+            const uint32_t bfull = PAIR ? cluster_map(bar_bfull, 0) : bar_bfull;
             pdl_wait();   // x is the predecessor's output
-            while (ok && gemm_next_seg(pos, run_hi, a, sg)) {
+            while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
                 for (int it = 2 * sg.s0; it < 2 * sg.s1 && ok; ++it) {
-                    const uint32_t bs = bi % GM_BSLOTS;
-                    ok = mbar_wait(bar_bempty + 8 * bs, ((bi / GM_BSLOTS) & 1) ^ 1, abort_flag, 2);
+                    const uint32_t bs = bi % T::B_SLOTS;
+                    ok = mbar_wait<PAIR>(bar_bempty + 8 * bs, ((bi / T::B_SLOTS) & 1) ^ 1, abort_flag, 2);
                     if (!ok) break;
-                    mbar_expect_tx(bar_bfull + 8 * bs, (uint32_t)(a.tn * 128));
-                    tma_load_2d(smem_u32(sB + bs * GM_B_BYTES), &tmap_x, it * GM_KSTAGE, sg.st * a.tn, bar_bfull + 8 * bs);
+                    if (rank == 0) mbar_expect_tx(bar_bfull + 8 * bs, (uint32_t)(a.tn * 128));
+                    if constexpr (PAIR) tma_load_2d_pair(smem_u32(sB + bs * T::B_BYTES), &tmap_x, it * GM_KSTAGE, sg.st * a.tn + rank * (sg.w / 2), bfull + 8 * bs);
+                    else tma_load_2d(smem_u32(sB + bs * T::B_BYTES), &tmap_x, it * GM_KSTAGE, sg.st * a.tn, bfull + 8 * bs);
                     ++bi;
                 }
             }
@@ -448,15 +494,15 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
         if (lane == 0) {
             uint32_t pi = 0;
             bool ok = true;
-            while (ok && gemm_next_seg(pos, run_hi, a, sg)) {
+            while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
                 const GemmOp& op = a.op[sg.op];
                 const int FB = frag_bytes(op.bits);
                 for (int s = sg.s0; s < sg.s1; ++s) {
                     const uint32_t ps = pi % GM_PSTAGES;
-                    ok = mbar_wait(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
+                    ok = mbar_wait<PAIR>(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
                     if (!ok) break;
                     mbar_expect_tx(bar_pfull + 8 * ps, (uint32_t)(sg.n_rt * FB));
-                    bulk_load(smem_u32(sP + ps * GM_P_BYTES), op.frags + frag_index(s, sg.rt * GM_FRAGS, op.NT) * FB, (uint32_t)(sg.n_rt * FB), bar_pfull + 8 * ps);
+                    if (sg.n_rt > 0) bulk_load(smem_u32(sP + ps * T::P_BYTES), op.frags + frag_index(s, sg.rt * GM_FRAGS + rank * T::FRAGS, op.NT) * FB, (uint32_t)(sg.n_rt * FB), bar_pfull + 8 * ps);
                     ++pi;
                 }
             }
@@ -465,33 +511,34 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
     } else if (warp == GM_MMA) {
         // ---------------- MMA issue ----------------------------------------------------------------
         uint32_t ai = 0, bi = 0, segc = 0;
-        bool ok = true;
-        while (ok && gemm_next_seg(pos, run_hi, a, sg)) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(sg.w >> 3) << 17) | (8u << 24);   // f16 x f16 -> f32, 128 x w
+        bool ok = rank == 0;
+        while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(sg.w >> 3) << 17) | ((PAIR ? 16u : 8u) << 24);   // f16 x f16 -> f32, 128 (a pair: 256) x w
             const uint32_t buf = n_buf == 2 ? (segc & 1u) : 0u, use = n_buf == 2 ? (segc >> 1) : segc;
             ++segc;
-            ok = mbar_wait_warp(bar_dempty + 8 * buf, (use & 1) ^ 1, abort_flag, 9);
+            ok = mbar_wait_warp<PAIR>(bar_dempty + 8 * buf, (use & 1) ^ 1, abort_flag, 9);
             if (!ok) break;
             tc_fence_after();
             const uint32_t td = __shfl_sync(0xffffffffu, tmem_base + buf * 128u, 0);
             const bool both = sg.n_rt > 8;
             for (int it = 2 * sg.s0; it < 2 * sg.s1 && ok; ++it) {
-                const uint32_t as = ai % GM_ASTAGES, bs = bi % GM_BSLOTS;
-                ok = mbar_wait_warp(bar_afull + 8 * as, (ai / GM_ASTAGES) & 1, abort_flag, 3) && mbar_wait_warp(bar_bfull + 8 * bs, (bi / GM_BSLOTS) & 1, abort_flag, 4);
+                const uint32_t as = ai % T::A_STAGES, bs = bi % T::B_SLOTS;
+                ok = mbar_wait_warp<PAIR>(bar_afull + 8 * as, (ai / T::A_STAGES) & 1, abort_flag, 3) && mbar_wait_warp<PAIR>(bar_bfull + 8 * bs, (bi / T::B_SLOTS) & 1, abort_flag, 4);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t bd = make_smem_desc(__shfl_sync(0xffffffffu, smem_u32(sB) + bs * GM_B_BYTES, 0));
-                const uint32_t ta = __shfl_sync(0xffffffffu, tmem_base + GM_ACOL0 + as * GM_ACOLS, 0);
+                const uint64_t bd = make_smem_desc(__shfl_sync(0xffffffffu, smem_u32(sB) + bs * T::B_BYTES, 0));
+                const uint32_t ta = __shfl_sync(0xffffffffu, tmem_base + GM_ACOL0 + as * T::A_COLS, 0);
                 const uint32_t more = it > 2 * sg.s0 ? 1u : 0u;
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < GM_KSTAGE / 16; ++k) {
-                        umma_f16_ts(td, ta + 8 * k, bd + 2 * k, idesc, k > 0 ? 1u : more);
-                        if (both) umma_f16_ts(td + d_cols, ta + 32 + 8 * k, bd + 2 * k, idesc, k > 0 ? 1u : more);
+                        if constexpr (PAIR) umma_f16_ts_pair(td, ta + 8 * k, bd + 2 * k, idesc, k > 0 ? 1u : more);
+                        else umma_f16_ts(td, ta + 8 * k, bd + 2 * k, idesc, k > 0 ? 1u : more);
+                        if (!PAIR && both) umma_f16_ts(td + d_cols, ta + 32 + 8 * k, bd + 2 * k, idesc, k > 0 ? 1u : more);
                     }
-                    umma_commit(bar_bempty + 8 * bs);
-                    umma_commit(bar_aempty + 8 * as);
-                    if (it + 1 == 2 * sg.s1) umma_commit(bar_dfull + 8 * buf);
+                    commit_all<PAIR>(bar_bempty + 8 * bs);
+                    commit_all<PAIR>(bar_aempty + 8 * as);
+                    if (it + 1 == 2 * sg.s1) commit_all<PAIR>(bar_dfull + 8 * buf);
                 }
                 __syncwarp();
                 ++ai; ++bi;
@@ -502,9 +549,12 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) __nanosleep(200000);   // let copies in flight land before the CTA's shared memory goes away
+    __syncwarp();
+    if constexpr (PAIR) cluster_sync_all();  // neither CTA leaves, or frees its TMEM, while the other's barriers, copies or instructions reach into it
     if (warp == GM_TMA) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(512) : "memory");
+        if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(512) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(512) : "memory");
     }
 }
 
@@ -521,36 +571,71 @@ EncodeTiledFn tensor_map_encoder() {
     return fn;
 }
 
-static cudaError_t launch_one(const CUtensorMap& tm, const GemmOutMaps& tmo, const GemmArgs& a, int grid, cudaStream_t s) {
-    auto kern = gemm_kernel;
+template <bool PAIR>
+static cudaError_t launch_one(const CUtensorMap& tm, const GemmOutMaps& tmo, const GemmArgs& a, int workers, cudaStream_t s) {
+    auto kern = gemm_kernel<PAIR>;
     static PerDeviceOnce configured;
     {
         const int rc = configured.run(current_device(), [&] {
-            return (int)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GM_SMEM);
+            return (int)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<PAIR>::SMEM);
         });
         if (rc != 0) return rc < 0 ? cudaErrorInvalidDevice : (cudaError_t)rc;
     }
-    cudaError_t e = launch_pdl(kern, dim3((unsigned)grid), dim3(GM_THREADS), GM_SMEM, s, tm, tmo, a);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(PAIR ? 2 * workers : workers)); cfg.blockDim = dim3(GM_THREADS); cfg.dynamicSmemBytes = Tile<PAIR>::SMEM; cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = PAIR ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tm, tmo, a);
     count_launch();
     return e;
 }
 
-// Token tiles of one width (a multiple of 16, at most GM_MAX_TN).
-static int token_tiles(int M) { return (M + GM_MAX_TN - 1) / GM_MAX_TN; }
+// How a launch for M tokens is cut: CTAs or pairs of them, token tiles of one width.
+struct GemmShape {
+    bool pair;
+    int n_st, tn;   // token tiles, tokens per tile
+    int workers;    // CTAs or pairs that the device holds
+};
+static GemmShape gemm_shape(const aq_handle_s* const* hs, int n, int M) {
+    GemmShape g;
+    const int sms = std::min(sm_count(), GM_MAX_GRID);
+    // Pairs dequantise a weight, and read it from L2, once per 256 tokens instead of 128, but fill and drain tiles of twice the
+    // size, and a tile costs them nearly the same whatever it holds: they pay where the tokens fill tiles of 256 (an even number of
+    // 128s, at least four) and a pair has about 48 stages (256 rows x 256 tokens x 64 k) of work.  Measured, us with single
+    // CTAs / pairs, 3 bits: 22016 x 4096 at 256 tokens 47.3 / 46.8, 257 57.9 / 68.5, 384 66.0 / 72.4, 448 82.4 / 75.3, 512 85.7 /
+    // 79.7, 640 103.5 / 104.5, 768 124.6 / 114.1; 32768 x 2048 at 512 71.7 / 69.1, 768 105.7 / 99.1; 4096 x 11008 at 256 30.5 /
+    // 31.3, 512 47.8 / 46.8; 4096 x 4096 at 512 (28 stages) 26.1 / 26.8, at 1024 (55) 43.8 / 37.7.
+    long long R = 0;
+    for (int i = 0; i < n; ++i) R += (hs[i]->NT + GM_FRAGS - 1) / GM_FRAGS;
+    const int t128 = (M + 127) / 128;
+    g.pair = t128 >= 4 && t128 % 2 == 0 && sms >= 2 && R * (t128 / 2) * hs[0]->KP * 4 >= 48LL * (sms / 2);
+    g.workers = g.pair ? sms / 2 : sms;
+    const int max_tn = g.pair ? Tile<true>::MAX_TN : Tile<false>::MAX_TN;
+    g.n_st = (M + max_tn - 1) / max_tn;
+    // (several tiles: a multiple of 32, the width of the epilogue's copies, which must not reach into the next tile; a pair's
+    // instruction takes multiples of 32)
+    g.tn = g.pair || g.n_st > 1 ? ((M + g.n_st - 1) / g.n_st + 31) / 32 * 32 : (M + 15) / 16 * 16;
+    return g;
+}
 
 // cut_runs for tiles of c1 units, remembered: finding the runs takes the host about 10 us, a stack asks for the same few
 // partitions again and again.
-static void cached_runs(long long total, long long c1, int grid, int* bounds) {
-    struct Entry { long long total, c1; int grid; int bounds[GM_MAX_GRID + 1]; };
+static void cached_runs(long long total, long long c1, int grid, int seg_cost, int* bounds) {
+    struct Entry { long long total, c1; int grid, seg_cost; int bounds[GM_MAX_GRID + 1]; };
     static std::mutex m;
     static std::vector<Entry> entries;   // (at most 64: the oldest makes room)
     std::lock_guard<std::mutex> lock(m);
     for (const Entry& e : entries)
-        if (e.total == total && e.c1 == c1 && e.grid == grid) { memcpy(bounds, e.bounds, sizeof(e.bounds)); return; }
+        if (e.total == total && e.c1 == c1 && e.grid == grid && e.seg_cost == seg_cost) { memcpy(bounds, e.bounds, sizeof(e.bounds)); return; }
     Entry e;
     memset(&e, 0, sizeof(e));
-    e.total = total; e.c1 = c1; e.grid = grid;
-    cut_runs(total, c1, grid, e.bounds);
+    e.total = total; e.c1 = c1; e.grid = grid; e.seg_cost = seg_cost;
+    cut_runs(total, c1, grid, e.bounds, seg_cost);
     memcpy(bounds, e.bounds, sizeof(e.bounds));
     if (entries.size() >= 64) entries.erase(entries.begin());
     entries.push_back(e);
@@ -574,18 +659,17 @@ cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x
         o.N = (int)hs[i]->N; o.NT = hs[i]->NT; o.R = (hs[i]->NT + GM_FRAGS - 1) / GM_FRAGS; o.bits = hs[i]->bits;
         rows += o.R;
     }
-    a.n_st = token_tiles(M);
-    // (several tiles: a multiple of 32, the width of the epilogue's copies, which must not reach into the next tile)
-    a.tn = a.n_st > 1 ? ((M + a.n_st - 1) / a.n_st + 31) / 32 * 32 : (M + 15) / 16 * 16;
+    const GemmShape shape = gemm_shape(hs, n, M);
+    a.n_st = shape.n_st; a.tn = shape.tn;
     const long long tiles = rows * a.n_st, total = tiles * 2 * a.n_slabs;   // in half slabs
-    int grid = sm_count() < GM_MAX_GRID ? sm_count() : GM_MAX_GRID;
+    int grid = shape.workers;
     if (total / 2 < grid) grid = (int)(total / 2);
     if (total > 0x7fffffffLL) return cudaErrorInvalidValue;
-    cached_runs(total, 2LL * a.n_slabs, grid, a.bounds);
+    cached_runs(total, 2LL * a.n_slabs, grid, shape.pair ? GM_PAIR_SEG_COST : GM_SEG_COST, a.bounds);
     CUtensorMap tm;
     const cuuint64_t dims[2] = {(cuuint64_t)hs[0]->K, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)hs[0]->K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)GM_KSTAGE, (cuuint32_t)a.tn};
+    const cuuint32_t box[2] = {(cuuint32_t)GM_KSTAGE, (cuuint32_t)(shape.pair ? a.tn / 2 : a.tn)};
     const cuuint32_t estr[2] = {1, 1};
     const CUresult r = enc(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x16), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -630,7 +714,7 @@ cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x
             e = cudaMemset2DAsync(o.out, (size_t)o.ldo * sizeof(float), 0, (size_t)o.N * sizeof(float), (size_t)M, s);
         if (e != cudaSuccess) return e;
     }
-    return launch_one(tm, tmo, a, grid, s);
+    return shape.pair ? launch_one<true>(tm, tmo, a, grid, s) : launch_one<false>(tm, tmo, a, grid, s);
 }
 
 cudaError_t launch_gemm(const aq_handle_s* h, const void* x16, const float* tok_scale, int M, float* out, int64_t ldo, bool out_ready, cudaStream_t s) {
@@ -719,8 +803,9 @@ bool gemm_stores_first(const aq_handle_s* const* hs, int n, int M, cudaStream_t 
     // zeros: 4096 x 4096 (16 tiles) at 32 tokens 18.5 / 15.2 us, 11008 x 4096 (86 tiles) at 200 tokens 46 / 42 us, eight 7B
     // layers (48 and 86 tiles) at 50 tokens 814 / 739 us; the other way round with 104 to 148 tiles, 18 expert layers at 512
     // tokens 1291 / 1381 us.
-    const long long tiles = R * token_tiles(M);
-    return tiles <= GM_MAX_TILES && 10 * tiles >= 7 * sm_count();
+    const GemmShape shape = gemm_shape(hs, n, M);
+    const long long tiles = R * shape.n_st;
+    return tiles <= GM_MAX_TILES && 10 * tiles >= 7 * shape.workers;
 }
 
 // True when launch_gemm_group accepts outputs preset by the caller (they are written through tensor maps).

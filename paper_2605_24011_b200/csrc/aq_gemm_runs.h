@@ -11,20 +11,23 @@ constexpr int GM_MAX_GRID = 192;   // CTAs of one launch (one per SM)
 // takes 1.03 to 1.04 of the time, 2 1.01 to 1.04, 3 1.00 to 1.02, 4 to 14 0.99 to 1.015; eight 7B layers at 200 tokens 1191,
 // 1156, 1139, 1136, 1133 (6), 1131 (9), 1135 us (14).
 constexpr int GM_SEG_COST = 9;
+// The same for a CTA pair, whose tiles are twice as wide: of 5, 9 and 15, in us, 4096 x 4096 at 1024 tokens 41.0, 42.1, 37.7,
+// 11008 x 4096 at 512 48.9, 46.1, 46.1, 12288 x 4096 52.9, 49.9, 49.8, 22016 x 4096 79.2, 79.1, 79.2.
+constexpr int GM_PAIR_SEG_COST = 15;
 
 // Cuts [0, total) into `grid` contiguous runs with even bounds (bounds[0] = 0 .. bounds[grid] = total).  The work is a
-// sequence of tiles of c1 units each.  A run costs its units plus GM_SEG_COST per tile it touches; the smallest budget under
+// sequence of tiles of c1 units each.  A run costs its units plus seg_cost per tile it touches; the smallest budget under
 // which a greedy walk places everything is found by bisection.
-inline void cut_runs(long long total, long long c1, int grid, int* bounds) {
+inline void cut_runs(long long total, long long c1, int grid, int* bounds, int seg_cost = GM_SEG_COST) {
     auto walk = [&](long long budget, int* out) {
         long long pos = 0;
         for (int c = 0; c < grid; ++c) {
             if (out) out[c] = (int)pos;
             long long left = budget;
             while (pos < total) {
-                const long long te = (pos / c1 + 1) * c1, need = GM_SEG_COST + (te - pos);
+                const long long te = (pos / c1 + 1) * c1, need = seg_cost + (te - pos);
                 if (need <= left) { pos = te; left -= need; continue; }
-                const long long take = (left - GM_SEG_COST) & ~1LL;
+                const long long take = (left - seg_cost) & ~1LL;
                 if (take >= 2) pos += take;
                 break;
             }
@@ -32,7 +35,7 @@ inline void cut_runs(long long total, long long c1, int grid, int* bounds) {
         if (out) out[grid] = (int)total;
         return pos >= total;
     };
-    long long lo = total / grid, hi = total / grid + 4 * GM_SEG_COST + 4;
+    long long lo = total / grid, hi = total / grid + 4 * seg_cost + 4;
     while (!walk(hi, nullptr)) hi *= 2;
     while (lo < hi) {
         const long long mid = (lo + hi) / 2;
