@@ -736,30 +736,39 @@ __global__ void __launch_bounds__(256) operand_rows_kernel(const uint16_t* __res
     const uint16_t* xr = x + m * K;
     __half* o = x16 + m * K;
     pdl_launch_dependents();
-    for (int64_t i = threadIdx.x; i < zero4; i += 256) zero[m * zero4 + i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto put = [&](int64_t k, const uint4& r) {   // eight consecutive elements from k
-        const uint2 lo = make_uint2(r.x, r.y), hi = make_uint2(r.z, r.w);
-        store_operand4(o, k, lo);
-        store_operand4(o, k + 4, hi);
-    };
-    if constexpr (!BF16) {
-        for (int64_t k = threadIdx.x * 8; k < K; k += 256 * 8) put(k, *reinterpret_cast<const uint4*>(xr + k));
-    } else {
-        auto convert = [&](int64_t k, float f, float& mx) {
-            const uint4 v = *reinterpret_cast<const uint4*>(xr + k);
-            const __nv_bfloat162* b = reinterpret_cast<const __nv_bfloat162*>(&v);
-            uint4 r;
-            __half2* h = reinterpret_cast<__half2*>(&r);
+    const int q8 = (int)(K >> 3), wid = (int)threadIdx.x & ~31;   // groups of eight elements (K is a multiple of 32); the warp's first thread
+    float mx = 0.f;
+    auto convert = [&](uint4& v, float f, bool on) {   // bfloat16 -> binary16, times f
+        uint32_t* w = reinterpret_cast<uint32_t*>(&v);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 p = __bfloat1622float2(b[i]);
-                h[i] = __floats2half2_rn(p.x * f, p.y * f);
-                mx = fmaxf(mx, fmaxf(fabsf(p.x), fabsf(p.y)));
+        for (int i = 0; i < 4; ++i) {
+            const float2 p = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(w + i));
+            const __half2 h = __floats2half2_rn(p.x * f, p.y * f);
+            w[i] = *reinterpret_cast<const uint32_t*>(&h);
+            if (on) mx = fmaxf(mx, fmaxf(fabsf(p.x), fabsf(p.y)));
+        }
+    };
+    auto rows = [&](float f) {
+        constexpr int STEPS = 4;   // groups per thread whose loads go out together
+        for (int i0 = 0; i0 + wid < q8; i0 += 256 * STEPS) {
+            uint4 v[STEPS];
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                v[n] = i < q8 ? *reinterpret_cast<const uint4*>(xr + 8 * (int64_t)i) : make_uint4(0u, 0u, 0u, 0u);
             }
-            put(k, r);
-        };
-        float mx = 0.f;
-        for (int64_t k = threadIdx.x * 8; k < K; k += 256 * 8) convert(k, 1.f, mx);   // K is a multiple of 32
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                if (i0 + 256 * n + wid >= q8) break;
+                if constexpr (BF16) convert(v[n], f, i < q8);
+                store_operand8(o, 8 * (int64_t)i, v[n], i < q8);
+            }
+        }
+    };
+    rows(1.f);
+    for (int64_t i = threadIdx.x; i < zero4; i += 256) zero[m * zero4 + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (BF16) {
         __shared__ float red[8];
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
@@ -773,8 +782,7 @@ __global__ void __launch_bounds__(256) operand_rows_kernel(const uint16_t* __res
             int e;
             frexpf(mx, &e);                       // mx = f 2^e, f in [0.5, 1)
             sc = ldexpf(1.f, e - 15);             // mx / sc in [2^14, 2^15)
-            float unused = 0.f;
-            for (int64_t k = threadIdx.x * 8; k < K; k += 256 * 8) convert(k, 1.f / sc, unused);
+            rows(1.f / sc);
         }
         if (threadIdx.x == 0) scale[m] = sc;
     }

@@ -220,68 +220,114 @@ __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __res
     const float4* t4 = src2 ? reinterpret_cast<const float4*>(src2 + m * K) : nullptr;
     __nv_bfloat16* xr = x + m * K;
     __half* hr = x16 + m * K;
-    const int64_t q4 = K >> 2;
+    const int q8 = (int)(K >> 3), wid = (int)threadIdx.x & ~31;   // groups of eight elements; the warp's first thread
     __shared__ float red[8];
-    float rms = 1.f;
-    if (in_op == AQ_IN_RMSNORM) {
-        float ss = 0.f;
-        for (int64_t k = threadIdx.x; k < q4; k += 256) {
-            const float4 v = s4[k];
-            ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
-        }
+    auto all = [&](float v, auto op) {   // op over the CTA
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+        for (int d = 16; d > 0; d >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, d));
         __syncthreads();
-        float tot = 0.f;
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+        __syncthreads();
+        v = red[0];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tot += red[i];
-        rms = rsqrtf(tot / (float)K + 1e-6f);
-        __syncthreads();
-    }
+        for (int i = 1; i < 8; ++i) v = op(v, red[i]);
+        return v;
+    };
     // the rounded vector, its binary16 copy as if no scaling were needed, and the row's largest magnitude
     float mx = 0.f;
-    for (int64_t k = threadIdx.x; k < q4; k += 256) {
-        float4 v = s4[k];
-        if (in_op == AQ_IN_SILU_MUL) {
-            const float4 u = t4[k];
+    auto emit = [&](int i, bool on, const float4& a, const float4& b) {
+        const __nv_bfloat162 p[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w), __floats2bfloat162_rn(b.x, b.y), __floats2bfloat162_rn(b.z, b.w)};
+        uint32_t r[4], h[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            r[e] = *reinterpret_cast<const uint32_t*>(&p[e]);
+            const float2 f = __bfloat1622float2(p[e]);
+            const __half2 w = __floats2half2_rn(f.x, f.y);
+            h[e] = *reinterpret_cast<const uint32_t*>(&w);
+            if (on) mx = fmaxf(mx, fmaxf(fabsf(f.x), fabsf(f.y)));
+        }
+        if (on) *reinterpret_cast<uint4*>(xr + 8 * (int64_t)i) = make_uint4(r[0], r[1], r[2], r[3]);
+        store_operand8(hr, 8 * (int64_t)i, make_uint4(h[0], h[1], h[2], h[3]), on);
+    };
+    // STEPS groups per thread at a time: their loads go out together
+    constexpr int STEPS = 2;
+    if (in_op == AQ_IN_RMSNORM) {
+        auto squares = [](const float4& v, float ss) { return fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, ss)))); };
+        auto scaled = [](const float4& v, float f) { return make_float4(v.x * f, v.y * f, v.z * f, v.w * f); };
+        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 a[STEPS], b[STEPS];   // rows of up to STEPS groups per thread stay in registers
+        float ss = 0.f;
+        for (int i0 = 0; i0 < q8; i0 += 256 * STEPS) {
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                a[n] = b[n] = none;
+                if (i < q8) { a[n] = s4[2 * i]; b[n] = s4[2 * i + 1]; }
+            }
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) ss = squares(b[n], squares(a[n], ss));
+        }
+        const float rms = rsqrtf(all(ss, [](float u, float v) { return u + v; }) / (float)K + 1e-6f);
+        for (int i0 = 0; i0 + wid < q8; i0 += 256 * STEPS) {
+            if (q8 > 256 * STEPS) {
+#pragma unroll
+                for (int n = 0; n < STEPS; ++n) {
+                    const int i = i0 + 256 * n + (int)threadIdx.x;
+                    if (i < q8) { a[n] = s4[2 * i]; b[n] = s4[2 * i + 1]; }
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                if (i0 + 256 * n + wid < q8) emit(i, i < q8, scaled(a[n], rms), scaled(b[n], rms));
+            }
+        }
+    } else {
+        const bool two = in_op == AQ_IN_SILU_MUL;
+        auto gated = [](float4 v, const float4& u) {
             v.x = v.x / (1.f + expf(-v.x)) * u.x; v.y = v.y / (1.f + expf(-v.y)) * u.y;
             v.z = v.z / (1.f + expf(-v.z)) * u.z; v.w = v.w / (1.f + expf(-v.w)) * u.w;
-        } else {
-            v.x *= rms; v.y *= rms; v.z *= rms; v.w *= rms;
+            return v;
+        };
+        for (int i0 = 0; i0 + wid < q8; i0 += 256 * STEPS) {
+            float4 a[STEPS], b[STEPS], c[STEPS], d[STEPS];
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                a[n] = b[n] = c[n] = d[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < q8) {
+                    a[n] = s4[2 * i]; b[n] = s4[2 * i + 1];
+                    if (two) { c[n] = t4[2 * i]; d[n] = t4[2 * i + 1]; }
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < STEPS; ++n) {
+                const int i = i0 + 256 * n + (int)threadIdx.x;
+                if (i0 + 256 * n + wid >= q8) break;
+                if (two) { a[n] = gated(a[n], c[n]); b[n] = gated(b[n], d[n]); }
+                emit(i, i < q8, a[n], b[n]);
+            }
         }
-        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-        uint2 r;
-        r.x = *reinterpret_cast<const uint32_t*>(&a); r.y = *reinterpret_cast<const uint32_t*>(&b);
-        *reinterpret_cast<uint2*>(xr + 4 * k) = r;
-        const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-        const __half2 ha = __floats2half2_rn(fa.x, fa.y), hb = __floats2half2_rn(fb.x, fb.y);
-        uint2 h;
-        h.x = *reinterpret_cast<const uint32_t*>(&ha); h.y = *reinterpret_cast<const uint32_t*>(&hb);
-        store_operand4(hr, 4 * k, h);
-        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(fa.x), fabsf(fa.y)), fmaxf(fabsf(fb.x), fabsf(fb.y))));
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();   // (also: this CTA's writes of x are visible to its own threads below)
-    mx = red[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) mx = fmaxf(mx, red[i]);
+    mx = all(mx, [](float u, float v) { return fmaxf(u, v); });
     float sc = 1.f;
     if (mx >= 32768.f && mx <= 3.0e38f) {
         int e;
         frexpf(mx, &e);
         sc = ldexpf(1.f, e - 15);
         const float inv = 1.f / sc;
-        for (int64_t k = threadIdx.x; k < q4; k += 256) {
-            const uint2 r = *reinterpret_cast<const uint2*>(xr + 4 * k);
-            const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.x));
-            const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.y));
-            const __half2 ha = __floats2half2_rn(fa.x * inv, fa.y * inv), hb = __floats2half2_rn(fb.x * inv, fb.y * inv);
-            uint2 h;
-            h.x = *reinterpret_cast<const uint32_t*>(&ha); h.y = *reinterpret_cast<const uint32_t*>(&hb);
-            store_operand4(hr, 4 * k, h);
+        for (int i0 = 0; i0 + wid < q8; i0 += 256) {
+            const int i = i0 + (int)threadIdx.x;
+            uint4 r = make_uint4(0u, 0u, 0u, 0u);
+            if (i < q8) r = *reinterpret_cast<const uint4*>(xr + 8 * (int64_t)i);   // (what this thread wrote)
+            uint32_t h[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[n]));
+                const __half2 w = __floats2half2_rn(f.x * inv, f.y * inv);
+                h[n] = *reinterpret_cast<const uint32_t*>(&w);
+            }
+            store_operand8(hr, 8 * (int64_t)i, make_uint4(h[0], h[1], h[2], h[3]), i < q8);
         }
     }
     if (threadIdx.x == 0) scale[m] = sc;

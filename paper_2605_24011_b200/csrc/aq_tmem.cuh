@@ -20,6 +20,22 @@ __device__ __forceinline__ void store_operand4(__half* row, int64_t k, const uin
     p[0] = v.x;
     p[4] = v.y;
 }
+// Eight consecutive elements per lane, from k (a multiple of 8) where on; lanes 4 i .. 4 i + 3 hold a block of 32 and are on
+// together; all lanes of the warp take part.  A lane's four pairs belong 16 bytes apart: the four lanes transpose them, and
+// each stores 16 bytes in one piece (as 4-byte stores they were twice the number of partly written sectors).
+__device__ __forceinline__ void store_operand8(__half* row, int64_t k, uint4 v, bool on) {
+    const bool odd = threadIdx.x & 1, up = threadIdx.x & 2;
+    uint32_t s0 = odd ? v.x : v.y, s1 = odd ? v.z : v.w;
+    s0 = __shfl_xor_sync(0xffffffffu, s0, 1);
+    s1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+    if (odd) { v.x = s0; v.z = s1; } else { v.y = s0; v.w = s1; }
+    s0 = up ? v.x : v.z; s1 = up ? v.y : v.w;
+    s0 = __shfl_xor_sync(0xffffffffu, s0, 2);
+    s1 = __shfl_xor_sync(0xffffffffu, s1, 2);
+    if (up) { v.x = s0; v.y = s1; } else { v.z = s0; v.w = s1; }
+    if (on) *reinterpret_cast<uint4*>(row + k) = v;
+}
+
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
