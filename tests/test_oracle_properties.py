@@ -122,6 +122,8 @@ def test_allocation_properties(data):
         assert cur[j] == b0 and ratio > 0
         cur[j] = b1
         nxt = S1.objective(S, cur, layer_of)
-        assert nxt < obj + 1e-18
+        # lower, but a layer's gain may be below the last place of the sum over the layers (a score of 2e-16 beside scores of 1).
+        # Each of up to 10 terms |S_j| eta < |S_j| and the squares' sum carry a few roundings of 2^-53: below 2^-48 (sum |S|)^2.
+        assert nxt <= obj + 2.0 ** -48 * np.abs(S).sum() ** 2
         obj = nxt
     assert cur == bits.tolist()
