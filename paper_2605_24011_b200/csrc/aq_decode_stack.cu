@@ -205,7 +205,9 @@ struct DsTail {
     int32_t pad_[2];
 };
 static_assert(sizeof(DsTail) == 32, "DsTail layout");
-constexpr int DS_TAIL_CHUNK = 2048;
+// Elements per chunk: four groups of four per lane of a warp, whose readings go out together.  (With 2048 read one group after the
+// other a launch ended 5 us later: an MLP of 4096 / 11008 and one token 30.7 us.)
+constexpr int DS_TAIL_CHUNK = 512;
 
 struct DsArgs {
     const DsPhase* phases;
@@ -1064,25 +1066,25 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag) == 0) {
 #pragma unroll 1
         for (int e = (int)blockIdx.x * RO::COLLECT_WARPS + cwarp; e < a.n_tails; e += (int)gridDim.x * RO::COLLECT_WARPS) {
-            const DsTail T = a.tails[e];
-            bool ok = true;
-            for (int i = lane * 4; i < T.n && ok; i += 128) {      // n is a multiple of 4
-                DsQuad q;
-                ds_ld_quad(T.src + i, q);
-                if (!ds_quad_complete(T.src + i, q, T.expect, wait_ns, &sh.abort_flag)) ok = false;
-                else {
-                    const float4 v = ds_quad_value(q);
-                    *reinterpret_cast<float4*>(T.out + i) = v;
-                    if (a.out != nullptr) {
-                        const int64_t o = (T.src - a.out_src) + i;
-                        float unused;
-                        if (o >= 0 && o < a.out_n) *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(a.out) + o) = ds_round4<BF16>(v, &unused);
-                    }
+            const DsTail T = a.tails[e];                           // (n is a multiple of 4)
+            DsQuad q[DS_TAIL_CHUNK / 128];
+#pragma unroll
+            for (int u = 0; u < DS_TAIL_CHUNK / 128; ++u)
+                if (lane * 4 + 128 * u < T.n) ds_ld_quad(T.src + lane * 4 + 128 * u, q[u]);
+#pragma unroll
+            for (int u = 0; u < DS_TAIL_CHUNK / 128; ++u) {
+                const int i = lane * 4 + 128 * u;
+                if (i >= T.n || !ds_quad_complete(T.src + i, q[u], T.expect, wait_ns, &sh.abort_flag)) break;
+                const float4 v = ds_quad_value(q[u]);
+                *reinterpret_cast<float4*>(T.out + i) = v;
+                if (a.out != nullptr) {
+                    const int64_t o = (T.src - a.out_src) + i;
+                    float unused;
+                    if (o >= 0 && o < a.out_n) *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(a.out) + o) = ds_round4<BF16>(v, &unused);
                 }
             }
         }
     }
-
     }   // (collect warps)
 
     // after a failed wait copies and tensor-core instructions may still be at work in this CTA: give them time
