@@ -670,6 +670,16 @@ __device__ __forceinline__ void ds_record(DsShared& sh, const DsArgs& a, int rw,
     }
 }
 
+// Asks for a phase's record and this CTA's tables for it, on one barrier.
+__device__ __forceinline__ void ds_fetch_record(DsShared& sh, const DsArgs& a, int q) {
+    const uint32_t bar = ds_smem(&sh.rec_bar[q % DS_RECS]);
+    uint64_t pol_keep;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
+    ds_expect_tx(bar, (uint32_t)(sizeof(DsPhase) + sizeof(DsCtaPhase)));
+    ds_bulk_load(ds_smem(&sh.rec[q % DS_RECS]), a.phases + q, (uint32_t)sizeof(DsPhase), bar, pol_keep);
+    ds_bulk_load(ds_smem(&sh.ctab[q % DS_RECS]), a.ctab + (size_t)q * gridDim.x + blockIdx.x, (uint32_t)sizeof(DsCtaPhase), bar, pol_keep);
+}
+
 // ---- the kernel ---------------------------------------------------------------------
 template <int MT, bool BF16>
 __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(const DsArgs a) {
@@ -683,25 +693,47 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     const u64 wait_ns = a.wait_ns;
     pdl_launch_dependents();   // (an attention step that follows may read its cache on the SMs this launch leaves first)
 
-    if (threadIdx.x == 0) {
+    // Up to two tokens: a thread per barrier, and the first phases' records are asked for by the thread that has set up theirs.
+    // (One thread for all of them, and the records after the CTA had met: an MLP of 2048 / 8192 took 4 to 9 % longer.  From three
+    // tokens on, with registers dealt by role, the former costs 40 bytes of spills and 3 % of a 7B-shaped pass.)
+    if constexpr (!RO::SHARES) {
+        if (threadIdx.x < DS_QUEUE) {
+            ds_mbar_init(ds_smem(&sh.full[threadIdx.x]), 1);
+            ds_mbar_init(ds_smem(&sh.empty[threadIdx.x]), DS_UNPACK_WARPS);
+        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + DS_MAX_STAGES) {
+            const int i = (int)threadIdx.x - 32;
+            ds_mbar_init(ds_smem(&sh.stored[i]), DS_UNPACK_WARPS);
+            ds_mbar_init(ds_smem(&sh.done[i]), 1);
+            ds_mbar_init(ds_smem(&sh.taken[i]), 4);
+        }
+    }
+    if (threadIdx.x == RO::COLLECT0 * 32) {
         sh.abort_flag = 0;
         sh.xphase = 0;
 #pragma unroll
         for (int i = 0; i < DS_RECORD_WARPS; ++i) sh.recorded[i] = 0;
 #pragma unroll 1
         for (int i = 0; i < DS_RECS; ++i) ds_mbar_init(ds_smem(&sh.rec_bar[i]), 1);
+        if constexpr (!RO::SHARES) {
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_async_smem();
+            if (a.n_phases > 0) ds_fetch_record(sh, a, 0);
+            if (a.n_phases > 1) ds_fetch_record(sh, a, 1);
+        } else {
 #pragma unroll 1
-        for (int i = 0; i < DS_QUEUE; ++i) {
-            ds_mbar_init(ds_smem(&sh.full[i]), 1);
-            ds_mbar_init(ds_smem(&sh.empty[i]), DS_UNPACK_WARPS);
-        }
+            for (int i = 0; i < DS_QUEUE; ++i) {
+                ds_mbar_init(ds_smem(&sh.full[i]), 1);
+                ds_mbar_init(ds_smem(&sh.empty[i]), DS_UNPACK_WARPS);
+            }
 #pragma unroll 1
-        for (int i = 0; i < DS_MAX_STAGES; ++i) {
-            ds_mbar_init(ds_smem(&sh.stored[i]), DS_UNPACK_WARPS);
-            ds_mbar_init(ds_smem(&sh.done[i]), 1);
-            ds_mbar_init(ds_smem(&sh.taken[i]), 4);
+            for (int i = 0; i < DS_MAX_STAGES; ++i) {
+                ds_mbar_init(ds_smem(&sh.stored[i]), DS_UNPACK_WARPS);
+                ds_mbar_init(ds_smem(&sh.done[i]), 1);
+                ds_mbar_init(ds_smem(&sh.taken[i]), 4);
+            }
         }
     }
+    __syncwarp();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ds_smem(&sh.tmem)), "n"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -734,17 +766,9 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     if constexpr (RO::SHARES) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RO::REGS_COLLECT));
     // ================= collect warps =================
     const int ctid = (int)threadIdx.x - RO::COLLECT0 * 32, cwarp = warp - RO::COLLECT0;
-    auto fetch_record = [&](int q) {   // the phase's record and this CTA's tables for it, on one barrier
-        const uint32_t bar = ds_smem(&sh.rec_bar[q % DS_RECS]);
-        uint64_t pol_keep;
-        asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
-        ds_expect_tx(bar, (uint32_t)(sizeof(DsPhase) + sizeof(DsCtaPhase)));
-        ds_bulk_load(ds_smem(&sh.rec[q % DS_RECS]), a.phases + q, (uint32_t)sizeof(DsPhase), bar, pol_keep);
-        ds_bulk_load(ds_smem(&sh.ctab[q % DS_RECS]), a.ctab + (size_t)q * gridDim.x + blockIdx.x, (uint32_t)sizeof(DsCtaPhase), bar, pol_keep);
-    };
-    if (ctid == 0) {
-        if (a.n_phases > 0) fetch_record(0);
-        if (a.n_phases > 1) fetch_record(1);
+    if (RO::SHARES && ctid == 0) {
+        if (a.n_phases > 0) ds_fetch_record(sh, a, 0);
+        if (a.n_phases > 1) ds_fetch_record(sh, a, 1);
     }
     DsPlace<MT> at;                    // of the next unit
     uint32_t turn = 0;                 // the team whose unit that is
@@ -760,7 +784,7 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
 #pragma unroll
             for (int i = 0; i < DS_RECORD_WARPS; ++i)
                 if (ph >= 2) ds_wait_count(&sh.recorded[i], ph - 2, wait_ns, &sh.abort_flag);
-            if (lane == 0) fetch_record(ph + 2);
+            if (lane == 0) ds_fetch_record(sh, a, ph + 2);
         }
         // every warp is through with phase ph - 1: the staged slabs are free
         if (ds_collect_sync_or<RO::CTHREADS>(*reinterpret_cast<volatile int*>(&sh.abort_flag))) break;
@@ -1065,7 +1089,7 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     // -- buffers no phase reads (and the last outputs): float32 copies for the caller, one chunk per warp --
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag) == 0) {
 #pragma unroll 1
-        for (int e = (int)blockIdx.x * RO::COLLECT_WARPS + cwarp; e < a.n_tails; e += (int)gridDim.x * RO::COLLECT_WARPS) {
+        for (int e = (int)blockIdx.x + (int)gridDim.x * cwarp; e < a.n_tails; e += (int)gridDim.x * RO::COLLECT_WARPS) {   // (few chunks: one per SM)
             const DsTail T = a.tails[e];                           // (n is a multiple of 4)
             DsQuad q[DS_TAIL_CHUNK / 128];
 #pragma unroll
