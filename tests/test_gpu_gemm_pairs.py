@@ -1,5 +1,6 @@
 """The prefill GEMM on CTA pairs (large products): row tiles whose second half is partly or wholly absent, two and three token
-tiles with a ragged last one, rows that leave binary16's range, outputs of any row length, and a wait that runs out."""
+tiles with a ragged last one, rows that leave binary16's range, outputs of any row length, a recorded launch, and a wait that
+runs out."""
 import time
 
 import numpy as np
@@ -43,6 +44,25 @@ def test_pairs(M, N, K, bits, dtype):
     got = y.double().cpu().numpy()
     assert np.isfinite(got).all()
     assert O.linear_excess(got[np.ix_(toks, rows)], want, T).max() <= 1.0
+
+
+def test_a_recorded_pair_launch_is_replayed_on_new_input():
+    M, N, K = 512, 11008, 4096
+    aq, h, x, rows, toks, want, T = _case(M, N, K, 2, "f16")
+    buf, y = torch.zeros_like(x), torch.empty((M, N), dtype=torch.float32, device="cuda")
+    aq.aq_linear(h, buf, y)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        aq.aq_linear(h, buf, y)
+    for scale in (1.0, 2.0):
+        buf.copy_(x * scale)
+        y.fill_(float("nan"))
+        g.replay()
+        torch.cuda.synchronize()
+        aq.aq_check()
+        assert O.linear_excess(y.double().cpu().numpy()[np.ix_(toks, rows)], scale * want, scale * T).max() <= 1.0
+    del g
 
 
 def test_a_wait_of_a_pair_runs_out_and_the_next_call_is_clean():
