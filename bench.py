@@ -628,9 +628,9 @@ def main():
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
 DECODE_TRAFFIC_BYTES = 8 * (355_696_384 + 4_406_784)
-# gemm_kernel: 21,203,456 + 4,608 bytes of DRAM traffic for one 11008 x 4096
+# gemm_kernel: 21,203,200 + 4,864 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
-PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_456 + 4_608) / 16_908_288)
+PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_200 + 4_864) / 16_908_288)
 
 
 def prefill_leg(aq, workloads, prog, out_buf, info, peaks, torch, gpu_index=0):
