@@ -627,7 +627,8 @@ def main():
 # the profile of a 4-layer pass of one token: 355,696,384 + 4,406,784 bytes for the first 4 layers (354,172,928
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
-DECODE_TRAFFIC_BYTES = 8 * (355_696_384 + 4_406_784)
+# (None: the kernel's last step and set-up have changed since.)
+DECODE_TRAFFIC_BYTES = None
 # gemm_kernel: 21,203,200 + 4,864 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
 PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_200 + 4_864) / 16_908_288)
