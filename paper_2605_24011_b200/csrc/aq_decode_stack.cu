@@ -77,7 +77,7 @@ template <int MT> struct DsRoles {
     static constexpr int WARPS = RECORD0 + DS_RECORD_WARPS, THREADS = WARPS * 32;
     static constexpr bool SHARES = MT > 2;      // registers per thread: 80 at the launch, then
     static constexpr int REGS_UNPACK = 56, REGS_COLLECT = 104, REGS_OTHER = 56;
-    static_assert(!SHARES || (DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80 && WARPS % 4 == 0), "the roles' registers fit");
+    static_assert(!SHARES || (DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80 && COLLECT0 % 4 == 0 && ISSUER % 4 == 0 && WARPS - ISSUER == 4), "the roles' registers fit, and no group of four has two shares");
 };
 constexpr int DS_MAX_COLLECT_WARPS = 12;
 constexpr int DS_FRAGS = 8;                 // 16-row tiles of a unit
@@ -752,16 +752,17 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     if (warp < DS_UNPACK_WARPS) {
         if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_UNPACK));
         ds_unpack_units<MT, BF16>(sh, wait_ns, tmem, warp >> 2, quarter, lane);
-    } else if (warp == RO::ISSUER) {
+    } else if (warp >= RO::ISSUER) {
+        // (one group of four warps: setmaxnreg is for a whole group, so it stands in front of the roles)
         if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
-        ds_issue_units<MT, BF16>(sh, a, tmem);
-    } else if (warp == RO::FEEDER) {
-        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
-        if (lane == 0) ds_feed(sh, a);
-        __syncwarp();
-    } else if (warp >= RO::RECORD0) {
-        if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_OTHER));
-        ds_record<BF16>(sh, a, warp - RO::RECORD0, lane);
+        if (warp == RO::ISSUER) {
+            ds_issue_units<MT, BF16>(sh, a, tmem);
+        } else if (warp == RO::FEEDER) {
+            if (lane == 0) ds_feed(sh, a);
+            __syncwarp();
+        } else {
+            ds_record<BF16>(sh, a, warp - RO::RECORD0, lane);
+        }
     } else {
     if constexpr (RO::SHARES) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RO::REGS_COLLECT));
     // ================= collect warps =================
