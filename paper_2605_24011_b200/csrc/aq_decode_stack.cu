@@ -59,6 +59,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "aq_decode_rings.h"
 #include "aq_decode_tc.cuh"
 #include "aq_internal.h"
 
@@ -88,18 +89,18 @@ constexpr int DS_XS_BYTES = DS_MAX_SLOTS * dt_slab_bytes(AQ_DECODE_MAX_M);
 // A unit's operands and sums in TMEM, A of both halves and D of both halves, and what goes with it (descriptor, scales, the
 // barrier that says they are there).  One token: five stages of both, refilled once the sums have been read.  Several tokens:
 // reading the sums takes longer than anything else, so A (two stages) is refilled as soon as the instructions have read it
-// and D (two as well) is written again once the sums have been read; unit n + 4 is not unpacked before unit n + 2 was issued,
-// which waited for the sums of unit n.
+// and D (two as well) is written again once the sums have been read (aq_decode_rings.h).
+constexpr int DS_MAX_STAGES = 5;
 template <int MT> struct DsStage {
     static constexpr int A_COLS = 2 * DtShape<MT>::A_COLS, D_COLS = 2 * DtShape<MT>::D_COLS;   // 64 + 32 / 128 + 128
     static constexpr bool SPLIT = MT > 1;
-    static constexpr int A = SPLIT ? 2 : 5, D = SPLIT ? 2 : 5, META = SPLIT ? 4 : 5;
-    static_assert(A * A_COLS + D * D_COLS <= 512 && META <= A + D, "fits TMEM; see above");
+    static constexpr int A = SPLIT ? DS_A_STAGES : 5, D = SPLIT ? DS_D_STAGES : 5, META = SPLIT ? DS_META_SLOTS : 5;
+    static_assert(A * A_COLS + D * D_COLS <= 512 && A <= DS_MAX_STAGES && D <= DS_MAX_STAGES && META <= DS_MAX_STAGES, "fits TMEM and the barriers");
+    static_assert(!SPLIT || ds_rings_hold(A, D, META, DsRoles<MT>::TEAMS), "a slot is written again only when its last unit is through with it");
     // first columns of stages (one token: a stage's sums lie behind its operand, one address serves both)
     __device__ static __forceinline__ uint32_t a_col(uint32_t s) { return s * (SPLIT ? A_COLS : A_COLS + D_COLS); }
     __device__ static __forceinline__ uint32_t d_col(uint32_t s) { return SPLIT ? A * A_COLS + s * D_COLS : a_col(s) + A_COLS; }
 };
-constexpr int DS_MAX_STAGES = 5;
 // A slot of a ring and how often the ring has gone round.
 template <int N> struct DsRing {
     uint32_t at = 0, use = 0;
