@@ -17,7 +17,7 @@
 //         across op and phase boundaries, so a phase starts with its first units
 //         waiting in TMEM;
 //       - the issuer (one thread) starts a unit's tensor-core instructions;
-//       - eight collect warps (twelve from three tokens on) form a phase's input, read
+//       - eight collect warps (twelve from five tokens on) form a phase's input, read
 //         the units' sums back, apply scales and minima and add the rows up in memory;
 //       - two record warps write the caller's copies of a phase's input.
 //     Four warps that each did all of this in turn, step after step, needed 1404
@@ -70,13 +70,17 @@ typedef unsigned long long u64;
 // Warps by role (a warp reaches the TMEM lanes of its quarter only: unpack and collect teams start at multiples of four).
 constexpr int DS_UNPACK_WARPS = 8;          // two teams of four: one per half (128 k) of a unit
 constexpr int DS_RECORD_WARPS = 2;
-// Collect warps: teams of four that take the units in turn.  One token: two teams.  Several tokens: a unit costs its team four
-// times as many instructions, so there are three, and the roles get registers by what they need.
+// Collect warps: teams of four that take the units in turn.  Two teams; three from five tokens on, where reading a unit's sums and
+// adding them sets the pace, with registers dealt to the roles by what they need (-Xptxas -v: 80 registers, 16 and 28 bytes
+// spilled for binary16 and bfloat16; two teams 90 to 96 and none to 4).  With three and four tokens a third team gains nothing
+// where units set the pace and costs where boundaries do, in us with three / two teams at 4 tokens: 8 blocks of the 7B shape 423 /
+// 419 (bfloat16 445 / 425), of the 2B shape 289 / 270, 18 expert blocks 373 / 340, MLP 4096 / 11008 36.9 / 34.8; at 5 and 8 tokens
+// 8 blocks of the 7B shape 504 / 527 and 556 / 579.
 template <int MT> struct DsRoles {
-    static constexpr int COLLECT_WARPS = MT <= 2 ? 8 : 12, TEAMS = COLLECT_WARPS / 4, CTHREADS = COLLECT_WARPS * 32;
+    static constexpr int COLLECT_WARPS = MT <= 4 ? 8 : 12, TEAMS = COLLECT_WARPS / 4, CTHREADS = COLLECT_WARPS * 32;
     static constexpr int COLLECT0 = DS_UNPACK_WARPS, ISSUER = COLLECT0 + COLLECT_WARPS, FEEDER = ISSUER + 1, RECORD0 = FEEDER + 1;
     static constexpr int WARPS = RECORD0 + DS_RECORD_WARPS, THREADS = WARPS * 32;
-    static constexpr bool SHARES = MT > 2;      // registers per thread: 80 at the launch, then
+    static constexpr bool SHARES = TEAMS == 3;      // registers per thread: 80 at the launch, then
     static constexpr int REGS_UNPACK = 56, REGS_COLLECT = 104, REGS_OTHER = 56;
     static_assert(!SHARES || (DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80 && COLLECT0 % 4 == 0 && ISSUER % 4 == 0 && WARPS - ISSUER == 4), "the roles' registers fit, and no group of four has two shares");
 };
@@ -694,9 +698,9 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     const u64 wait_ns = a.wait_ns;
     pdl_launch_dependents();   // (an attention step that follows may read its cache on the SMs this launch leaves first)
 
-    // Up to two tokens: a thread per barrier, and the first phases' records are asked for by the thread that has set up theirs.
-    // (One thread for all of them, and the records after the CTA had met: an MLP of 2048 / 8192 took 4 to 9 % longer.  From three
-    // tokens on, with registers dealt by role, the former costs 40 bytes of spills and 3 % of a 7B-shaped pass.)
+    // Two teams: a thread per barrier, and the first phases' records are asked for by the thread that has set up theirs.
+    // (One thread for all of them, and the records after the CTA had met: an MLP of 2048 / 8192 took 4 to 9 % longer.  With
+    // registers dealt by role the former costs 40 bytes of spills and 3 % of a 7B-shaped pass.)
     if constexpr (!RO::SHARES) {
         if (threadIdx.x < DS_QUEUE) {
             ds_mbar_init(ds_smem(&sh.full[threadIdx.x]), 1);
