@@ -17,8 +17,8 @@
 //         across op and phase boundaries, so a phase starts with its first units
 //         waiting in TMEM;
 //       - the issuer (one thread) starts a unit's tensor-core instructions;
-//       - eight collect warps (twelve from five tokens on) form a phase's input, read
-//         the units' sums back, apply scales and minima and add the rows up in memory;
+//       - eight or twelve collect warps (ds_teams) form a phase's input, read the units'
+//         sums back, apply scales and minima and add the rows up in memory;
 //       - two record warps write the caller's copies of a phase's input.
 //     Four warps that each did all of this in turn, step after step, needed 1404
 //     us for a 7B-shaped pass of one token (software-pipelined: 1398); the roles
@@ -56,6 +56,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <numeric>
 #include <type_traits>
 #include <vector>
 
@@ -70,14 +71,11 @@ typedef unsigned long long u64;
 // Warps by role (a warp reaches the TMEM lanes of its quarter only: unpack and collect teams start at multiples of four).
 constexpr int DS_UNPACK_WARPS = 8;          // two teams of four: one per half (128 k) of a unit
 constexpr int DS_RECORD_WARPS = 2;
-// Collect warps: teams of four that take the units in turn.  Two teams; three from five tokens on, where reading a unit's sums and
-// adding them sets the pace, with registers dealt to the roles by what they need (-Xptxas -v: 80 registers, 16 and 28 bytes
-// spilled for binary16 and bfloat16; two teams 90 to 96 and none to 4).  With three and four tokens a third team gains nothing
-// where units set the pace and costs where boundaries do, in us with three / two teams at 4 tokens: 8 blocks of the 7B shape 423 /
-// 419 (bfloat16 445 / 425), of the 2B shape 289 / 270, 18 expert blocks 373 / 340, MLP 4096 / 11008 36.9 / 34.8; at 5 and 8 tokens
-// 8 blocks of the 7B shape 504 / 527 and 556 / 579.
-template <int MT> struct DsRoles {
-    static constexpr int COLLECT_WARPS = MT <= 4 ? 8 : 12, TEAMS = COLLECT_WARPS / 4, CTHREADS = COLLECT_WARPS * 32;
+// Collect warps: teams of four that take the units in turn, two or three (ds_teams).  With three, registers are dealt to the roles
+// by what they need (-Xptxas -v: 80 registers, 16 and 28 bytes spilled for binary16 and bfloat16; two teams 90 to 96 registers,
+// none to 4 bytes spilled, with eight tokens 16 and 20).
+template <int NTEAMS> struct DsRoles {
+    static constexpr int TEAMS = NTEAMS, COLLECT_WARPS = 4 * TEAMS, CTHREADS = COLLECT_WARPS * 32;
     static constexpr int COLLECT0 = DS_UNPACK_WARPS, ISSUER = COLLECT0 + COLLECT_WARPS, FEEDER = ISSUER + 1, RECORD0 = FEEDER + 1;
     static constexpr int WARPS = RECORD0 + DS_RECORD_WARPS, THREADS = WARPS * 32;
     static constexpr bool SHARES = TEAMS == 3;      // registers per thread: 80 at the launch, then
@@ -100,7 +98,6 @@ template <int MT> struct DsStage {
     static constexpr bool SPLIT = MT > 1;
     static constexpr int A = SPLIT ? DS_A_STAGES : 5, D = SPLIT ? DS_D_STAGES : 5, META = SPLIT ? DS_META_SLOTS : 5;
     static_assert(A * A_COLS + D * D_COLS <= 512 && A <= DS_MAX_STAGES && D <= DS_MAX_STAGES && META <= DS_MAX_STAGES, "fits TMEM and the barriers");
-    static_assert(!SPLIT || ds_rings_hold(A, D, META, DsRoles<MT>::TEAMS), "a slot is written again only when its last unit is through with it");
     // first columns of stages (one token: a stage's sums lie behind its operand, one address serves both)
     __device__ static __forceinline__ uint32_t a_col(uint32_t s) { return s * (SPLIT ? A_COLS : A_COLS + D_COLS); }
     __device__ static __forceinline__ uint32_t d_col(uint32_t s) { return SPLIT ? A * A_COLS + s * D_COLS : a_col(s) + A_COLS; }
@@ -226,6 +223,7 @@ struct DsArgs {
     int n_ops;
     int n_tails;
     int M;
+    int late;                         // several tokens: a unit is unpacked only when the sums of the last one in its stage have been read
     // the caller's rounded output: the tail chunks that convert [out_src, out_src + out_n) also write it (null: nobody does)
     void* out;
     const u64* out_src;
@@ -412,9 +410,9 @@ static_assert(sizeof(DsShared) <= 227 * 1024, "fits an SM");
 template <int MT>
 __device__ __forceinline__ void ds_commit(const float (&acc)[MT], u64* out, const void* res, bool res_plain, int row, int N, int M) {
     if (row >= N) return;
-    if constexpr (MT > 1) {
+    if constexpr (MT > 2) {
         // (what a sum costs here, times 1024 per unit, is a third of the collect warps' instructions: the limits are looked at
-        // once for all tokens)
+        // once for all tokens; with two tokens that only delays the first, 18 expert blocks 269 -> 275 us)
         float mx = 0.f;
         bool clean = true;
 #pragma unroll
@@ -504,9 +502,10 @@ __device__ __forceinline__ void ds_feed(DsShared& sh, const DsArgs& a) {
 
 // An unpack warp: its two fragments (rows 32 quarter .. + 31) of half `half` of every unit.
 template <int MT, bool BF16>
-__device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint32_t tmem, int half, int quarter, int lane) {
+__device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint32_t tmem, bool late, int half, int quarter, int lane) {
     using ST = DsStage<MT>;
     using SH = DtShape<MT>;
+    const uint32_t released = ds_smem(late ? sh.taken : sh.done);   // several tokens: by which barriers
     DsPlace<MT> at;
     for (uint32_t n = 0;; ++n) {
         const uint32_t e = n % DS_QUEUE;
@@ -518,12 +517,12 @@ __device__ __forceinline__ void ds_unpack_units(DsShared& sh, u64 wait_ns, uint3
         const uint8_t* fr = sh.ring + (d.w & 0xFFFFFu) + (half ? (d.w >> 20) << 8 : 0u) + (uint32_t)(quarter * 2 * fb);
         const uint4 dm = *reinterpret_cast<const uint4*>(fr + (lane >> 4) * fb + (lane & 15) * 16);
         const uint32_t ta = tmem + ST::a_col(at.a().at) + (uint32_t)(half * SH::A_COLS) + ((uint32_t)(quarter * 32) << 16);
-        // the stage is free once its last unit's instructions have completed (one token: and its sums have been read)
+        // the stage is free once its last unit's instructions have completed (one token, and late: and its sums have been read)
         auto stage_free = [&]() {
             if (at.a().use == 0) return true;
             if constexpr (!ST::SPLIT) return ds_warp_wait(ds_smem(&sh.taken[at.a().at]), (at.a().use - 1) & 1u, wait_ns, &sh.abort_flag);
             const uint32_t before = n - ST::A;   // the unit that had the stage
-            return ds_warp_wait(ds_smem(&sh.done[before % ST::D]), (before / ST::D) & 1u, wait_ns, &sh.abort_flag);
+            return ds_warp_wait(released + 8 * (before % ST::D), (before / ST::D) & 1u, wait_ns, &sh.abort_flag);
         };
         if constexpr (MT == 1) {
             uint32_t va[16], vb[16];
@@ -686,10 +685,11 @@ __device__ __forceinline__ void ds_fetch_record(DsShared& sh, const DsArgs& a, i
 }
 
 // ---- the kernel ---------------------------------------------------------------------
-template <int MT, bool BF16>
-__global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(const DsArgs a) {
+template <int MT, int TEAMS, bool BF16>
+__global__ void __launch_bounds__(DsRoles<TEAMS>::THREADS, 1) decode_stack_kernel(const DsArgs a) {
     using ST = DsStage<MT>;
-    using RO = DsRoles<MT>;
+    using RO = DsRoles<TEAMS>;
+    static_assert(!ST::SPLIT || ds_rings_hold(ST::A, ST::D, ST::META, TEAMS), "a slot is written again only when its last unit is through with it");
     extern __shared__ __align__(128) uint8_t ds_smem_raw[];
     DsShared& sh = *reinterpret_cast<DsShared*>(ds_smem_raw);
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(DsRoles<MT>::THREADS, 1) decode_stack_kernel(c
     }
     if (warp < DS_UNPACK_WARPS) {
         if constexpr (RO::SHARES) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(RO::REGS_UNPACK));
-        ds_unpack_units<MT, BF16>(sh, wait_ns, tmem, warp >> 2, quarter, lane);
+        ds_unpack_units<MT, BF16>(sh, wait_ns, tmem, a.late != 0, warp >> 2, quarter, lane);
     } else if (warp == RO::ISSUER) {
         ds_issue_units<MT, BF16>(sh, a, tmem);
     } else if (warp == RO::FEEDER) {
@@ -1139,6 +1139,8 @@ struct DecodePlan {
     int n_ops = 0;
     int n_phases = 0;
     int n_tails = 0;
+    bool late = false;            // ds_late, ds_teams of its phases
+    int teams = 2;
     int device = 0;
     bool pinned = false;          // recorded into a CUDA graph: its device tables must outlive the plan cache's turnover
     std::vector<char> in_tails;   // per buffer: the tail chunks convert it (no phase reads it)
@@ -1350,6 +1352,34 @@ bool build_decode_tables(const aq_stack_t* p, const StackPlan& plan, int M, int 
     return true;
 }
 
+// Collect teams for M tokens.  Reading a unit's sums and adding them sets the pace from five tokens on, and a third team helps there;
+// so do its threads where every CTA reads whole rows for the row norms and they save it a step (256 or 384 threads, a group of
+// four elements each).  With three and four tokens it gains nothing where units set the pace and costs where boundaries do, and
+// with seven and eight the same holds for whole rows of which it saves no step.  Measured, us with two / three teams: 18 expert
+// blocks (K = 1024) 340 / 373 at 4 tokens, 402 / 396 at 5, 443 / 471 at 7, 457 / 482 at 8; 8 blocks of the 2B shape (2048) 270 / 289
+// at 4, 355 / 341 at 5, 359 / 350 at 6, 386 / 395 at 7, 400 / 405 at 8; of the 7B shape (shares from 5 tokens on) 421 / 423 at 4,
+// 525 / 492 at 5, 578 / 547 at 8; 8 blocks of 1280 / 5120 (two steps / one) 208 / 188 at 5, 242 / 224 at 8.
+static int ds_teams(const std::vector<DsPhase>& phases, int M) {
+    if (M <= 4) return 2;
+    if (M <= 6) return 3;
+    bool whole_rows = false;
+    for (const DsPhase& P : phases) {
+        if (P.in_op != AQ_IN_RMSNORM || P.norm != nullptr) continue;
+        const int q4 = P.K / 4, two = DsRoles<2>::CTHREADS, three = DsRoles<3>::CTHREADS;
+        if ((q4 + two - 1) / two != (q4 + three - 1) / three) return 3;
+        whole_rows = true;
+    }
+    return whole_rows ? 2 : 3;
+}
+// Whether the operand of unit n + 2 is unpacked only when the sums of unit n have been read, not as soon as its instructions have
+// completed.  At once is better where a phase is many units long; where it is not, unit n + 2 belongs to the next phase, and
+// unpacking it takes issue slots from the sums that everybody is waiting for.  The line lies at the units a CTA meets of a phase, on
+// average; us at once / late: two teams, 18 expert blocks (0.9 units) 285 / 272 at 2 tokens, 335 / 320 at 4, 474 / 457 at 8; 8 blocks
+// of 2048 / 8192 (3.1) 212 / 209 at 4, 2304 / 8192 (3.5) 240 / 236, 2560 / 8192 (4.0) 245 / 243, 3072 / 8192 (5.0) 221 / 223 at 2, of
+// the 7B shape (10) 344 / 348 at 2; three teams, 5 tokens: expert 407 / 396, 1536 / 6144 (1.7) 200.7 / 198.6, 2048 / 6144 (2.4) 248 /
+// 251, 3072 / 8192 315 / 325, 7B shape 492 / 509.
+static bool ds_late(int64_t units, int64_t cta_phases, int teams) { return units < (teams == 2 ? 4 : 2) * cta_phases; }
+
 // What a pass needs before its first launch: x as float32 (groups of eight) and zeros in the packed sums.  One kernel in place of
 // a conversion and a memset: a pass of a small program takes 15 us, and each launch before the big one added 1.5.
 template <bool BF16>
@@ -1380,16 +1410,16 @@ __global__ void __launch_bounds__(256) begin_pass_kernel(const uint4* __restrict
     for (int64_t i = i0; i < zero16; i += step) zero[i] = make_uint4(0, 0, 0, 0);
 }
 
-template <int MT, bool BF16>
+template <int MT, int TEAMS, bool BF16>
 static cudaError_t launch_ds(const DsArgs& a, int grid, cudaStream_t s) {
-    auto kern = decode_stack_kernel<MT, BF16>;
+    auto kern = decode_stack_kernel<MT, TEAMS, BF16>;
     static PerDeviceOnce configured;
     {
         const int rc = configured.run(current_device(), [&] {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsShared));
             if (e != cudaSuccess) return (int)e;
             int per_sm = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DsRoles<MT>::THREADS, sizeof(DsShared));
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DsRoles<TEAMS>::THREADS, sizeof(DsShared));
             if (e != cudaSuccess) return (int)e;
             return per_sm < 1 ? (int)cudaErrorCooperativeLaunchTooLarge : 0;
         });
@@ -1397,7 +1427,7 @@ static cudaError_t launch_ds(const DsArgs& a, int grid, cudaStream_t s) {
     }
     DsArgs args = a;
     void* params[1] = {&args};
-    cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3((unsigned)grid), dim3(DsRoles<MT>::THREADS), params,
+    cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3((unsigned)grid), dim3(DsRoles<TEAMS>::THREADS), params,
                                                 sizeof(DsShared), s);
     if (e == cudaSuccess) count_launch();
     return e;
@@ -1471,6 +1501,8 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
         };
         std::vector<int32_t> unit_total(grid, 0);
         for (size_t i = 0; i < ctab.size(); ++i) unit_total[i % grid] += ctab[i].total;
+        dp->teams = ds_teams(phases, M);
+        dp->late = ds_late(std::accumulate(unit_total.begin(), unit_total.end(), (int64_t)0), (int64_t)phases.size() * grid, dp->teams);
         dp->n_ops = (int)feed_ops.size();
         feed_ops.push_back(DsFeedOp{});   // (the feeder reads one op ahead)
         xoff.resize(xoff.size() + grid, 0);
@@ -1499,6 +1531,7 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
     a.n_phases = dp->n_phases;
     a.n_tails = dp->n_tails;
     a.M = M;
+    a.late = dp->late ? 1 : 0;
     a.wait_ns = g_wait_ns;
     a.out = nullptr; a.out_src = nullptr; a.out_n = 0;
     if (out != nullptr && out_buf >= 1 && out_buf < p->n_bufs && dp->in_tails[out_buf] &&
@@ -1521,10 +1554,11 @@ int launch_decode_stack(const aq_stack_t* p, const StackPlan& plan, int M, aq_dt
     }
     if (e == cudaSuccess) {
         const bool bf = (dt == AQ_BF16);
-        if (M == 1) e = bf ? launch_ds<1, true>(a, grid, s) : launch_ds<1, false>(a, grid, s);
-        else if (M == 2) e = bf ? launch_ds<2, true>(a, grid, s) : launch_ds<2, false>(a, grid, s);
-        else if (M <= 4) e = bf ? launch_ds<4, true>(a, grid, s) : launch_ds<4, false>(a, grid, s);
-        else e = bf ? launch_ds<8, true>(a, grid, s) : launch_ds<8, false>(a, grid, s);
+        if (M == 1) e = bf ? launch_ds<1, 2, true>(a, grid, s) : launch_ds<1, 2, false>(a, grid, s);
+        else if (M == 2) e = bf ? launch_ds<2, 2, true>(a, grid, s) : launch_ds<2, 2, false>(a, grid, s);
+        else if (M <= 4) e = bf ? launch_ds<4, 2, true>(a, grid, s) : launch_ds<4, 2, false>(a, grid, s);
+        else if (dp->teams == 2) e = bf ? launch_ds<8, 2, true>(a, grid, s) : launch_ds<8, 2, false>(a, grid, s);
+        else e = bf ? launch_ds<8, 3, true>(a, grid, s) : launch_ds<8, 3, false>(a, grid, s);
     }
     if (e != cudaSuccess) { *err = e; return -1; }
     return 0;

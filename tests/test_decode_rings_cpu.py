@@ -31,11 +31,11 @@ SRC = textwrap.dedent(r"""
         }
         bool has(int x, int y) { return x == y || before[x][y]; }
     };
-    static bool sound(int a, int d, int meta, int teams) {
+    static bool sound(int a, int d, int meta, int teams, bool late) {   // late: the operand's stage is filled again after the sums have been read
         Order o;
         for (int n = 0; n < N; ++n) {
             if (n) { o.after(o.U(n), o.U(n - 1)); o.after(o.I(n), o.I(n - 1)); o.after(o.F(n), o.F(n - 1)); }
-            if (n >= a) o.after(o.U(n), o.F(n - a));
+            if (n >= a) o.after(o.U(n), late ? o.C(n - a) : o.F(n - a));
             if (n >= d) o.after(o.I(n), o.C(n - d));
             if (n >= teams) o.after(o.C(n), o.C(n - teams));
             o.after(o.I(n), o.U(n)); o.after(o.F(n), o.I(n)); o.after(o.C(n), o.F(n));
@@ -56,7 +56,7 @@ SRC = textwrap.dedent(r"""
             if (!wait(n, meta, n ? o.I(n - 1) : -1, o.I(n), U)) return false;          // issuer: the operand is there
             if (!wait(n, meta, before_c, o.C(n), U)) return false;                     // collect: the same, then
             if (!wait(n, d, o.U(n), o.C(n), F)) return false;                          // ... its instructions
-            if (n + a < N && !wait(n, d, o.U(n + a - 1), o.U(n + a), F)) return false;  // unpack: the operand has been read
+            if (n + a < N && !(late ? wait(n, d, o.U(n + a - 1), o.U(n + a), C) : wait(n, d, o.U(n + a - 1), o.U(n + a), F))) return false;  // unpack
             if (n + d < N && !wait(n, d, o.I(n + d - 1), o.I(n + d), C)) return false;  // issuer: the sums have been read
         }
         return true;
@@ -66,10 +66,10 @@ SRC = textwrap.dedent(r"""
         for (int teams = 1; teams <= 3; ++teams) for (int a = 1; a <= 4; ++a) for (int d = 1; d <= 4; ++d) for (int m = 1; m <= 8; ++m)
             if (ds_rings_hold(a, d, m, teams)) {
                 ++accepted;
-                if (!sound(a, d, m, teams)) { std::printf("accepted, but not sound: A %d D %d META %d, %d teams\n", a, d, m, teams); return 1; }
+                if (!sound(a, d, m, teams, false) || !sound(a, d, m, teams, true)) { std::printf("accepted, but not sound: A %d D %d META %d, %d teams\n", a, d, m, teams); return 1; }
             }
         for (int teams = 2; teams <= 3; ++teams)
-            if (!ds_rings_hold(DS_A_STAGES, DS_D_STAGES, DS_META_SLOTS, teams) || sound(2, 2, 3, teams)) { std::printf("%d teams\n", teams); return 1; }
+            if (!ds_rings_hold(DS_A_STAGES, DS_D_STAGES, DS_META_SLOTS, teams) || sound(2, 2, 3, teams, false)) { std::printf("%d teams\n", teams); return 1; }
         std::printf("OK %d\n", accepted);
         return accepted > 50 ? 0 : 1;
     }

@@ -62,6 +62,16 @@ def test_wide_magnitudes(M, dtype, bits):
     _run(M, 512, 96, dtype, (bits,), True)
 
 
+@pytest.mark.parametrize("M,K,N,dtype", [
+    (2, 1024, 2048, "f16"), (4, 1024, 2048, "bf16"), (6, 1024, 2048, "f16"), (8, 1024, 2048, "bf16"), (7, 1536, 2048, "f16"),   # under a unit
+    (2, 2048, 13312, "bf16"), (3, 2048, 13312, "f16"), (5, 2048, 13312, "bf16"), (7, 2048, 13312, "f16"), (8, 2560, 13312, "bf16"),   # 4.3, 5.3
+])
+def test_units_per_phase(M, K, N, dtype):
+    """Phases of a few and of many units per CTA: two and three collect teams, operands unpacked after the sums have been read and
+    after the instructions have."""
+    _run(M, K, N, dtype, (3, 2, 4), False)
+
+
 def _emulated(d, m, q, x):
     """y and sum |x w| of the several-token arithmetic with binary16 activations, rounding where it rounds: the two half sums of
     a block are joined in binary32, two multiply-adds bring the block into the unit's sum (256 k), units are added in steps of
