@@ -83,7 +83,7 @@ static_assert(GM_DQ_WARPS * GM_REGS_DQ + GM_EP_WARPS * GM_REGS_EP + 4 * GM_REGS_
 // What depends on whether a tile belongs to one CTA or to a pair of them.
 template <bool PAIR> struct Tile {
     static constexpr int FRAGS = PAIR ? GM_FRAGS / 2 : GM_FRAGS;   // 16-row tiles a CTA dequantises
-    static constexpr int MAX_TN = PAIR ? 256 : 128;                // tokens per tile (UMMA N)
+    static constexpr int MAX_TN = PAIR ? GM_PAIR_TOKENS : GM_TOKENS;   // tokens per tile (UMMA N)
     static constexpr int B_BYTES = 128 * 128;                      // token slot: 128 tokens x 64 k (of a pair each CTA holds half of the tile's tokens)
     static constexpr int B_SLOTS = PAIR ? 7 : 5;
     static constexpr int P_BYTES = FRAGS * frag_bytes(4);          // packed fragments of one slab (largest width)
@@ -595,32 +595,10 @@ static cudaError_t launch_one(const CUtensorMap& tm, const GemmOutMaps& tmo, con
     return e;
 }
 
-// How a launch for M tokens is cut: CTAs or pairs of them, token tiles of one width.
-struct GemmShape {
-    bool pair;
-    int n_st, tn;   // token tiles, tokens per tile
-    int workers;    // CTAs or pairs that the device holds
-};
-static GemmShape gemm_shape(const aq_handle_s* const* hs, int n, int M) {
-    GemmShape g;
-    const int sms = std::min(sm_count(), GM_MAX_GRID);
-    // Pairs dequantise a weight, and read it from L2, once per 256 tokens instead of 128, but fill and drain tiles of twice the
-    // size, and a tile costs them nearly the same whatever it holds: they pay where the tokens fill tiles of 256 (an even number of
-    // 128s, at least four) and a pair has about 48 stages (256 rows x 256 tokens x 64 k) of work.  Measured, us with single
-    // CTAs / pairs, 3 bits: 22016 x 4096 at 256 tokens 47.3 / 46.8, 257 57.9 / 68.5, 384 66.0 / 72.4, 448 82.4 / 75.3, 512 85.7 /
-    // 79.7, 640 103.5 / 104.5, 768 124.6 / 114.1; 32768 x 2048 at 512 71.7 / 69.1, 768 105.7 / 99.1; 4096 x 11008 at 256 30.5 /
-    // 31.3, 512 47.8 / 46.8; 4096 x 4096 at 512 (28 stages) 26.1 / 26.8, at 1024 (55) 43.8 / 37.7.
+static GemmShape shape_of(const aq_handle_s* const* hs, int n, int M) {
     long long R = 0;
     for (int i = 0; i < n; ++i) R += (hs[i]->NT + GM_FRAGS - 1) / GM_FRAGS;
-    const int t128 = (M + 127) / 128;
-    g.pair = t128 >= 4 && t128 % 2 == 0 && sms >= 2 && R * (t128 / 2) * hs[0]->KP * 4 >= 48LL * (sms / 2);
-    g.workers = g.pair ? sms / 2 : sms;
-    const int max_tn = g.pair ? Tile<true>::MAX_TN : Tile<false>::MAX_TN;
-    g.n_st = (M + max_tn - 1) / max_tn;
-    // (several tiles: a multiple of 32, the width of the epilogue's copies, which must not reach into the next tile; a pair's
-    // instruction takes multiples of 32)
-    g.tn = g.pair || g.n_st > 1 ? ((M + g.n_st - 1) / g.n_st + 31) / 32 * 32 : (M + 15) / 16 * 16;
-    return g;
+    return gemm_shape(R, hs[0]->KP, M, sm_count());
 }
 
 // cut_runs for tiles of c1 units, remembered: finding the runs takes the host about 10 us, a stack asks for the same few
@@ -659,7 +637,7 @@ cudaError_t launch_gemm_group(const aq_handle_s* const* hs, int n, const void* x
         o.N = (int)hs[i]->N; o.NT = hs[i]->NT; o.R = (hs[i]->NT + GM_FRAGS - 1) / GM_FRAGS; o.bits = hs[i]->bits;
         rows += o.R;
     }
-    const GemmShape shape = gemm_shape(hs, n, M);
+    const GemmShape shape = shape_of(hs, n, M);
     a.n_st = shape.n_st; a.tn = shape.tn;
     const long long tiles = rows * a.n_st, total = tiles * 2 * a.n_slabs;   // in half slabs
     int grid = shape.workers;
@@ -804,15 +782,13 @@ bool gemm_stores_first(const aq_handle_s* const* hs, int n, int M, cudaStream_t 
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
     if (cap != cudaStreamCaptureStatusNone) return false;
-    long long R = 0;
-    for (int i = 0; i < n; ++i) R += (hs[i]->NT + GM_FRAGS - 1) / GM_FRAGS;
     // Stores first saves writing the zeros, but where a tile is shared by CTAs that all reach it at the same time the others
     // wait 3 to 5 us for the first one's stores; from about two CTAs per tile on, zeros are cheaper.  Measured, stores first /
     // zeros: 4096 x 4096 (16 tiles) at 32 tokens 18.5 / 15.2 us, 11008 x 4096 (86 tiles) at 200 tokens 46 / 42 us, eight 7B
     // layers (48 and 86 tiles) at 50 tokens 814 / 739 us; the other way round with 104 to 148 tiles, 18 expert layers at 512
     // tokens 1291 / 1381 us.
-    const GemmShape shape = gemm_shape(hs, n, M);
-    const long long tiles = R * shape.n_st;
+    const GemmShape shape = shape_of(hs, n, M);
+    const long long tiles = shape.tiles;
     return tiles <= GM_MAX_TILES && 10 * tiles >= 7 * shape.workers;
 }
 

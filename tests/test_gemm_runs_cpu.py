@@ -71,6 +71,37 @@ SRC = textwrap.dedent(r"""
     }
 """)
 
+SHAPE = textwrap.dedent(r"""
+    #include <cstdio>
+    #include "aq_gemm_runs.h"
+    int main() {
+        long long N, K; int M, sms;
+        while (std::scanf("%lld %lld %d %d", &N, &K, &M, &sms) == 4) {
+            const aq::GemmShape g = aq::gemm_shape((N + 255) / 256, (int)((K + 255) / 256), M, sms);
+            std::printf("%d %d %d %d %lld\n", g.pair, g.n_st, g.tn, g.workers, g.tiles);
+        }
+    }
+""")
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+@pytest.mark.parametrize("pair,N,K,M,sms", [
+    (1, 22016, 4096, 512, 148), (1, 22016, 4096, 385, 148), (0, 22016, 4096, 384, 148), (0, 22016, 4096, 640, 148), (1, 4096, 4096, 1024, 148),
+    (0, 4096, 4096, 512, 148), (0, 22016, 4096, 512, 1),
+    (0, 512, 65536, 448, 148), (0, 128, 131072, 400, 148), (0, 768, 32768, 768, 148), (1, 1024, 16384, 1024, 148),      # few row tiles
+    (0, 65536, 256, 1024, 148), (0, 32768, 1024, 512, 148), (1, 32768, 1280, 512, 148),                                  # short rows
+    (0, 2048, 16384, 2048, 148), (0, 3072, 16384, 2048, 148), (1, 2304, 16384, 2048, 148), (1, 2304, 8192, 4096, 148),   # 64 MB of tokens
+    (1, 4096, 11008, 4096, 148), (1, 11008, 4096, 8192, 148),
+])
+def test_pairs_where_they_pay(tmp_path, pair, N, K, M, sms):
+    src, exe = tmp_path / "shape.cpp", tmp_path / "shape"
+    src.write_text(SHAPE)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", HDR, str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], input=f"{N} {K} {M} {sms}", capture_output=True, text=True, check=True)
+    got, n_st, tn, workers, tiles = map(int, r.stdout.split())
+    assert got == pair and workers == (sms // 2 if pair else sms) and tiles == n_st * -(-N // 256)
+    assert tn <= (256 if pair else 128) and tn % 32 == 0 and (n_st - 1) * tn < M <= n_st * tn
+
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
 def test_gemm_runs_partition(tmp_path):
