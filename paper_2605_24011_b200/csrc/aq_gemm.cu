@@ -176,11 +176,12 @@ __device__ __forceinline__ void give_up(volatile int* abort_flag, int code) {
     if constexpr (PAIR) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32((const void*)abort_flag), cluster_rank() ^ 1u)), "r"(1) : "memory");
     atomicCAS(&g_gemm_status, 0, code);
 }
-// Bounded wait.  Returns false when the limit ran out or another role (of either CTA of a pair) gave up.
-template <bool PAIR>
+// Bounded wait.  Returns false when the limit ran out or another role (of either CTA of a pair) gave up.  OWN: every arrival comes from
+// this CTA; of a pair the others may come from its partner, so they are waited for at cluster scope (0 to 1 % of a product).
+template <bool PAIR, bool OWN = !PAIR>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code) {
     for (uint32_t i = 0; i < GM_SPIN_LIMIT; ++i) {
-        if (mbar_try(bar, parity)) return true;
+        if (OWN ? mbar_try(bar, parity) : mbar_try_cluster(bar, parity)) return true;
         if (i > 2000) {
             __nanosleep(40);
             if (*abort_flag) return false;
@@ -189,9 +190,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     give_up<PAIR>(abort_flag, code);
     return false;
 }
-template <bool PAIR>
+template <bool PAIR, bool OWN = !PAIR>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code) {
-    return __all_sync(0xffffffffu, mbar_wait<PAIR>(bar, parity, abort_flag, code));
+    return __all_sync(0xffffffffu, mbar_wait<PAIR, OWN>(bar, parity, abort_flag, code));
 }
 // Arrive on a barrier of the CTA that issues the instructions: given as a cluster address for a pair, as a local one otherwise.
 template <bool PAIR>
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             for (int s = sg.s0; s < sg.s1 && ok; ++s, ++n) {
                 if ((int)(n % T::DQ_GROUPS) != group) continue;
                 const uint32_t ps = n % GM_PSTAGES, parity = (n / T::DQ_GROUPS) & 1;   // (of the group's two A stages)
-                ok = mbar_wait_warp<PAIR>(bar_pfull + 8 * ps, (n / GM_PSTAGES) & 1, abort_flag, 5);
+                ok = mbar_wait_warp<PAIR, true>(bar_pfull + 8 * ps, (n / GM_PSTAGES) & 1, abort_flag, 5);
                 if (!ok) break;
                 const uint8_t* frags = sP + ps * T::P_BYTES + ft * frag_bytes(bits);
                 if (bits == 2) ok = dequant_slab<2, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
                 const int FB = frag_bytes(op.bits);
                 for (int s = sg.s0; s < sg.s1; ++s) {
                     const uint32_t ps = pi % GM_PSTAGES;
-                    ok = mbar_wait<PAIR>(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
+                    ok = mbar_wait<PAIR, true>(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
                     if (!ok) break;
                     mbar_expect_tx(bar_pfull + 8 * ps, (uint32_t)(sg.n_rt * FB));
                     if (sg.n_rt > 0) bulk_load(smem_u32(sP + ps * T::P_BYTES), op.frags + frag_index(s, sg.rt * GM_FRAGS + rank * T::FRAGS, op.NT) * FB, (uint32_t)(sg.n_rt * FB), bar_pfull + 8 * ps);
