@@ -88,11 +88,11 @@ inline void cut_runs(long long total, long long c1, int grid, int* bounds, int s
 }
 
 // Cost of the run [lo, hi) under the model above.
-inline long long run_cost(long long lo, long long hi, long long c1) {
+inline long long run_cost(long long lo, long long hi, long long c1, int seg_cost = GM_SEG_COST) {
     long long cost = 0;
     for (long long pos = lo; pos < hi;) {
         const long long te = (pos / c1 + 1) * c1, end = te < hi ? te : hi;
-        cost += GM_SEG_COST + (end - pos);
+        cost += seg_cost + (end - pos);
         pos = end;
     }
     return cost;

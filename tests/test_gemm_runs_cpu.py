@@ -1,6 +1,6 @@
 """Host logic of the prefill GEMM's scheduler: `csrc/aq_gemm_runs.h` (how the (row tile, token tile, half k-slab)
-work is cut into one contiguous run per CTA), compiled with the host compiler alone and driven from a small C++
-program.  Checked for many shapes: the bounds partition the work (ascending, even, first 0, last total), the run that
+work is cut into one contiguous run per CTA or pair of CTAs), compiled with the host compiler alone and driven from a
+small C++ program.  Checked for many shapes, for CTAs and for pairs: the bounds partition the work (ascending, even, first 0, last total), the run that
 holds a tile's last slab starts inside that tile or covers the tile whole (what the store-first protocol of the kernel
 relies on), and the most expensive run is never more expensive than under the equal cut it replaced."""
 import os
@@ -9,6 +9,8 @@ import subprocess
 import textwrap
 
 import pytest
+
+from gemm_rule import gemm_shape
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 HDR = os.path.join(ROOT, "paper_2605_24011_b200", "csrc")
@@ -21,18 +23,20 @@ SRC = textwrap.dedent(r"""
     using namespace aq;
     #define CHECK(c) do { if (!(c)) { std::printf("FAIL line %d: %s (n_slabs %lld R %lld M %d grid %d)\n", __LINE__, #c, n_slabs, R, M, grid); return 1; } } while (0)
 
-    // the same derivation of the tile structure as the launcher's: tiles of 256 rows x up to 128 tokens, half slabs
-    static int one(long long n_slabs, long long R, int M, int grid) {
-        const long long n_st = (M + 127) / 128, c1 = 2 * n_slabs, total = R * n_st * c1;
+    // the launcher's tiles: 256 rows x up to 128 tokens for a CTA, 256 for a pair; work in half slabs
+    static int one(long long n_slabs, long long R, int M, int grid, bool pair) {
+        const int tokens = pair ? GM_PAIR_TOKENS : GM_TOKENS, seg = pair ? GM_PAIR_SEG_COST : GM_SEG_COST;
+        if (pair) grid /= 2;
+        const long long n_st = (M + tokens - 1) / tokens, c1 = 2 * n_slabs, total = R * n_st * c1;
         if (total / 2 < grid) grid = (int)(total / 2);
         if (grid < 1) return 0;
         std::vector<int> b(grid + 1, -1);
-        cut_runs(total, c1, grid, b.data());
+        cut_runs(total, c1, grid, b.data(), seg);
         CHECK(b[0] == 0 && b[grid] == total);
         long long worst = 0;
         for (int c = 0; c < grid; ++c) {
             CHECK(b[c] <= b[c + 1] && b[c] % 2 == 0);
-            worst = std::max(worst, run_cost(b[c], b[c + 1], c1));
+            worst = std::max(worst, run_cost(b[c], b[c + 1], c1, seg));
         }
         // a run that contains a tile's last unit and does not start inside that tile covers the tile whole
         for (int c = 0; c < grid; ++c) {
@@ -46,11 +50,11 @@ SRC = textwrap.dedent(r"""
         long long worst_equal = 0;
         for (int c = 0; c < grid; ++c) {
             const long long lo = (total * c / grid) & ~1LL, hi = (c + 1 == grid) ? total : ((total * (c + 1) / grid) & ~1LL);
-            worst_equal = std::max(worst_equal, run_cost(lo, hi, c1));
+            worst_equal = std::max(worst_equal, run_cost(lo, hi, c1, seg));
         }
         CHECK(worst <= worst_equal);
         // and no run costs more than the work spread evenly plus what one tile and its pieces can add
-        CHECK(worst <= total / grid + c1 + 4 * GM_SEG_COST + 2 || worst <= worst_equal);
+        CHECK(worst <= total / grid + c1 + 4 * seg + 2 || worst <= worst_equal);
         return 0;
     }
 
@@ -63,26 +67,15 @@ SRC = textwrap.dedent(r"""
         for (int M : Ms) for (long long K : Ks) for (long long N : Ns) for (int g : grids) {
             const long long n_slabs = (K + 255) / 256 * 2, R = (N + 255) / 256;
             if (n_slabs * R * 16 > 2000000000LL) continue;
-            if (one(n_slabs, R, M, g)) return 1;
-            ++n;
+            for (bool pair : {false, true}) {
+                if (one(n_slabs, R, M, g, pair)) return 1;
+                ++n;
+            }
         }
         std::printf("OK %d\n", n);
         return 0;
     }
 """)
-
-SHAPE = textwrap.dedent(r"""
-    #include <cstdio>
-    #include "aq_gemm_runs.h"
-    int main() {
-        long long N, K; int M, sms;
-        while (std::scanf("%lld %lld %d %d", &N, &K, &M, &sms) == 4) {
-            const aq::GemmShape g = aq::gemm_shape((N + 255) / 256, (int)((K + 255) / 256), M, sms);
-            std::printf("%d %d %d %d %lld\n", g.pair, g.n_st, g.tn, g.workers, g.tiles);
-        }
-    }
-""")
-
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
 @pytest.mark.parametrize("pair,N,K,M,sms", [
@@ -94,11 +87,7 @@ SHAPE = textwrap.dedent(r"""
     (1, 4096, 11008, 4096, 148), (1, 11008, 4096, 8192, 148),
 ])
 def test_pairs_where_they_pay(tmp_path, pair, N, K, M, sms):
-    src, exe = tmp_path / "shape.cpp", tmp_path / "shape"
-    src.write_text(SHAPE)
-    subprocess.run(["g++", "-std=c++17", "-O1", "-I", HDR, str(src), "-o", str(exe)], check=True)
-    r = subprocess.run([str(exe)], input=f"{N} {K} {M} {sms}", capture_output=True, text=True, check=True)
-    got, n_st, tn, workers, tiles = map(int, r.stdout.split())
+    got, n_st, tn, workers, tiles = gemm_shape(tmp_path, N, K, M, sms)
     assert got == pair and workers == (sms // 2 if pair else sms) and tiles == n_st * -(-N // 256)
     assert tn <= (256 if pair else 128) and tn % 32 == 0 and (n_st - 1) * tn < M <= n_st * tn
 

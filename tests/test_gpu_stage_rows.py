@@ -1,5 +1,6 @@
-"""The staging kernels of the prefill path at the edges of what a thread and a CTA hold: rows of one block, rows that fill the
-registers of 256 threads (4096) and a block more, twice that and a block more, and rows that leave binary16's range."""
+"""The staging kernels of the prefill path at the edges of what a thread and a CTA hold.  For bfloat16: rows of one block, rows that
+fill the registers of 256 threads (4096) and a block more, twice that and a block more, and rows that leave binary16's range.  The
+kernel for binary16 reads four elements per thread and step at any row length; it gets the same rows."""
 import pytest
 
 from oracle import aq_oracle as O
