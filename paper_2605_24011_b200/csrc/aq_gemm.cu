@@ -166,7 +166,8 @@ __device__ __forceinline__ bool gemm_next_seg(int& pos, int hi, const GemmArgs& 
     while (sg.op + 1 < a.n_ops && r >= a.op[sg.op].R) { r -= a.op[sg.op].R; ++sg.op; }
     sg.rt = r;
     sg.w = min(a.tn, (a.M - sg.st * a.tn + (PAIR ? 31 : 15)) & ~(PAIR ? 31 : 15));
-    sg.n_rt = max(0, min(Tile<PAIR>::FRAGS, a.op[sg.op].NT - r * GM_FRAGS - rank * Tile<PAIR>::FRAGS));
+    sg.n_rt = min(Tile<PAIR>::FRAGS, a.op[sg.op].NT - r * GM_FRAGS - rank * Tile<PAIR>::FRAGS);
+    if (PAIR) sg.n_rt = max(0, sg.n_rt);
     return true;
 }
 
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
         // TMEM lanes 32 quarter .. + 31 of row half rh: fragments 8 rh + 2 quarter and the next of the tile
         const int quarter = warp & 3, rh = PAIR ? 0 : (warp >> 2) & 1, group = warp / T::DQ_GROUP, ft = 8 * rh + 2 * quarter;
         const uint32_t tmem_a = tmem_base + GM_ACOL0 + (uint32_t)(group * 2 * T::A_COLS + rh * 32) + ((uint32_t)(quarter * 32) << 16);
-        const uint32_t ae = bar_aempty + 16 * group, af = PAIR ? cluster_map(bar_afull + 16 * group, 0) : bar_afull + 16 * group;
+        const uint32_t af_pair = PAIR ? cluster_map(bar_afull + 16 * group, 0) : 0;
         uint32_t n = 0;   // slabs of the run so far
         bool ok = true;
         while (ok && gemm_next_seg<PAIR>(pos, run_hi, a, rank, sg)) {
@@ -341,6 +342,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
                 ok = mbar_wait_warp<PAIR, true>(bar_pfull + 8 * ps, (n / GM_PSTAGES) & 1, abort_flag, 5);
                 if (!ok) break;
                 const uint8_t* frags = sP + ps * T::P_BYTES + ft * frag_bytes(bits);
+                const uint32_t ae = bar_aempty + 16 * group, af = PAIR ? af_pair : bar_afull + 16 * group;
                 if (bits == 2) ok = dequant_slab<2, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
                 else if (bits == 3) ok = dequant_slab<3, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
                 else ok = dequant_slab<4, PAIR>(frags, n_have, lane, tmem_a, bar_pempty + 8 * ps, ae, af, parity, abort_flag);
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
             };
             // two register sets: the TMEM load of the next 32 columns is in flight while this one is staged
             uint32_t va[32], vb[32];
-            if (n_all > 0) tmem_ld32(column(0), va);
+            if (!PAIR || n_all > 0) tmem_ld32(column(0), va);
             for (int c = 0; c < n_all; c += 2) {
                 tmem_ld_wait();
                 if (c + 1 < n_all) tmem_ld32(column(c + 1), vb);
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) gemm_kernel(const __grid_consta
                     ok = mbar_wait<PAIR, true>(bar_pempty + 8 * ps, ((pi / GM_PSTAGES) & 1) ^ 1, abort_flag, 1);
                     if (!ok) break;
                     mbar_expect_tx(bar_pfull + 8 * ps, (uint32_t)(sg.n_rt * FB));
-                    if (sg.n_rt > 0) bulk_load(smem_u32(sP + ps * T::P_BYTES), op.frags + frag_index(s, sg.rt * GM_FRAGS + rank * T::FRAGS, op.NT) * FB, (uint32_t)(sg.n_rt * FB), bar_pfull + 8 * ps);
+                    if (!PAIR || sg.n_rt > 0) bulk_load(smem_u32(sP + ps * T::P_BYTES), op.frags + frag_index(s, sg.rt * GM_FRAGS + rank * T::FRAGS, op.NT) * FB, (uint32_t)(sg.n_rt * FB), bar_pfull + 8 * ps);
                     ++pi;
                 }
             }
