@@ -209,6 +209,10 @@ __global__ void __launch_bounds__(256) stage_kernel(const float* __restrict__ sr
 // (kept for the caller) it writes the binary16 operand x16 the GEMM reads -- exact wherever a bfloat16 value lies
 // inside binary16's range; a row with a magnitude of 2^15 or more is divided by the power of two that brings its
 // largest one below 2^15, kept in scale[m] (1 otherwise) and undone by the GEMM's epilogue.
+// STEPS: groups of eight elements a thread has in flight at a time; two (54 registers, four CTAs per SM) while that many CTAs hold all
+// rows, one (40 registers, six) for more rows.  us with two / one: 18 expert blocks at 600 tokens 1253 / 1226, at 768 1363 / 1322, at
+// 1024 1566 / 1513 (four elements at a time, 32 registers 1516); at 50 tokens 640 with two, 681 with four elements.
+template <int STEPS>
 __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __restrict__ src, const float* __restrict__ src2, int in_op,
                                                               int64_t K, __nv_bfloat16* __restrict__ x, __half* __restrict__ x16,
                                                               float* __restrict__ scale, const PresetList pre) {
@@ -249,8 +253,6 @@ __global__ void __launch_bounds__(256) stage_rows_bf16_kernel(const float* __res
         if (on) *reinterpret_cast<uint4*>(xr + 8 * (int64_t)i) = make_uint4(r[0], r[1], r[2], r[3]);
         store_operand8(hr, 8 * (int64_t)i, make_uint4(h[0], h[1], h[2], h[3]), on);
     };
-    // STEPS groups per thread at a time: their loads go out together
-    constexpr int STEPS = 2;
     if (in_op == AQ_IN_RMSNORM) {
         auto squares = [](const float4& v, float ss) { return fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, ss)))); };
         auto scaled = [](const float4& v, float f) { return make_float4(v.x * f, v.y * f, v.z * f, v.w * f); };
@@ -418,7 +420,8 @@ static cudaError_t run_stack(const aq_stack_t* p, const StackPlan& plan, const T
             pre.first = (!decode && dt == AQ_BF16) ? (unsigned)M : g;
             if (decode) stage_kernel<T><<<g, 256, 0, s>>>(buf(f.src), s2, (int)f.in_op, K, total4, stage, nullptr, pre);
             else if (dt == AQ_BF16) {
-                e = launch_pdl(stage_rows_bf16_kernel, dim3(pre.first + pre.ctas()), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K,
+                auto kern = M > 4 * sm_count() ? stage_rows_bf16_kernel<1> : stage_rows_bf16_kernel<2>;
+                e = launch_pdl(kern, dim3(pre.first + pre.ctas()), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K,
                                reinterpret_cast<__nv_bfloat16*>(stage), reinterpret_cast<__half*>(ws + plan.x16_off[i]),
                                reinterpret_cast<float*>(ws + plan.rs_off[i]), pre);
             } else e = launch_pdl(stage_kernel<T>, dim3(pre.first + pre.ctas()), dim3(256), 0, s, (const float*)buf(f.src), s2, (int)f.in_op, K, total4, stage,

@@ -11,11 +11,9 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype", ("bf16", "f16"))
-@pytest.mark.parametrize("K,I", [(32, 4128), (4128, 96), (8224, 32), (96, 8224), (4096, 2048 + 32)])
-def test_staged_rows(K, I, dtype):
+def _staged_rows(M, K, I, dtype, rows=None):
     from paper_2605_24011_b200 import aq
-    M, bits = 9, 3
+    bits = 3
     quant, handles = {}, []
     for i, (name, n, k) in enumerate((("plain", 32, K), ("gate", I, K), ("up", I, K), ("down", 32, I))):
         W = synth.weights(n, k, 61, i)
@@ -35,4 +33,17 @@ def test_staged_rows(K, I, dtype):
     out = torch.empty((M, 32), dtype=tdt, device="cuda")
     aq.aq_stack_forward(prog, x.cuda(), out, 4, M, ws)
     aq.aq_check()
-    check_program(prog, [(0, "plain"), (0, "gate"), (0, "up"), (0, "down")], ws, M, tdt, quant)
+    check_program(prog, [(0, "plain"), (0, "gate"), (0, "up"), (0, "down")], ws, M, tdt, quant, rows=rows)
+
+
+@pytest.mark.parametrize("dtype", ("bf16", "f16"))
+@pytest.mark.parametrize("K,I", [(32, 4128), (4128, 96), (8224, 32), (96, 8224), (4096, 2048 + 32)])
+def test_staged_rows(K, I, dtype):
+    _staged_rows(9, K, I, dtype)
+
+
+@pytest.mark.parametrize("K,I", [(32, 2048), (2080, 96), (4128, 2048 + 32)])   # (256 threads hold 2048)
+def test_more_rows_than_ctas_at_once(K, I):
+    """bfloat16: a thread has one group of eight elements in flight instead of two."""
+    M = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 9
+    _staged_rows(M, K, I, "bf16", rows=[0, 5, 6, M // 2, M - 10, M - 9, M - 1])
