@@ -4,13 +4,17 @@
 //
 // Bound: HBM traffic, (bits+1)/8 bytes read + sizeof(out) bytes written per
 // weight.  One warp per fragment (16 rows x 128 k): the warp reads its
-// fragment with 16-byte loads and writes row segments of 64 / 128 bytes.  A CTA
-// takes 64 rows x 256 k and the CTAs go along the rows first, so that what is
-// being written at one time is a few whole rows; stored with an evict-first hint.
-// Measured against CTAs that went down the columns: 16384 x 8192 at 3 bits into
-// binary16 63.9 -> 58.8 us (5.25 -> 5.71 TB/s), 8192 x 8192 at 4 bits into
-// float32 75.5 -> 72.2, 4096 x 4096 10.4 -> 10.3, 5000 x 1056 6.2 both; whole
-// rows of 1024 k per CTA instead 58.5, 72.5, 10.2 and 6.7.
+// fragment with 16-byte loads and writes row segments of 64 / 128 bytes, with an
+// evict-first hint.  A CTA takes 64 rows x 256 k.  CTAs go along the rows, so that
+// what is being written at one time is a few whole rows, and the slabs are counted
+// through, so that an odd number of them leaves no warp idle; float32 rows of up
+// to 3200 go down the columns, whose CTAs read what lies together.  Times of the
+// kernel, us, down the columns without the hint / along the rows / down with the
+// hint: binary16, 16384 x 8192 at 3 bits 63.2 / 56.5 (5.94 TB/s) / 63.7, 16384 x
+// 3072 24.1 / 18.5 / 19.7, 15811 x 352 at 2 bits 4.48 / 4.10 / 4.48 (with pairs of
+// slabs 4.83); float32, 16384 x 8192 142 / 136 / 142, 16384 x 4096 72.7 / 66.4 /
+// 69.2, 2603 x 3104 11.3 / 11.7 / 11.1, 4899 x 2080 at 4 bits 13.4 / 14.1 / 13.3,
+// 2220 x 1088 at 2 bits 4.8 / 6.2 / 4.8.
 #include "aq_internal.h"
 #include "aq_layout.cuh"
 
@@ -54,16 +58,17 @@ __device__ __forceinline__ void decode_unit(const SlotWords<BITS>& sw, const uin
     }
 }
 
-template <int BITS, typename T>
+// n: slabs of 128 k that exist (along the rows), groups of four row tiles (down the columns)
+template <int BITS, typename T, bool DOWN>
 __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict__ frags, int64_t N, int64_t K, int NT,
-                                                      int KP, T* __restrict__ out) {
+                                                      unsigned n, T* __restrict__ out) {
     constexpr int FB = frag_bytes(BITS);
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int warp = threadIdx.x >> 5;
-    const unsigned rt = blockIdx.x / (unsigned)KP;
-    const int64_t R = (int64_t)rt * 4 + (warp >> 1);
-    const int64_t S = (int64_t)(blockIdx.x - rt * (unsigned)KP) * 2 + (warp & 1);
-    if (R >= NT) return;
+    const unsigned at = DOWN ? blockIdx.x : 2 * blockIdx.x + (warp & 1), rest = at % n;
+    const int64_t R = (int64_t)(DOWN ? rest : at / n) * 4 + (warp >> 1);
+    const int64_t S = DOWN ? 2 * (int64_t)(at / n) + (warp & 1) : rest;
+    if (R >= NT || S * 128 >= K) return;
     const uint8_t* fb = frags + frag_index(S, R, NT) * FB;
     LaneCodes<BITS> lc;
     load_lane_codes<BITS>(lc, fb, lane);
@@ -92,15 +97,19 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
     }
 }
 
+template <int BITS, typename T, bool DOWN>
+static void launch_as(const aq_handle_s* h, void* out, cudaStream_t s) {
+    const int64_t slabs = (h->K + 127) / 128, groups = (h->NT + 3) / 4;
+    const unsigned grid = (unsigned)(DOWN ? (slabs + 1) / 2 * groups : (slabs * groups + 1) / 2);
+    dequant_kernel<BITS, T, DOWN><<<grid, 256, 0, s>>>(h->frags, h->N, h->K, h->NT, (unsigned)(DOWN ? groups : slabs), (T*)out);
+}
+
 template <int BITS>
 static cudaError_t launch_bits(const aq_handle_s* h, void* out, aq_dtype_t dt, cudaStream_t s) {
-    const unsigned grid = (unsigned)((int64_t)h->KP * ((h->NT + 3) / 4));
-    if (dt == AQ_F16)
-        dequant_kernel<BITS, __half><<<grid, 256, 0, s>>>(h->frags, h->N, h->K, h->NT, h->KP, (__half*)out);
-    else if (dt == AQ_BF16)
-        dequant_kernel<BITS, __nv_bfloat16><<<grid, 256, 0, s>>>(h->frags, h->N, h->K, h->NT, h->KP, (__nv_bfloat16*)out);
-    else
-        dequant_kernel<BITS, float><<<grid, 256, 0, s>>>(h->frags, h->N, h->K, h->NT, h->KP, (float*)out);
+    if (dt == AQ_F16) launch_as<BITS, __half, false>(h, out, s);
+    else if (dt == AQ_BF16) launch_as<BITS, __nv_bfloat16, false>(h, out, s);
+    else if (h->K > 3200) launch_as<BITS, float, false>(h, out, s);
+    else launch_as<BITS, float, true>(h, out, s);
     count_launch();
     return cudaGetLastError();
 }
