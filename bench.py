@@ -597,8 +597,8 @@ def main():
         "roofline": {"bound": "hbm", "achieved": value / world, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": (value / world) / peaks["hbm_gbs"], "traffic": DECODE_TRAFFIC_BYTES,
                      "peak_source": peaks["source"],
-                     "kernel": "decode_stack_kernel (one launch per pass; time = whole pass incl. its two glue kernels)",
-                     "traffic_note": "dram bytes of the 4-layer ncu capture scaled by packed bytes to 32 layers",
+                     "kernel": "decode_stack_kernel (one launch per pass; time = whole pass incl. the kernel that widens its input)",
+                     "traffic_note": DECODE_TRAFFIC_BYTES and "dram bytes of the 4-layer ncu capture scaled by packed bytes to 32 layers",
                      "algorithmic_bytes_per_step": packed},
     }
 
@@ -624,14 +624,13 @@ def main():
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of the decode kernel per stack pass, from the ncu capture summarised in
-# the profile of a 4-layer pass of one token: 355,696,384 + 4,406,784 bytes for the first 4 layers (354,172,928
+# the profile of a 4-layer pass of one token: 355,714,560 + 4,011,008 bytes for the first 4 layers (354,172,928
 # packed bytes), times 8 for the 32 layers (every byte is read once, so traffic grows with the packed bytes).
 # Set to None whenever the kernel changes, until the capture has been taken again.
-# (None: the kernel's last step and set-up have changed since.)
-DECODE_TRAFFIC_BYTES = None
-# gemm_kernel: 21,203,200 + 4,864 bytes of DRAM traffic for one 11008 x 4096
+DECODE_TRAFFIC_BYTES = 8 * (355_714_560 + 4_011_008)
+# gemm_kernel: 21,203,200 + 69,632 bytes of DRAM traffic for one 11008 x 4096
 # 2-bit launch (16,908,288 packed bytes), scaled by packed bytes to the 224 matrices of one pass
-PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_200 + 4_864) / 16_908_288)
+PREFILL_TRAFFIC_BYTES = round(2_833_383_424 * (21_203_200 + 69_632) / 16_908_288)
 
 
 def prefill_leg(aq, workloads, prog, out_buf, info, peaks, torch, gpu_index=0):

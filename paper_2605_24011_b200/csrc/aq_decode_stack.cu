@@ -42,11 +42,11 @@
 // warps set the pace: a team of four takes 1.7 us per unit, 0.7 to read the sums and
 // apply the block scales and 1 for 1024 red.adds, and a boundary costs about 9 us, most
 // of it the wait for the slowest CTA and the exchange of row norms.  Two teams, with A
-// kept until the sums were read and one multiply-add per value, took 2304 us for a 7B-shaped
-// pass, three teams with operand and sums released on their own 2090 (M = 4 with
-// instrumentation 447 -> 383 thousand cycles for four layers, M = 2 no difference).  Neither
+// kept until the sums were read and one multiply-add per value, took 2306 us for a 7B-shaped
+// pass, two teams with operand and sums released on their own 2278, three 2180.  Neither
 // the L2 rate of the adds (204 ns per 1024 of them with every SM adding) nor the polls
-// (pauses of 32 to 250 ns in them changed nothing) is the limit.
+// (pauses of 32 to 250 ns in them changed nothing) is the limit.  The order in which the
+// compiler lays out the roles moves these figures by up to 8 %: measure after any change.
 //
 // Every wait is bounded: when one runs out the kernel raises a status word,
 // gives copies in flight time to land and returns.

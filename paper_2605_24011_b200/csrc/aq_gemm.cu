@@ -10,12 +10,11 @@
 // two, undone in the epilogue through tok_scale).
 //
 // Bound: by its flops the tensor cores (dense contraction, 2 M flops per weight).  In
-// fact no unit is full: 11008 x 4096 at 512 tokens keeps the tensor pipe 47 % active, L2
-// at 20 % of its rate, issue slots at 38 %; the dequantise warps wait 40 % of their time for
-// instructions to release a stage, and with one instruction in eight the call still takes 37
-// of 48 us, so hand-overs, fill, epilogue and uneven runs (172 tiles on 148 SMs) share the
-// rest.  With few tokens it is the chain of latencies from launch to sums (2.7 us), epilogue
-// and adds.
+// fact no unit is full: 11008 x 4096 at 512 tokens (pairs, 86 tiles on 74 of them) keeps
+// the tensor pipe 51 % active, L2 at 21 % of its rate, issue slots at 26 % (single CTAs: 47,
+// 20 and 38 %); the start (4 us to the first instruction), drains of 128 KB per SM and
+// pieces of tiles added through L2 share the rest.  With few tokens it is the chain of
+// latencies from launch to sums (2.7 us), epilogue and adds.
 //
 // tcgen05 UMMA, 256 weight rows x up to 128 tokens per tile:
 //   A (M side, 2 x 128) = weight rows, dequantised by sixteen warps from the packed
@@ -37,8 +36,9 @@
 // Large products run on CTA pairs (tcgen05 cta_group::2, one instruction over 256 rows and up to 256 tokens; each CTA
 // dequantises its 128 rows and holds half of the tokens): half the dequantisation, half the packed bytes and half the
 // operand reads from shared memory per flop.  In an instrumented copy 64 k of a tile (512 cycles of instructions) take 595
-// cycles instead of 880, yet a pass gains 3 to 4 % only: the chip is at its power limit by then (22016 x 4096 at 512 tokens in a
-// loop: 987 W, 1.66 GHz of 1.97; cuBLAS 993 W at 1.34), so it is the energy of dequantising, moving and adding that counts.  Deeper rings (4 to 7 token slots, 4 to 7 epilogue chunks per warp) change nothing.
+// cycles instead of 880; products gain 5 to 12 %, a 7B-shaped pass of 512 tokens 3 to 4 %.  22016 x 4096 at 512 tokens: 1190
+// TFLOP/s over 50 ms, 1029 over 5 s, when the chip is at its power limit (985 W, 1.61 GHz of 1.97; cuBLAS 1593 and 1359, 1.31
+// GHz).  Deeper rings (4 to 7 token slots, 4 to 7 epilogue chunks per warp) change nothing.
 //
 // One persistent CTA, or pair, per SM (or two).  The work -- (row tile, token tile, 128-k slab)
 // triples -- is cut into contiguous runs, one per CTA, balanced for slabs plus a
@@ -789,7 +789,9 @@ bool gemm_stores_first(const aq_handle_s* const* hs, int n, int M, cudaStream_t 
     // wait 3 to 5 us for the first one's stores; from about two CTAs per tile on, zeros are cheaper.  Measured, stores first /
     // zeros: 4096 x 4096 (16 tiles) at 32 tokens 18.5 / 15.2 us, 11008 x 4096 (86 tiles) at 200 tokens 46 / 42 us, eight 7B
     // layers (48 and 86 tiles) at 50 tokens 814 / 739 us; the other way round with 104 to 148 tiles, 18 expert layers at 512
-    // tokens 1291 / 1381 us.
+    // tokens 1291 / 1381 us.  On pairs (74, so from 52 tiles on): 44 tiles (2688 x 8192 at 1024 tokens) 55.9 / 52.5 us, 48 (4096 x
+    // 4096 at 768) 37.1 / 33.7; 60 (5003 x 4000 at 768) 39.4 / 42.0, 64 (4096 x 4096 at 1024) 40.2 / 41.4, but with twice the columns
+    // 75.5 / 72.0, 86 (11008 x 4096 at 512) 52.2 / 54.6.
     const GemmShape shape = shape_of(hs, n, M);
     const long long tiles = shape.tiles;
     return tiles <= GM_MAX_TILES && 10 * tiles >= 7 * shape.workers;

@@ -55,7 +55,8 @@ inline GemmShape gemm_shape(long long R, int KP, int M, int sms) {
 // 1156, 1139, 1136, 1133 (6), 1131 (9), 1135 us (14).
 constexpr int GM_SEG_COST = 9;
 // The same for a CTA pair, whose tiles are twice as wide: of 5, 9 and 15, in us, 4096 x 4096 at 1024 tokens 41.0, 42.1, 37.7,
-// 11008 x 4096 at 512 48.9, 46.1, 46.1, 12288 x 4096 52.9, 49.9, 49.8, 22016 x 4096 79.2, 79.1, 79.2.
+// 11008 x 4096 at 512 48.9, 46.1, 46.1, 12288 x 4096 52.9, 49.9, 49.8, 22016 x 4096 79.2, 79.1, 79.2.  Over 75 products that pairs
+// take, 400 to 1024 tokens, against 15: 9 takes 1.006 of the time (geometric mean; 0.97 to 1.11), 12 1.002, 21 1.009.
 constexpr int GM_PAIR_SEG_COST = 15;
 
 // Cuts [0, total) into `grid` contiguous runs with even bounds (bounds[0] = 0 .. bounds[grid] = total).  The work is a
