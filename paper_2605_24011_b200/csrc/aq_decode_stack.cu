@@ -80,7 +80,8 @@ template <int NTEAMS> struct DsRoles {
     static constexpr int WARPS = RECORD0 + DS_RECORD_WARPS, THREADS = WARPS * 32;
     static constexpr bool SHARES = TEAMS == 3;      // registers per thread: 80 at the launch, then
     static constexpr int REGS_UNPACK = 56, REGS_COLLECT = 104, REGS_OTHER = 56;
-    static_assert(!SHARES || (DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80 && COLLECT0 % 4 == 0 && ISSUER % 4 == 0 && WARPS - ISSUER == 4), "the roles' registers fit, and no group of four has two shares");
+    static_assert(!SHARES || DS_UNPACK_WARPS * REGS_UNPACK + COLLECT_WARPS * REGS_COLLECT + 4 * REGS_OTHER <= WARPS * 80, "the roles' registers fit");
+    static_assert(!SHARES || (COLLECT0 % 4 == 0 && ISSUER % 4 == 0 && WARPS - ISSUER == 4), "no group of four has two shares");
 };
 constexpr int DS_MAX_COLLECT_WARPS = 12;
 constexpr int DS_FRAGS = 8;                 // 16-row tiles of a unit
@@ -90,7 +91,7 @@ constexpr int DS_MAX_SLOTS = 6;             // staged slabs per phase per CTA
 constexpr int DS_XS_BYTES = DS_MAX_SLOTS * dt_slab_bytes(AQ_DECODE_MAX_M);
 // A unit's operands and sums in TMEM, A of both halves and D of both halves, and what goes with it (descriptor, scales, the
 // barrier that says they are there).  One token: five stages of both, refilled once the sums have been read.  Several tokens:
-// reading the sums takes longer than anything else, so A (two stages) is refilled as soon as the instructions have read it
+// reading the sums takes longer than anything else, so A (two stages) is refilled as soon as the instructions have read it (ds_late: where that pays)
 // and D (two as well) is written again once the sums have been read (aq_decode_rings.h).
 constexpr int DS_MAX_STAGES = 5;
 template <int MT> struct DsStage {

@@ -8,7 +8,8 @@
 // evict-first hint.  A CTA takes 64 rows x 256 k.  CTAs go along the rows, so that
 // what is being written at one time is a few whole rows, and the slabs are counted
 // through, so that an odd number of them leaves no warp idle; float32 rows of up
-// to 3200 go down the columns, whose CTAs read what lies together.  Times of the
+// to 3200 go down the columns, whose CTAs read what lies together, unless there is
+// only one CTA per SM (3406 x 576 at 4 bits 4.8 us down, 4.2 along the rows).  Times of the
 // kernel, us, down the columns without the hint / along the rows / down with the
 // hint: binary16, 16384 x 8192 at 3 bits 63.2 / 56.5 (5.94 TB/s) / 63.7, 16384 x
 // 3072 24.1 / 18.5 / 19.7, 15811 x 352 at 2 bits 4.48 / 4.10 / 4.48 (with pairs of
@@ -97,9 +98,12 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint8_t* __restrict_
     }
 }
 
+static int64_t slabs_of(const aq_handle_s* h) { return (h->K + 127) / 128; }
+static int64_t groups_of(const aq_handle_s* h) { return (h->NT + 3) / 4; }
+
 template <int BITS, typename T, bool DOWN>
 static void launch_as(const aq_handle_s* h, void* out, cudaStream_t s) {
-    const int64_t slabs = (h->K + 127) / 128, groups = (h->NT + 3) / 4;
+    const int64_t slabs = slabs_of(h), groups = groups_of(h);
     const unsigned grid = (unsigned)(DOWN ? (slabs + 1) / 2 * groups : (slabs * groups + 1) / 2);
     dequant_kernel<BITS, T, DOWN><<<grid, 256, 0, s>>>(h->frags, h->N, h->K, h->NT, (unsigned)(DOWN ? groups : slabs), (T*)out);
 }
@@ -108,7 +112,7 @@ template <int BITS>
 static cudaError_t launch_bits(const aq_handle_s* h, void* out, aq_dtype_t dt, cudaStream_t s) {
     if (dt == AQ_F16) launch_as<BITS, __half, false>(h, out, s);
     else if (dt == AQ_BF16) launch_as<BITS, __nv_bfloat16, false>(h, out, s);
-    else if (h->K > 3200) launch_as<BITS, float, false>(h, out, s);
+    else if (h->K > 3200 || slabs_of(h) * groups_of(h) <= 2 * sm_count()) launch_as<BITS, float, false>(h, out, s);
     else launch_as<BITS, float, true>(h, out, s);
     count_launch();
     return cudaGetLastError();
